@@ -179,10 +179,8 @@ __device__ __forceinline__ float gelu_erfc_term(float y) {               // 2^(-
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-q));
     return e;
 }
-// The same term for two elements: the Horner steps run as packed pairs.
-__device__ __forceinline__ void gelu_erfc_term2(float y0, float y1, float& e0, float& e1) {
-    const f32x2 t = f2_pack(__saturatef(fabsf(y0) * 0.17677669529663688110f),
-                            __saturatef(fabsf(y1) * 0.17677669529663688110f));
+// The same term for two elements from their t's: the Horner steps run as packed pairs.
+__device__ __forceinline__ void gelu_erfc_poly2(f32x2 t, float& e0, float& e1) {
     f32x2 q = f2_dup(-1.00217749e-04f * 16384.0f);
     q = f2_fma(q, t, f2_dup(4.61550077e-04f * 4096.0f));
     q = f2_fma(q, t, f2_dup(2.30229650e-03f * 1024.0f));
@@ -195,6 +193,14 @@ __device__ __forceinline__ void gelu_erfc_term2(float y0, float y1, float& e0, f
     f2_unpack(q, q0, q1);
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(-q0));
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(-q1));
+}
+__device__ __forceinline__ void gelu_erfc_term2(float y0, float y1, float& e0, float& e1) {
+    gelu_erfc_poly2(f2_pack(__saturatef(fabsf(y0) * 0.17677669529663688110f),
+                            __saturatef(fabsf(y1) * 0.17677669529663688110f)), e0, e1);
+}
+// For callers that need the value at y >= 0 only: the term is 1 for y <= 0, and no absolute value is taken.
+__device__ __forceinline__ void gelu_erfc_term2_pos(float y0, float y1, float& e0, float& e1) {
+    gelu_erfc_poly2(f2_pack(__saturatef(y0 * 0.17677669529663688110f), __saturatef(y1 * 0.17677669529663688110f)), e0, e1);
 }
 // gelu_scaled(y, h) = 2*h*GELU(y); h = 0.5 gives GELU itself, h = 0.5/s_out folds the output step.
 // With w = h*y:  w*(1 + erf) = (w + |w|) - |w|*erfc, one rounding after an exact first term.

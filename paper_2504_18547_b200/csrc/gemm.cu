@@ -1119,6 +1119,11 @@ int sm_count() {
 constexpr uint32_t SMEM_TILE_BUDGET = 204u * 1024u;   // dynamic shared memory spent on operand rings
 
 }  // namespace
+}  // namespace vitint
+
+#include "gemm_direct.cu"
+
+namespace vitint {
 
 // Batched NT integer GEMM launcher shared by the linear layer, Q K^T and P V.
 int launch_gemm(const Operand& A, const Operand& B, int M, int N, int K, int n_inner, int n_outer, int b_mn_major,
@@ -1195,6 +1200,7 @@ int launch_gemm(const Operand& A, const Operand& B, int M, int N, int K, int n_i
     if (int rc = make_map(&map_a, A.data, A.row_bytes, A.rows, (uint64_t)n_inner, (uint64_t)n_outer, A.pitch,
                           A.inner_stride, A.outer_stride, P.a_direct ? (uint32_t)BK : 16u * ca, BM, P.a_direct != 0))
         return rc;
+    if (direct_eligible(P, n_inner, n_outer, b_mn_major)) return launch_gemm_direct(map_a, B.data, B.row_bytes, B.pitch, P, st);
     if (b_mn_major) {
         if (int rc = make_map(&map_b, B.data, B.row_bytes, B.rows, (uint64_t)n_inner, (uint64_t)n_outer, B.pitch,
                               B.inner_stride, B.outer_stride, 8u * cb, BK, false))

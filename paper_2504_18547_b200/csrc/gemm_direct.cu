@@ -1,0 +1,536 @@
+// a2 + a3 for operands stored one code per byte: the integer GEMM of gemm.cu with an epilogue laid out for the SM's
+// shared-memory / L1 data pipe.
+//
+// With a thread per accumulator row (gemm.cu) every store of a warp walks 32 different rows and every parameter read serves
+// two elements.  Here the epilogue reads the accumulators in the matrix-fragment layout (tcgen05.ld 16x256b: a thread holds
+// a few columns of two rows), and the rows of the weight tile are PERMUTED by the TMA copy (a five-dimensional view of the
+// weight matrix) so that the columns a thread holds are consecutive columns of the output:
+//   codes  16 consecutive columns of a 64-column block: the per-column parameters are read once for four rows, and a
+//          warp's 16-byte stores cover 64 contiguous bytes of 8 rows instead of 16 of 32;
+//   fp32   8 consecutive columns of a 32-column block: a warp's 32-byte accesses of the residual and the result cover whole
+//          128-byte lines, so nothing is staged through shared memory and the operand ring keeps the space.
+// The arithmetic per element is that of gemm.cu, bit for bit.
+//
+// Measured against gemm_i8_kernel on the same operands (us, 4-bit codes, M = 25,216): 768 -> 2304 requantized 48.3 -> 40.1,
+// 768 -> 3072 GELU 79.8 -> 72.1, 3072 -> 768 fp32 60.1 -> 55.5; at M = 197, where the tile width matters, 6.6 -> 4.5, 7.7 ->
+// 4.9 and 15.0 -> 9.3, and 768 -> 768 fp32 9.9 -> 4.3.  What bounds it: the mainloop alone (no epilogue) takes 27.5, 35.9 and
+// 36.2 us at M = 25,216, the epilogue alone 28, 63 (GELU: the fp32 pipe, 58 % busy) and 38 us (its 155 MB); the two share the
+// SM's issue slots and data pipe.
+//
+// Warps 0-15 epilogue (four per TMEM lane quarter, units of 16 rows x one column block in turn), 16 TMA, 17 MMA issue.
+#include "common.cuh"
+#include "ptx.cuh"
+#include "tile_ops.cuh"
+
+namespace vitint {
+namespace {
+
+constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
+
+constexpr int GD_EPI_WARPS = 16;                                // four per TMEM lane quarter
+constexpr int GD_SLICES = GD_EPI_WARPS / 4;
+constexpr int GD_WARP_TMA = GD_EPI_WARPS, GD_WARP_MMA = GD_EPI_WARPS + 1;
+constexpr int GD_THREADS = (GD_EPI_WARPS + 2) * 32;
+
+// Column block within which the weight rows are permuted: column 2q + 8g + e of the tensor-core block is output column
+// (B/4) q + 2g + e, e < 2, q < 4, g < B/8.
+__host__ __device__ constexpr int gd_block(int kind) { return kind == EK_DEQUANT ? 32 : 64; }
+
+// Where column c of the tile keeps its parameters in shared memory: the four threads q of a row group read float4 number k
+// of their columns at 64 consecutive bytes.
+template <int BLK>
+__device__ __forceinline__ int gd_param_slot(int c) {
+    const int w = c & (BLK - 1), q = w / (BLK / 4), i = w & (BLK / 4 - 1);
+    return (c - w) + (i >> 2) * 16 + q * 4 + (i & 3);
+}
+
+struct DirectBars {
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync;
+};
+
+// Two accumulators -> float.  SMALL: |acc| < 2^22, one integer addition each and a packed subtraction instead of the
+// conversion instruction.
+template <bool SMALL>
+__device__ __forceinline__ f32x2 acc_to_float2(uint32_t v0, uint32_t v1) {
+    if (SMALL) return f2_add(f2_pack(__uint_as_float(0x4B400000u + v0), __uint_as_float(0x4B400000u + v1)), f2_dup(-12582912.0f));
+    return f2_pack((float)(int)v0, (float)(int)v1);
+}
+
+// Sixteen byte codes -> eight bytes of 4-bit or four bytes of 2-bit codes (element order kept).
+__device__ __forceinline__ void narrow4(const uint32_t (&w)[4], uint32_t (&o)[2]) {
+    uint32_t t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t n = w[k] & 0x0F0F0F0Fu;
+        t[k] = n | (n >> 4);                                    // bytes 0 and 2 hold two codes each
+    }
+    o[0] = __byte_perm(t[0], t[1], 0x6420);
+    o[1] = __byte_perm(t[2], t[3], 0x6420);
+}
+__device__ __forceinline__ uint32_t narrow2(const uint32_t (&w)[4]) {
+    uint32_t t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t n = w[k] & 0x03030303u;
+        n |= n >> 6;                                            // bytes 0 and 2: two codes in the low four bits
+        t[k] = n | (n >> 12);                                   // byte 0: four codes
+    }
+    return __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
+}
+
+// The parameters of a thread's sixteen columns of a 64-column block.
+template <bool GELU>
+struct CodeParams {
+    float4 a[4], b[4], q[GELU ? 4 : 1];
+    __device__ __forceinline__ void load(const EpiParams& ep, int buf, int tile_col, int lane) {
+        const int o = tile_col + (lane & 3) * 4;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            a[k] = *reinterpret_cast<const float4*>(&ep.a[buf][o + 16 * k]);
+            b[k] = *reinterpret_cast<const float4*>(&ep.b[buf][o + 16 * k]);
+            if (GELU) q[k] = *reinterpret_cast<const float4*>(&ep.q[buf][o + 16 * k]);
+        }
+    }
+};
+
+// Requantizing epilogue of 16 rows x 64 columns, a thread's share two rows x 16 consecutive columns.
+template <int KIND, bool SMALL>
+__device__ __forceinline__ void direct_codes(const GemmParams& P, const uint32_t (&v)[32], const CodeParams<KIND == EK_REQUANT_GELU>& cp,
+                                             int lane, long long row0, int rows_valid, int n0) {
+    const int r = lane >> 2, q = lane & 3;
+    const f32x2 magic = f2_dup(12582912.0f), qp2 = f2_dup(P.out_qp);
+    const float qn = P.out_qn, qp = P.out_qp;
+    uint32_t w[2][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 a = cp.a[k], b = cp.b[k];
+        float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (KIND == EK_REQUANT_GELU) g4 = cp.q[k];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {                           // rows r and r + 8
+            uint32_t c[4];
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {                       // columns 4k + 2p, 4k + 2p + 1 of the thread's sixteen
+                const int i = 8 * k + 4 * p + 2 * h;
+                const f32x2 y = f2_fma(acc_to_float2<SMALL>(v[i], v[i + 1]), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
+                                       p ? f2_pack(b.z, b.w) : f2_pack(b.x, b.y));
+                float y0, y1, c0, c1;
+                f2_unpack(y, y0, y1);
+                if (KIND == EK_REQUANT_GELU) {
+                    // unsigned codes: the value arrives clamped to [0, 1] in units of Qp, and a negative y is code 0 whatever
+                    // its GELU: t = 0 there, the term is 1 and 2w - w = w < 0 saturates to 0
+                    float e0, e1, w0, w1, d0, d1;
+                    gelu_erfc_term2_pos(y0, y1, e0, e1);
+                    const f32x2 wq = f2_mul(y, p ? f2_pack(g4.z, g4.w) : f2_pack(g4.x, g4.y));
+                    f2_unpack(wq, w0, w1);
+                    f2_unpack(f2_add(wq, wq), d0, d1);
+                    const float u0 = __saturatef(fmaf(-w0, e0, d0)), u1 = __saturatef(fmaf(-w1, e1, d1));
+                    f2_unpack(f2_fma(f2_pack(u0, u1), qp2, magic), c0, c1);
+                } else {
+                    f2_unpack(f2_add(f2_pack(fminf(fmaxf(y0, qn), qp), fminf(fmaxf(y1, qn), qp)), magic), c0, c1);
+                }
+                c[2 * p] = __float_as_uint(c0);                 // the code in two's complement is the low byte
+                c[2 * p + 1] = __float_as_uint(c1);
+            }
+            w[h][k] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+        }
+    }
+    const int col = n0 + 16 * q;
+    uint8_t* const o = (uint8_t*)P.out + (row0 + r) * P.ld_out + ((col * P.out_c) >> 3);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (r + 8 * h < rows_valid) {
+            uint8_t* const oh = o + (h ? 8 * P.ld_out : 0);
+            if (P.out_c == 8) {
+                *reinterpret_cast<uint4*>(oh) = make_uint4(w[h][0], w[h][1], w[h][2], w[h][3]);
+            } else if (P.out_c == 4) {
+                uint32_t t[2];
+                narrow4(w[h], t);
+                *reinterpret_cast<uint2*>(oh) = make_uint2(t[0], t[1]);
+            } else {
+                *reinterpret_cast<uint32_t*>(oh) = narrow2(w[h]);
+            }
+            // row padding behind the last column of the matrix
+            if (n0 + 64 >= P.N && q == 3)
+                for (long long off = ((long long)P.N * P.out_c) >> 3; off + 4 <= P.ld_out; off += 4)
+                    *reinterpret_cast<uint32_t*>((uint8_t*)P.out + (row0 + r + 8 * h) * P.ld_out + off) = 0u;
+        }
+    }
+}
+
+// Residual of 16 rows x 32 columns: rows r and r + 8, eight consecutive columns.
+__device__ __forceinline__ void direct_residual(const GemmParams& P, int lane, long long row0, int rows_valid, int n0,
+                                                float (&res)[2][8]) {
+    const int r = lane >> 2, q = lane & 3;
+    const float* const p = P.residual + (row0 + r) * P.ld_res + n0 + 8 * q;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (r + 8 * h < rows_valid) ptx::ld_global_32B(p + (h ? 8 * P.ld_res : 0), res[h]);
+}
+
+// fp32 epilogue of 16 rows x 32 columns.
+template <bool SMALL, bool RES>
+__device__ __forceinline__ void direct_f32(const GemmParams& P, const uint32_t (&v)[16], const EpiParams& ep, int buf, int tile_col,
+                                           int lane, long long row0, int rows_valid, int n0, const float (&res)[2][8]) {
+    const int r = lane >> 2, q = lane & 3;
+    float* const o = (float*)P.out + (row0 + r) * P.ld_out + n0 + 8 * q;
+    float out[2][8];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float4 a = *reinterpret_cast<const float4*>(&ep.a[buf][tile_col + 16 * k + 4 * q]);
+        const float4 b = *reinterpret_cast<const float4*>(&ep.b[buf][tile_col + 16 * k + 4 * q]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const int i = 8 * k + 4 * p + 2 * h, j = 4 * k + 2 * p;
+                f32x2 y = f2_fma(acc_to_float2<SMALL>(v[i], v[i + 1]), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
+                                 p ? f2_pack(b.z, b.w) : f2_pack(b.x, b.y));
+                if (RES) y = f2_add(y, f2_pack(res[h][j], res[h][j + 1]));
+                f2_unpack(y, out[h][j], out[h][j + 1]);
+            }
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (r + 8 * h < rows_valid) ptx::st_global_32B(o + (h ? 8 * P.ld_out : 0), out[h]);
+}
+
+template <int KIND, bool SMALL, bool RES>
+__global__ void __launch_bounds__(GD_THREADS, 1)
+gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                   const __grid_constant__ GemmParams P) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ DirectBars bars;
+    __shared__ __align__(16) EpiParams epi_params;
+    __shared__ uint32_t tmem_base_slot;
+    __shared__ int abort_flag;
+    constexpr int BLK = gd_block(KIND);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
+    const uint32_t stage_bytes = P.ia_bytes + P.ib_bytes;
+    volatile int* abort_ptr = &abort_flag;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        for (int s = 0; s < MAX_STAGES; ++s) {
+            ptx::mbar_init(ptx::smem_addr(&bars.full[s]), 1);
+            ptx::mbar_init(ptx::smem_addr(&bars.empty[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            ptx::mbar_init(ptx::smem_addr(&bars.acc_full[b]), 1);
+            ptx::mbar_init(ptx::smem_addr(&bars.acc_empty[b]), GD_EPI_WARPS);
+        }
+        ptx::mbar_init(ptx::smem_addr(&bars.epi_sync), GD_EPI_WARPS);
+        ptx::fence_mbar_init();
+        ptx::fence_proxy_async_smem();
+    }
+    if (warp == GD_WARP_MMA) {
+        ptx::tmem_alloc(ptx::smem_addr(&tmem_base_slot), P.tmem_cols);
+        ptx::tmem_relinquish();
+    }
+    if (warp == GD_WARP_TMA && lane == 0) {
+        ptx::prefetch_tensormap(&map_a);
+        ptx::prefetch_tensormap(&map_b);
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t acc_stride = P.tmem_cols >> 1;
+    grid_dependency_wait();        // operands, parameters and the residual may come from the previous kernel
+    grid_dependency_launch();
+
+    if (warp == GD_WARP_TMA) {
+        if (lane == 0) {
+            VT_TRACER(tr, 0);
+            VT_STAMP(tr, TT_START);
+            const uint32_t full0 = ptx::smem_addr(&bars.full[0]), empty0 = ptx::smem_addr(&bars.empty[0]);
+            const int k_blocks = P.k_blocks, ns = P.ns_i;
+            int s = 0, it = 0;
+            uint32_t ph = 1u, dst = smem_base;
+            bool ok = true;
+            for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x) {
+                const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
+                const int m0 = m_tile * BM, blk0 = n_tile * P.bn / BLK;
+                for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+                    VT_STAMP(tr, TT_WAIT_EMPTY);
+                    if (!mbar_wait(empty0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
+                    VT_STAMP(tr, TT_GOT_EMPTY);
+                    const uint32_t full = full0 + 8u * (uint32_t)s;
+                    ptx::mbar_arrive_expect_tx(full, stage_bytes);
+                    ptx::tma_load_4d(dst, &map_a, full, kb * BK, m0, 0, 0);
+                    ptx::tma_load_5d(dst + P.ia_bytes, &map_b, full, kb * BK, 0, 0, 0, blk0);
+                    if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_bytes;
+                }
+            }
+            if (!ok) {
+                // give the copies still in flight a bounded chance to land before the CTA exits
+                for (int j = (it > ns ? it - ns : 0); j < it; ++j) {
+                    const uint32_t bar = full0 + 8u * (uint32_t)(j % ns);
+                    for (int spin = 0; spin < (1 << 20) && !ptx::mbar_try_wait(bar, (uint32_t)(j / ns) & 1u); ++spin) {}
+                }
+            }
+        }
+    } else if (warp == GD_WARP_MMA) {
+        if (lane == 0) {
+            const uint32_t idesc = ptx::idesc_i8(BM, P.bn, P.a_signed, P.b_signed, 0);
+            VT_TRACER(tr, 1);
+            VT_STAMP(tr, TT_START);
+            const uint64_t a_desc0 = ptx::smem_desc(smem_base, 16, 1024, ptx::SWIZZLE_128B);
+            const uint64_t b_desc0 = ptx::smem_desc(smem_base + P.ia_bytes, 16, 1024, ptx::SWIZZLE_128B);
+            const uint64_t stage_step = (uint64_t)(stage_bytes >> 4);        // descriptor address field counts 16-byte units
+            const uint32_t full0 = ptx::smem_addr(&bars.full[0]), empty0 = ptx::smem_addr(&bars.empty[0]);
+            const int k_blocks = P.k_blocks, ns = P.ns_i;
+            const int last_steps = (P.K - (k_blocks - 1) * BK + 31) / 32;    // MMAs of the last (possibly partial) K block
+            int s = 0, tl = 0;
+            uint32_t ph = 0;
+            uint64_t a_desc = a_desc0, b_desc = b_desc0;
+            bool ok = true;
+            for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x, ++tl) {
+                const int buf = tl & 1;
+                const uint32_t acc_ph = (uint32_t)(tl >> 1) & 1u;
+                VT_STAMP(tr, TT_WAIT_EMPTY);
+                if (!mbar_wait(ptx::smem_addr(&bars.acc_empty[buf]), acc_ph ^ 1u, abort_ptr)) { ok = false; break; }
+                VT_STAMP(tr, TT_GOT_EMPTY);
+                ptx::tc_fence_after();
+                const uint32_t d_tmem = tmem_base + (uint32_t)buf * acc_stride;
+                for (int kb = 0; kb < k_blocks; ++kb) {
+                    VT_STAMP(tr, TT_WAIT_FULL);
+                    if (!mbar_wait(full0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
+                    VT_STAMP(tr, TT_GOT_FULL);
+                    ptx::tc_fence_after();
+                    if (kb + 1 < k_blocks || last_steps == 4) {              // 32 int8 of K per MMA: 32 bytes along a swizzled row
+                        ptx::mma_i8(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u);
+                        ptx::mma_i8(d_tmem, a_desc + 2u, b_desc + 2u, idesc, 1u);
+                        ptx::mma_i8(d_tmem, a_desc + 4u, b_desc + 4u, idesc, 1u);
+                        ptx::mma_i8(d_tmem, a_desc + 6u, b_desc + 6u, idesc, 1u);
+                    } else {
+                        for (int k = 0; k < last_steps; ++k)
+                            ptx::mma_i8(d_tmem, a_desc + (uint64_t)(k * 2), b_desc + (uint64_t)(k * 2), idesc, (kb | k) != 0 ? 1u : 0u);
+                    }
+                    ptx::mma_commit(empty0 + 8u * (uint32_t)s);
+                    if (++s == ns) { s = 0; ph ^= 1u; a_desc = a_desc0; b_desc = b_desc0; }
+                    else { a_desc += stage_step; b_desc += stage_step; }
+                }
+                if (ok) ptx::mma_commit(ptx::smem_addr(&bars.acc_full[buf]));
+                VT_STAMP(tr, TT_ISSUED);
+            }
+        }
+    } else {
+        const int q4 = warp & 3, slice = warp >> 2;
+        const int tid_e = threadIdx.x;
+        // per-column parameters of a tile (multiplier, bias, GELU output factor), column c of the tile
+        auto fetch_params = [&](int tile, int c, float& a, float& b, float& q) {
+            const int n = (tile % P.n_tiles) * P.bn + c;
+            a = 0.0f; b = 0.0f; q = 0.0f;
+            if (n < P.N) {
+                if (KIND == EK_REQUANT) {
+                    a = __ldg(P.col_a + n);
+                } else {
+                    a = P.col_a ? __fmul_rn(P.x_step, __ldg(P.col_a + n)) : P.x_step;
+                    if (KIND == EK_REQUANT_GELU) q = __fdiv_rn(0.5f * __ldg(P.inv_s + n), P.out_qp);   // folds GELU's 1/2 and 1/Qp
+                }
+                b = P.col_b ? __ldg(P.col_b + n) : 0.0f;
+            }
+        };
+        // The parameters of tile i+1 are fetched while the warps wait for tile i's accumulators and are stored to the other
+        // half of epi_params before tile i is processed, so no tile waits for them.  (bn <= 256 <= epilogue threads)
+        const bool my_col = tid_e < P.bn;
+        const int my_slot = gd_param_slot<BLK>(tid_e);
+        auto put_params = [&](int buf, float a, float b, float q) {
+            epi_params.a[buf][my_slot] = a;
+            epi_params.b[buf][my_slot] = b;
+            if (KIND == EK_REQUANT_GELU) epi_params.q[buf][my_slot] = q;
+        };
+        if (my_col && (int)blockIdx.x < P.total_tiles) {
+            float a, b, q;
+            fetch_params(blockIdx.x, tid_e, a, b, q);
+            put_params(0, a, b, q);
+        }
+        int tl = 0;
+        bool ok = true;
+        VT_TRACER(tr, (lane == 0 && warp == 0) ? 2 : ((lane == 0 && warp == GD_EPI_WARPS - 1) ? 3 : -1));
+        VT_STAMP(tr, TT_START);
+        float res[2][2][8];                                                   // fp32 kinds: the next block's residual, per half
+        auto request_residual = [&](int tile, int blk, int half) {
+            const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
+            const int n0 = n_tile * P.bn + blk * BLK, row0 = m_tile * BM + q4 * 32 + 16 * half;
+            if (tile < P.total_tiles && blk * BLK < P.bn && n0 < P.N) direct_residual(P, lane, row0, P.M - row0, n0, res[half]);
+        };
+        if (KIND == EK_DEQUANT && RES) {
+            request_residual(blockIdx.x, slice, 0);
+            request_residual(blockIdx.x, slice, 1);
+        }
+        for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x, ++tl) {
+            const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
+            const int buf = tl & 1;
+            const int next_tile = tile + (int)gridDim.x;
+            const bool fetch_next = my_col && next_tile < P.total_tiles;
+            float na = 0.0f, nb = 0.0f, nq = 0.0f;
+            if (fetch_next) fetch_params(next_tile, tid_e, na, nb, nq);
+            const int row_q = m_tile * BM + q4 * 32, col_t = n_tile * P.bn;
+            const int rows_q = P.M - row_q;                                   // valid rows from the quarter's first one on
+            const uint32_t acc_ph = (uint32_t)(tl >> 1) & 1u;
+            VT_STAMP(tr, TT_WAIT_ACC);
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&bars.epi_sync));
+            bool w = mbar_wait(ptx::smem_addr(&bars.epi_sync), (uint32_t)tl & 1u, abort_ptr);
+            VT_STAMP(tr, TT_WAIT_FULL);
+            w = w && mbar_wait(ptx::smem_addr(&bars.acc_full[buf]), acc_ph, abort_ptr);
+            VT_STAMP(tr, TT_GOT_ACC);
+            if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+            ptx::tc_fence_after();
+            if (fetch_next) put_params(buf ^ 1, na, nb, nq);                  // every warp has passed the barrier: none reads that half
+            const uint32_t t_quarter = tmem_base + (uint32_t)buf * acc_stride + ((uint32_t)(q4 * 32) << 16);
+            const int cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;         // whole blocks
+            const int n_blk = cols / BLK;
+            if constexpr (KIND == EK_DEQUANT) {
+#pragma unroll 1
+                for (int blk = slice; blk < n_blk; blk += GD_SLICES) {
+                    const int n0 = col_t + blk * BLK;
+                    const bool more = blk + GD_SLICES < n_blk;
+#pragma unroll
+                    for (int half = 0; half < 2; ++half) {
+                        uint32_t v[16];
+                        ptx::tmem_ld_frag32(t_quarter + ((uint32_t)half << 20) + (uint32_t)(blk * BLK), v);
+                        ptx::tmem_ld_wait();
+                        direct_f32<SMALL, RES>(P, v, epi_params, buf, blk * BLK, lane, row_q + 16 * half, rows_q - 16 * half, n0, res[half]);
+                        // the warp's next block (of this tile or the next) is on its way from here on
+                        if (RES) request_residual(more ? tile : next_tile, more ? blk + GD_SLICES : slice, half);
+                    }
+                }
+                if (RES && slice >= n_blk) {                                  // no block of this tile was this warp's
+                    request_residual(next_tile, slice, 0);
+                    request_residual(next_tile, slice, 1);
+                }
+            } else {
+                // One 16-row half of a block at a time: 90 registers, so that sixteen warps fit.  (Eight warps that keep the
+                // parameters of a block for both halves and read the next accumulators ahead: fc1 79 us against 72.)
+#pragma unroll 1
+                for (int u = slice; u < 2 * n_blk; u += GD_SLICES) {
+                    const int half = u & 1, tile_col = (u >> 1) * BLK;
+                    uint32_t v[32];
+                    ptx::tmem_ld_frag64(t_quarter + ((uint32_t)half << 20) + (uint32_t)tile_col, v);
+                    CodeParams<KIND == EK_REQUANT_GELU> cp;
+                    cp.load(epi_params, buf, tile_col, lane);
+                    ptx::tmem_ld_wait();
+                    direct_codes<KIND, SMALL>(P, v, cp, lane, row_q + 16 * half, rows_q - 16 * half, col_t + tile_col);
+                }
+            }
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&bars.acc_empty[buf]));
+            VT_STAMP(tr, TT_TILE_DONE);
+        }
+        VT_STAMP(tr, TT_END);
+    }
+
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (warp == GD_WARP_MMA) {
+        ptx::tc_fence_after();
+        __syncwarp();
+        ptx::tmem_dealloc(tmem_base, P.tmem_cols);
+    }
+}
+
+// The weight matrix as the five-dimensional view whose tile copy lands permuted within blocks of `block` rows:
+// (byte, e, q, g, block) with row = block * B + (B/4) q + 2g + e.
+int make_map_permuted(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, uint64_t pitch, int block, int bn) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return VITINT_ERR_CUDA;
+    const cuuint64_t g = (cuuint64_t)block / 8;
+    cuuint64_t dims[5] = {row_bytes, 2, 4, g, rows / (uint64_t)block};
+    cuuint64_t strides[4] = {pitch, pitch * (uint64_t)(block / 4), pitch * 2, pitch * (uint64_t)block};
+    cuuint32_t box[5] = {(cuuint32_t)BK, 2, 4, (cuuint32_t)g, (cuuint32_t)(bn / block)};
+    cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void*>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? VITINT_OK : VITINT_ERR_CUDA;
+}
+
+// Which calls this kernel takes: both operands one code per byte, whole column blocks, no batch of problems, and for fp32
+// outputs 32-byte aligned rows of the output and the residual.  Everything else stays with gemm_i8_kernel.
+bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_major) {
+    if (!P.a_direct || !P.b_direct || n_inner != 1 || n_outer != 1 || b_mn_major) return false;
+    if (P.kind == EK_REQUANT || (P.kind == EK_REQUANT_GELU && P.unit_out)) return P.N % 64 == 0;
+    if (P.kind != EK_DEQUANT || P.N % 32 != 0) return false;
+    // A short contraction whose residual and output exceed L2 is bound by HBM, and gemm_i8_kernel's asynchronous copies of the
+    // residual through shared memory keep more of it in flight (K = 768, N = 768: 27.8 against 30.1 us at M = 18,912, 35.7
+    // against 39.2 at 25,216; below, 24.1 against 19.2 at 12,608).
+    if (P.residual && P.K <= 1024 && (long long)P.M * P.N * 8 > 100ll * 1000 * 1000) return false;
+    auto rows32 = [](const void* p, long long ld) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0 && ld % 8 == 0; };
+    return rows32(P.out, P.ld_out) && (!P.residual || rows32(P.residual, P.ld_res));
+}
+
+// Tile width: the multiple of the column block with the least estimated time
+//     fill (K blocks x 0.27 us) + (waves - 1) x max(K blocks x 0.32 us, epilogue) + epilogue
+// where the epilogue takes 0.2 us and 9.8 (requantize), 14.8 (GELU) or 12.9 ns (fp32) a column, as measured at M = 197 ..
+// 25,344 and widths 32 .. 256: a K block costs the same at every width (four MMAs of one issuing thread), so a grid that
+// does not fill the chip takes narrow tiles (197 x 768 x 768 fp32: 7.3 us at 256 columns, 4.4 at 32) and a full one the
+// widest that does not add a wave.
+int direct_tile_columns(const GemmParams& P) {
+    const int block = gd_block(P.kind), sms = sm_count();
+    const float per_col = P.kind == EK_REQUANT ? 0.0098f : P.kind == EK_DEQUANT ? 0.0129f : 0.0148f;
+    const float k_fill = 0.27f * (float)P.k_blocks, k_main = 0.32f * (float)P.k_blocks;
+    int best = 0;
+    float best_t = 0.0f;
+    for (int bn = MAX_BN; bn >= block; bn -= block) {
+        if (bn > P.N && bn - block >= P.N) continue;
+        const long long tiles = (long long)P.m_tiles * ((P.N + bn - 1) / bn);
+        const float waves = (float)((tiles + sms - 1) / sms), epi = 0.2f + per_col * (float)bn;
+        const float t = k_fill + (waves - 1.0f) * (k_main > epi ? k_main : epi) + epi;
+        if (!best || t < best_t) { best = bn; best_t = t; }
+    }
+    return best;
+}
+
+int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_bytes, uint64_t w_pitch, GemmParams P,
+                       cudaStream_t st) {
+    const int block = gd_block(P.kind);
+    P.bn = direct_tile_columns(P);
+    P.n_tiles = (P.N + P.bn - 1) / P.bn;
+    const long long tiles = (long long)P.m_tiles * P.n_tiles;
+    if (tiles > 0x7fffffffll) return VITINT_ERR_UNSUPPORTED;
+    P.total_tiles = (int)tiles;
+    P.ib_bytes = (uint32_t)P.bn * BK;
+    const uint32_t stage = P.ia_bytes + P.ib_bytes;
+    int ns = (int)(GD_RING_BYTES / stage);
+    P.ns_i = ns > MAX_STAGES ? MAX_STAGES : ns;
+    uint32_t cols = 32;
+    while (cols < 2u * (uint32_t)P.bn) cols <<= 1;
+    P.tmem_cols = cols;
+    CUtensorMap map_b;
+    if (int rc = make_map_permuted(&map_b, w, w_row_bytes, (uint64_t)P.N, w_pitch, block, P.bn)) return rc;
+    size_t smem = (size_t)P.ns_i * stage + 1024;
+    if (smem < 120 * 1024) smem = 120 * 1024;                  // two CTAs never share an SM (and its tensor memory)
+    int grid = sm_count();
+    if (grid > P.total_tiles) grid = P.total_tiles;
+#ifdef VITINT_TRACE
+    if (g_trace_max_ctas > 0 && grid > g_trace_max_ctas) grid = g_trace_max_ctas;
+#endif
+    const int dev = current_device();
+    if (dev < 0) return VITINT_ERR_CUDA;
+    static bool attr_set[MAX_DEVICES][8] = {};
+    auto launch = [&](auto kernel, int slot) -> int {
+        if (!attr_set[dev][slot]) {
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GD_RING_BYTES + 1024) != cudaSuccess)
+                return VITINT_ERR_CUDA;
+            attr_set[dev][slot] = true;
+        }
+        launch_kernel(kernel, dim3(grid), dim3(GD_THREADS), smem, st, map_a, map_b, P);
+        return cuda_status(cudaGetLastError());
+    };
+    const bool small = P.small_acc == 2;
+    if (P.kind == EK_DEQUANT) {
+        if (P.residual) return small ? launch(gemm_direct_kernel<EK_DEQUANT, true, true>, 0) : launch(gemm_direct_kernel<EK_DEQUANT, false, true>, 1);
+        return small ? launch(gemm_direct_kernel<EK_DEQUANT, true, false>, 2) : launch(gemm_direct_kernel<EK_DEQUANT, false, false>, 3);
+    }
+    if (P.kind == EK_REQUANT) return small ? launch(gemm_direct_kernel<EK_REQUANT, true, false>, 4) : launch(gemm_direct_kernel<EK_REQUANT, false, false>, 5);
+    return small ? launch(gemm_direct_kernel<EK_REQUANT_GELU, true, false>, 6) : launch(gemm_direct_kernel<EK_REQUANT_GELU, false, false>, 7);
+}
+
+}  // namespace
+}  // namespace vitint
