@@ -374,6 +374,61 @@ int vitint_layernorm_compare_quantize(const float* x, int64_t rows, int64_t cols
                                       const uint8_t* flip, float n_eps, const vitint_codes* out, float* stats,
                                       void* stream);
 
+/* A stack of integerized encoder layers run by one call: per layer
+ *   LayerNorm + quantize -> QKV linear -> attention core -> projection + residual
+ *   -> LayerNorm + quantize -> fc1 (GELU, requantized) -> fc2 + residual,
+ * each stage exactly the entry point of this header that the fields name (the attention core is one fused launch, or
+ * vitint_qk -> softmax -> vitint_pv where `attention` says so).  Layer i > 0 reads what layer i - 1 wrote: layer i writes
+ * buf[i & 1], the last one `out`.
+ *   vitint_encoder_forward          enqueues the launches one by one.
+ *   vitint_encoder_plan_create      records the same launches once as a CUDA graph (and enqueues, on `stream`, the kernels
+ *                                   that fill the tables of the Eq. 4 and bounded softmax where a layer uses them).
+ *   vitint_encoder_plan_run         runs the recorded launches with this call's x and out: one graph launch instead of
+ *                                   seven or more launches per layer.  On a stream that is being captured the launches are
+ *                                   enqueued one by one.  Safe to call from several threads; calls that overlap on the GPU
+ *                                   share the layers' buffers and must be ordered by the caller.
+ * The descriptors' device memory (weights, parameters, buffers) is the caller's and must outlive the plan; a plan belongs to
+ * the device that was current when it was created.  Errors: those of the stages, INVALID_ARG, CUDA. */
+typedef enum {
+    VITINT_ATTN_EXP_CORE = 0,        /* vitint_attention_core_prepared, `table` filled by vitint_attention_exp_table */
+    VITINT_ATTN_SHIFT_CORE = 1,      /* vitint_attention_core_shift */
+    VITINT_ATTN_EXP = 2,             /* vitint_qk -> vitint_softmax_quantize -> vitint_pv */
+    VITINT_ATTN_EXP_BOUNDED = 3,     /* vitint_qk -> vitint_softmax_quantize_bounded -> vitint_pv */
+    VITINT_ATTN_SHIFT = 4            /* vitint_qk -> vitint_softmax_shift_quantize -> vitint_pv */
+} vitint_attention_kind;
+
+typedef struct {
+    int32_t batch, tokens, heads, bits;
+    int32_t attention;               /* vitint_attention_kind */
+    int32_t compare_layernorm;       /* 0: vitint_layernorm_quantize, 1: vitint_layernorm_compare_quantize */
+    int32_t score_bound;             /* ATTN_EXP_BOUNDED */
+    int32_t reserved_;
+    float eps, n_eps, ln_step, q_step, k_step, v_step, p_step, o_step, g_step;
+    float c;                         /* softmax scale: c (ATTN_EXP, ATTN_EXP_BOUNDED) or c2 (ATTN_SHIFT) */
+    const float *ln1_gamma, *ln1_beta, *ln2_gamma, *ln2_beta;      /* compare_layernorm == 0 */
+    const float *ln1_refs, *ln2_refs;                              /* compare_layernorm == 1 */
+    const uint8_t *ln1_flip, *ln2_flip;
+    float* ln_stats;
+    vitint_codes w_qkv, w_proj, w_fc1, w_fc2;
+    const float *alpha_qkv, *beta_qkv, *alpha_o;
+    const float *proj_step, *proj_bias, *fc1_step, *fc1_bias, *fc2_step, *fc2_bias, *inv_g_step;
+    vitint_codes x1, qkv, p, o, x2, g;                             /* activation codes; p: unfused attention only */
+    int32_t* scores;                                               /* unfused attention only */
+    int64_t ld_scores;
+    float* h;                                                      /* fp32 [batch*tokens, dim] between the two halves */
+    void* table;
+    size_t table_bytes;
+} vitint_encoder_layer_desc;
+
+typedef struct vitint_encoder_plan vitint_encoder_plan;
+
+int vitint_encoder_forward(const vitint_encoder_layer_desc* layers, int32_t n_layers, float* const buf[2], const float* x,
+                           float* out, void* stream);
+int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layers, int32_t n_layers, float* const buf[2], void* stream,
+                               vitint_encoder_plan** plan);
+int vitint_encoder_plan_run(vitint_encoder_plan* plan, const float* x, float* out, void* stream);
+void vitint_encoder_plan_destroy(vitint_encoder_plan* plan);
+
 /* Host-side helpers (no device work, HOST pointers): the constants that the method absorbs into the stage behind a
  * contraction, computed in fp64 and rounded once to fp32.
  *   vitint_fold_requant (Eq. 2, "equivalent bias" and "post-scaling factor" followed by a quantizer of step

@@ -37,6 +37,21 @@ class _Slabs(Structure):
                 ("head_stride_bytes", c_int64), ("bits", c_int32), ("is_signed", c_int32)]
 
 
+class _EncoderLayerDesc(Structure):
+    _fields_ = ([(n, c_int32) for n in ("batch", "tokens", "heads", "bits", "attention", "compare_layernorm", "score_bound", "reserved_")]
+                + [(n, c_float) for n in ("eps", "n_eps", "ln_step", "q_step", "k_step", "v_step", "p_step", "o_step", "g_step", "c")]
+                + [(n, c_void_p) for n in ("ln1_gamma", "ln1_beta", "ln2_gamma", "ln2_beta", "ln1_refs", "ln2_refs", "ln1_flip",
+                                           "ln2_flip", "ln_stats")]
+                + [(n, _Codes) for n in ("w_qkv", "w_proj", "w_fc1", "w_fc2")]
+                + [(n, c_void_p) for n in ("alpha_qkv", "beta_qkv", "alpha_o", "proj_step", "proj_bias", "fc1_step", "fc1_bias",
+                                           "fc2_step", "fc2_bias", "inv_g_step")]
+                + [(n, _Codes) for n in ("x1", "qkv", "p", "o", "x2", "g")]
+                + [("scores", c_void_p), ("ld_scores", c_int64), ("h", c_void_p), ("table", c_void_p), ("table_bytes", c_size_t)])
+
+
+ATTN_EXP_CORE, ATTN_SHIFT_CORE, ATTN_EXP, ATTN_EXP_BOUNDED, ATTN_SHIFT = range(5)
+
+
 class _AttentionDesc(Structure):
     _fields_ = [("batch", c_int32), ("tokens", c_int32), ("heads", c_int32), ("bits", c_int32),
                 ("w_qkv", _Codes), ("alpha_qkv", c_void_p), ("beta_qkv", c_void_p),
@@ -93,6 +108,12 @@ def lib():
         L.vitint_attention_block.argtypes = [POINTER(_Codes), POINTER(_AttentionDesc), c_void_p, c_int64,
                                              POINTER(_Codes), POINTER(_Codes), POINTER(_Codes), c_void_p, c_size_t,
                                              c_void_p]
+        bufs = POINTER(c_void_p)
+        L.vitint_encoder_forward.argtypes = [POINTER(_EncoderLayerDesc), c_int32, bufs, c_void_p, c_void_p, c_void_p]
+        L.vitint_encoder_plan_create.argtypes = [POINTER(_EncoderLayerDesc), c_int32, bufs, c_void_p, POINTER(c_void_p)]
+        L.vitint_encoder_plan_run.argtypes = [c_void_p, c_void_p, c_void_p, c_void_p]
+        L.vitint_encoder_plan_destroy.argtypes = [c_void_p]
+        L.vitint_encoder_plan_destroy.restype = None
         L.vitint_layernorm_compare_quantize.argtypes = [c_void_p, c_int64, c_int64, c_int64, c_void_p, c_void_p, c_float,
                                                         POINTER(_Codes), c_void_p, c_void_p]
         L.vitint_linear_e2m1.argtypes = [POINTER(_Codes), POINTER(_Codes), c_void_p, c_int64, c_void_p, c_void_p]
@@ -139,8 +160,22 @@ def _check(code: int, where: str):
         raise VitintError(code, where)
 
 
+_raw_stream = None
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    """The current stream's handle.  torch.cuda.current_stream() builds a Stream object (3.2 us a call); once it has
+    initialised CUDA the handle itself is asked for (0.2 us)."""
+    global _raw_stream
+    if _raw_stream is None:
+        handle = torch.cuda.current_stream().cuda_stream
+        get, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if get is not None and device is not None:
+            _raw_stream = lambda: get(device())
+        else:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        return handle
+    return _raw_stream()
 
 
 def _ptr(t):
@@ -474,6 +509,30 @@ def vitint_attention_core_noalloc(qkv: Codes, batch: int, heads: int, tokens: in
                                                float(p_step), p_bits, _ptr(alpha_o), _ptr(beta_o), byref(do),
                                                _stream()), "vitint_attention_core_noalloc")
     return out
+
+
+class EncoderPlan:
+    """The launches of a stack of encoder layers recorded as a CUDA graph (vitint_encoder_plan_*).  descs: one
+    _EncoderLayerDesc per layer; bufs: the two fp32 buffers between the layers (None for a single layer).  The memory the
+    descriptors name belongs to the caller and must outlive the plan."""
+
+    def __init__(self, descs: list, bufs=None):
+        arr = (_EncoderLayerDesc * len(descs))(*descs)
+        ptrs = None if bufs is None else (c_void_p * 2)(*[b.data_ptr() for b in bufs])
+        handle = c_void_p()
+        _check(lib().vitint_encoder_plan_create(arr, len(descs), ptrs, _stream(), byref(handle)), "vitint_encoder_plan_create")
+        self._handle = handle.value
+        self._run, self._destroy = lib().vitint_encoder_plan_run, lib().vitint_encoder_plan_destroy
+
+    def run(self, x: torch.Tensor, out: torch.Tensor) -> None:
+        code = self._run(self._handle, x.data_ptr(), out.data_ptr(), _stream())
+        if code != 0:
+            raise VitintError(code, "vitint_encoder_plan_run")
+
+    def __del__(self):
+        if getattr(self, "_handle", None):
+            self._destroy(self._handle)
+            self._handle = None
 
 
 @dataclass

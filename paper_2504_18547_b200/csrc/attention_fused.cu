@@ -592,6 +592,17 @@ extern "C" size_t vitint_attention_core_workspace_bytes(int32_t bits) {
 }
 
 namespace vitint {
+// Fills the tables of vitint_attention_core_shift for these steps.
+int attention_shift_table(int bits, float q_step, float k_step, void* table, size_t table_bytes, cudaStream_t st) {
+    const size_t need = vitint_attention_core_shift_workspace_bytes(bits);
+    if (need == 0) return VITINT_ERR_UNSUPPORTED;
+    if (!table || (reinterpret_cast<uintptr_t>(table) & 255u) || table_bytes < need) return VITINT_ERR_WORKSPACE;
+    const int m = 1 << (container_bits(bits) - 1), smax = 64 * m * m;
+    const float c2 = (float)((double)(float)((double)q_step * (double)k_step / 8.0) * 1.4426950408889634);
+    launch_kernel(shift_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (uint32_t*)table,
+                  reinterpret_cast<short*>((uint32_t*)table + (2 * smax + 1)), smax, c2);
+    return cuda_status(cudaGetLastError());
+}
 int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tokens, int smax, const float* table, float p_step,
                           float p_qp, const float* alpha_o, const float* beta_o, const vitint_codes* o_out, cudaStream_t st);
 }
@@ -711,9 +722,9 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
             return VITINT_ERR_CUDA;
     }
     if (build_table) {
-        if (shift) launch_kernel(shift_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (uint32_t*)workspace,
-                                 reinterpret_cast<short*>((uint32_t*)workspace + (2 * smax + 1)), smax, c2);
-        else launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
+        if (shift) {
+            if (int rc = attention_shift_table(qkv->bits, q_step, k_step, workspace, workspace_bytes, st)) return rc;
+        } else launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
         if (cudaGetLastError() != cudaSuccess) return VITINT_ERR_CUDA;
     }
     int grid = sm_count();

@@ -5,6 +5,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <tuple>
+#include <vector>
+
 #include "vitint.h"
 
 namespace vitint {
@@ -40,9 +43,34 @@ int cuda_status(cudaError_t e);
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// While a LaunchRecorder is active on the calling thread, launch_kernel() does not launch: it appends a kernel node to the
+// recorder's graph (behind the previous one, with a programmatic edge -- the form a captured programmatic launch takes), or,
+// once the graph is instantiated, rewrites the parameters of the instance's next node.  encoder.cu is its only user.
+struct LaunchRecorder {
+    cudaGraph_t graph = nullptr;              // being built ...
+    cudaGraphExec_t exec = nullptr;           // ... or instantiated: update the nodes first_node, first_node + 1, ...
+    std::vector<cudaGraphNode_t>* nodes = nullptr;
+    size_t next = 0;
+    cudaError_t error = cudaSuccess;
+    cudaError_t record(const cudaKernelNodeParams& p);
+};
+inline thread_local LaunchRecorder* t_recorder = nullptr;
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                                  Args... args) {
+    if (t_recorder) {
+        std::tuple<KArgs...> values(static_cast<KArgs>(args)...);
+        void* ptrs[sizeof...(KArgs) + 1];
+        std::apply([&](auto&... v) { int i = 0; ((ptrs[i++] = (void*)&v), ...); }, values);
+        cudaKernelNodeParams p = {};
+        p.func = (void*)kernel;
+        p.gridDim = grid;
+        p.blockDim = block;
+        p.sharedMemBytes = (unsigned)smem;
+        p.kernelParams = ptrs;
+        return t_recorder->record(p);
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;

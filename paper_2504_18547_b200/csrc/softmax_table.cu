@@ -97,6 +97,15 @@ int launch_softmax_table(const int32_t* s, int64_t rows, int cols, int64_t ld_s,
 }
 
 }  // namespace
+
+// Fills the table of vitint_softmax_quantize_bounded.
+int softmax_bounded_table(float c, int score_bound, void* table, size_t table_bytes, cudaStream_t st) {
+    if (!table || (reinterpret_cast<uintptr_t>(table) & 255u) || table_bytes < vitint_softmax_table_workspace_bytes(score_bound))
+        return VITINT_ERR_WORKSPACE;
+    launch_kernel(exp_table_kernel, dim3((2 * score_bound + 1 + 255) / 256), dim3(256), 0, st, (float*)table, score_bound, c);
+    return cuda_status(cudaGetLastError());
+}
+
 }  // namespace vitint
 
 using namespace vitint;
@@ -129,10 +138,8 @@ extern "C" int vitint_softmax_quantize_bounded(const int32_t* s, int64_t rows, i
     const int vec_p = (p_f32 && aligned16(p_f32) && ld_p % 4 == 0) ? 1 : 0;
     cudaStream_t st = (cudaStream_t)stream;
     float* table = (float*)workspace;
-    if (!table_ready) {
-        launch_kernel(exp_table_kernel, dim3((2 * score_bound + 1 + 255) / 256), dim3(256), 0, st, table, (int)score_bound, c);
-        if (int rc = cuda_status(cudaGetLastError())) return rc;
-    }
+    if (!table_ready)
+        if (int rc = softmax_bounded_table(c, score_bound, table, workspace_bytes, st)) return rc;
     uint8_t* o = (uint8_t*)p_out->data;
     if (cb == 2) return launch_softmax_table<2>(s, rows, cols, ld_s, table, score_bound, p_step, o, p_out->pitch_bytes, p_f32, ld_p, (float)qp, vec_p, st);
     if (cb == 4) return launch_softmax_table<4>(s, rows, cols, ld_s, table, score_bound, p_step, o, p_out->pitch_bytes, p_f32, ld_p, (float)qp, vec_p, st);

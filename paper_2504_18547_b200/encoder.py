@@ -25,7 +25,8 @@ def _dev(a, device):
 class EncoderLayer:
     def __init__(self, batch: int, tokens: int, heads: int, mlp_dim: int, bits: int, prm: dict, device="cuda",
                  eps: float = 1e-6, widen_weights: bool = True, fused_attention: bool = True,
-                 wide_activations: bool = True, softmax: str = "exp", layernorm: str = "fp32"):
+                 wide_activations: bool = True, softmax: str = "exp", layernorm: str = "fp32", plan: bool = True):
+        """plan: record the layer's launches once as a graph that forward() then launches (a stack records its own)."""
         self.batch, self.tokens, self.heads, self.bits, self.eps = batch, tokens, heads, bits, eps
         self.dim = D = heads * 64
         self.mlp_dim = F = mlp_dim
@@ -113,10 +114,98 @@ class EncoderLayer:
         self.epi_o = B.Epilogue(mode=B.EPI_REQUANT, alpha=self.alpha_o, out_bits=bits, out_signed=True, out_container=ca)
         self.epi_fc1 = B.Epilogue(mode=B.EPI_REQUANT, act=1, inv_out_step=self.inv_s_g, out_bits=bits, out_signed=False,
                                   out_container=ca)
+        self._plan = self._plan_for = None
+        if plan:
+            self._replan()
+
+    def _signature(self) -> list:
+        """Everything a plan takes from this layer, as plain values: the addresses of its weights, parameters and buffers,
+        and its scalars.  A plan is used only while it equals the one the plan was made for."""
+        w, s, b = self.w, self.s_w, self.bias
+        v = [self.s_ln, self.s_q, self.s_k, self.s_v, self.s_p, self.s_o, self.s_g, self.eps, self.batch, self.tokens,
+             self.x1.data.data_ptr(), self.qkv.data.data_ptr(), self.O.data.data_ptr(), self.x2.data.data_ptr(),
+             self.g.data.data_ptr(), self.h.data_ptr(), self.alpha_qkv.data_ptr(), self.beta_qkv.data_ptr(),
+             self.alpha_o.data_ptr(), self.inv_s_g.data_ptr(), w["qkv"].data.data_ptr(), w["proj"].data.data_ptr(),
+             w["fc1"].data.data_ptr(), w["fc2"].data.data_ptr(), s["proj"].data_ptr(), s["fc1"].data_ptr(),
+             s["fc2"].data_ptr(), b["proj"].data_ptr(), b["fc1"].data_ptr(), b["fc2"].data_ptr()]
+        if self.layernorm == "compare":
+            (r1, f1), (r2, f2) = self.ln_refs
+            v += [r1.data_ptr(), f1.data_ptr(), r2.data_ptr(), f2.data_ptr(), self.ln_stats.data_ptr(), self.n_eps]
+        else:
+            v += [self.ln1_g.data_ptr(), self.ln1_b.data_ptr(), self.ln2_g.data_ptr(), self.ln2_b.data_ptr()]
+        if self.fused_attention:
+            v.append(self.attn_table.data_ptr())
+        else:
+            v += [self.S.data_ptr(), self.P.data.data_ptr(), self.c, self.c2]
+            if self.sm_table is not None:
+                v.append(self.sm_table.data_ptr())
+        return v
+
+    def _desc(self):
+        d = B._EncoderLayerDesc()
+        d.batch, d.tokens, d.heads, d.bits = self.batch, self.tokens, self.heads, self.bits
+        d.eps, d.ln_step, d.g_step = self.eps, self.s_ln, self.s_g
+        d.q_step, d.k_step, d.v_step, d.p_step, d.o_step = self.s_q, self.s_k, self.s_v, self.s_p, self.s_o
+        p = lambda t: t.data_ptr()
+        if self.layernorm == "compare":
+            d.compare_layernorm, d.n_eps, d.ln_stats = 1, self.n_eps, p(self.ln_stats)
+            (r1, f1), (r2, f2) = self.ln_refs
+            d.ln1_refs, d.ln1_flip, d.ln2_refs, d.ln2_flip = p(r1), p(f1), p(r2), p(f2)
+        else:
+            d.ln1_gamma, d.ln1_beta, d.ln2_gamma, d.ln2_beta = p(self.ln1_g), p(self.ln1_b), p(self.ln2_g), p(self.ln2_b)
+        d.w_qkv, d.w_proj, d.w_fc1, d.w_fc2 = (self.w[n].desc() for n in ("qkv", "proj", "fc1", "fc2"))
+        d.alpha_qkv, d.beta_qkv, d.alpha_o, d.inv_g_step = p(self.alpha_qkv), p(self.beta_qkv), p(self.alpha_o), p(self.inv_s_g)
+        d.proj_step, d.fc1_step, d.fc2_step = (p(self.s_w[n]) for n in ("proj", "fc1", "fc2"))
+        d.proj_bias, d.fc1_bias, d.fc2_bias = (p(self.bias[n]) for n in ("proj", "fc1", "fc2"))
+        d.x1, d.qkv, d.o, d.x2, d.g = self.x1.desc(), self.qkv.desc(), self.O.desc(), self.x2.desc(), self.g.desc()
+        d.h = p(self.h)
+        table = None
+        if self.fused_attention:
+            d.attention = B.ATTN_SHIFT_CORE if self.softmax == "shift" else B.ATTN_EXP_CORE
+            table = self.attn_table
+        else:
+            d.scores, d.ld_scores, d.p = p(self.S), self.ld_s, self.P.desc()
+            if self.softmax == "shift":
+                d.attention, d.c = B.ATTN_SHIFT, self.c2
+            elif self.sm_table is not None:
+                d.attention, d.c, d.score_bound, table = B.ATTN_EXP_BOUNDED, self.c, self.score_bound, self.sm_table
+            else:
+                d.attention, d.c = B.ATTN_EXP, self.c
+        if table is not None:
+            d.table, d.table_bytes = p(table), table.numel()
+        return d
+
+    def _tables_filled(self):
+        """Making a plan fills the tables of the attention variants that build theirs on first use."""
+        if self.fused_attention and self.softmax == "shift":
+            self.attn_table_ready = True
+        elif not self.fused_attention and self.sm_table is not None:
+            self.sm_table_ready = True
+
+    def _replan(self):
+        """Records the layer's launches.  Where a stage does not take the layer's shape or steps there is no plan, and
+        forward() reports the error of that stage."""
+        self._plan_for, self._plan = self._signature(), None
+        try:
+            self._plan = B.EncoderPlan([self._desc()])
+        except B.VitintError:
+            return
+        self._tables_filled()
+
+    def _plain_io(self, x: torch.Tensor, out: torch.Tensor) -> bool:
+        """Whether x and out are dense matrices of the layer's shape (what a plan takes)."""
+        shape = (self.rows, self.dim)
+        return x.shape == shape and out.shape == shape and x.is_contiguous() and out.is_contiguous()
 
     def forward(self, x: torch.Tensor, out: torch.Tensor, events: list | None = None) -> torch.Tensor:
         """x, out: fp32 [batch*tokens, dim] on the device.  `events`, when given, receives
         len(self.stages)+1 recorded CUDA events bracketing the stages."""
+        if events is None and self._plan is not None and self._plain_io(x, out):
+            if self._plan_for != self._signature():
+                self._replan()
+            if self._plan is not None:
+                self._plan.run(x, out)
+                return out
         def mark():
             if events is not None:
                 e = torch.cuda.Event(enable_timing=True)
@@ -193,11 +282,33 @@ class EncoderStack:
 
     def __init__(self, layer_params: list, batch: int, tokens: int, heads: int, mlp_dim: int, bits: int,
                  device="cuda", **kw):
+        kw = dict(kw, plan=False)
         self.layers = [EncoderLayer(batch, tokens, heads, mlp_dim, bits, prm, device, **kw) for prm in layer_params]
         rows, dim = batch * tokens, heads * 64
         self.buf = [torch.empty((rows, dim), dtype=torch.float32, device=device) for _ in range(2)]
+        self._plan = self._plan_for = None
+        if self.layers:
+            self._replan()
+
+    def _signature(self) -> list:
+        return [l._signature() for l in self.layers] + [b.data_ptr() for b in self.buf]
+
+    def _replan(self):
+        self._plan_for, self._plan = self._signature(), None
+        try:
+            self._plan = B.EncoderPlan([l._desc() for l in self.layers], self.buf)
+        except B.VitintError:
+            return
+        for l in self.layers:
+            l._tables_filled()
 
     def forward(self, x: torch.Tensor, out: torch.Tensor) -> torch.Tensor:
+        if self._plan is not None and self.layers[0]._plain_io(x, out):
+            if self._plan_for != self._signature():
+                self._replan()
+            if self._plan is not None:
+                self._plan.run(x, out)
+                return out
         cur = x
         n = len(self.layers)
         for i, layer in enumerate(self.layers):

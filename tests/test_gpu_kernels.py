@@ -63,3 +63,94 @@ def test_linear_fp32_dispatch_boundary(M, N):
                          vt.Epilogue(mode=vt.EPI_DEQUANT_F32, residual=dev(res)))
     want = vo.epilogue_dequant(vo.matmul_i32(qx, qw), np.float32(0.37), s_w, bias, res)
     assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+# ---- recorded layers: the plan against the same launches one by one ------------------------------------------------
+def small_layer(kw, layer=0, cfg=None):
+    from paper_2504_18547_b200.encoder import EncoderLayer
+    cfg = cfg or si.BlockConfig("plan", 2, kw.pop("tokens", 50), 128, 2, kw.pop("bits", 4), mlp_dim=320)
+    return cfg, EncoderLayer(cfg.batch, cfg.tokens, cfg.heads, cfg.mlp_dim, cfg.bits, si.layer_parameters(cfg, layer), **kw)
+
+
+def one_by_one(layer, x):
+    """The layer with an event after every stage: the launches, not the plan."""
+    out = torch.empty_like(x)
+    layer.forward(x, out, events=[])
+    return out
+
+
+@pytest.mark.parametrize("kw", [{}, {"softmax": "shift", "layernorm": "compare"}, {"bits": 8}, {"fused_attention": False, "bits": 3},
+                                {"softmax": "shift", "fused_attention": False}, {"tokens": 300}, {"wide_activations": False, "bits": 2}],
+                         ids=lambda kw: "-".join(f"{k}_{v}" for k, v in kw.items()) or "plain")
+def test_layer_plan_equals_its_launches(kw):
+    cfg, layer = small_layer(dict(kw))
+    assert layer._plan is not None
+    for i in range(3):                                       # other inputs in other buffers, one of them on another stream
+        x = dev(si.normal(300 + i, (cfg.rows, cfg.dim)))
+        out = torch.full_like(x, float("nan"))
+        stream = torch.cuda.Stream() if i == 1 else torch.cuda.current_stream()
+        stream.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(stream):
+            layer.forward(x, out)
+        torch.cuda.synchronize()
+        assert torch.equal(out, one_by_one(layer, x))
+    # an output whose rows start on 16 bytes only, a strided input, and a replaced parameter
+    flat = torch.empty(cfg.rows * cfg.dim + 4, device="cuda")
+    odd = flat[4:].view(cfg.rows, cfg.dim)
+    layer.forward(x, odd)
+    assert torch.equal(odd, out)
+    wide = torch.zeros((cfg.rows, cfg.dim + 4), device="cuda")
+    wide[:, :cfg.dim] = x
+    layer.forward(wide[:, :cfg.dim], odd)
+    assert torch.equal(odd, out)
+    layer.bias["fc2"] = layer.bias["fc2"] + 1.0
+    layer.forward(x, odd)
+    assert torch.equal(odd, one_by_one(layer, x)) and not torch.equal(odd, out)
+
+
+def test_layer_plan_inside_a_captured_graph():
+    cfg, layer = small_layer({})
+    x, out = dev(si.normal(310, (cfg.rows, cfg.dim))), torch.empty((cfg.rows, cfg.dim), device="cuda")
+    layer.forward(x, out)
+    want = out.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        layer.forward(x, out)
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+
+
+def test_stack_plan_from_two_threads():
+    import threading
+    from paper_2504_18547_b200.encoder import EncoderStack
+    cfg = si.BlockConfig("plan", 1, 40, 64, 1, 4, mlp_dim=128)
+    stacks = [EncoderStack([si.layer_parameters(cfg, l + 5 * k) for l in range(3)], 1, 40, 1, 128, 4) for k in range(2)]
+    xs = [dev(si.normal(320 + i, (40, 64))) for i in range(6)]
+    want = [[], []]
+    for k, st in enumerate(stacks):
+        for x in xs:
+            cur = x
+            for l in st.layers:
+                cur = one_by_one(l, cur)
+            want[k].append(cur)
+    torch.cuda.synchronize()
+    got, errors = [[], []], []
+
+    def work(k):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for x in xs:
+                    got[k].append(stacks[k].forward(x, torch.empty_like(x)))
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:                               # noqa: BLE001 -- reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not errors
+    for k in range(2):
+        for a, b in zip(got[k], want[k]):
+            assert torch.equal(a, b)
