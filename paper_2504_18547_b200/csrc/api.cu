@@ -5,6 +5,25 @@ namespace vitint {
 
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? VITINT_OK : VITINT_ERR_CUDA; }
 
+cudaError_t LaunchRecorder::record(const cudaKernelNodeParams& p) {
+    if (error != cudaSuccess) return error;
+    if (exec) {
+        error = next < nodes->size() ? cudaGraphExecKernelNodeSetParams(exec, (*nodes)[next], &p) : cudaErrorInvalidValue;
+    } else {
+        cudaGraphNode_t node;
+        error = cudaGraphAddKernelNode(&node, graph, nullptr, 0, &p);
+        if (error == cudaSuccess && !nodes->empty()) {
+            cudaGraphEdgeData edge = {};
+            edge.from_port = cudaGraphKernelNodePortProgrammatic;
+            edge.type = cudaGraphDependencyTypeProgrammatic;
+            error = cudaGraphAddDependencies_v2(graph, &nodes->back(), &node, &edge, 1);
+        }
+        if (error == cudaSuccess) nodes->push_back(node);
+    }
+    ++next;
+    return error;
+}
+
 int check_codes(const vitint_codes* c) {
     if (!c || !c->data) return VITINT_ERR_INVALID_ARG;
     if (!valid_bits(c->bits) || (c->is_signed != 0 && c->is_signed != 1)) return VITINT_ERR_INVALID_ARG;

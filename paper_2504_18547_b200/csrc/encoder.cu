@@ -10,25 +10,6 @@
 
 namespace vitint {
 
-cudaError_t LaunchRecorder::record(const cudaKernelNodeParams& p) {
-    if (error != cudaSuccess) return error;
-    if (exec) {
-        error = next < nodes->size() ? cudaGraphExecKernelNodeSetParams(exec, (*nodes)[next], &p) : cudaErrorInvalidValue;
-    } else {
-        cudaGraphNode_t node;
-        error = cudaGraphAddKernelNode(&node, graph, nullptr, 0, &p);
-        if (error == cudaSuccess && !nodes->empty()) {
-            cudaGraphEdgeData edge = {};
-            edge.from_port = cudaGraphKernelNodePortProgrammatic;
-            edge.type = cudaGraphDependencyTypeProgrammatic;
-            error = cudaGraphAddDependencies_v2(graph, &nodes->back(), &node, &edge, 1);
-        }
-        if (error == cudaSuccess) nodes->push_back(node);
-    }
-    ++next;
-    return error;
-}
-
 namespace {
 
 enum Stage { ST_LN1, ST_QKV, ST_ATTENTION, ST_PROJ, ST_LN2, ST_FC1, ST_FC2, NUM_STAGES };

@@ -48,6 +48,7 @@ struct GemmParams {
     int bn, m_tiles, n_tiles, n_inner, total_tiles, k_blocks;
     int ca, cb, a_signed, b_signed, shift, b_mn_major;
     int a_direct, b_direct;            // operand already int8: TMA writes the operand ring itself
+    int reorder;                       // gemm_direct_kernel: both operands packed alike, unpacked in the cheaper order of k
     int small_acc;                     // |acc| < 2^22: int -> float without a conversion instruction
     int unit_out;                      // GELU + unsigned requantization: the GELU multiplier carries 1/Qp and values clamp to [0, 1]
     int epi_warps;                     // EPI_WARPS, or MAX_EPI_WARPS when both operands come straight from TMA

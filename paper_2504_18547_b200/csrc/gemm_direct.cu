@@ -1,5 +1,4 @@
-// a2 + a3 for operands stored one code per byte: the integer GEMM of gemm.cu with an epilogue laid out for the SM's
-// shared-memory / L1 data pipe.
+// a2 + a3: the integer GEMM of gemm.cu with an epilogue laid out for the SM's shared-memory / L1 data pipe.
 //
 // With a thread per accumulator row (gemm.cu) every store of a warp walks 32 different rows and every parameter read serves
 // two elements.  Here the epilogue reads the accumulators in the matrix-fragment layout (tcgen05.ld 16x256b: a thread holds
@@ -17,7 +16,12 @@
 // 36.2 us at M = 25,216, the epilogue alone 28, 63 (GELU: the fp32 pipe, 58 % busy) and 38 us (its 155 MB); the two share the
 // SM's issue slots and data pipe.
 //
-// Warps 0-15 epilogue (four per TMEM lane quarter, units of 16 rows x one column block in turn), 16 TMA, 17 MMA issue.
+// Warps 0-15 epilogue (four per TMEM lane quarter, units of 16 rows x one column block in turn), 16 TMA, 17 MMA issue.  With
+// bit-packed operands (PACKED) warps 8-15 expand them instead: two groups of four warps take K blocks in turn, and where both
+// operands are packed alike the codes of a chunk keep the order in which masks and shifts produce them (the contraction does
+// not mind), 12 operations for 32 codes instead of 20 and their sign left in the high bits.  12,608 x 768 -> 3072 of 4-bit
+// packed codes, requantized: 81 -> 48 us (one group 63, two 58, reordered 48); 3072 -> 768 fp32 104 -> 52; 197 x 192 -> 576
+// 7.6 -> 4.3.  What is left above the byte-stored form (29 us) is the expansion: ALU and shared-memory traffic.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"
@@ -26,11 +30,10 @@ namespace vitint {
 namespace {
 
 constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
-
-constexpr int GD_EPI_WARPS = 16;                                // four per TMEM lane quarter
-constexpr int GD_SLICES = GD_EPI_WARPS / 4;
-constexpr int GD_WARP_TMA = GD_EPI_WARPS, GD_WARP_MMA = GD_EPI_WARPS + 1;
-constexpr int GD_THREADS = (GD_EPI_WARPS + 2) * 32;
+constexpr int GD_THREADS = 18 * 32;
+constexpr int GD_UNPACK_WARPS = 8;
+__host__ __device__ constexpr int gd_epi_warps(bool packed) { return packed ? 16 - GD_UNPACK_WARPS : 16; }
+constexpr int GD_WARP_TMA = 16, GD_WARP_MMA = 17;
 
 // Column block within which the weight rows are permuted: column 2q + 8g + e of the tensor-core block is output column
 // (B/4) q + 2g + e, e < 2, q < 4, g < B/8.
@@ -45,13 +48,42 @@ __device__ __forceinline__ int gd_param_slot(int c) {
 }
 
 struct DirectBars {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync;
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync, p_full[MAX_STAGES], p_empty[MAX_STAGES];
 };
 
-// Two accumulators -> float.  SMALL: |acc| < 2^22, one integer addition each and a packed subtraction instead of the
-// conversion instruction.
-template <bool SMALL>
-__device__ __forceinline__ f32x2 acc_to_float2(uint32_t v0, uint32_t v1) {
+// One packed operand tile, `rows` rows of 16 C bytes -> rows of 128 int8 (128-byte swizzle), by 128 threads: thread t expands
+// chunk t % C of rows t / C, t / C + 128 / C, ... (always the same row of an eight-row group, so nothing but two pointers
+// changes along the way).
+template <int C, int SGN, bool REORDER>
+__device__ __forceinline__ void direct_unpack_tile(const uint8_t* src, uint8_t* dst, int rows, int t) {
+    constexpr int STEP = 128 / C;
+    const int r = t / C, sw = r & 7, oc = (t % C) * (8 / C);
+    src += t * 16;
+    dst += r * 128;
+#pragma unroll 4
+    for (; rows > 0; rows -= STEP, src += 2048, dst += STEP * 128)
+        if (rows >= STEP || r < rows) {
+            const uint4 in = *reinterpret_cast<const uint4*>(src);
+            if (REORDER) expand_chunk_reordered<C, SGN>(in, dst, oc, sw);
+            else expand_chunk<C, SGN>(in, dst, oc, sw);
+        }
+}
+__device__ __forceinline__ void direct_unpack(int c, int is_signed, int reorder, const uint8_t* src, uint8_t* dst, int rows, int t) {
+    if (c == 4) {
+        if (reorder) is_signed ? direct_unpack_tile<4, 1, true>(src, dst, rows, t) : direct_unpack_tile<4, 0, true>(src, dst, rows, t);
+        else is_signed ? direct_unpack_tile<4, 1, false>(src, dst, rows, t) : direct_unpack_tile<4, 0, false>(src, dst, rows, t);
+    } else {
+        if (reorder) is_signed ? direct_unpack_tile<2, 1, true>(src, dst, rows, t) : direct_unpack_tile<2, 0, true>(src, dst, rows, t);
+        else is_signed ? direct_unpack_tile<2, 1, false>(src, dst, rows, t) : direct_unpack_tile<2, 0, false>(src, dst, rows, t);
+    }
+}
+
+// Two accumulators (times 2^shift where signed codes were unpacked into the high bits of their bytes) -> float.  SMALL: the
+// unscaled sums stay below 2^22, one integer addition each and a packed subtraction instead of the conversion instruction;
+// otherwise 2^-shift rides on the multiplier.
+template <bool SMALL, bool PACKED>
+__device__ __forceinline__ f32x2 acc_to_float2(uint32_t v0, uint32_t v1, int shift) {
+    if (SMALL && PACKED) { v0 = (uint32_t)((int)v0 >> shift); v1 = (uint32_t)((int)v1 >> shift); }
     if (SMALL) return f2_add(f2_pack(__uint_as_float(0x4B400000u + v0), __uint_as_float(0x4B400000u + v1)), f2_dup(-12582912.0f));
     return f2_pack((float)(int)v0, (float)(int)v1);
 }
@@ -94,7 +126,7 @@ struct CodeParams {
 };
 
 // Requantizing epilogue of 16 rows x 64 columns, a thread's share two rows x 16 consecutive columns.
-template <int KIND, bool SMALL>
+template <int KIND, bool SMALL, bool PACKED>
 __device__ __forceinline__ void direct_codes(const GemmParams& P, const uint32_t (&v)[32], const CodeParams<KIND == EK_REQUANT_GELU>& cp,
                                              int lane, long long row0, int rows_valid, int n0) {
     const int r = lane >> 2, q = lane & 3;
@@ -112,7 +144,7 @@ __device__ __forceinline__ void direct_codes(const GemmParams& P, const uint32_t
 #pragma unroll
             for (int p = 0; p < 2; ++p) {                       // columns 4k + 2p, 4k + 2p + 1 of the thread's sixteen
                 const int i = 8 * k + 4 * p + 2 * h;
-                const f32x2 y = f2_fma(acc_to_float2<SMALL>(v[i], v[i + 1]), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
+                const f32x2 y = f2_fma(acc_to_float2<SMALL, PACKED>(v[i], v[i + 1], P.shift), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
                                        p ? f2_pack(b.z, b.w) : f2_pack(b.x, b.y));
                 float y0, y1, c0, c1;
                 f2_unpack(y, y0, y1);
@@ -169,7 +201,7 @@ __device__ __forceinline__ void direct_residual(const GemmParams& P, int lane, l
 }
 
 // fp32 epilogue of 16 rows x 32 columns.
-template <bool SMALL, bool RES>
+template <bool SMALL, bool RES, bool PACKED>
 __device__ __forceinline__ void direct_f32(const GemmParams& P, const uint32_t (&v)[16], const EpiParams& ep, int buf, int tile_col,
                                            int lane, long long row0, int rows_valid, int n0, const float (&res)[2][8]) {
     const int r = lane >> 2, q = lane & 3;
@@ -184,7 +216,7 @@ __device__ __forceinline__ void direct_f32(const GemmParams& P, const uint32_t (
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
                 const int i = 8 * k + 4 * p + 2 * h, j = 4 * k + 2 * p;
-                f32x2 y = f2_fma(acc_to_float2<SMALL>(v[i], v[i + 1]), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
+                f32x2 y = f2_fma(acc_to_float2<SMALL, PACKED>(v[i], v[i + 1], P.shift), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
                                  p ? f2_pack(b.z, b.w) : f2_pack(b.x, b.y));
                 if (RES) y = f2_add(y, f2_pack(res[h][j], res[h][j + 1]));
                 f2_unpack(y, out[h][j], out[h][j + 1]);
@@ -195,7 +227,7 @@ __device__ __forceinline__ void direct_f32(const GemmParams& P, const uint32_t (
         if (r + 8 * h < rows_valid) ptx::st_global_32B(o + (h ? 8 * P.ld_out : 0), out[h]);
 }
 
-template <int KIND, bool SMALL, bool RES>
+template <int KIND, bool SMALL, bool RES, bool PACKED>
 __global__ void __launch_bounds__(GD_THREADS, 1)
 gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                    const __grid_constant__ GemmParams P) {
@@ -205,23 +237,30 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     constexpr int BLK = gd_block(KIND);
+    constexpr int EPI_W = gd_epi_warps(PACKED), SLICES = EPI_W / 4;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
+    uint8_t* const smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     const uint32_t stage_bytes = P.ia_bytes + P.ib_bytes;
+    const uint32_t packed_off = (uint32_t)P.ns_i * stage_bytes, stage_packed = P.pa_bytes + P.pb_bytes;     // packed operands' ring
     volatile int* abort_ptr = &abort_flag;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < MAX_STAGES; ++s) {
-            ptx::mbar_init(ptx::smem_addr(&bars.full[s]), 1);
+            ptx::mbar_init(ptx::smem_addr(&bars.full[s]), PACKED ? GD_UNPACK_WARPS / 2 + ((P.a_direct || P.b_direct) ? 1 : 0) : 1);
             ptx::mbar_init(ptx::smem_addr(&bars.empty[s]), 1);
+            if (PACKED) {
+                ptx::mbar_init(ptx::smem_addr(&bars.p_full[s]), 1);
+                ptx::mbar_init(ptx::smem_addr(&bars.p_empty[s]), GD_UNPACK_WARPS / 2);
+            }
         }
         for (int b = 0; b < 2; ++b) {
             ptx::mbar_init(ptx::smem_addr(&bars.acc_full[b]), 1);
-            ptx::mbar_init(ptx::smem_addr(&bars.acc_empty[b]), GD_EPI_WARPS);
+            ptx::mbar_init(ptx::smem_addr(&bars.acc_empty[b]), EPI_W);
         }
-        ptx::mbar_init(ptx::smem_addr(&bars.epi_sync), GD_EPI_WARPS);
+        ptx::mbar_init(ptx::smem_addr(&bars.epi_sync), EPI_W);
         ptx::fence_mbar_init();
         ptx::fence_proxy_async_smem();
     }
@@ -247,28 +286,47 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             VT_STAMP(tr, TT_START);
             const uint32_t full0 = ptx::smem_addr(&bars.full[0]), empty0 = ptx::smem_addr(&bars.empty[0]);
             const int k_blocks = P.k_blocks, ns = P.ns_i;
-            int s = 0, it = 0;
-            uint32_t ph = 1u, dst = smem_base;
+            int s = 0, it = 0, sp = 0;
+            uint32_t ph = 1u, dst = smem_base, php = 1u;
             bool ok = true;
+            const uint32_t direct_bytes = PACKED ? (P.a_direct ? P.ia_bytes : 0u) + (P.b_direct ? P.ib_bytes : 0u) : stage_bytes;
+            const int a_step = P.a_direct ? BK : 16 * P.ca, b_step = P.b_direct ? BK : 16 * P.cb;         // bytes of a row per K block
             for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x) {
                 const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
                 const int m0 = m_tile * BM, blk0 = n_tile * P.bn / BLK;
                 for (int kb = 0; kb < k_blocks; ++kb, ++it) {
-                    VT_STAMP(tr, TT_WAIT_EMPTY);
-                    if (!mbar_wait(empty0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
-                    VT_STAMP(tr, TT_GOT_EMPTY);
                     const uint32_t full = full0 + 8u * (uint32_t)s;
-                    ptx::mbar_arrive_expect_tx(full, stage_bytes);
-                    ptx::tma_load_4d(dst, &map_a, full, kb * BK, m0, 0, 0);
-                    ptx::tma_load_5d(dst + P.ia_bytes, &map_b, full, kb * BK, 0, 0, 0, blk0);
+                    uint32_t a_dst = dst, b_dst = dst + P.ia_bytes, a_bar = full, b_bar = full;
+                    if (PACKED) {
+                        const uint32_t p_full = ptx::smem_addr(&bars.p_full[sp]), p_dst = smem_base + packed_off + (uint32_t)sp * stage_packed;
+                        if (!mbar_wait(ptx::smem_addr(&bars.p_empty[sp]), php, abort_ptr)) { ok = false; break; }
+                        ptx::mbar_arrive_expect_tx(p_full, stage_packed);
+                        if (!P.a_direct) { a_dst = p_dst; a_bar = p_full; }
+                        if (!P.b_direct) { b_dst = p_dst + P.pa_bytes; b_bar = p_full; }
+                        if (++sp == P.ns_p) { sp = 0; php ^= 1u; }
+                    }
+                    if (!PACKED || direct_bytes) {
+                        VT_STAMP(tr, TT_WAIT_EMPTY);
+                        if (!mbar_wait(empty0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
+                        VT_STAMP(tr, TT_GOT_EMPTY);
+                        ptx::mbar_arrive_expect_tx(full, direct_bytes);
+                    }
+                    ptx::tma_load_4d(a_dst, &map_a, a_bar, kb * a_step, m0, 0, 0);
+                    ptx::tma_load_5d(b_dst, &map_b, b_bar, kb * b_step, 0, 0, 0, blk0);
                     if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_bytes;
                 }
             }
             if (!ok) {
                 // give the copies still in flight a bounded chance to land before the CTA exits
-                for (int j = (it > ns ? it - ns : 0); j < it; ++j) {
-                    const uint32_t bar = full0 + 8u * (uint32_t)(j % ns);
-                    for (int spin = 0; spin < (1 << 20) && !ptx::mbar_try_wait(bar, (uint32_t)(j / ns) & 1u); ++spin) {}
+                for (int j = (it > MAX_STAGES ? it - MAX_STAGES : 0); j <= it; ++j) {
+                    if (PACKED && j + P.ns_p > it) {
+                        const uint32_t bar = ptx::smem_addr(&bars.p_full[j % P.ns_p]);
+                        for (int spin = 0; spin < (1 << 20) && !ptx::mbar_try_wait(bar, (uint32_t)(j / P.ns_p) & 1u); ++spin) {}
+                    }
+                    if (direct_bytes && j + ns > it) {
+                        const uint32_t bar = full0 + 8u * (uint32_t)(j % ns);
+                        for (int spin = 0; spin < (1 << 20) && !ptx::mbar_try_wait(bar, (uint32_t)(j / ns) & 1u); ++spin) {}
+                    }
                 }
             }
         }
@@ -282,7 +340,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             const uint64_t stage_step = (uint64_t)(stage_bytes >> 4);        // descriptor address field counts 16-byte units
             const uint32_t full0 = ptx::smem_addr(&bars.full[0]), empty0 = ptx::smem_addr(&bars.empty[0]);
             const int k_blocks = P.k_blocks, ns = P.ns_i;
-            const int last_steps = (P.K - (k_blocks - 1) * BK + 31) / 32;    // MMAs of the last (possibly partial) K block
+            // MMAs of the last (possibly partial) K block; 64 two-bit codes share a chunk, whose reordered codes fill two steps
+            int last_steps = (P.K - (k_blocks - 1) * BK + 31) / 32;
+            if (PACKED && P.reorder && P.ca == 2) last_steps = (last_steps + 1) & ~1;
             int s = 0, tl = 0;
             uint32_t ph = 0;
             uint64_t a_desc = a_desc0, b_desc = b_desc0;
@@ -317,9 +377,40 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 VT_STAMP(tr, TT_ISSUED);
             }
         }
+    } else if (PACKED && warp >= EPI_W) {
+        // Packed codes -> int8 operand tiles: 48 KB for a K block of a 128 x 256 tile.  Two groups of four warps take K blocks
+        // in turn, so that one group's waits, shared-memory latency and proxy fence run beside the other's work.
+        const int grp = (warp - EPI_W) >> 2, tid_u = threadIdx.x - (EPI_W + 4 * grp) * 32;
+        const int ns = P.ns_i, ns_p = P.ns_p;
+        int s = grp % ns, sp = grp % ns_p;
+        uint32_t ph = 1u, php = 0u;
+        bool ok = true;
+        int kb = grp, tile = blockIdx.x;
+        while (kb >= P.k_blocks) { kb -= P.k_blocks; tile += gridDim.x; }
+        while (ok && tile < P.total_tiles) {
+            bool w = mbar_wait(ptx::smem_addr(&bars.p_full[sp]), php, abort_ptr);
+            w = w && mbar_wait(ptx::smem_addr(&bars.empty[s]), ph, abort_ptr);
+            if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+            ptx::tc_fence_after();
+            const uint8_t* pa = smem_gen + packed_off + (size_t)sp * stage_packed;
+            uint8_t* ia = smem_gen + (size_t)s * stage_bytes;
+            if (!P.a_direct) direct_unpack(P.ca, P.a_signed, P.reorder, pa, ia, BM, tid_u);
+            if (!P.b_direct) direct_unpack(P.cb, P.b_signed, P.reorder, pa + P.pa_bytes, ia + P.ia_bytes, P.bn, tid_u);
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                ptx::mbar_arrive(ptx::smem_addr(&bars.full[s]));
+                ptx::mbar_arrive(ptx::smem_addr(&bars.p_empty[sp]));
+            }
+            if ((s += 2) >= ns) { s -= ns; ph ^= 1u; }
+            if ((sp += 2) >= ns_p) { sp -= ns_p; php ^= 1u; }
+            kb += 2;
+            while (kb >= P.k_blocks) { kb -= P.k_blocks; tile += gridDim.x; }
+        }
     } else {
         const int q4 = warp & 3, slice = warp >> 2;
         const int tid_e = threadIdx.x;
+        const float down = __int_as_float((127 - (SMALL ? 0 : P.shift)) << 23);
         // per-column parameters of a tile (multiplier, bias, GELU output factor), column c of the tile
         auto fetch_params = [&](int tile, int c, float& a, float& b, float& q) {
             const int n = (tile % P.n_tiles) * P.bn + c;
@@ -332,6 +423,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     if (KIND == EK_REQUANT_GELU) q = __fdiv_rn(0.5f * __ldg(P.inv_s + n), P.out_qp);   // folds GELU's 1/2 and 1/Qp
                 }
                 b = P.col_b ? __ldg(P.col_b + n) : 0.0f;
+                if (PACKED) a *= down;
             }
         };
         // The parameters of tile i+1 are fetched while the warps wait for tile i's accumulators and are stored to the other
@@ -350,7 +442,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         }
         int tl = 0;
         bool ok = true;
-        VT_TRACER(tr, (lane == 0 && warp == 0) ? 2 : ((lane == 0 && warp == GD_EPI_WARPS - 1) ? 3 : -1));
+        VT_TRACER(tr, (lane == 0 && warp == 0) ? 2 : ((lane == 0 && warp == EPI_W - 1) ? 3 : -1));
         VT_STAMP(tr, TT_START);
         float res[2][2][8];                                                   // fp32 kinds: the next block's residual, per half
         auto request_residual = [&](int tile, int blk, int half) {
@@ -387,17 +479,17 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             const int n_blk = cols / BLK;
             if constexpr (KIND == EK_DEQUANT) {
 #pragma unroll 1
-                for (int blk = slice; blk < n_blk; blk += GD_SLICES) {
+                for (int blk = slice; blk < n_blk; blk += SLICES) {
                     const int n0 = col_t + blk * BLK;
-                    const bool more = blk + GD_SLICES < n_blk;
+                    const bool more = blk + SLICES < n_blk;
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         uint32_t v[16];
                         ptx::tmem_ld_frag32(t_quarter + ((uint32_t)half << 20) + (uint32_t)(blk * BLK), v);
                         ptx::tmem_ld_wait();
-                        direct_f32<SMALL, RES>(P, v, epi_params, buf, blk * BLK, lane, row_q + 16 * half, rows_q - 16 * half, n0, res[half]);
+                        direct_f32<SMALL, RES, PACKED>(P, v, epi_params, buf, blk * BLK, lane, row_q + 16 * half, rows_q - 16 * half, n0, res[half]);
                         // the warp's next block (of this tile or the next) is on its way from here on
-                        if (RES) request_residual(more ? tile : next_tile, more ? blk + GD_SLICES : slice, half);
+                        if (RES) request_residual(more ? tile : next_tile, more ? blk + SLICES : slice, half);
                     }
                 }
                 if (RES && slice >= n_blk) {                                  // no block of this tile was this warp's
@@ -408,14 +500,14 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 // One 16-row half of a block at a time: 90 registers, so that sixteen warps fit.  (Eight warps that keep the
                 // parameters of a block for both halves and read the next accumulators ahead: fc1 79 us against 72.)
 #pragma unroll 1
-                for (int u = slice; u < 2 * n_blk; u += GD_SLICES) {
+                for (int u = slice; u < 2 * n_blk; u += SLICES) {
                     const int half = u & 1, tile_col = (u >> 1) * BLK;
                     uint32_t v[32];
                     ptx::tmem_ld_frag64(t_quarter + ((uint32_t)half << 20) + (uint32_t)tile_col, v);
                     CodeParams<KIND == EK_REQUANT_GELU> cp;
                     cp.load(epi_params, buf, tile_col, lane);
                     ptx::tmem_ld_wait();
-                    direct_codes<KIND, SMALL>(P, v, cp, lane, row_q + 16 * half, rows_q - 16 * half, col_t + tile_col);
+                    direct_codes<KIND, SMALL, PACKED>(P, v, cp, lane, row_q + 16 * half, rows_q - 16 * half, col_t + tile_col);
                 }
             }
             ptx::tc_fence_before();
@@ -437,30 +529,31 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 
 // The weight matrix as the five-dimensional view whose tile copy lands permuted within blocks of `block` rows:
 // (byte, e, q, g, block) with row = block * B + (B/4) q + 2g + e.
-int make_map_permuted(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, uint64_t pitch, int block, int bn) {
+int make_map_permuted(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows, uint64_t pitch, int block, int bn,
+                      int container) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return VITINT_ERR_CUDA;
     const cuuint64_t g = (cuuint64_t)block / 8;
     cuuint64_t dims[5] = {row_bytes, 2, 4, g, rows / (uint64_t)block};
     cuuint64_t strides[4] = {pitch, pitch * (uint64_t)(block / 4), pitch * 2, pitch * (uint64_t)block};
-    cuuint32_t box[5] = {(cuuint32_t)BK, 2, 4, (cuuint32_t)g, (cuuint32_t)(bn / block)};
+    cuuint32_t box[5] = {(cuuint32_t)(16 * container), 2, 4, (cuuint32_t)g, (cuuint32_t)(bn / block)};
     cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<void*>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, container == 8 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? VITINT_OK : VITINT_ERR_CUDA;
 }
 
-// Which calls this kernel takes: both operands one code per byte, whole column blocks, no batch of problems, and for fp32
-// outputs 32-byte aligned rows of the output and the residual.  Everything else stays with gemm_i8_kernel.
+// Which calls this kernel takes: whole column blocks, no batch of problems, and for fp32 outputs 32-byte aligned rows of the
+// output and the residual.  Everything else stays with gemm_i8_kernel.
 bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_major) {
-    if (!P.a_direct || !P.b_direct || n_inner != 1 || n_outer != 1 || b_mn_major) return false;
+    if (n_inner != 1 || n_outer != 1 || b_mn_major) return false;
     if (P.kind == EK_REQUANT || (P.kind == EK_REQUANT_GELU && P.unit_out)) return P.N % 64 == 0;
     if (P.kind != EK_DEQUANT || P.N % 32 != 0) return false;
     // A short contraction whose residual and output exceed L2 is bound by HBM, and gemm_i8_kernel's asynchronous copies of the
     // residual through shared memory keep more of it in flight (K = 768, N = 768: 27.8 against 30.1 us at M = 18,912, 35.7
     // against 39.2 at 25,216; below, 24.1 against 19.2 at 12,608).
-    if (P.residual && P.K <= 1024 && (long long)P.M * P.N * 8 > 100ll * 1000 * 1000) return false;
+    if (P.a_direct && P.b_direct && P.residual && P.K <= 1024 && (long long)P.M * P.N * 8 > 100ll * 1000 * 1000) return false;
     auto rows32 = [](const void* p, long long ld) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0 && ld % 8 == 0; };
     return rows32(P.out, P.ld_out) && (!P.residual || rows32(P.residual, P.ld_res));
 }
@@ -490,21 +583,34 @@ int direct_tile_columns(const GemmParams& P) {
 int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_bytes, uint64_t w_pitch, GemmParams P,
                        cudaStream_t st) {
     const int block = gd_block(P.kind);
+    const bool packed = !P.a_direct || !P.b_direct;
     P.bn = direct_tile_columns(P);
     P.n_tiles = (P.N + P.bn - 1) / P.bn;
     const long long tiles = (long long)P.m_tiles * P.n_tiles;
     if (tiles > 0x7fffffffll) return VITINT_ERR_UNSUPPORTED;
     P.total_tiles = (int)tiles;
     P.ib_bytes = (uint32_t)P.bn * BK;
-    const uint32_t stage = P.ia_bytes + P.ib_bytes;
-    int ns = (int)(GD_RING_BYTES / stage);
-    P.ns_i = ns > MAX_STAGES ? MAX_STAGES : ns;
+    P.pb_bytes = P.b_direct ? 0u : (uint32_t)P.bn * 16u * (uint32_t)P.cb;
+    const uint32_t stage = P.ia_bytes + P.ib_bytes, stage_p = P.pa_bytes + P.pb_bytes;
+    int ns, ns_p = 0;
+    if (packed) {
+        P.reorder = !P.a_direct && !P.b_direct && P.ca == P.cb ? 1 : 0;
+        ns = 3;
+        while (ns > 2 && (uint32_t)ns * stage + 2u * stage_p > GD_RING_BYTES) --ns;
+        ns_p = (int)((GD_RING_BYTES - (uint32_t)ns * stage) / stage_p);
+        if (ns_p > MAX_STAGES) ns_p = MAX_STAGES;
+    } else {
+        ns = (int)(GD_RING_BYTES / stage);
+        if (ns > MAX_STAGES) ns = MAX_STAGES;
+    }
+    P.ns_i = ns;
+    P.ns_p = ns_p;
     uint32_t cols = 32;
     while (cols < 2u * (uint32_t)P.bn) cols <<= 1;
     P.tmem_cols = cols;
     CUtensorMap map_b;
-    if (int rc = make_map_permuted(&map_b, w, w_row_bytes, (uint64_t)P.N, w_pitch, block, P.bn)) return rc;
-    size_t smem = (size_t)P.ns_i * stage + 1024;
+    if (int rc = make_map_permuted(&map_b, w, w_row_bytes, (uint64_t)P.N, w_pitch, block, P.bn, P.b_direct ? 8 : P.cb)) return rc;
+    size_t smem = (size_t)ns * stage + (size_t)ns_p * stage_p + 1024;
     if (smem < 120 * 1024) smem = 120 * 1024;                  // two CTAs never share an SM (and its tensor memory)
     int grid = sm_count();
     if (grid > P.total_tiles) grid = P.total_tiles;
@@ -513,7 +619,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
 #endif
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
-    static bool attr_set[MAX_DEVICES][8] = {};
+    static bool attr_set[MAX_DEVICES][16] = {};
     auto launch = [&](auto kernel, int slot) -> int {
         if (!attr_set[dev][slot]) {
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GD_RING_BYTES + 1024) != cudaSuccess)
@@ -523,13 +629,17 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
         launch_kernel(kernel, dim3(grid), dim3(GD_THREADS), smem, st, map_a, map_b, P);
         return cuda_status(cudaGetLastError());
     };
-    const bool small = P.small_acc == 2;
-    if (P.kind == EK_DEQUANT) {
-        if (P.residual) return small ? launch(gemm_direct_kernel<EK_DEQUANT, true, true>, 0) : launch(gemm_direct_kernel<EK_DEQUANT, false, true>, 1);
-        return small ? launch(gemm_direct_kernel<EK_DEQUANT, true, false>, 2) : launch(gemm_direct_kernel<EK_DEQUANT, false, false>, 3);
-    }
-    if (P.kind == EK_REQUANT) return small ? launch(gemm_direct_kernel<EK_REQUANT, true, false>, 4) : launch(gemm_direct_kernel<EK_REQUANT, false, false>, 5);
-    return small ? launch(gemm_direct_kernel<EK_REQUANT_GELU, true, false>, 6) : launch(gemm_direct_kernel<EK_REQUANT_GELU, false, false>, 7);
+    auto by_operands = [&](auto small) -> int {
+        constexpr bool S = decltype(small)::value;
+        constexpr int s0 = S ? 0 : 8;
+        if (P.kind == EK_DEQUANT) {
+            if (packed) return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, true>, s0) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, true>, s0 + 1);
+            return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, false>, s0 + 2) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, false>, s0 + 3);
+        }
+        if (P.kind == EK_REQUANT) return packed ? launch(gemm_direct_kernel<EK_REQUANT, S, false, true>, s0 + 4) : launch(gemm_direct_kernel<EK_REQUANT, S, false, false>, s0 + 5);
+        return packed ? launch(gemm_direct_kernel<EK_REQUANT_GELU, S, false, true>, s0 + 6) : launch(gemm_direct_kernel<EK_REQUANT_GELU, S, false, false>, s0 + 7);
+    };
+    return P.small_acc ? by_operands(std::true_type{}) : by_operands(std::false_type{});
 }
 
 }  // namespace

@@ -75,6 +75,20 @@ __device__ __forceinline__ void expand_chunk(uint4 in, uint8_t* row, int oc0, in
 }
 
 
+// The same codes in another order within the chunk -- all low fields of the four words first, then the next ones: no byte
+// permutes, 12 instead of 20 operations for 32 four-bit codes.  For contractions whose two operands go through this function
+// with the same C: the order of k is the same on both sides.
+template <int C, int SGN>
+__device__ __forceinline__ void expand_chunk_reordered(uint4 in, uint8_t* row, int oc0, int sw) {
+    constexpr uint32_t MASK = C == 4 ? (SGN ? 0xF0F0F0F0u : 0x0F0F0F0Fu) : (SGN ? 0xC0C0C0C0u : 0x03030303u);
+#pragma unroll
+    for (int f = 0; f < 8 / C; ++f) {
+        const int s = SGN ? 8 - C - C * f : C * f;                // left (signed: into the high bits) or right
+        auto field = [&](uint32_t w) { return (SGN ? w << s : w >> s) & MASK; };
+        *reinterpret_cast<uint4*>(row + (((oc0 + f) ^ sw) << 4)) = make_uint4(field(in.x), field(in.y), field(in.z), field(in.w));
+    }
+}
+
 // Rows of 64 int8 (64 codes each), 64-byte swizzle: row r lives at r*64 and its 16-byte chunk
 // cc at slot cc ^ ((r >> 1) & 3).  This one layout serves a K-contiguous operand with K = 64
 // (SBO = 512) and an N-contiguous operand with N = 64 (eight K rows per 512-byte group).

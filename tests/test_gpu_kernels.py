@@ -154,3 +154,42 @@ def test_stack_plan_from_two_threads():
     for k in range(2):
         for a, b in zip(got[k], want[k]):
             assert torch.equal(a, b)
+
+
+# ---- bit-packed operands: both packed alike (the reordered unpacking), packed unlike, one of them byte-stored; K at the
+# ---- edges of a 32-code MMA step, a 64-code chunk and a 128-code block
+@pytest.mark.parametrize("M,K,N", [(1, 16, 64), (33, 33, 64), (129, 96, 128), (130, 200, 192), (197, 1000, 320), (2000, 160, 1152)])
+@pytest.mark.parametrize("bx,bw", [(4, 4), (2, 2), (3, 4), (2, 4), (4, 2)])
+@pytest.mark.parametrize("xs", [True, False])
+def test_linear_packed_operands(M, K, N, bx, bw, xs):
+    qx, qw = rand_codes(121 + M, (M, K), bx, xs), rand_codes(122 + N, (N, K), bw, True)
+    acc = vo.matmul_i32(qx, qw)
+    spread = max(float(np.abs(acc).mean()), 1.0)
+    alpha = ((np.abs(si.normal(123, (N,), 0.0, 0.2)) + 0.5) * 2 / spread).astype(np.float32)
+    beta, res = si.normal(124, (N,), 0.0, 0.3), si.normal(125, (M, N))
+    px, pw = to_codes(qx, bx, xs), to_codes(qw, bw, True)
+    for x, w in ((px, pw), (px, vt.vitint_widen(pw)), (vt.vitint_widen(px), pw)):
+        q = vt.vitint_linear(x, 1.0, w, None, None, vt.Epilogue(mode=vt.EPI_REQUANT, alpha=dev(alpha), beta=dev(beta), out_bits=4,
+                                                                out_signed=True))
+        assert np.array_equal(from_codes(q), vo.epilogue_requant(acc, alpha, beta, 4, True)) and padding_is_zero(q)
+        y = vt.vitint_linear(x, 0.75, w, dev(alpha), dev(beta), vt.Epilogue(mode=vt.EPI_DEQUANT_F32, residual=dev(res)))
+        want = vo.epilogue_dequant(acc, np.float32(0.75), alpha, beta, res)
+        assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+def test_linear_packed_large_sums():
+    """Sums beyond 2^22 (converted with their power-of-two scale) and the largest the packed path takes."""
+    M, K, N = 130, 8000, 64
+    qx, qw = np.full((M, K), -8, np.int16), rand_codes(131, (N, K), 4, True)
+    qw[0], qw[1] = -8, 7
+    acc = vo.matmul_i32(qx, qw)
+    s_w = np.full(N, 1e-4, np.float32)
+    y = vt.vitint_linear(to_codes(qx, 4, True), 0.75, to_codes(qw, 4, True), dev(s_w), None, vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+    want = vo.epilogue_dequant(acc, np.float32(0.75), s_w)
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+    K = 70000                                               # 70000 * 64 > 2^22
+    qx, qw = rand_codes(132, (M, K), 4, True), rand_codes(133, (N, K), 4, True)
+    qx[0], qw[0] = -8, -8
+    y = vt.vitint_linear(to_codes(qx, 4, True), 0.75, to_codes(qw, 4, True), dev(s_w), None, vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+    want = vo.epilogue_dequant(vo.matmul_i32(qx, qw), np.float32(0.75), s_w)
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
