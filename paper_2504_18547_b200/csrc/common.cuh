@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "vitint.h"
@@ -33,6 +34,42 @@ inline void code_range(int bits, int is_signed, int* qn, int* qp) {
 int check_codes(const vitint_codes* c);
 
 int cuda_status(cudaError_t e);
+
+// Per-device caches (a process may use several GPUs): SM count, and which kernels already carry their
+// shared-memory opt-in on that device.
+constexpr int MAX_DEVICES = 64;
+inline int current_device() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return -1;
+    return dev;
+}
+inline int sm_count() {
+    static int n[MAX_DEVICES] = {};
+    const int dev = current_device();
+    if (dev < 0) return 1;
+    if (!n[dev]) {
+        int v = 0;
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        n[dev] = v > 0 ? v : 1;
+    }
+    return n[dev];
+}
+
+typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+inline EncodeTiledFn encode_fn() {
+    static EncodeTiledFn fn = nullptr;
+    if (!fn) {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult qres;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
+            qres == cudaDriverEntryPointSuccess)
+            fn = (EncodeTiledFn)p;
+    }
+    return fn;
+}
 
 // ---- programmatic dependent launch ---------------------------------------------------------
 // Every kernel of the library is launched with programmatic stream serialization: its CTAs may

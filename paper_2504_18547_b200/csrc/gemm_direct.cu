@@ -6,6 +6,8 @@
 // weight matrix) so that the columns a thread holds are consecutive columns of the output:
 //   codes  16 consecutive columns of a 64-column block: the per-column parameters are read once for four rows, and a
 //          warp's 16-byte stores cover 64 contiguous bytes of 8 rows instead of 16 of 32;
+//   norm   (QKV projection with the per-head quantizing LayerNorm) the Q and K tiles keep the weights' order, a thread walks a
+//          row's 64 columns of a head;
 //   fp32   8 consecutive columns of a 32-column block: a warp's 32-byte accesses of the residual and the result cover whole
 //          128-byte lines, so nothing is staged through shared memory and the operand ring keeps the space.
 // The arithmetic per element is that of gemm.cu, bit for bit.
@@ -30,10 +32,11 @@ namespace vitint {
 namespace {
 
 constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
-constexpr int GD_THREADS = 18 * 32;
+// Epilogue, unpack, TMA and MMA warps.  Eighteen warps leave a thread 96 registers; the norm kind, whose threads hold a head's
+// 64 channels, takes twelve epilogue warps (three heads of a 192-column tile for each lane quarter) and 128 registers.
 constexpr int GD_UNPACK_WARPS = 8;
-__host__ __device__ constexpr int gd_epi_warps(bool packed) { return packed ? 16 - GD_UNPACK_WARPS : 16; }
-constexpr int GD_WARP_TMA = 16, GD_WARP_MMA = 17;
+__host__ __device__ constexpr int gd_epi_warps(int kind, bool packed) { return packed ? 16 - GD_UNPACK_WARPS : kind == EK_QKV_NORM ? 12 : 16; }
+__host__ __device__ constexpr int gd_threads(int kind, bool packed) { return (gd_epi_warps(kind, packed) + (packed ? GD_UNPACK_WARPS : 0) + 2) * 32; }
 
 // Column block within which the weight rows are permuted: column 2q + 8g + e of the tensor-core block is output column
 // (B/4) q + 2g + e, e < 2, q < 4, g < B/8.
@@ -46,6 +49,11 @@ __device__ __forceinline__ int gd_param_slot(int c) {
     const int w = c & (BLK - 1), q = w / (BLK / 4), i = w & (BLK / 4 - 1);
     return (c - w) + (i >> 2) * 16 + q * 4 + (i & 3);
 }
+
+// What only one kind of epilogue needs: the weights in their own order for the norm kind's Q and K tiles.
+struct NoExtra { int unused; };
+struct NormExtra { CUtensorMap map_w; };
+template <int KIND> using DirectExtra = std::conditional_t<KIND == EK_QKV_NORM, NormExtra, NoExtra>;
 
 struct DirectBars {
     uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync, p_full[MAX_STAGES], p_empty[MAX_STAGES];
@@ -227,17 +235,162 @@ __device__ __forceinline__ void direct_f32(const GemmParams& P, const uint32_t (
         if (r + 8 * h < rows_valid) ptx::st_global_32B(o + (h ? 8 * P.ld_out : 0), out[h]);
 }
 
+// ---- QKV projection with the per-head quantizing LayerNorm of Section IV-C (Eq. 5 statistics, comparator of Fig. 5(b)) -----
+// A thread owns the 64 channels of a head of one accumulator row.  It walks them in order through the recurrence of Eq. 5
+//     delta = y_i - mu;  mu += delta / i;  S += delta * (y_i - mu)          (one rounded fp32 operation each)
+// with y_i = fma(float(acc_i), s_x s_w[i], b_i), forms V = S + n*eps, reads the accumulators a second time and finds each level
+// as Qn + number of references r with copysign(d*d, d) > V*r, d = y - mu (negated where the gain is negative): the count is
+// guessed from d / sqrt(V) (folded from a uniform quantizer, the references are the signed squares of equally spaced points)
+// and proven by two comparisons, formed exactly as defined, around it; where they fail all references are compared.  The fp32 Q
+// and K never exist in memory.  Both passes are rolled loops over 16 columns: unrolled over the 64 their code streams through
+// the instruction cache once per head, and that, not arithmetic, set the pace (one 197-row tile 9.8 us, of which the levels 6).
+// 12,672 x 384 -> 1152 (DeiT-S width, batch 64, 3-bit): 49 -> 31 us, 197 x 192 -> 576: 16.3 -> 6.5, against eight warps that
+// searched the references by four dependent shared-memory loads.
+constexpr int GD_NORM_REFS = 18;                               // -inf, up to 15 references, +inf, padded
+struct NormTables {
+    float ref[2][64][GD_NORM_REFS];
+    float4 guess[2][64];                                       // inv, off: count ~ rint(top * sat((y - mu) / sqrt(V) * inv + off)); sign of the gain
+    float2 step[64];                                           // i and RN(1/i)
+};
+
+__device__ __noinline__ uint32_t norm_count_all(const float* r, float ds, float V) {
+    uint32_t cnt = 0;
+    for (int t = 1; r[t] < INFINITY; ++t) cnt += ds > __fmul_rn(V, r[t]) ? 1u : 0u;
+    return cnt;
+}
+
+template <bool SMALL, bool PACKED>
+__device__ __forceinline__ void direct_norm_head(const GemmParams& P, const EpiParams& ep, int buf, uint32_t taddr, int tile_col,
+                                                 const NormTables& nt, int seg, long long row, bool row_ok, int col) {
+    float mu = 0.0f, S = 0.0f;
+    // statistics, in channel order
+#pragma unroll 1
+    for (int c0 = 0; c0 < 64; c0 += 16) {
+        uint32_t v[16];
+        ptx::tmem_ld16(taddr + (uint32_t)c0, v);
+        const float4* const pa = reinterpret_cast<const float4*>(&ep.a[buf][tile_col + c0]);
+        const float4* const pb = reinterpret_cast<const float4*>(&ep.b[buf][tile_col + c0]);
+        const float4* const ps = reinterpret_cast<const float4*>(&nt.step[c0]);
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int i4 = 0; i4 < 4; ++i4) {
+            const float4 a4 = pa[i4], b4 = pb[i4], s01 = ps[2 * i4], s23 = ps[2 * i4 + 1];
+            float y[4];
+            f2_unpack(f2_fma(acc_to_float2<SMALL, PACKED>(v[4 * i4], v[4 * i4 + 1], P.shift), f2_pack(a4.x, a4.y), f2_pack(b4.x, b4.y)), y[0], y[1]);
+            f2_unpack(f2_fma(acc_to_float2<SMALL, PACKED>(v[4 * i4 + 2], v[4 * i4 + 3], P.shift), f2_pack(a4.z, a4.w), f2_pack(b4.z, b4.w)), y[2], y[3]);
+            const float fi[4] = {s01.x, s01.z, s23.x, s23.z}, ri[4] = {s01.y, s01.w, s23.y, s23.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const float delta = __fadd_rn(y[j], -mu);
+                // RN(delta / i): quotient estimate, exact remainder in one FMA, one correction
+                const float q0 = __fmul_rn(delta, ri[j]);
+                const float rem = __fmaf_rn(-q0, fi[j], delta);
+                mu = __fadd_rn(mu, __fmaf_rn(rem, ri[j], q0));
+                S = __fadd_rn(S, __fmul_rn(delta, __fadd_rn(y[j], -mu)));
+            }
+        }
+    }
+    const float V = __fadd_rn(S, P.n_eps);
+    if (P.norm_stats != nullptr && row_ok) {
+        const int heads = P.norm_dim >> 6, head = (col - seg * P.norm_dim) >> 6;
+        *reinterpret_cast<float2*>(P.norm_stats + ((long long)seg * P.M * heads + row * heads + head) * 2) = make_float2(mu, V);
+    }
+    // levels
+    const f32x2 nmu2 = f2_dup(-mu), rs2 = f2_dup(rsqrtf(V)), V2 = f2_dup(V), top2 = f2_dup((float)((1 << P.norm_bits) - 1));
+    uint8_t* o = (uint8_t*)P.out + row * P.ld_out + (((long long)col * P.out_c) >> 3);
+    const uint32_t qn_low = ((uint32_t)P.norm_qn & 0x7Fu) * 0x01010101u, qn_top = ((uint32_t)P.norm_qn & 0x80u) * 0x01010101u;
+    uint32_t ref0 = ptx::smem_addr(&nt.ref[seg][0][0]) - 0x4B400000u * 4u;         // the guess is 1.5*2^23 + count: times four an address
+#pragma unroll 1
+    for (int c0 = 0; c0 < 64; c0 += 16) {
+        uint32_t v[16], w[4];
+        ptx::tmem_ld16(taddr + (uint32_t)c0, v);
+        const float4* const pa = reinterpret_cast<const float4*>(&ep.a[buf][tile_col + c0]);
+        const float4* const pb = reinterpret_cast<const float4*>(&ep.b[buf][tile_col + c0]);
+        const float4* const pg = &nt.guess[seg][c0];
+        ptx::tmem_ld_wait();
+#pragma unroll
+        for (int i4 = 0; i4 < 4; ++i4) {
+            const float4 a4 = pa[i4], b4 = pb[i4];
+            float ds[4];
+            uint32_t g[4];
+            bool proven = true;
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+                const int i = 4 * i4 + 2 * p;
+                const float4 ga = pg[i], gb = pg[i + 1];
+                const f32x2 y = f2_fma(acc_to_float2<SMALL, PACKED>(v[i], v[i + 1], P.shift), p ? f2_pack(a4.z, a4.w) : f2_pack(a4.x, a4.y),
+                                       p ? f2_pack(b4.z, b4.w) : f2_pack(b4.x, b4.y));
+                const f32x2 delta = f2_add(y, nmu2), d = f2_mul(delta, f2_pack(ga.z, gb.z));             // exact sign change
+                float d0, d1, q0, q1, u0, u1, g0, g1, l0, l1, h0, h1;
+                f2_unpack(d, d0, d1);
+                f2_unpack(f2_mul(d, d), q0, q1);
+                ds[2 * p] = copysignf(q0, d0);
+                ds[2 * p + 1] = copysignf(q1, d1);
+                f2_unpack(f2_mul(delta, rs2), u0, u1);
+                u0 = __saturatef(fmaf(u0, ga.x, ga.y));
+                u1 = __saturatef(fmaf(u1, gb.x, gb.y));
+                f2_unpack(f2_fma(f2_pack(u0, u1), top2, f2_dup(12582912.0f)), g0, g1);
+                g[2 * p] = __float_as_uint(g0);
+                g[2 * p + 1] = __float_as_uint(g1);
+                const uint32_t r0 = g[2 * p] * 4u + ref0, r1 = g[2 * p + 1] * 4u + ref0;
+                f2_unpack(f2_mul(V2, f2_pack(ptx::ld_shared_f32(r0 + 4 * i * GD_NORM_REFS), ptx::ld_shared_f32(r1 + 4 * (i + 1) * GD_NORM_REFS))), l0, l1);
+                f2_unpack(f2_mul(V2, f2_pack(ptx::ld_shared_f32(r0 + 4 * (i * GD_NORM_REFS + 1)), ptx::ld_shared_f32(r1 + 4 * ((i + 1) * GD_NORM_REFS + 1)))), h0, h1);
+                proven = proven && ds[2 * p] > l0 && !(ds[2 * p] > h0) && ds[2 * p + 1] > l1 && !(ds[2 * p + 1] > h1);
+            }
+            uint32_t n = (g[0] + (g[1] << 8) + (g[2] << 16) + (g[3] << 24)) - 0x4B400000u * 0x01010101u;
+            if (!proven) {
+                n = 0;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) n |= norm_count_all(nt.ref[seg][c0 + 4 * i4 + j], ds[j], V) << (8 * j);
+            }
+            w[i4] = (n + qn_low) ^ qn_top;                      // Qn added to every byte (none overflows: low bits, then the top bit)
+        }
+        if (row_ok) {
+            if (P.out_c == 8) {
+                *reinterpret_cast<uint4*>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+            } else if (P.out_c == 4) {
+                uint32_t t[2];
+                narrow4(w, t);
+                *reinterpret_cast<uint2*>(o) = make_uint2(t[0], t[1]);
+            } else {
+                *reinterpret_cast<uint32_t*>(o) = narrow2(w);
+            }
+        }
+        o += 2 * P.out_c;
+        ref0 += 4u * 16u * GD_NORM_REFS;
+    }
+}
+
+// A tile's rows and columns.  The norm kind numbers its tiles by column first, Q and K before V, so that the cheap V tiles
+// fill the last round, and no tile crosses from one of the three segments into the next.
+template <int KIND>
+__device__ __forceinline__ void direct_tile(const GemmParams& P, int tile, int& m_tile, int& col_t, int& cols) {
+    if (KIND == EK_QKV_NORM) {
+        const int n = tile / P.m_tiles, per_seg = P.n_tiles / 3;
+        m_tile = tile - n * P.m_tiles;
+        const int seg = n / per_seg, off = (n - seg * per_seg) * P.bn;
+        col_t = seg * P.norm_dim + off;
+        cols = P.norm_dim - off < P.bn ? P.norm_dim - off : P.bn;
+    } else {
+        m_tile = tile / P.n_tiles;
+        col_t = (tile - m_tile * P.n_tiles) * P.bn;
+        cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;                       // whole blocks
+    }
+}
+
 template <int KIND, bool SMALL, bool RES, bool PACKED>
-__global__ void __launch_bounds__(GD_THREADS, 1)
+__global__ void __launch_bounds__(gd_threads(KIND, PACKED), 1)
 gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                   const __grid_constant__ GemmParams P) {
+                   const __grid_constant__ DirectExtra<KIND> X, const __grid_constant__ GemmParams P) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ DirectBars bars;
     __shared__ __align__(16) EpiParams epi_params;
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
+    __shared__ __align__(16) std::conditional_t<KIND == EK_QKV_NORM, NormTables, float4> norm_tab[1];
     constexpr int BLK = gd_block(KIND);
-    constexpr int EPI_W = gd_epi_warps(PACKED), SLICES = EPI_W / 4;
+    constexpr int EPI_W = gd_epi_warps(KIND, PACKED), SLICES = EPI_W / 4;
+    constexpr int WARP_TMA_D = gd_threads(KIND, PACKED) / 32 - 2, WARP_MMA_D = WARP_TMA_D + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
@@ -264,11 +417,11 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         ptx::fence_mbar_init();
         ptx::fence_proxy_async_smem();
     }
-    if (warp == GD_WARP_MMA) {
+    if (warp == WARP_MMA_D) {
         ptx::tmem_alloc(ptx::smem_addr(&tmem_base_slot), P.tmem_cols);
         ptx::tmem_relinquish();
     }
-    if (warp == GD_WARP_TMA && lane == 0) {
+    if (warp == WARP_TMA_D && lane == 0) {
         ptx::prefetch_tensormap(&map_a);
         ptx::prefetch_tensormap(&map_b);
     }
@@ -280,7 +433,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     grid_dependency_wait();        // operands, parameters and the residual may come from the previous kernel
     grid_dependency_launch();
 
-    if (warp == GD_WARP_TMA) {
+    if (warp == WARP_TMA_D) {
         if (lane == 0) {
             VT_TRACER(tr, 0);
             VT_STAMP(tr, TT_START);
@@ -292,8 +445,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             const uint32_t direct_bytes = PACKED ? (P.a_direct ? P.ia_bytes : 0u) + (P.b_direct ? P.ib_bytes : 0u) : stage_bytes;
             const int a_step = P.a_direct ? BK : 16 * P.ca, b_step = P.b_direct ? BK : 16 * P.cb;         // bytes of a row per K block
             for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x) {
-                const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
-                const int m0 = m_tile * BM, blk0 = n_tile * P.bn / BLK;
+                int m_tile, col_t, cols;
+                direct_tile<KIND>(P, tile, m_tile, col_t, cols);
+                const int m0 = m_tile * BM, blk0 = col_t / BLK;
                 for (int kb = 0; kb < k_blocks; ++kb, ++it) {
                     const uint32_t full = full0 + 8u * (uint32_t)s;
                     uint32_t a_dst = dst, b_dst = dst + P.ia_bytes, a_bar = full, b_bar = full;
@@ -312,7 +466,12 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                         ptx::mbar_arrive_expect_tx(full, direct_bytes);
                     }
                     ptx::tma_load_4d(a_dst, &map_a, a_bar, kb * a_step, m0, 0, 0);
-                    ptx::tma_load_5d(b_dst, &map_b, b_bar, kb * b_step, 0, 0, 0, blk0);
+                    if constexpr (KIND == EK_QKV_NORM) {
+                        if (col_t < 2 * P.norm_dim) ptx::tma_load_4d(b_dst, &X.map_w, b_bar, kb * b_step, col_t, 0, 0);
+                        else ptx::tma_load_5d(b_dst, &map_b, b_bar, kb * b_step, 0, 0, 0, blk0);
+                    } else {
+                        ptx::tma_load_5d(b_dst, &map_b, b_bar, kb * b_step, 0, 0, 0, blk0);
+                    }
                     if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_bytes;
                 }
             }
@@ -330,7 +489,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 }
             }
         }
-    } else if (warp == GD_WARP_MMA) {
+    } else if (warp == WARP_MMA_D) {
         if (lane == 0) {
             const uint32_t idesc = ptx::idesc_i8(BM, P.bn, P.a_signed, P.b_signed, 0);
             VT_TRACER(tr, 1);
@@ -413,24 +572,34 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         const float down = __int_as_float((127 - (SMALL ? 0 : P.shift)) << 23);
         // per-column parameters of a tile (multiplier, bias, GELU output factor), column c of the tile
         auto fetch_params = [&](int tile, int c, float& a, float& b, float& q) {
-            const int n = (tile % P.n_tiles) * P.bn + c;
+            int m_tile, col_t, cols;
+            direct_tile<KIND>(P, tile, m_tile, col_t, cols);
+            const int n = col_t + c;
             a = 0.0f; b = 0.0f; q = 0.0f;
-            if (n < P.N) {
+            if (c < cols) {
                 if (KIND == EK_REQUANT) {
                     a = __ldg(P.col_a + n);
+                } else if (KIND == EK_QKV_NORM && col_t >= 2 * P.norm_dim) {   // V: folded requantization
+                    a = __ldg(P.v_alpha + (n - 2 * P.norm_dim));
                 } else {
                     a = P.col_a ? __fmul_rn(P.x_step, __ldg(P.col_a + n)) : P.x_step;
                     if (KIND == EK_REQUANT_GELU) q = __fdiv_rn(0.5f * __ldg(P.inv_s + n), P.out_qp);   // folds GELU's 1/2 and 1/Qp
                 }
-                b = P.col_b ? __ldg(P.col_b + n) : 0.0f;
+                if (KIND == EK_QKV_NORM && col_t >= 2 * P.norm_dim) b = P.v_beta ? __ldg(P.v_beta + (n - 2 * P.norm_dim)) : 0.0f;
+                else b = P.col_b ? __ldg(P.col_b + n) : 0.0f;
                 if (PACKED) a *= down;
             }
         };
         // The parameters of tile i+1 are fetched while the warps wait for tile i's accumulators and are stored to the other
         // half of epi_params before tile i is processed, so no tile waits for them.  (bn <= 256 <= epilogue threads)
         const bool my_col = tid_e < P.bn;
-        const int my_slot = gd_param_slot<BLK>(tid_e);
-        auto put_params = [&](int buf, float a, float b, float q) {
+        auto put_params = [&](int tile, int buf, float a, float b, float q) {
+            int my_slot = gd_param_slot<BLK>(tid_e);
+            if (KIND == EK_QKV_NORM) {
+                int m_tile, col_t, cols;
+                direct_tile<KIND>(P, tile, m_tile, col_t, cols);
+                if (col_t < 2 * P.norm_dim) my_slot = tid_e;                  // Q and K: columns in order
+            }
             epi_params.a[buf][my_slot] = a;
             epi_params.b[buf][my_slot] = b;
             if (KIND == EK_REQUANT_GELU) epi_params.q[buf][my_slot] = q;
@@ -438,7 +607,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         if (my_col && (int)blockIdx.x < P.total_tiles) {
             float a, b, q;
             fetch_params(blockIdx.x, tid_e, a, b, q);
-            put_params(0, a, b, q);
+            put_params(blockIdx.x, 0, a, b, q);
         }
         int tl = 0;
         bool ok = true;
@@ -446,22 +615,41 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         VT_STAMP(tr, TT_START);
         float res[2][2][8];                                                   // fp32 kinds: the next block's residual, per half
         auto request_residual = [&](int tile, int blk, int half) {
-            const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
-            const int n0 = n_tile * P.bn + blk * BLK, row0 = m_tile * BM + q4 * 32 + 16 * half;
-            if (tile < P.total_tiles && blk * BLK < P.bn && n0 < P.N) direct_residual(P, lane, row0, P.M - row0, n0, res[half]);
+            int m_tile, col_t, cols;
+            direct_tile<KIND>(P, tile, m_tile, col_t, cols);
+            const int n0 = col_t + blk * BLK, row0 = m_tile * BM + q4 * 32 + 16 * half;
+            if (tile < P.total_tiles && blk * BLK < cols) direct_residual(P, lane, row0, P.M - row0, n0, res[half]);
         };
+        if constexpr (KIND == EK_QKV_NORM) {
+            // read by every epilogue warp after the first tile's group barrier
+            const int nt = (1 << P.norm_bits) - 1;
+            for (int i = tid_e; i < 2 * 64; i += EPI_W * 32) {
+                const int set = i >> 6, c = i & 63;
+                const float* r = P.norm_refs + (size_t)i * nt;
+                float* const dst = norm_tab[0].ref[set][c];
+                dst[0] = -INFINITY;
+                for (int t = 0; t < GD_NORM_REFS - 1; ++t) dst[t + 1] = t < nt ? __ldg(r + t) : INFINITY;
+                const float r0 = __ldg(r), r1 = __ldg(r + nt - 1), sgn = (P.norm_flip != nullptr && __ldg(P.norm_flip + i)) ? -1.0f : 1.0f;
+                const float rho0 = copysignf(sqrtf(fabsf(r0)), r0), rho1 = copysignf(sqrtf(fabsf(r1)), r1);
+                float inv = (float)(nt - 1) / (rho1 - rho0);
+                if (!(inv < 1e30f)) inv = 0.0f;
+                norm_tab[0].guess[set][c] = make_float4(inv * sgn / (float)nt, (0.5f - rho0 * inv) / (float)nt, sgn, 0.0f);
+                if (set == 0) norm_tab[0].step[c] = make_float2((float)(c + 1), __frcp_rn((float)(c + 1)));
+            }
+        }
         if (KIND == EK_DEQUANT && RES) {
             request_residual(blockIdx.x, slice, 0);
             request_residual(blockIdx.x, slice, 1);
         }
         for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x, ++tl) {
-            const int m_tile = tile / P.n_tiles, n_tile = tile - m_tile * P.n_tiles;
+            int m_tile, col_t, cols;
+            direct_tile<KIND>(P, tile, m_tile, col_t, cols);
             const int buf = tl & 1;
             const int next_tile = tile + (int)gridDim.x;
             const bool fetch_next = my_col && next_tile < P.total_tiles;
             float na = 0.0f, nb = 0.0f, nq = 0.0f;
             if (fetch_next) fetch_params(next_tile, tid_e, na, nb, nq);
-            const int row_q = m_tile * BM + q4 * 32, col_t = n_tile * P.bn;
+            const int row_q = m_tile * BM + q4 * 32;
             const int rows_q = P.M - row_q;                                   // valid rows from the quarter's first one on
             const uint32_t acc_ph = (uint32_t)(tl >> 1) & 1u;
             VT_STAMP(tr, TT_WAIT_ACC);
@@ -473,9 +661,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             VT_STAMP(tr, TT_GOT_ACC);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             ptx::tc_fence_after();
-            if (fetch_next) put_params(buf ^ 1, na, nb, nq);                  // every warp has passed the barrier: none reads that half
+            if (fetch_next) put_params(next_tile, buf ^ 1, na, nb, nq);                  // every warp has passed the barrier: none reads that half
             const uint32_t t_quarter = tmem_base + (uint32_t)buf * acc_stride + ((uint32_t)(q4 * 32) << 16);
-            const int cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;         // whole blocks
             const int n_blk = cols / BLK;
             if constexpr (KIND == EK_DEQUANT) {
 #pragma unroll 1
@@ -497,17 +684,26 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     request_residual(next_tile, slice, 1);
                 }
             } else {
+                bool norm = false;
+                if constexpr (KIND == EK_QKV_NORM) {
+                    norm = col_t < 2 * P.norm_dim;                            // a Q or K tile
+#pragma unroll 1
+                    for (int blk = slice; norm && blk < n_blk; blk += SLICES)
+                        direct_norm_head<SMALL, PACKED>(P, epi_params, buf, t_quarter + (uint32_t)(blk * 64), blk * 64, norm_tab[0],
+                                                        col_t >= P.norm_dim ? 1 : 0, row_q + lane, lane < rows_q, col_t + blk * 64);
+                }
+                constexpr int CK = KIND == EK_QKV_NORM ? EK_REQUANT : KIND;
                 // One 16-row half of a block at a time: 90 registers, so that sixteen warps fit.  (Eight warps that keep the
                 // parameters of a block for both halves and read the next accumulators ahead: fc1 79 us against 72.)
 #pragma unroll 1
-                for (int u = slice; u < 2 * n_blk; u += SLICES) {
+                for (int u = slice; !norm && u < 2 * n_blk; u += SLICES) {
                     const int half = u & 1, tile_col = (u >> 1) * BLK;
                     uint32_t v[32];
                     ptx::tmem_ld_frag64(t_quarter + ((uint32_t)half << 20) + (uint32_t)tile_col, v);
-                    CodeParams<KIND == EK_REQUANT_GELU> cp;
+                    CodeParams<CK == EK_REQUANT_GELU> cp;
                     cp.load(epi_params, buf, tile_col, lane);
                     ptx::tmem_ld_wait();
-                    direct_codes<KIND, SMALL, PACKED>(P, v, cp, lane, row_q + 16 * half, rows_q - 16 * half, col_t + tile_col);
+                    direct_codes<CK, SMALL, PACKED>(P, v, cp, lane, row_q + 16 * half, rows_q - 16 * half, col_t + tile_col);
                 }
             }
             ptx::tc_fence_before();
@@ -520,7 +716,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 
     ptx::tc_fence_before();
     __syncthreads();
-    if (warp == GD_WARP_MMA) {
+    if (warp == WARP_MMA_D) {
         ptx::tc_fence_after();
         __syncwarp();
         ptx::tmem_dealloc(tmem_base, P.tmem_cols);
@@ -548,6 +744,7 @@ int make_map_permuted(CUtensorMap* map, const void* base, uint64_t row_bytes, ui
 // output and the residual.  Everything else stays with gemm_i8_kernel.
 bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_major) {
     if (n_inner != 1 || n_outer != 1 || b_mn_major) return false;
+    if (P.kind == EK_QKV_NORM) return true;
     if (P.kind == EK_REQUANT || (P.kind == EK_REQUANT_GELU && P.unit_out)) return P.N % 64 == 0;
     if (P.kind != EK_DEQUANT || P.N % 32 != 0) return false;
     // A short contraction whose residual and output exceed L2 is bound by HBM, and gemm_i8_kernel's asynchronous copies of the
@@ -566,13 +763,14 @@ bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_maj
 // widest that does not add a wave.
 int direct_tile_columns(const GemmParams& P) {
     const int block = gd_block(P.kind), sms = sm_count();
-    const float per_col = P.kind == EK_REQUANT ? 0.0098f : P.kind == EK_DEQUANT ? 0.0129f : 0.0148f;
+    const int segments = P.kind == EK_QKV_NORM ? 3 : 1, width = P.N / segments;
+    const float per_col = P.kind == EK_QKV_NORM ? 0.017f : P.kind == EK_REQUANT ? 0.0098f : P.kind == EK_DEQUANT ? 0.0129f : 0.0148f;
     const float k_fill = 0.27f * (float)P.k_blocks, k_main = 0.32f * (float)P.k_blocks;
     int best = 0;
     float best_t = 0.0f;
-    for (int bn = MAX_BN; bn >= block; bn -= block) {
-        if (bn > P.N && bn - block >= P.N) continue;
-        const long long tiles = (long long)P.m_tiles * ((P.N + bn - 1) / bn);
+    for (int bn = P.kind == EK_QKV_NORM ? 192 : MAX_BN; bn >= block; bn -= block) {
+        if (bn > width && bn - block >= width) continue;
+        const long long tiles = (long long)P.m_tiles * ((width + bn - 1) / bn) * segments;
         const float waves = (float)((tiles + sms - 1) / sms), epi = 0.2f + per_col * (float)bn;
         const float t = k_fill + (waves - 1.0f) * (k_main > epi ? k_main : epi) + epi;
         if (!best || t < best_t) { best = bn; best_t = t; }
@@ -585,22 +783,23 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     const int block = gd_block(P.kind);
     const bool packed = !P.a_direct || !P.b_direct;
     P.bn = direct_tile_columns(P);
-    P.n_tiles = (P.N + P.bn - 1) / P.bn;
+    P.n_tiles = P.kind == EK_QKV_NORM ? 3 * ((P.norm_dim + P.bn - 1) / P.bn) : (P.N + P.bn - 1) / P.bn;
     const long long tiles = (long long)P.m_tiles * P.n_tiles;
     if (tiles > 0x7fffffffll) return VITINT_ERR_UNSUPPORTED;
     P.total_tiles = (int)tiles;
     P.ib_bytes = (uint32_t)P.bn * BK;
     P.pb_bytes = P.b_direct ? 0u : (uint32_t)P.bn * 16u * (uint32_t)P.cb;
     const uint32_t stage = P.ia_bytes + P.ib_bytes, stage_p = P.pa_bytes + P.pb_bytes;
+    const uint32_t ring = GD_RING_BYTES - (P.kind == EK_QKV_NORM ? 8u * 1024u : 0u);     // beside 12 KB of static reference tables
     int ns, ns_p = 0;
     if (packed) {
         P.reorder = !P.a_direct && !P.b_direct && P.ca == P.cb ? 1 : 0;
         ns = 3;
-        while (ns > 2 && (uint32_t)ns * stage + 2u * stage_p > GD_RING_BYTES) --ns;
-        ns_p = (int)((GD_RING_BYTES - (uint32_t)ns * stage) / stage_p);
+        while (ns > 2 && (uint32_t)ns * stage + 2u * stage_p > ring) --ns;
+        ns_p = (int)((ring - (uint32_t)ns * stage) / stage_p);
         if (ns_p > MAX_STAGES) ns_p = MAX_STAGES;
     } else {
-        ns = (int)(GD_RING_BYTES / stage);
+        ns = (int)(ring / stage);
         if (ns > MAX_STAGES) ns = MAX_STAGES;
     }
     P.ns_i = ns;
@@ -619,19 +818,29 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
 #endif
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
-    static bool attr_set[MAX_DEVICES][16] = {};
-    auto launch = [&](auto kernel, int slot) -> int {
+    static bool attr_set[MAX_DEVICES][20] = {};
+    const int threads = gd_threads(P.kind, packed);
+    auto launch_with = [&](auto kernel, int slot, const auto& extra) -> int {
         if (!attr_set[dev][slot]) {
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GD_RING_BYTES + 1024) != cudaSuccess)
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring + 1024) != cudaSuccess)
                 return VITINT_ERR_CUDA;
             attr_set[dev][slot] = true;
         }
-        launch_kernel(kernel, dim3(grid), dim3(GD_THREADS), smem, st, map_a, map_b, P);
+        launch_kernel(kernel, dim3(grid), dim3(threads), smem, st, map_a, map_b, extra, P);
         return cuda_status(cudaGetLastError());
     };
+    auto launch = [&](auto kernel, int slot) -> int { return launch_with(kernel, slot, NoExtra{}); };
     auto by_operands = [&](auto small) -> int {
         constexpr bool S = decltype(small)::value;
-        constexpr int s0 = S ? 0 : 8;
+        constexpr int s0 = S ? 0 : 10;
+        if (P.kind == EK_QKV_NORM) {
+            NormExtra extra;
+            if (int rc = make_map(&extra.map_w, w, w_row_bytes, (uint64_t)P.N, 1, 1, w_pitch, w_pitch * P.N, w_pitch * P.N,
+                                  P.b_direct ? (uint32_t)BK : 16u * P.cb, (uint32_t)P.bn, P.b_direct != 0))
+                return rc;
+            return packed ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, true>, s0 + 8, extra)
+                          : launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false>, s0 + 9, extra);
+        }
         if (P.kind == EK_DEQUANT) {
             if (packed) return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, true>, s0) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, true>, s0 + 1);
             return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, false>, s0 + 2) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, false>, s0 + 3);

@@ -1,28 +1,39 @@
 // Quantizing LayerNorm of Section IV-C: the running statistics of Eq. 5 and the division- and
-// square-root-free comparator of Fig. 5(b), as two kernels.
+// square-root-free comparator of Fig. 5(b), in one kernel.
 //
-//   ln_running_stats_kernel    one thread per row walks the row in order:
-//                                delta = x_i - mu;  mu += delta / i;  S += delta * (x_i - mu)
-//                              every operation a single round-to-nearest fp32 one (no contraction), the
-//                              division by i exact-rounded through a reciprocal and one correction step.
-//                              Writes (mu, V = S + n*eps) per row.
-//   ln_compare_quantize_kernel level = Qn + number of references exceeded.  With d = x - mu (negated where
-//                              gamma < 0) the sign logic of the figure collapses into one comparison of
-//                              signed squares,  copysign(d*d, d) > V * r,  r = sgn(c) c^2 / n the caller's
-//                              signed reference.  The references of a column ascend, fp32 multiplication
-//                              by V > 0 keeps their order, so the comparisons are true up to some index
-//                              and false after it: the count is found by bisection (b comparisons for
-//                              2^b - 1 references) with the candidate references kept in registers.
+//   statistics  one thread per row walks the row in order:
+//                 delta = x_i - mu;  mu += delta / i;  S += delta * (x_i - mu)
+//               every operation a single round-to-nearest fp32 one (no contraction), the
+//               division by i exact-rounded through a reciprocal and one correction step.
+//   comparator  level = Qn + number of references exceeded.  With d = x - mu (negated where
+//               gamma < 0) the sign logic of the figure collapses into one comparison of
+//               signed squares,  copysign(d*d, d) > V * r,  r = sgn(c) c^2 / n the caller's
+//               signed reference.  The references of a column ascend, so the comparisons are true up to some
+//               index and false after it.  Folded from a uniform quantizer they are the signed squares of equally
+//               spaced points, so the index is guessed from d / sqrt(V) (two operations) and two comparisons around
+//               the guess, formed exactly as defined, prove it; where they do not, all references are compared.
+//
+// What bounds it.  The recurrence is a chain of five dependent fp32 operations per element (20 cycles, 768 elements: 8 us)
+// and cannot be split without changing the order of Eq. 5 and with it the bits; one CTA per SM walks all its rows at once, one
+// lane each, while TMA keeps the next chunks of columns coming and the other warps lay out the references.  Its levels it finds
+// afterwards with all warps, the rows coming from L2.  As two kernels -- statistics, then a bisection over references held in
+// registers, 42 instructions an element -- 12,608 x 768 took 39 us and 25,216 x 768 74 us; as one 25 and 38, of which the walk
+// 13 and 17.  (Requesting the next task's rows ahead of the present one's levels: no change.)
 #include "common.cuh"
 #include "ptx.cuh"
+#include "tile_ops.cuh"
 
 namespace vitint {
 namespace {
 
-constexpr int LNC_ROWS_PER_THREAD = 16;
-constexpr int LNC_BATCH = 4;            // rows whose loads are issued together
-
-constexpr int LNS_MAX_COLS = 4096;    // (float(i), RN(1/i)) pairs tabulated in shared memory
+constexpr int LNC_THREADS = 512, LNC_WARPS = LNC_THREADS / 32;
+constexpr int LNC_CHUNK = 64;                  // columns per staged chunk: two TMA boxes of 32, 128-byte swizzle (a lane reads its own
+                                               // row in 16-byte pieces without bank conflicts)
+constexpr int LNC_MAX_BUFFERS = 6;
+constexpr int LNC_MAX_ROWS = 192;              // rows a CTA walks at once (six warps)
+constexpr int LNC_SLAB = 768, LNC_QUARTER = LNC_SLAB / 4;     // columns whose references are in shared memory at a time
+constexpr int LNC_ROW_BATCH = 4;               // rows of one comparator task: their loads are issued together
+constexpr int LNS_MAX_COLS = 4096;
 
 // One step of Eq. 5 for element xi, i = fi: every operation a single rounded fp32 one.  The update of S
 // belonging to the PREVIOUS element (its delta in pd, its value in px; mu is still that element's mean) is
@@ -42,186 +53,290 @@ __device__ __forceinline__ void running_step(float xi, float fi, float r, float&
     px = xi;
 }
 
-// One warp per 32 rows, a thread walks one row -- but the row reaches the thread through shared memory: the warp
-// copies a 128-column chunk of its 32 rows with coalesced 16-byte asynchronous copies (lane l takes the l-th float4 of
-// every row: 512 contiguous bytes per row) into a [32][132]-float buffer, and each thread then reads its own row from
-// there (132 floats per row: the lanes' 16-byte reads fall on different bank groups).  Read straight from global
-// memory, every load instruction of the warp touched 32 different lines, and the load path took as long as the
-// dependent chain itself.  Two buffers: the next chunk is on its way while this one is walked.
-constexpr int LNS_CHUNK = 128;                 // columns per staged chunk
-constexpr int LNS_ROW_FLOATS = LNS_CHUNK + 4;  // padded row of the staging buffer
-__global__ void __launch_bounds__(32)
-ln_running_stats_kernel(const float* __restrict__ x, int64_t rows, int cols, int64_t ldx, float n_eps,
-                        float* __restrict__ stats) {
-    // (float(i), RN(1/i)) for every column: one broadcast shared-memory read per element instead of a
-    // conversion and a reciprocal (both run on the quarter-rate unit) in front of the dependent chain
-    extern __shared__ __align__(16) float2 inv_tab[];
-    float* const stage = reinterpret_cast<float*>(inv_tab + ((cols + 1) & ~1));          // 16-byte aligned behind the table
-    const int lane = threadIdx.x;
-    for (int i = lane; i < cols; i += 32) {
-        const float fi = (float)(i + 1);
-        inv_tab[i] = make_float2(fi, __frcp_rn(fi));
-    }
-    __syncwarp();
-    grid_dependency_wait();        // x may come from the previous kernel of the stream
-    grid_dependency_launch();
-    const int64_t row0 = (int64_t)blockIdx.x * 32;
-    const int n_chunks = (cols + LNS_CHUNK - 1) / LNS_CHUNK;
-    auto request = [&](int c, float* buf) {
-        const int col = c * LNS_CHUNK + lane * 4;
-        if (col < cols) {                                                              // cols is a multiple of 4
-#pragma unroll 8
-            for (int r = 0; r < 32; ++r) {
-                const int64_t row = row0 + r < rows ? row0 + r : rows - 1;             // a surplus row repeats the last one
-                ptx::cp_async16(ptx::smem_addr(buf + r * LNS_ROW_FLOATS + lane * 4), x + row * ldx + col);
-            }
-        }
-        ptx::cp_async_commit();
-    };
-    float mu = 0.0f, S = 0.0f, pd = 0.0f, px = 0.0f;
-    request(0, stage);
-    for (int c = 0; c < n_chunks; ++c) {
-        float* const buf = stage + (c & 1) * 32 * LNS_ROW_FLOATS;
-        if (c + 1 < n_chunks) {
-            request(c + 1, stage + ((c + 1) & 1) * 32 * LNS_ROW_FLOATS);
-            ptx::cp_async_wait<1>();
-        } else {
-            ptx::cp_async_wait<0>();
-        }
-        __syncwarp();                                                                  // every lane's copies have landed
-        const float4* mine = reinterpret_cast<const float4*>(buf + lane * LNS_ROW_FLOATS);
-        const float2* tab = inv_tab + c * LNS_CHUNK;
-        const int nv = (cols - c * LNS_CHUNK < LNS_CHUNK ? cols - c * LNS_CHUNK : LNS_CHUNK) >> 2;
-        if (nv == LNS_CHUNK / 4) {
-#pragma unroll 8
-            for (int v = 0; v < LNS_CHUNK / 4; ++v) {
-                const float4 e4 = mine[v];
-                const float e[4] = {e4.x, e4.y, e4.z, e4.w};
+struct LncShape {
+    int cols, rows_cta, nbuf;
+    uint32_t off_ref, off_col, off_stage, buf_bytes;
+};
+
+// References of columns slab0 .. slab0 + 767 in shared memory, [NT + 2][768] with -inf and +inf around them and column c at
+// (c % 4) * 192 + c / 4, so that the lanes of a warp (four neighbouring columns each) read different banks whatever their
+// levels; and per column inv, off and the sign of the gain, for the guess  count ~ rint(NT * sat((x - mu) / sqrt(V) * inv + off)):
+// with the references as signed roots rho, inv = (NT - 1) / (rho_last - rho_first) / NT (negated for a negative gain),
+// off = (1/2 - rho_first * (NT - 1) / (rho_last - rho_first)) / NT.
+template <int NT>
+__device__ __forceinline__ void lnc_load_refs(float* s_ref, float* s_col, const LncShape& sh, int slab0, const float* __restrict__ refs,
+                                              const uint8_t* __restrict__ flip, int t0, int nthreads) {
+    const int n = min(LNC_SLAB, sh.cols - slab0);
+    for (int c = t0; c < n; c += nthreads) {
+        float* const dst = s_ref + (c & 3) * LNC_QUARTER + (c >> 2);
+        float first = 0.0f, last = 0.0f;
+        dst[0] = -INFINITY;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 t = tab[4 * v + j];
-                    running_step(e[j], t.x, t.y, mu, S, pd, px);
-                }
-            }
-        } else {
-            for (int v = 0; v < nv; ++v) {
-                const float4 e4 = mine[v];
-                const float e[4] = {e4.x, e4.y, e4.z, e4.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 t = tab[4 * v + j];
-                    running_step(e[j], t.x, t.y, mu, S, pd, px);
-                }
-            }
+        for (int t = 0; t < NT; ++t) {
+            const float r = __ldg(refs + (int64_t)(slab0 + c) * NT + t);
+            if (t == 0) first = r;
+            if (t == NT - 1) last = r;
+            dst[(t + 1) * LNC_SLAB] = r;
         }
-        __syncwarp();                                                                  // the buffer is free for the chunk after next
-    }
-    S = __fadd_rn(S, __fmul_rn(pd, __fadd_rn(px, -mu)));      // the last element's term
-    const int64_t row = row0 + lane;
-    if (row < rows) {
-        stats[2 * row] = mu;
-        stats[2 * row + 1] = __fadd_rn(S, n_eps);
+        dst[(NT + 1) * LNC_SLAB] = INFINITY;
+        const float rho0 = copysignf(sqrtf(fabsf(first)), first), rho1 = copysignf(sqrtf(fabsf(last)), last);
+        float inv = __fdividef((float)(NT - 1), rho1 - rho0);
+        if (!(inv < 1e30f)) inv = 0.0f;
+        const float sgn = (flip && __ldg(flip + slab0 + c)) ? -1.0f : 1.0f;
+        s_col[c] = inv * sgn * (1.0f / NT);
+        s_col[LNC_SLAB + c] = (0.5f - rho0 * inv) * (1.0f / NT);
+        s_col[2 * LNC_SLAB + c] = sgn;
     }
 }
 
-// Block (32, 4): lane = four adjacent columns, threadIdx.y = a group of LNC_ROWS_PER_THREAD rows.
 template <int BITS, int C>
-__global__ void __launch_bounds__(128)
-ln_compare_quantize_kernel(const float* __restrict__ x, int64_t rows, int cols, int64_t ldx,
-                           const float* __restrict__ refs, const uint8_t* __restrict__ flip,
-                           const float* __restrict__ stats, uint8_t* __restrict__ out, int64_t pitch, int qn) {
-    grid_dependency_wait();
-    grid_dependency_launch();
+__global__ void __launch_bounds__(LNC_THREADS, 1)
+ln_compare_quantize_kernel(const __grid_constant__ CUtensorMap map_x, const float* __restrict__ x, int64_t rows, int64_t ldx,
+                           const float* __restrict__ refs, const uint8_t* __restrict__ flip, float n_eps, float* __restrict__ stats,
+                           uint8_t* __restrict__ out, int64_t pitch, int qn, const __grid_constant__ LncShape sh) {
+    extern __shared__ uint8_t lnc_raw[];
+    __shared__ float2 s_stat[LNC_MAX_ROWS];                     // (mu, V) of the CTA's rows
+    __shared__ uint64_t full[LNC_MAX_BUFFERS], empty[LNC_MAX_BUFFERS];
+    __shared__ int abort_flag;
     constexpr int NT = (1 << BITS) - 1;
     constexpr int LANES_PER_WORD = 8 / C;                       // lanes whose 4 codes share one 32-bit word
-    const int lane = threadIdx.x;
-    const int col = (blockIdx.x * 32 + lane) * 4;
-    const bool col_ok = col < cols;                             // cols is a multiple of 4
-    float r[4][NT];
-    float sgn[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        sgn[j] = (col_ok && flip && flip[col + j]) ? -1.0f : 1.0f;
-#pragma unroll
-        for (int t = 0; t < NT; ++t) r[j][t] = col_ok ? __ldg(refs + (int64_t)(col + j) * NT + t) : 0.0f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint8_t* const smem = lnc_raw + ((1024u - (ptx::smem_addr(lnc_raw) & 1023u)) & 1023u);
+    float2* const tab = reinterpret_cast<float2*>(smem);        // (float(i), RN(1/i)) of every column
+    float* const s_ref = reinterpret_cast<float*>(smem + sh.off_ref);
+    float* const s_col = reinterpret_cast<float*>(smem + sh.off_col);
+    uint8_t* const stage = smem + sh.off_stage;
+    const int cols = sh.cols, nbuf = sh.nbuf;
+    const int walkers = (sh.rows_cta + 31) / 32;
+
+    if (threadIdx.x == 0) {
+        abort_flag = 0;
+        for (int b = 0; b < nbuf; ++b) {
+            ptx::mbar_init(ptx::smem_addr(&full[b]), 1);
+            ptx::mbar_init(ptx::smem_addr(&empty[b]), (uint32_t)walkers);
+        }
+        ptx::fence_mbar_init();
+        ptx::fence_proxy_async_smem();
     }
+    for (int i = threadIdx.x; i < cols; i += LNC_THREADS) {
+        const float fi = (float)(i + 1);
+        tab[i] = make_float2(fi, __frcp_rn(fi));
+    }
+    __syncthreads();
+    grid_dependency_wait();        // x may come from the previous kernel of the stream
+    grid_dependency_launch();
+    const int n_chunks = (cols + LNC_CHUNK - 1) / LNC_CHUNK;
     const int words_per_row = (int)(pitch / 4);
-    const int word = (blockIdx.x * 32 + lane) / LANES_PER_WORD;
-    const int64_t row0 = ((int64_t)blockIdx.y * 4 + threadIdx.y) * LNC_ROWS_PER_THREAD;
-    // Rows go in batches of LNC_BATCH: the loads of the next batch are in flight while this batch's levels are
-    // found (a single row per thread would leave too few bytes in flight to keep HBM busy).
-    float4 xb[LNC_BATCH], xb_next[LNC_BATCH];
-    float2 mb[LNC_BATCH], mb_next[LNC_BATCH];
-    auto load_batch = [&](int64_t first, float4 (&xv)[LNC_BATCH], float2 (&mv)[LNC_BATCH]) {
-#pragma unroll
-        for (int k = 0; k < LNC_BATCH; ++k) {
-            const int64_t row = first + k;
-            const bool ok = row < rows && row < row0 + LNC_ROWS_PER_THREAD;
-            mv[k] = ok ? __ldg(reinterpret_cast<const float2*>(stats) + row) : make_float2(0.f, 1.f);
-            xv[k] = (ok && col_ok) ? __ldg(reinterpret_cast<const float4*>(x + row * ldx + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    };
-    load_batch(row0, xb_next, mb_next);
-    for (int rb = 0; rb < LNC_ROWS_PER_THREAD; rb += LNC_BATCH) {
-        if (row0 + rb >= rows) break;                            // uniform across the warp
-#pragma unroll
-        for (int k = 0; k < LNC_BATCH; ++k) { xb[k] = xb_next[k]; mb[k] = mb_next[k]; }
-        load_batch(row0 + rb + LNC_BATCH, xb_next, mb_next);
-#pragma unroll
-      for (int k = 0; k < LNC_BATCH; ++k) {
-        const int64_t row = row0 + rb + k;
-        if (row >= rows) break;                                  // uniform across the warp
-        const float4 xv = xb[k];
-        const float mu = mb[k].x, V = mb[k].y;
-        const float e[4] = {xv.x, xv.y, xv.z, xv.w};
-        uint32_t bits = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float d = __fmul_rn(__fadd_rn(e[j], -mu), sgn[j]);        // exact sign change
-            const float ds = copysignf(__fmul_rn(d, d), d);
-            float cand[NT > 1 ? NT / 2 : 1];
-            int cnt = 0;
-            {
-                constexpr int half = (NT + 1) / 2;
-                const bool p = ds > __fmul_rn(V, r[j][half - 1]);
-                cnt = p ? half : 0;
-#pragma unroll
-                for (int i = 0; i < half - 1; ++i) cand[i] = p ? r[j][i + half] : r[j][i];
+    // a lane covers four columns; with sub-byte containers the words up to the pitch are written (as zero) past the last column
+    const int lanes_total = max(cols / 4, words_per_row * LANES_PER_WORD);
+    constexpr uint32_t FIELDS = 1u | (1u << C) | (1u << (2 * C)) | (1u << (3 * C));
+    const uint32_t qn_low = ((uint32_t)qn & ((1u << (C - 1)) - 1u)) * FIELDS, qn_top = ((uint32_t)qn & (1u << (C - 1))) * FIELDS;
+    int slab_in = -1;                                           // first column of the references in shared memory
+    int buf = 0;                                                // of the walkers and of the producer: next buffer and its phase
+    uint32_t ph = 0u;
+    bool ok = true;
+    for (int64_t row0 = (int64_t)blockIdx.x * sh.rows_cta; row0 < rows; row0 += (int64_t)gridDim.x * sh.rows_cta) {
+        const int n_rows = rows - row0 < sh.rows_cta ? (int)(rows - row0) : sh.rows_cta;
+        // ---- statistics ----
+        if (warp < walkers) {
+            float mu = 0.0f, S = 0.0f, pd = 0.0f, px = 0.0f;
+            const int my_row = min(warp * 32 + lane, sh.rows_cta - 1), r7 = my_row & 7;
+            for (int c = 0; c < n_chunks; ++c) {
+                const bool w = mbar_wait(ptx::smem_addr(&full[buf]), ph, &abort_flag);
+                if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
+                const uint8_t* mine = stage + (size_t)buf * sh.buf_bytes + my_row * 128;
+                const float4* t4 = reinterpret_cast<const float4*>(tab + c * LNC_CHUNK);   // two columns' pairs
+                const int box = sh.buf_bytes >> 1;
+                // four elements of the row and their (i, 1/i); the next four are read before these are walked
+                struct Four { float4 e, ta, tb; };
+                auto read = [&](int v) {
+                    return Four{*reinterpret_cast<const float4*>(mine + (v >> 3) * box + (((v & 7) ^ r7) << 4)), t4[2 * v], t4[2 * v + 1]};
+                };
+                const int nv = (cols - c * LNC_CHUNK < LNC_CHUNK ? cols - c * LNC_CHUNK : LNC_CHUNK) >> 2;
+                Four cur = read(0);
+#pragma unroll 4
+                for (int v = 0; v < nv; ++v) {
+                    const Four next = read(v + 1 < nv ? v + 1 : v);
+                    running_step(cur.e.x, cur.ta.x, cur.ta.y, mu, S, pd, px);
+                    running_step(cur.e.y, cur.ta.z, cur.ta.w, mu, S, pd, px);
+                    running_step(cur.e.z, cur.tb.x, cur.tb.y, mu, S, pd, px);
+                    running_step(cur.e.w, cur.tb.z, cur.tb.w, mu, S, pd, px);
+                    cur = next;
+                }
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&empty[buf]));
+                if (++buf == nbuf) { buf = 0; ph ^= 1u; }
             }
-#pragma unroll
-            for (int half = (NT + 1) / 4; half >= 1; half >>= 1) {
-                const bool p = ds > __fmul_rn(V, cand[half - 1]);
-                cnt += p ? half : 0;
-#pragma unroll
-                for (int i = 0; i < half - 1; ++i) cand[i] = p ? cand[i + half] : cand[i];
+            if (ok && warp * 32 + lane < n_rows) {
+                S = __fadd_rn(S, __fmul_rn(pd, __fadd_rn(px, -mu)));                   // the last element's term
+                const float2 st = make_float2(mu, __fadd_rn(S, n_eps));
+                s_stat[my_row] = st;
+                reinterpret_cast<float2*>(stats)[row0 + my_row] = st;
             }
-            bits |= ((uint32_t)(qn + cnt) & ((1u << C) - 1u)) << (C * j);
+        } else if (warp == LNC_WARPS - 1) {
+            if (lane == 0) {
+                const uint32_t bytes = (uint32_t)sh.rows_cta * 128u;
+                int c = 0;
+                for (; c < n_chunks; ++c) {
+                    if (!mbar_wait(ptx::smem_addr(&empty[buf]), ph ^ 1u, &abort_flag)) { ok = false; break; }
+                    const uint32_t bar = ptx::smem_addr(&full[buf]), dst = ptx::smem_addr(stage) + (uint32_t)buf * sh.buf_bytes;
+                    const bool two = c * LNC_CHUNK + 32 < cols;
+                    ptx::mbar_arrive_expect_tx(bar, two ? 2u * bytes : bytes);
+                    ptx::tma_load_3d(dst, &map_x, bar, c * LNC_CHUNK, (int)row0, 0);
+                    if (two) ptx::tma_load_3d(dst + (sh.buf_bytes >> 1), &map_x, bar, c * LNC_CHUNK + 32, (int)row0, 0);
+                    if (++buf == nbuf) { buf = 0; ph ^= 1u; }
+                }
+                if (!ok) {
+                    // give the copies still in flight a bounded chance to land before the CTA exits
+                    for (int j = 0; j < nbuf; ++j)
+                        for (int spin = 0; spin < (1 << 20) && !ptx::mbar_try_wait(ptx::smem_addr(&full[j]), j < buf ? ph : ph ^ 1u); ++spin) {}
+                }
+            }
+            __syncwarp();
+        } else if (slab_in != 0) {
+            lnc_load_refs<NT>(s_ref, s_col, sh, 0, refs, flip, threadIdx.x - walkers * 32, LNC_THREADS - (walkers + 1) * 32);
         }
-        if (!col_ok) bits = 0;
-        // gather 8/C neighbouring lanes into one 32-bit word
-        if (C == 4) {
-            bits |= __shfl_xor_sync(0xffffffffu, bits, 1) << 16;
-        } else if (C == 2) {
-            bits |= __shfl_xor_sync(0xffffffffu, bits, 1) << 8;
-            bits |= __shfl_xor_sync(0xffffffffu, bits, 2) << 16;
+        slab_in = 0;
+        if (!__syncthreads_and(ok ? 1 : 0)) return;
+
+        // ---- comparator ----
+        for (int slab0 = 0; slab0 < lanes_total * 4; slab0 += LNC_SLAB) {
+            if (slab0 != slab_in && slab0 < cols) {
+                __syncthreads();
+                lnc_load_refs<NT>(s_ref, s_col, sh, slab0, refs, flip, threadIdx.x, LNC_THREADS);
+                slab_in = slab0;
+                __syncthreads();
+            }
+            const int groups = (min(lanes_total - slab0 / 4, LNC_QUARTER) + 31) / 32;      // of 32 lanes
+            const int batches = (n_rows + LNC_ROW_BATCH - 1) / LNC_ROW_BATCH;
+            for (int task = warp; task < groups * batches; task += LNC_WARPS) {
+                const int batch = task / groups, grp = task - batch * groups;
+                const int ql = grp * 32 + lane;                                            // the lane's four columns within the slab
+                const int col = slab0 + ql * 4;
+                const bool col_ok = col < cols;
+                const int rb = batch * LNC_ROW_BATCH;
+                const float* xp = x + (row0 + rb) * ldx + col;
+                float4 xb[LNC_ROW_BATCH];
+#pragma unroll
+                for (int k = 0; k < LNC_ROW_BATCH; ++k, xp += ldx)
+                    xb[k] = (col_ok && rb + k < n_rows) ? __ldg(reinterpret_cast<const float4*>(xp)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const int qs = col_ok ? ql : 0;
+                const float4 inv4 = *reinterpret_cast<const float4*>(s_col + 4 * qs), off4 = *reinterpret_cast<const float4*>(s_col + LNC_SLAB + 4 * qs);
+                const float4 sgn4 = *reinterpret_cast<const float4*>(s_col + 2 * LNC_SLAB + 4 * qs);
+                const float inv[4] = {inv4.x, inv4.y, inv4.z, inv4.w}, off[4] = {off4.x, off4.y, off4.z, off4.w};
+                const f32x2 sgn[2] = {f2_pack(sgn4.x, sgn4.y), f2_pack(sgn4.z, sgn4.w)};
+                // the guess arrives as 1.5*2^23 + count: times the row of references it is an address, the constant folded into the base
+                const uint32_t ref0 = ptx::smem_addr(s_ref) + 4u * (uint32_t)qs - 0x4B400000u * (4u * LNC_SLAB);
+                uint8_t* o = out + (row0 + rb) * pitch + (int64_t)((slab0 / 4 + ql) / LANES_PER_WORD) * 4;
+                const bool writes = (lane % LANES_PER_WORD) == 0 && ql < LNC_QUARTER && (slab0 / 4 + ql) / LANES_PER_WORD < words_per_row;
+#pragma unroll
+                for (int k = 0; k < LNC_ROW_BATCH; ++k, o += pitch) {
+                    if (rb + k >= n_rows) break;                                           // uniform across the warp
+                    const float2 st = s_stat[rb + k];
+                    const float V = st.y;
+                    const f32x2 nm2 = f2_dup(-st.x), rs2 = f2_dup(rsqrtf(V)), V2 = f2_dup(V);
+                    const f32x2 xs[2] = {f2_pack(xb[k].x, xb[k].y), f2_pack(xb[k].z, xb[k].w)};
+                    float ds[4];
+                    uint32_t g[4];
+                    bool proven = true;
+#pragma unroll
+                    for (int p = 0; p < 2; ++p) {
+                        const f32x2 delta = f2_add(xs[p], nm2), d = f2_mul(delta, sgn[p]);                 // exact sign change
+                        float d0, d1, q0, q1, u0, u1, g0, g1, l0, l1, h0, h1;
+                        f2_unpack(d, d0, d1);
+                        f2_unpack(f2_mul(d, d), q0, q1);
+                        ds[2 * p] = copysignf(q0, d0);
+                        ds[2 * p + 1] = copysignf(q1, d1);
+                        f2_unpack(f2_mul(delta, rs2), u0, u1);
+                        u0 = __saturatef(fmaf(u0, inv[2 * p], off[2 * p]));
+                        u1 = __saturatef(fmaf(u1, inv[2 * p + 1], off[2 * p + 1]));
+                        f2_unpack(f2_fma(f2_pack(u0, u1), f2_dup((float)NT), f2_dup(12582912.0f)), g0, g1);
+                        g[2 * p] = __float_as_uint(g0);
+                        g[2 * p + 1] = __float_as_uint(g1);
+                        const uint32_t r0 = g[2 * p] * (4u * LNC_SLAB) + (ref0 + 8u * p * LNC_QUARTER);
+                        const uint32_t r1 = g[2 * p + 1] * (4u * LNC_SLAB) + (ref0 + (8u * p + 4u) * LNC_QUARTER);
+                        f2_unpack(f2_mul(V2, f2_pack(ptx::ld_shared_f32(r0), ptx::ld_shared_f32(r1))), l0, l1);   // reference count - 1
+                        f2_unpack(f2_mul(V2, f2_pack(ptx::ld_shared_f32(r0 + 4 * LNC_SLAB), ptx::ld_shared_f32(r1 + 4 * LNC_SLAB))), h0, h1);
+                        proven = proven && ds[2 * p] > l0 && !(ds[2 * p] > h0) && ds[2 * p + 1] > l1 && !(ds[2 * p + 1] > h1);
+                    }
+                    uint32_t n = (g[0] + (g[1] << C) + (g[2] << (2 * C)) + (g[3] << (3 * C))) -
+                                 0x4B400000u * (1u + (1u << C) + (1u << (2 * C)) + (1u << (3 * C)));
+                    if (!proven && col_ok) {
+                        n = 0;
+                        const float* my_ref = s_ref + qs;
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            uint32_t cnt = 0;
+#pragma unroll 1
+                            for (int t = 1; t <= NT; ++t) cnt += ds[j] > __fmul_rn(V, my_ref[j * LNC_QUARTER + t * LNC_SLAB]) ? 1u : 0u;
+                            n |= cnt << (C * j);
+                        }
+                    }
+                    // counts to levels: Qn added to each field (no field overflows: its low bits, then its top bit by an exclusive or)
+                    uint32_t bits = col_ok ? (n + qn_low) ^ qn_top : 0u;
+                    // gather 8/C neighbouring lanes into one 32-bit word
+                    if (C == 4) {
+                        bits |= __shfl_xor_sync(0xffffffffu, bits, 1) << 16;
+                    } else if (C == 2) {
+                        bits |= __shfl_xor_sync(0xffffffffu, bits, 1) << 8;
+                        bits |= __shfl_xor_sync(0xffffffffu, bits, 2) << 16;
+                    }
+                    if (writes) *reinterpret_cast<uint32_t*>(o) = bits;
+                }
+            }
         }
-        if ((lane % LANES_PER_WORD) == 0 && word < words_per_row)
-            *reinterpret_cast<uint32_t*>(out + row * pitch + (int64_t)word * 4) = bits;
-      }
+        __syncthreads();                                                                   // s_stat is free for the next rows
     }
+}
+
+inline uint32_t lnc_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
+
+template <int BITS, int C>
+int launch_ln_compare(cudaStream_t st, const float* x, int64_t rows, int cols, int64_t ldx, const float* refs, const uint8_t* flip,
+                      float n_eps, float* stats, uint8_t* out, int64_t pitch, int qn) {
+    // all SMs, as many rounds as 192 rows a CTA make necessary, the rows spread evenly over them
+    const int64_t sms = sm_count(), rounds = (rows + sms * LNC_MAX_ROWS - 1) / (sms * LNC_MAX_ROWS);
+    LncShape sh{};
+    sh.cols = cols;
+    sh.rows_cta = (int)((rows + sms * rounds - 1) / (sms * rounds));
+    sh.rows_cta = sh.rows_cta < 8 ? 8 : sh.rows_cta;
+    sh.off_ref = lnc_up((uint32_t)cols * 8u, 16);
+    sh.off_col = sh.off_ref + (uint32_t)((1 << BITS) + 1) * LNC_SLAB * 4u;
+    sh.off_stage = lnc_up(sh.off_col + 3u * LNC_SLAB * 4u, 1024);
+    sh.buf_bytes = 2u * lnc_up((uint32_t)sh.rows_cta * 128u, 1024);
+    const uint32_t budget = 222u * 1024u;
+    sh.nbuf = (int)((budget - sh.off_stage) / sh.buf_bytes);
+    if (sh.nbuf > LNC_MAX_BUFFERS) sh.nbuf = LNC_MAX_BUFFERS;
+    if (sh.nbuf < 2) return VITINT_ERR_UNSUPPORTED;
+    const size_t smem = sh.off_stage + (size_t)sh.nbuf * sh.buf_bytes + 1024;
+    const int dev = current_device();
+    if (dev < 0) return VITINT_ERR_CUDA;
+    static bool attr_set[MAX_DEVICES] = {};
+    if (!attr_set[dev]) {
+        if (cudaFuncSetAttribute(ln_compare_quantize_kernel<BITS, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)budget + 1024) != cudaSuccess)
+            return VITINT_ERR_CUDA;
+        attr_set[dev] = true;
+    }
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return VITINT_ERR_CUDA;
+    CUtensorMap map_x;
+    cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, 1}, strides[2] = {(cuuint64_t)ldx * 4, (cuuint64_t)ldx * 4 * (cuuint64_t)rows};
+    cuuint32_t box[3] = {32, (cuuint32_t)sh.rows_cta, 1}, estr[3] = {1, 1, 1};
+    if (fn(&map_x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(x), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return VITINT_ERR_CUDA;
+    const int64_t ctas = (rows + sh.rows_cta - 1) / sh.rows_cta;
+    launch_kernel(ln_compare_quantize_kernel<BITS, C>, dim3((unsigned)(ctas < sms ? ctas : sms)), dim3(LNC_THREADS), smem, st, map_x, x, rows,
+                  ldx, refs, flip, n_eps, stats, out, pitch, qn, sh);
+    return cuda_status(cudaGetLastError());
 }
 
 template <int BITS>
-int launch_ln_compare(int c, dim3 grid, cudaStream_t st, const float* x, int64_t rows, int cols, int64_t ldx,
-                      const float* refs, const uint8_t* flip, const float* stats, uint8_t* out, int64_t pitch, int qn) {
-    const dim3 block(32, 4);
-    if (c == 2)
-        launch_kernel(ln_compare_quantize_kernel<BITS, 2>, grid, block, 0, st, x, rows, cols, ldx, refs, flip, stats, out, pitch, qn);
-    else if (c == 4)
-        launch_kernel(ln_compare_quantize_kernel<BITS, 4>, grid, block, 0, st, x, rows, cols, ldx, refs, flip, stats, out, pitch, qn);
-    else
-        launch_kernel(ln_compare_quantize_kernel<BITS, 8>, grid, block, 0, st, x, rows, cols, ldx, refs, flip, stats, out, pitch, qn);
-    return cuda_status(cudaGetLastError());
+int launch_ln_compare_bits(int c, cudaStream_t st, const float* x, int64_t rows, int cols, int64_t ldx, const float* refs,
+                           const uint8_t* flip, float n_eps, float* stats, uint8_t* out, int64_t pitch, int qn) {
+    if (c == 2) return launch_ln_compare<BITS, 2>(st, x, rows, cols, ldx, refs, flip, n_eps, stats, out, pitch, qn);
+    if (c == 4) return launch_ln_compare<BITS, 4>(st, x, rows, cols, ldx, refs, flip, n_eps, stats, out, pitch, qn);
+    return launch_ln_compare<BITS, 8>(st, x, rows, cols, ldx, refs, flip, n_eps, stats, out, pitch, qn);
 }
 
 }  // namespace
@@ -238,28 +353,15 @@ extern "C" int vitint_layernorm_compare_quantize(const float* x, int64_t rows, i
     if (!(n_eps > 0.0f && n_eps < INFINITY)) return VITINT_ERR_INVALID_ARG;
     if (out->bits == 8 || cols % 4 != 0 || cols > LNS_MAX_COLS) return VITINT_ERR_UNSUPPORTED;
     if (!aligned16(x) || ldx % 4 != 0 || (reinterpret_cast<uintptr_t>(stats) & 7u) != 0) return VITINT_ERR_ALIGNMENT;
+    if (rows > 0x7fffffff) return VITINT_ERR_UNSUPPORTED;
     const int c = codes_container(out);
-    // one lane covers four columns; with sub-byte containers 8/c lanes share an output word, and the words up
-    // to the pitch are written (as zero) by the lanes past the last column
-    const int64_t lanes_cols = cols / 4, lanes_pitch = (out->pitch_bytes / 4) * (8 / c);
-    const int64_t lanes = lanes_cols > lanes_pitch ? lanes_cols : lanes_pitch;
     int qn, qp;
     code_range(out->bits, out->is_signed, &qn, &qp);
     cudaStream_t st = (cudaStream_t)stream;
-    const size_t stats_smem = (size_t)((cols + 1) & ~(int64_t)1) * sizeof(float2) + 2 * 32 * LNS_ROW_FLOATS * sizeof(float);
-    if (stats_smem > 48 * 1024 &&
-        cudaFuncSetAttribute(ln_running_stats_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stats_smem) != cudaSuccess)
-        return VITINT_ERR_CUDA;
-    launch_kernel(ln_running_stats_kernel, dim3((unsigned)((rows + 31) / 32)), dim3(32), stats_smem, st, x, rows, (int)cols, ldx,
-                  n_eps, stats);
-    if (int rc = cuda_status(cudaGetLastError())) return rc;
-    const int64_t row_groups = (rows + 4 * LNC_ROWS_PER_THREAD - 1) / (4 * LNC_ROWS_PER_THREAD);
-    if (row_groups > 65535) return VITINT_ERR_UNSUPPORTED;
-    const dim3 grid((unsigned)((lanes + 31) / 32), (unsigned)row_groups);
     uint8_t* o = (uint8_t*)out->data;
     switch (out->bits) {
-        case 2: return launch_ln_compare<2>(c, grid, st, x, rows, (int)cols, ldx, refs, flip, stats, o, out->pitch_bytes, qn);
-        case 3: return launch_ln_compare<3>(c, grid, st, x, rows, (int)cols, ldx, refs, flip, stats, o, out->pitch_bytes, qn);
-        default: return launch_ln_compare<4>(c, grid, st, x, rows, (int)cols, ldx, refs, flip, stats, o, out->pitch_bytes, qn);
+        case 2: return launch_ln_compare_bits<2>(c, st, x, rows, (int)cols, ldx, refs, flip, n_eps, stats, o, out->pitch_bytes, qn);
+        case 3: return launch_ln_compare_bits<3>(c, st, x, rows, (int)cols, ldx, refs, flip, n_eps, stats, o, out->pitch_bytes, qn);
+        default: return launch_ln_compare_bits<4>(c, st, x, rows, (int)cols, ldx, refs, flip, n_eps, stats, o, out->pitch_bytes, qn);
     }
 }

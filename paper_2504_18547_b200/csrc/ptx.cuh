@@ -60,6 +60,12 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
     return ok != 0;
 }
 
+__device__ __forceinline__ float ld_shared_f32(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+    return v;
+}
+
 // Asynchronous 16-byte copy global -> shared by the calling thread (both addresses 16-byte aligned),
 // grouped and awaited per thread.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {

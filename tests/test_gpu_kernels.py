@@ -193,3 +193,81 @@ def test_linear_packed_large_sums():
     y = vt.vitint_linear(to_codes(qx, 4, True), 0.75, to_codes(qw, 4, True), dev(s_w), None, vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
     want = vo.epilogue_dequant(vo.matmul_i32(qx, qw), np.float32(0.75), s_w)
     assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+# ---- comparator LayerNorm: column slabs, staged chunks and rounds of rows; references no uniform quantizer would give ------
+def compare_case(rows, cols, bits, seed, refs=None):
+    x = si.normal(seed, (rows, cols), 0.3, 1.7)
+    g, b = si.normal(seed + 1, (cols,), 1.0, 0.02), si.normal(seed + 2, (cols,), 0.0, 0.02)
+    g[::3] *= -1
+    step = si.gaussian_lsq_step(1.0, bits)
+    n_eps = float(np.float32(np.float64(cols) * np.float64(np.float32(1e-6))))
+    r, f = vt.fold_layernorm_references(g, b, step, bits, True, cols)
+    return x, (r if refs is None else refs(r)), f, n_eps
+
+
+def compare_reference(x, refs, flip, n_eps, bits):
+    """The definition: Eq. 5 in fp32, then the count of references exceeded."""
+    mu, s = np.zeros(x.shape[0], np.float32), np.zeros(x.shape[0], np.float32)
+    for i in range(x.shape[1]):
+        delta = x[:, i] - mu
+        mu = mu + delta / np.float32(i + 1)
+        s = s + delta * (x[:, i] - mu)
+    v = s + np.float32(n_eps)
+    d = (x - mu[:, None]) * np.where(flip, np.float32(-1), np.float32(1))
+    ds = np.copysign(d * d, d)
+    cnt = np.zeros(x.shape, np.int16)
+    with np.errstate(invalid="ignore"):
+        for t in range(refs.shape[1]):
+            cnt += ds > v[:, None] * refs[:, t]
+    return cnt - (1 << (bits - 1))
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 4), (7, 64), (33, 68), (300, 772), (149, 1540), (28500, 64)])
+@pytest.mark.parametrize("bits,cont", [(2, 0), (3, 8), (4, 0), (4, 8)])
+def test_compare_layernorm_tiling(rows, cols, bits, cont):
+    x, refs, flip, n_eps = compare_case(rows, cols, bits, 400 + cols)
+    out = vt.Codes.empty(rows, cols, bits, True, container=cont)
+    out.data.fill_(0xA5)
+    got, _ = vt.vitint_layernorm_compare_quantize(dev(x), dev(refs), dev(flip), n_eps, bits, True, out=out)
+    assert np.array_equal(from_codes(got), compare_reference(x, refs, flip, n_eps, bits)) and padding_is_zero(got)
+
+
+@pytest.mark.parametrize("warp", ["squeezed", "equal", "huge"])
+def test_compare_layernorm_references_that_are_not_uniform(warp):
+    """Ascending references for which the count cannot be guessed: it is found all the same."""
+    def refs(r):
+        if warp == "equal":
+            return np.repeat(r[:, 7:8], r.shape[1], axis=1)
+        if warp == "huge":
+            return np.sort(r * np.float32(1e30), axis=1)
+        return np.sort((np.sign(r) * np.abs(r) ** 3 * 1e3).astype(np.float32), axis=1)
+    x, refs_, flip, n_eps = compare_case(90, 256, 4, 450, refs)
+    got, _ = vt.vitint_layernorm_compare_quantize(dev(x), dev(refs_), dev(flip), n_eps, 4, True)
+    assert np.array_equal(from_codes(got), compare_reference(x, refs_, flip, n_eps, 4))
+
+
+@pytest.mark.parametrize("M,heads,bits", [(1, 1, 2), (129, 3, 4), (300, 5, 3), (2000, 7, 4)])
+@pytest.mark.parametrize("packed", [False, True])
+def test_qkv_norm_tiles_and_references(M, heads, bits, packed):
+    """Segments that end inside a tile, packed operands, and references no uniform quantizer would give."""
+    D, K = 64 * heads, 96
+    qx, qw = rand_codes(461, (M, K), bits, True), rand_codes(462, (3 * D, K), bits, True)
+    acc = vo.matmul_i32(qx, qw)
+    s_w = (np.abs(si.normal(463, (3 * D,), 0.0, 0.01)) + 1e-3).astype(np.float32)
+    bias = si.normal(464, (3 * D,), 0.0, 0.05)
+    y = vo.epilogue_dequant(acc, np.float32(0.5), s_w, bias)
+    rf = [compare_case(2, 64, bits, 470 + k) for k in range(2)]
+    n_eps = rf[0][3]
+    alpha, beta = np.full(D, 0.3, np.float32), si.normal(465, (D,), 0.0, 0.3)
+    x, w = to_codes(qx, bits, True), to_codes(qw, bits, True)
+    if not packed:
+        x, w = byte_codes(qx, bits, True), byte_codes(qw, bits, True)
+    for odd in (False, True):
+        refs = [np.sort((np.sign(r) * np.abs(r) ** 3 * 1e3).astype(np.float32), axis=1) if odd else r for _, r, _, _ in rf]
+        flips = [f for _, _, f, _ in rf]
+        got, _ = vt.vitint_linear_qkv_norm(x, 0.5, w, dev(s_w), dev(bias), dev(np.stack(refs)), dev(np.stack(flips)), n_eps,
+                                           dev(alpha), dev(beta), bits)
+        want = [compare_reference(y[:, k * D:(k + 1) * D].reshape(M * heads, 64), refs[k], flips[k], n_eps, bits).reshape(M, D)
+                for k in range(2)] + [vo.epilogue_requant(acc[:, 2 * D:], alpha, beta, bits, True)]
+        assert np.array_equal(from_codes(got), np.concatenate(want, axis=1)) and padding_is_zero(got)
