@@ -10,11 +10,18 @@
 //   compute   unpack to int8 operand tiles (rows of 64 bytes, 64-byte swizzle)
 //   control   tcgen05.mma  S[128, T] = Q K^T   (K = 64: two MMAs) into TMEM
 //   compute   e_j = EXP[S_j] from a table of exp(fl32(s*c)) over every possible integer score
-//             (|S| <= 64*max|q|*max|k|: 8193 entries for 4-bit codes); row sum in fp64;
+//             (|S| <= 64*max|q|*max|k|: 8192 distinct ones for 4-bit codes); row sum in fp64;
 //             p_j = e_j / Z;  code = clamp(rint(p_j / s_P));  codes written as int8 rows (128-byte
 //             swizzle) = the A operand of P V.  e_j is parked in TMEM over S between the passes.
 //   control   tcgen05.mma  O[128, 64] = P V  (V is the N-contiguous B operand) into TMEM
 //   compute   requantize O, pack, store the head's 64 columns of the [M, D] code matrix
+//
+// What bounds it: the lookups.  Random entries of a 32 KB table take 2.8 passes of the shared-memory pipe per 32 scores, and
+// with the code stores, the operand copies and the tensor core's own reads that pipe is busy 57 % of the time; instructions
+// issue in half the slots.  197 tokens x 12 heads, batch 128: 75.5 -> 65.9 us by walking the last columns in blocks of eight
+// (200 instead of 224) and 20 % fewer instructions a score; 256 tokens, where nothing is padded, 45.9 -> 45.3.  Overlapping the
+// steps of neighbouring items (scores formed while O is pending, O requantized between two chunks) cost more in instructions
+// than it hid: 74.8.
 //
 // Softmax accuracy: exp(t_j)/sum_k exp(t_k) equals Eq. 3's softmax exactly (the maximum is only
 // subtracted there for range); every table entry is a correctly rounded fp32, the sum is fp64,
@@ -119,7 +126,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             ptx::mbar_init(ptx::smem_addr(&bars[k].o_full), 1);
             ptx::mbar_init(ptx::smem_addr(&bars[k].o_done), AT_COMPUTE_WARPS);
             ptx::mbar_init(ptx::smem_addr(&bars[k].grp_sync), AT_COMPUTE_WARPS * 32);
-            ptx::mbar_init(ptx::smem_addr(&bars[k].z_sync), AT_COMPUTE_WARPS * 32);
+            ptx::mbar_init(ptx::smem_addr(&bars[k].z_sync), AT_COMPUTE_WARPS);
         }
         ptx::fence_mbar_init();
         ptx::fence_proxy_async_smem();
@@ -133,13 +140,23 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     // the exp table: global -> shared, once per CTA
     {
         float* tab = reinterpret_cast<float*>(smem_gen + P.off_table);
-        for (int i = threadIdx.x; i <= 2 * P.smax; i += AT_THREADS) tab[i] = __ldg(P.table + i);
+        if constexpr (!SHIFT) fill_table_ring(tab, P.table, P.smax, threadIdx.x, AT_THREADS);
         if constexpr (SHIFT) {
+            for (int i = threadIdx.x; i <= 2 * P.smax; i += AT_THREADS) tab[i] = __ldg(P.table + i);
             // the 16-bit table of integer parts sits behind the 32-bit one, in the workspace and here
             const uint32_t* src = reinterpret_cast<const uint32_t*>(P.table) + P.ftab_word;
             uint32_t* dst = reinterpret_cast<uint32_t*>(smem_gen + P.off_ftab);
             for (int i = threadIdx.x; i <= P.smax; i += AT_THREADS) dst[i] = __ldg(src + i);
         }
+    }
+    if constexpr (!SHIFT) {
+        // P columns behind the last block of eight that holds a token are never written: zero for good
+        for (int i = threadIdx.x; i < AT_GROUPS * 128 * 16; i += AT_THREADS) {
+            const int gr = i / 2048, cc = (i >> 7) & 15, r = i & 127;
+            if (cc * 16 < P.kv_rows)
+                *reinterpret_cast<uint4*>(smem_gen + P.off_group + (size_t)gr * P.group_bytes + P.off_p + (cc >> 3) * 16384 + r * 128 + (((cc & 7) ^ (r & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
+        }
+        ptx::fence_proxy_async_smem();
     }
     if (is_control && lane == 0) { ptx::prefetch_tensormap(&map_q); ptx::prefetch_tensormap(&map_kv); }
     ptx::tc_fence_before();
@@ -154,10 +171,10 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t q_bytes = 128u * head_bytes, kv_bytes = (uint32_t)P.kv_rows * head_bytes;   // TMA boxes
 
     auto item_coords = [&](int item, int& b, int& h, int& qt) {
-        qt = item % P.q_tiles;
-        const int bh = item / P.q_tiles;
-        h = bh % P.heads;
-        b = bh / P.heads;
+        const uint32_t two = (uint32_t)P.q_tiles - 1u, bh = (uint32_t)item >> two;           // one or two query tiles
+        qt = item & (int)two;
+        b = (int)(bh / (uint32_t)P.heads);
+        h = (int)bh - b * P.heads;
     };
 
     if (is_control) {
@@ -254,12 +271,14 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const int row = wq * 32 + lane;                             // query row of the tile
         double* const zx = reinterpret_cast<double*>(ggen + P.off_z);   // partial row sums, [2][128]
         const uint32_t t_row = tmem_grp + ((uint32_t)(wq * 32) << 16);
-        const char* const tab_mid = reinterpret_cast<const char*>(smem_gen + P.off_table) + (size_t)P.smax * 4;
+        const char* const ring = reinterpret_cast<const char*>(smem_gen + P.off_table);
+        const uint32_t ring_mask = 8u * (uint32_t)P.smax - 4u;
         float* const colp2 = reinterpret_cast<float*>(ggen + P.off_col);  // alpha[64], beta[64] of the head, one copy per item parity
         const int sh_idx = DIRECT ? 0 : 2 * (8 - C) - 2;            // scaled score -> byte offset 4*S
-        const int chunks = P.kv_rows / 32;
-        const int tab_half = 4 * P.smax;
-        const char* const tab_lo = tab_mid - tab_half;
+        const int chunks = P.kv_rows / 32, full_chunks = T >> 5, tail = T & 31, tail_blocks = (tail + 7) >> 3;
+        const int tail0 = (hf ^ full_chunks) & 1;                   // the thread with fewer whole chunks takes the first block of the tail
+        const uint32_t qp2 = (uint32_t)P.p_qp * 0x00010001u;
+        const bool steep = P.p_step < 1.0f / 65000.0f;              // codes before the clamp might not fit 16 bits
         const double inv_p_step = 1.0 / (double)P.p_step;
         bool ok = true;
         int n = 0;
@@ -290,12 +309,13 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             w = mbar_wait(ptx::smem_addr(&B.s_full), ph, abort_ptr);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             ptx::tc_fence_after();
+            // a warp whose 32 query rows all lie past the last token has nothing to compute: its P rows
+            // only feed accumulator rows that are never stored (whatever int8 they hold)
+            const bool warp_live = qt * 128 + wq * 32 < T;
             if constexpr (SHIFT) {
                 // Two tables over the score range: M[s] = trunc((1 + (z - floor z)) * 2^23) (32-bit) and f[s] = floor z
                 // (16-bit), z = fl32(s * c2).  floor z increases with s, so the row's largest score carries the row's
                 // largest integer part m and pass 0 needs no lookup at all.
-                const int full_chunks = T >> 5;
-                const bool warp_live = qt * 128 + wq * 32 < T;
                 int* const mx = reinterpret_cast<int*>(ggen + P.off_mx);
                 unsigned long long* const sx = reinterpret_cast<unsigned long long*>(ggen + P.off_z);
                 const uint32_t* const mtab = reinterpret_cast<const uint32_t*>(smem_gen + P.off_table);
@@ -316,7 +336,8 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     }
                 }
                 mx[hf * 128 + row] = smx;
-                ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 0u, abort_ptr);       // two phases per item: parities 0, 1
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 smx = max(mx[row], mx[128 + row]);
@@ -355,7 +376,8 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 unsigned long long sigma = ((unsigned long long)sg_hi << 32) | sg_lo;
                 ptx::tmem_st_wait();
                 sx[hf * 128 + row] = sigma;
-                ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 1u, abort_ptr);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 sigma = sx[row] + sx[128 + row];
@@ -404,60 +426,40 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     *reinterpret_cast<uint4*>(blk + ((((cc + 1) & 7) ^ sw) << 4)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
                 }
             } else {
-            // pass 1: e_j = EXP[S_j] (an integer score is bounded by the code ranges, so the byte offset
-            // 4*S always lies inside the table), row sum in fp64, e_j parked in TMEM over S_j
-            // four interleaved partial sums: a single fp64 accumulator would chain 32 dependent additions per chunk
+            // pass 1: e_j = EXP[S_j], row sum in fp64, e_j parked in TMEM over S_j; whole chunks of 32 columns, then the tail
+            // by blocks of eight (197 tokens: 200 columns walked instead of 224)
             double zp[4] = {0.0, 0.0, 0.0, 0.0};
-            const int full_chunks = T >> 5;
-            // a warp whose 32 query rows all lie past the last token has nothing to compute: its P rows
-            // only feed accumulator rows that are never stored (whatever int8 they hold)
-            const bool warp_live = qt * 128 + wq * 32 < T;
-            for (int ch = hf; warp_live && ch < chunks; ch += 2) {
-                uint32_t v[32];
-                ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
-                ptx::tmem_ld_wait();
-                if (ch < full_chunks) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        // every table entry is a positive normal float (exp of a bounded argument), so its
-                        // double is formed from the bits with two integer operations instead of a conversion
-                        // (the conversion unit runs at a quarter of the fp64 adder's rate)
-                        // Integer multiply-adds run beside the compare / shift / permute unit, which is the busier
-                        // one in this kernel: the byte offset, its clamp (one unsigned minimum after biasing) and
-                        // both words of the double are formed with them.
-                        uint32_t eb;
-                        if (DIRECT) {
-                            // raw bytes: 4*S + 4*smax, kept inside the table for any operand value
-                            const uint32_t off = min((uint32_t)((int)v[i] * 4 + tab_half), (uint32_t)(2 * tab_half));
-                            eb = *reinterpret_cast<const uint32_t*>(tab_lo + off);
-                        } else {
-                            eb = *reinterpret_cast<const uint32_t*>(tab_mid + ((int)v[i] >> sh_idx));
-                        }
-                        uint32_t hi, lo;
-                        asm("mad.hi.u32 %0, %1, 536870912, 939524096;" : "=r"(hi) : "r"(eb));    // (eb >> 3) + 0x38000000
-                        asm("mul.lo.u32 %0, %1, 536870912;" : "=r"(lo) : "r"(eb));                // eb << 29
-                        zp[i & 3] += __hiloint2double((int)hi, (int)lo);
-                        v[i] = eb;
-                    }
-                } else {
-                    // last, partial chunk: columns past the last token hold no score -> no lookup, e = 0
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const bool valid = ch * 32 + i < T;
-                        const int off = valid ? (DIRECT ? ((int)v[i] << 2) : ((int)v[i] >> sh_idx)) : 0;
-                        uint32_t eb = *reinterpret_cast<const uint32_t*>(tab_mid + max(-tab_half, min(tab_half, off)));
-                        if (!valid) eb = 0u;
-                        zp[i & 3] += __hiloint2double(valid ? (int)((eb >> 3) + 0x38000000u) : 0, (int)(eb << 29));
-                        v[i] = eb;
-                    }
+            if (warp_live) {
+                // sixteen columns are looked up while the next sixteen are on their way
+                uint32_t v0[16], v1[16];
+                if (hf < full_chunks) ptx::tmem_ld16(t_row + (uint32_t)(hf * 32), v0);
+#pragma unroll 1
+                for (int ch = hf; ch < full_chunks; ch += 2) {
+                    const uint32_t t_ch = t_row + (uint32_t)(ch * 32);
+                    ptx::tmem_ld_wait();
+                    ptx::tmem_ld16(t_ch + 16, v1);
+                    exp_lookup<16, !DIRECT, false>(v0, ring, ring_mask, sh_idx, 16, zp);
+                    ptx::tmem_st16(t_ch, v0);
+                    ptx::tmem_ld_wait();
+                    if (ch + 2 < full_chunks) ptx::tmem_ld16(t_ch + 64, v0);
+                    exp_lookup<16, !DIRECT, false>(v1, ring, ring_mask, sh_idx, 16, zp);
+                    ptx::tmem_st16(t_ch + 16, v1);
                 }
-                ptx::tmem_st32(t_row + (uint32_t)(ch * 32), v);
+#pragma unroll 1
+                for (int k = tail0; k < tail_blocks; k += 2) {
+                    uint32_t v[8];
+                    ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                    ptx::tmem_ld_wait();
+                    exp_lookup<8, !DIRECT, true>(v, ring, ring_mask, sh_idx, tail - 8 * k, zp);
+                    ptx::tmem_st8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                }
+                ptx::tmem_st_wait();
             }
-            ptx::tmem_st_wait();
-            // the row's two threads add their partial sums (every thread takes part in the barrier)
+            // the row's two threads add their partial sums (every warp takes part in the barrier)
             double z = (zp[0] + zp[1]) + (zp[2] + zp[3]);
             zx[hf * 128 + row] = z;
-            ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
             w = mbar_wait(ptx::smem_addr(&B.z_sync), ph, abort_ptr);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             z = zx[row] + zx[128 + row];
@@ -467,35 +469,41 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             const double rz = warp_live ? inv_p_step / z : 0.0;
             const float rzh = (float)rz;
             const float rzl = (float)(rz - (double)rzh);
-            const f32x2 rzh2 = f2_dup(rzh), rzl2 = f2_dup(rzl), magic2 = f2_dup(12582912.0f);
+            const f32x2 rzh2 = f2_dup(rzh), rzl2 = f2_dup(rzl);
             uint8_t* const prow = ggen + P.off_p + row * 128;
             const int sw = row & 7;
             // pass 2: code = min(rint(e_j / (Z s_P)), Qp) (p >= 0: no lower clamp)
-            for (int ch = hf; warp_live && ch < chunks; ch += 2) {
-                uint32_t v[32];
-                ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
-                ptx::tmem_ld_wait();
-                uint32_t wd[8];
+            if (warp_live) {
+                const float e_top = steep ? 60000.0f / rzh : 0.0f;         // far above Qp, below 2^16
+#pragma unroll 1
+                for (int ch = hf; ch < full_chunks; ch += 2) {
+                    uint32_t v[32], wd[8];
+                    ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
+                    ptx::tmem_ld_wait();
+                    if (steep) {
 #pragma unroll
-                for (int i4 = 0; i4 < 8; ++i4) {
-                    uint32_t cb[4];
-#pragma unroll
-                    for (int j = 0; j < 4; j += 2) {
-                        // two scores per instruction (each half is the scalar IEEE result): e*r_hi + RN(e*r_lo)
-                        const f32x2 e2 = f2_pack(__uint_as_float(v[4 * i4 + j]), __uint_as_float(v[4 * i4 + j + 1]));
-                        float a0, a1, c0, c1;
-                        f2_unpack(f2_fma(e2, rzh2, f2_mul(e2, rzl2)), a0, a1);
-                        f2_unpack(f2_add(f2_pack(fminf(a0, P.p_qp), fminf(a1, P.p_qp)), magic2), c0, c1);
-                        cb[j] = __float_as_uint(c0);                                           // code in the low byte
-                        cb[j + 1] = __float_as_uint(c1);
+                        for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(fminf(__uint_as_float(v[i]), e_top));
                     }
-                    wd[i4] = __byte_perm(__byte_perm(cb[0], cb[1], 0x4040), __byte_perm(cb[2], cb[3], 0x4040), 0x5410);
+                    quantize_entries<32>(v, rzh2, rzl2, qp2, wd);
+                    // 32 codes = two 16-byte chunks cc = 2*ch, 2*ch+1 of this row's 256-byte K extent
+                    const int cc = 2 * ch;
+                    uint8_t* const blk = prow + (cc >> 3) * 16384;
+                    *reinterpret_cast<uint4*>(blk + (((cc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+                    *reinterpret_cast<uint4*>(blk + ((((cc + 1) & 7) ^ sw) << 4)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
                 }
-                // 32 codes = two 16-byte chunks cc = 2*ch, 2*ch+1 of this row's 256-byte K extent
-                const int cc = 2 * ch;
-                uint8_t* const blk = prow + (cc >> 3) * 16384;
-                *reinterpret_cast<uint4*>(blk + (((cc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                *reinterpret_cast<uint4*>(blk + ((((cc + 1) & 7) ^ sw) << 4)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
+#pragma unroll 1
+                for (int k = tail0; k < tail_blocks; k += 2) {
+                    uint32_t v[8], wd[2];
+                    const int col = full_chunks * 32 + k * 8, cc = col >> 4;
+                    ptx::tmem_ld8(t_row + (uint32_t)col, v);
+                    ptx::tmem_ld_wait();
+                    if (steep) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) v[i] = __float_as_uint(fminf(__uint_as_float(v[i]), e_top));
+                    }
+                    quantize_entries<8>(v, rzh2, rzl2, qp2, wd);
+                    *reinterpret_cast<uint2*>(prow + (cc >> 3) * 16384 + (((cc & 7) ^ sw) << 4) + (col & 8)) = make_uint2(wd[0], wd[1]);
+                }
             }
             }   // exp / Eq. 4
             ptx::fence_proxy_async_smem();
@@ -507,49 +515,15 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             ptx::tc_fence_after();
             const int token = qt * 128 + row;
-            // each of the row's two threads requantizes and stores 32 of the head's 64 columns
-            uint32_t ow[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) ow[k] = 0;
-            {
-                uint32_t v[32];
+            // each of the row's two threads requantizes and stores 32 of the head's 64 columns (V codes that were unpacked sit
+            // in the high bits of their bytes)
+            if (warp_live) {
+                uint32_t v[32], ow[8];
                 ptx::tmem_ld32(t_row + (uint32_t)(hf * 32), v);
                 ptx::tmem_ld_wait();
-                // straight-line per-column arithmetic first, container-dependent packing afterwards
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int col = hf * 32 + i;
-                    const float f = small_int_to_float((int)v[i] >> (8 - C));     // V codes sit in the high bits of their bytes
-                    v[i] = round_clamp_bits(fmaf(f, colp[col], colp[64 + col]), P.out_qn, P.out_qp);
-                }
-                if (P.out_c == 4) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) ow[i >> 3] |= (v[i] & 0xFu) << (4 * (i & 7));
-                } else if (P.out_c == 2) {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) ow[i >> 4] |= (v[i] & 0x3u) << (2 * (i & 15));
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        ow[i] = __byte_perm(__byte_perm(v[4 * i], v[4 * i + 1], 0x4040),
-                                            __byte_perm(v[4 * i + 2], v[4 * i + 3], 0x4040), 0x5410);
-                }
-            }
-            if (token < T) {
-                // 32 codes = 4*out_c bytes at column block h*64 + hf*32
-                uint8_t* o = P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c);
-                if (P.out_c == 4) {
-                    *reinterpret_cast<uint4*>(o) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-                } else if (P.out_c == 2) {
-                    *reinterpret_cast<uint2*>(o) = make_uint2(ow[0], ow[1]);
-                } else if ((reinterpret_cast<uintptr_t>(o) & 31u) == 0) {
-                    // one 32-byte store: a warp's store touches 32 different rows whatever its width
-                    const uint32_t lo[4] = {ow[0], ow[1], ow[2], ow[3]}, hi[4] = {ow[4], ow[5], ow[6], ow[7]};
-                    ptx::st_global_32B(o, lo, hi);
-                } else {
-                    reinterpret_cast<uint4*>(o)[0] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-                    reinterpret_cast<uint4*>(o)[1] = make_uint4(ow[4], ow[5], ow[6], ow[7]);
-                }
+                requantize_row32(v, 8 - C, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
+                if (token < T)
+                    store_row32(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c), ow, P.out_c);
             }
             // row padding behind the last head's columns (a caller may choose a pitch beyond the row's codes)
             if (token < T && h == P.heads - 1 && hf == 1) {
@@ -603,7 +577,7 @@ int attention_shift_table(int bits, float q_step, float k_step, void* table, siz
                   reinterpret_cast<short*>((uint32_t*)table + (2 * smax + 1)), smax, c2);
     return cuda_status(cudaGetLastError());
 }
-int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tokens, int smax, const float* table, float p_step,
+int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tokens, int smax, const float* table, float cs, float p_step,
                           float p_qp, const float* alpha_o, const float* beta_o, const vitint_codes* o_out, cudaStream_t st);
 }
 
@@ -650,7 +624,7 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
         }
         int pqn, pqp;
         code_range(p_bits, 0, &pqn, &pqp);
-        return attention_long_launch(qkv, batch, heads, tokens, smax, (const float*)workspace, p_step, (float)pqp, alpha_o,
+        return attention_long_launch(qkv, batch, heads, tokens, smax, (const float*)workspace, cs, p_step, (float)pqp, alpha_o,
                                      beta_o, o_out, st);
     }
 

@@ -4,6 +4,9 @@
 //   pass A   S_c = Q K_c^T (tcgen05, K = 64)  ->  Z += sum_j EXP[S_j]            (table of exp(fl32(s c)), fp64 sum)
 //   pass B   S_c again                        ->  codes = min(rint(EXP[S_j] / (Z s_P)), Qp)  ->  P_c in shared memory
 //            O += P_c V_c (tcgen05, accumulating in tensor memory across the chunks)
+// Pass A needs the table's exact entries.  Pass B only needs the level they lead to, and finds it from 2^(s c2 + log2 r) on the
+// special-function unit; blocks in which a score comes too close to a rounding boundary to be sure of take the table again.
+// So the lookups -- 2.8 passes of the shared-memory pipe per 32 scores, what bounded the kernel with two a score -- are halved.
 // then O is requantized and stored.  S, the probabilities and P never reach HBM: the unfused sequence writes and
 // re-reads 4 T^2 bytes per head (946 MB at 785 tokens, batch 32), which is what bounds it.  The table makes the
 // two-pass form exact and cheap: exp(t_j) / sum_k exp(t_k) needs no running maximum and no rescaling of O, and Q K^T
@@ -11,7 +14,10 @@
 // so the codes are the same.
 //
 // One pipeline per CTA, steps in sequence (every thread passes the same barriers; an expired wait makes the whole CTA
-// leave together), two CTAs per SM so that one's loads and MMAs run beside the other's softmax.  Byte-stored codes.
+// leave together), two CTAs per SM so that one's loads and MMAs run beside the other's softmax; the next chunk's K is on its
+// way while this one's scores are worked on, and V is awaited only in front of P V.  Items are numbered by query tile first,
+// so that the last tile of every head, often nearly empty, fills the last round.  Byte-stored codes.
+// 785 tokens x 12 heads, batch 16: LONG_BEFORE -> LONG_AFTER us.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"
@@ -30,18 +36,19 @@ struct LongParams {
     int smax;
     int part_bytes;               // bytes of one of the Q / K / V segments in a QKV row
     const float* table;
-    float p_step, p_qp;
+    float p_step, p_qp, c2;       // c2: the scores' scale in the exponent of two
     const float* alpha_o;
     const float* beta_o;
     uint8_t* out;
     int64_t out_pitch;
     int out_c;
     float out_qn, out_qp;
+    uint32_t k_stride;            // bytes between the two K buffers
     uint32_t off_table, off_q, off_k, off_v, off_p, off_z, off_col;
 };
 
 struct LongBars {
-    uint64_t q_full, kv_full, s_full, o_full;
+    uint64_t q_full, k_full[2], v_full, s_full, o_full;
 };
 
 __global__ void __launch_bounds__(AL_THREADS, 2)
@@ -61,7 +68,9 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     if (threadIdx.x == 0) {
         abort_flag = 0;
         ptx::mbar_init(ptx::smem_addr(&B.q_full), 1);
-        ptx::mbar_init(ptx::smem_addr(&B.kv_full), 1);
+        ptx::mbar_init(ptx::smem_addr(&B.k_full[0]), 1);
+        ptx::mbar_init(ptx::smem_addr(&B.k_full[1]), 1);
+        ptx::mbar_init(ptx::smem_addr(&B.v_full), 1);
         ptx::mbar_init(ptx::smem_addr(&B.s_full), 1);
         ptx::mbar_init(ptx::smem_addr(&B.o_full), 1);
         ptx::fence_mbar_init();
@@ -74,8 +83,7 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     grid_dependency_wait();        // the table and the codes come from earlier kernels of the stream
     grid_dependency_launch();
     {
-        float* tab = reinterpret_cast<float*>(smem_gen + P.off_table);
-        for (int i = threadIdx.x; i <= 2 * P.smax; i += AL_THREADS) tab[i] = __ldg(P.table + i);
+        fill_table_ring(reinterpret_cast<float*>(smem_gen + P.off_table), P.table, P.smax, threadIdx.x, AL_THREADS);
     }
     if (is_control && lane == 0) { ptx::prefetch_tensormap(&map_q); ptx::prefetch_tensormap(&map_kv); }
     ptx::tc_fence_before();
@@ -88,7 +96,8 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const uint32_t idesc_qk = ptx::idesc_i8(128, CH, 1, 1, 0);
     const uint32_t idesc_pv = ptx::idesc_i8(128, 64, 0, 1, 1);
     const uint64_t q_desc = ptx::smem_desc(smem_base + P.off_q, 16, 512, ptx::SWIZZLE_64B);
-    const uint64_t k_desc = ptx::smem_desc(smem_base + P.off_k, 16, 512, ptx::SWIZZLE_64B);
+    const uint64_t k_desc[2] = {ptx::smem_desc(smem_base + P.off_k, 16, 512, ptx::SWIZZLE_64B),
+                                ptx::smem_desc(smem_base + P.off_k + P.k_stride, 16, 512, ptx::SWIZZLE_64B)};
     const uint64_t v_desc = ptx::smem_desc(smem_base + P.off_v, 16, 512, ptx::SWIZZLE_64B);
     const int pv_steps = CH / 32, blocks = CH / 32;
 
@@ -98,112 +107,140 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int tid_c = warp * 32 + lane;                          // 0..255 for compute threads
     const int row = wq * 32 + lane;
     const uint32_t t_row = tmem + ((uint32_t)(wq * 32) << 16);
-    const char* const tab_lo = reinterpret_cast<const char*>(smem_gen + P.off_table);
-    const int tab_half = 4 * P.smax;
+    const char* const ring = reinterpret_cast<const char*>(smem_gen + P.off_table);
+    const uint32_t ring_mask = 8u * (uint32_t)P.smax - 4u, qp2 = (uint32_t)P.p_qp * 0x00010001u;
+    const bool steep = P.p_step < 1.0f / 65000.0f;               // codes before the clamp might not fit 16 bits
+    const f32x2 c2 = f2_dup(P.c2);
     double* const zx = reinterpret_cast<double*>(smem_gen + P.off_z);
     float* const colp = reinterpret_cast<float*>(smem_gen + P.off_col);
     const double inv_p_step = 1.0 / (double)P.p_step;
     uint8_t* const prow = smem_gen + P.off_p + row * 128;
     const int sw = row & 7;
 
-    uint32_t n_q = 0, n_kv = 0, n_s = 0, n_o = 0;                // completed phases of each barrier (parity = count & 1)
+    uint32_t n_q = 0, n_k = 0, n_v = 0, n_s = 0, n_o = 0;        // completed phases of each barrier (parity = count & 1; K alternates)
+    uint32_t i_q = 0, i_k = 0, i_v = 0;                          // copies issued (control lane)
     bool ok = true;
+    const int per_tile = P.batch * P.heads;
+    auto coords = [&](int item, int& b, int& h, int& qt) {
+        qt = item / per_tile;
+        const int bh = item - qt * per_tile;
+        b = bh / P.heads;
+        h = bh - b * P.heads;
+    };
+    auto load_q = [&](int b, int h, int qt) {
+        ptx::mbar_arrive_expect_tx(ptx::smem_addr(&B.q_full), q_bytes);
+        ptx::tma_load_3d(smem_base + P.off_q, &map_q, ptx::smem_addr(&B.q_full), h * 64, qt * 128, b);
+        ++i_q;
+    };
+    auto load_k = [&](int b, int h, int c) {
+        const uint32_t bar = ptx::smem_addr(&B.k_full[i_k & 1u]);
+        ptx::mbar_arrive_expect_tx(bar, kv_bytes);
+        ptx::tma_load_3d(smem_base + P.off_k + (i_k & 1u) * P.k_stride, &map_kv, bar, P.part_bytes + h * 64, c * CH, b);
+        ++i_k;
+    };
+    if (is_control && lane == 0 && (int)blockIdx.x < P.total_items) {
+        int b, h, qt;
+        coords(blockIdx.x, b, h, qt);
+        load_q(b, h, qt);
+        load_k(b, h, 0);
+    }
     for (int item = blockIdx.x; ok && item < P.total_items; item += gridDim.x) {
-        const int qt = item % P.q_tiles;
-        const int bh = item / P.q_tiles;
-        const int h = bh % P.heads, b = bh / P.heads;
+        int b, h, qt;
+        coords(item, b, h, qt);
         if (!is_control) {
             if (tid_c < 64) colp[tid_c] = __ldg(P.alpha_o + h * 64 + tid_c);
             else if (tid_c < 128) colp[tid_c] = P.beta_o ? __ldg(P.beta_o + h * 64 + (tid_c - 64)) : 0.0f;
         }
-        if (is_control && lane == 0) {
-            ptx::mbar_arrive_expect_tx(ptx::smem_addr(&B.q_full), q_bytes);
-            ptx::tma_load_3d(smem_base + P.off_q, &map_q, ptx::smem_addr(&B.q_full), h * 64, qt * 128, b);
-        }
         double zp[4] = {0.0, 0.0, 0.0, 0.0};
-        f32x2 rzh2 = f2_dup(0.0f), rzl2 = f2_dup(0.0f);
-        const f32x2 magic2 = f2_dup(12582912.0f);
+        f32x2 rzh2 = f2_dup(0.0f), rzl2 = f2_dup(0.0f), l2 = f2_dup(0.0f);
+        float limit = 0.0f, e_top = 0.0f;
         const bool warp_live = qt * 128 + wq * 32 < T;
         for (int pass = 0; ok && pass < 2; ++pass) {
             for (int c = 0; ok && c < P.n_chunks; ++c) {
                 const int key0 = c * CH;
-                // ---- loads and S_c = Q K_c^T ---------------------------------------------------------------
+                // ---- S_c = Q K_c^T; the next chunk's K and this one's V are requested behind it -------------------------
                 bool w = true;
                 if (is_control && lane == 0) {
-                    const uint32_t bar = ptx::smem_addr(&B.kv_full);
-                    ptx::mbar_arrive_expect_tx(bar, pass ? 2u * kv_bytes : kv_bytes);
-                    ptx::tma_load_3d(smem_base + P.off_k, &map_kv, bar, P.part_bytes + h * 64, key0, b);
-                    if (pass) ptx::tma_load_3d(smem_base + P.off_v, &map_kv, bar, 2 * P.part_bytes + h * 64, key0, b);
                     if (pass == 0 && c == 0) w = mbar_wait(ptx::smem_addr(&B.q_full), n_q & 1u, abort_ptr);
-                    w = w && mbar_wait(bar, n_kv & 1u, abort_ptr);
+                    w = w && mbar_wait(ptx::smem_addr(&B.k_full[n_k & 1u]), (n_k >> 1) & 1u, abort_ptr);
                     if (w) {
                         ptx::tc_fence_after();
+                        const uint64_t kd = k_desc[n_k & 1u];
                         for (int k = 0; k < 2; ++k)
-                            ptx::mma_i8(tmem, q_desc + (uint64_t)(k * 2), k_desc + (uint64_t)(k * 2), idesc_qk, k);
+                            ptx::mma_i8(tmem, q_desc + (uint64_t)(k * 2), kd + (uint64_t)(k * 2), idesc_qk, k);
                         ptx::mma_commit(ptx::smem_addr(&B.s_full));
+                        // (the other K buffer was read by the product before this one, which every thread has awaited)
+                        if (c + 1 < P.n_chunks) load_k(b, h, c + 1);
+                        else if (pass == 0) load_k(b, h, 0);
+                        else if (item + (int)gridDim.x < P.total_items) {
+                            int b2, h2, q2;
+                            coords(item + gridDim.x, b2, h2, q2);
+                            load_k(b2, h2, 0);
+                        }
+                        if (pass) {
+                            // (the V before it has been read: the last P V has been awaited)
+                            ptx::mbar_arrive_expect_tx(ptx::smem_addr(&B.v_full), kv_bytes);
+                            ptx::tma_load_3d(smem_base + P.off_v, &map_kv, ptx::smem_addr(&B.v_full), 2 * P.part_bytes + h * 64, key0, b);
+                            ++i_v;
+                        }
                     }
                 }
                 if (pass == 0 && c == 0) ++n_q;
-                ++n_kv;
-                // every thread waits for S (the control lane included, so that K may be overwritten afterwards)
+                ++n_k;
                 w = w && mbar_wait(ptx::smem_addr(&B.s_full), n_s & 1u, abort_ptr);
                 ++n_s;
                 if (!__syncthreads_and(w ? 1 : 0)) { ok = false; break; }
                 ptx::tc_fence_after();
-                const bool tail = key0 + CH > T;                        // columns past the last token in this chunk
+                if (is_control && lane == 0 && pass == 1 && c + 1 == P.n_chunks && item + (int)gridDim.x < P.total_items) {
+                    // Q has been read for the last time
+                    int b2, h2, q2;
+                    coords(item + gridDim.x, b2, h2, q2);
+                    load_q(b2, h2, q2);
+                }
                 if (!is_control && warp_live) {
                     if (pass == 0) {
                         // ---- pass A: row sum of the table entries ------------------------------------------
+#pragma unroll 1
                         for (int blk = hf; blk < blocks; blk += 2) {
-                            if (key0 + blk * 32 >= T) break;
-                            uint32_t v[32];
-                            ptx::tmem_ld32(t_row + (uint32_t)(blk * 32), v);
+                            const int n_valid = T - (key0 + blk * 32);                  // columns of this block that are tokens
+                            if (n_valid <= 0) break;
+                            uint32_t v0[16], v1[16];
+                            ptx::tmem_ld16(t_row + (uint32_t)(blk * 32), v0);
                             ptx::tmem_ld_wait();
-#pragma unroll
-                            for (int i = 0; i < 32; ++i) {
-                                const uint32_t off = min((uint32_t)((int)v[i] * 4 + tab_half), (uint32_t)(2 * tab_half));
-                                const uint32_t eb = *reinterpret_cast<const uint32_t*>(tab_lo + off);
-                                // a table entry is a positive normal float: its double from the bits, two integer operations
-                                uint32_t hi, lo;
-                                asm("mad.hi.u32 %0, %1, 536870912, 939524096;" : "=r"(hi) : "r"(eb));
-                                asm("mul.lo.u32 %0, %1, 536870912;" : "=r"(lo) : "r"(eb));
-                                const bool valid = !tail || key0 + blk * 32 + i < T;
-                                zp[i & 3] += valid ? __hiloint2double((int)hi, (int)lo) : 0.0;
+                            ptx::tmem_ld16(t_row + (uint32_t)(blk * 32 + 16), v1);
+                            if (n_valid >= 32) {
+                                exp_lookup<16, false, false>(v0, ring, ring_mask, 0, 16, zp);
+                                ptx::tmem_ld_wait();
+                                exp_lookup<16, false, false>(v1, ring, ring_mask, 0, 16, zp);
+                            } else {
+                                exp_lookup<16, false, true>(v0, ring, ring_mask, 0, n_valid, zp);
+                                ptx::tmem_ld_wait();
+                                if (n_valid > 16) exp_lookup<16, false, true>(v1, ring, ring_mask, 0, n_valid - 16, zp);
                             }
                         }
                     } else {
                         // ---- pass B: codes of this chunk into the P tile -----------------------------------
-                        for (int blk = hf; blk < blocks; blk += 2) {
-                            uint32_t v[32];
-                            ptx::tmem_ld32(t_row + (uint32_t)(blk * 32), v);
-                            ptx::tmem_ld_wait();
-                            uint32_t wd[8];
+#pragma unroll 1
+                        for (int p16 = hf; p16 < 2 * blocks; p16 += 2) {               // the row's threads take 16 columns in turn
+                            const int n_valid = T - (key0 + p16 * 16);
+                            uint32_t wd[4] = {0u, 0u, 0u, 0u};
+                            if (n_valid > 0) {
+                                uint32_t v[16];
+                                ptx::tmem_ld16(t_row + (uint32_t)(p16 * 16), v);
+                                ptx::tmem_ld_wait();
+                                bool sure = !steep && n_valid >= 16;
+                                if (sure) sure = quantize_scores<16>(v, c2, l2, P.p_qp, limit, wd);
+                                if (!__all_sync(0xffffffffu, sure)) {
+                                    double unused[4] = {0.0, 0.0, 0.0, 0.0};
+                                    exp_lookup<16, false, true>(v, ring, ring_mask, 0, n_valid, unused);
+                                    if (steep) {
 #pragma unroll
-                            for (int i4 = 0; i4 < 8; ++i4) {
-                                uint32_t cb[4];
-#pragma unroll
-                                for (int j = 0; j < 4; j += 2) {
-                                    float e[2];
-#pragma unroll
-                                    for (int u = 0; u < 2; ++u) {
-                                        const int i = 4 * i4 + j + u;
-                                        const uint32_t off = min((uint32_t)((int)v[i] * 4 + tab_half), (uint32_t)(2 * tab_half));
-                                        const float ev = *reinterpret_cast<const float*>(tab_lo + off);
-                                        e[u] = (!tail || key0 + blk * 32 + i < T) ? ev : 0.0f;
+                                        for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(fminf(__uint_as_float(v[i]), e_top));
                                     }
-                                    const f32x2 e2 = f2_pack(e[0], e[1]);
-                                    float a0, a1, c0, c1;
-                                    f2_unpack(f2_fma(e2, rzh2, f2_mul(e2, rzl2)), a0, a1);
-                                    f2_unpack(f2_add(f2_pack(fminf(a0, P.p_qp), fminf(a1, P.p_qp)), magic2), c0, c1);
-                                    cb[j] = __float_as_uint(c0);
-                                    cb[j + 1] = __float_as_uint(c1);
+                                    quantize_entries<16>(v, rzh2, rzl2, qp2, wd);
                                 }
-                                wd[i4] = __byte_perm(__byte_perm(cb[0], cb[1], 0x4040), __byte_perm(cb[2], cb[3], 0x4040), 0x5410);
                             }
-                            const int cc = 2 * blk;
-                            uint8_t* const pblk = prow + (cc >> 3) * 16384;
-                            *reinterpret_cast<uint4*>(pblk + (((cc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                            *reinterpret_cast<uint4*>(pblk + ((((cc + 1) & 7) ^ sw) << 4)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
+                            *reinterpret_cast<uint4*>(prow + (p16 >> 3) * 16384 + (((p16 & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
                         }
                         ptx::fence_proxy_async_smem();
                     }
@@ -212,17 +249,22 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 __syncthreads();                                        // S has been read; the P tile is complete
                 if (pass == 1) {
                     // ---- O += P_c V_c ----------------------------------------------------------------------
+                    w = true;
                     if (is_control && lane == 0) {
-                        ptx::tc_fence_after();
-                        for (int ks = 0; ks < pv_steps; ++ks) {
-                            const uint64_t p_desc = ptx::smem_desc(smem_base + P.off_p + (uint32_t)(ks >> 2) * 16384u, 16, 1024,
-                                                                   ptx::SWIZZLE_128B) + (uint64_t)((ks & 3) * 2);
-                            ptx::mma_i8(tmem + AL_O_COL, p_desc, v_desc + (uint64_t)(ks * 128), idesc_pv, (c > 0 || ks > 0) ? 1 : 0);
+                        w = mbar_wait(ptx::smem_addr(&B.v_full), n_v & 1u, abort_ptr);
+                        if (w) {
+                            ptx::tc_fence_after();
+                            for (int ks = 0; ks < pv_steps; ++ks) {
+                                const uint64_t p_desc = ptx::smem_desc(smem_base + P.off_p + (uint32_t)(ks >> 2) * 16384u, 16, 1024,
+                                                                       ptx::SWIZZLE_128B) + (uint64_t)((ks & 3) * 2);
+                                ptx::mma_i8(tmem + AL_O_COL, p_desc, v_desc + (uint64_t)(ks * 128), idesc_pv, (c > 0 || ks > 0) ? 1 : 0);
+                            }
+                            ptx::mma_commit(ptx::smem_addr(&B.o_full));
                         }
-                        ptx::mma_commit(ptx::smem_addr(&B.o_full));
                     }
-                    // K, V and the P tile are reused by the next chunk: everyone waits for the MMAs that read them
-                    w = mbar_wait(ptx::smem_addr(&B.o_full), n_o & 1u, abort_ptr);
+                    ++n_v;
+                    // V and the P tile are reused by the next chunk: everyone waits for the MMAs that read them
+                    w = w && mbar_wait(ptx::smem_addr(&B.o_full), n_o & 1u, abort_ptr);
                     ++n_o;
                     if (!__syncthreads_and(w ? 1 : 0)) { ok = false; break; }
                 }
@@ -238,6 +280,13 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     const float rzh = (float)rz;
                     rzh2 = f2_dup(rzh);
                     rzl2 = f2_dup((float)(rz - (double)rzh));
+                    e_top = 60000.0f / rzh;                             // (steep only) far above Qp, below 2^16
+                    // Pass B's exponent is s c2 + l.  Where the code is not 0 the exponent lies in [-1, 8], so |s c2| <= |l| + 8,
+                    // and the roundings of c2, of l and of the FMA and the error of log2f leave at most (4 |l| + 40) 2^-24 in it
+                    // and ln 2 times that, plus exp2's 2^-22, relative in the argument.
+                    const float l = log2f(rzh);
+                    l2 = f2_dup(l);
+                    limit = 0.5f - (P.p_qp + 1.0f) * 1.25f * ((4.0f * fabsf(l) + 40.0f) * 4.1316e-8f + 2.4e-7f);
                 }
                 __syncthreads();                                        // zx may be rewritten by the next item
             }
@@ -247,38 +296,12 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         ptx::tc_fence_after();
         if (!is_control) {
             const int token = qt * 128 + row;
-            uint32_t ow[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) ow[k] = 0;
-            uint32_t v[32];
+            uint32_t v[32], ow[8];
             ptx::tmem_ld32(t_row + AL_O_COL + (uint32_t)(hf * 32), v);
             ptx::tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-                const int col = hf * 32 + i;
-                v[i] = round_clamp_bits(fmaf(small_int_to_float((int)v[i]), colp[col], colp[64 + col]), P.out_qn, P.out_qp);
-            }
-            if (P.out_c == 4) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) ow[i >> 3] |= (v[i] & 0xFu) << (4 * (i & 7));
-            } else if (P.out_c == 2) {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) ow[i >> 4] |= (v[i] & 0x3u) << (2 * (i & 15));
-            } else {
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                    ow[i] = __byte_perm(__byte_perm(v[4 * i], v[4 * i + 1], 0x4040), __byte_perm(v[4 * i + 2], v[4 * i + 3], 0x4040), 0x5410);
-            }
+            requantize_row32(v, 0, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
             if (token < T) {
-                uint8_t* o = P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c);
-                if (P.out_c == 4) {
-                    *reinterpret_cast<uint4*>(o) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-                } else if (P.out_c == 2) {
-                    *reinterpret_cast<uint2*>(o) = make_uint2(ow[0], ow[1]);
-                } else {
-                    reinterpret_cast<uint4*>(o)[0] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-                    reinterpret_cast<uint4*>(o)[1] = make_uint4(ow[4], ow[5], ow[6], ow[7]);
-                }
+                store_row32(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c), ow, P.out_c);
                 if (h == P.heads - 1 && hf == 1) {
                     uint8_t* const orow = P.out + ((long long)b * T + token) * P.out_pitch;
                     for (long long off = (long long)P.heads * (8 * P.out_c); off + 4 <= P.out_pitch; off += 4)
@@ -289,10 +312,15 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         ptx::tc_fence_before();
         __syncthreads();                                                // O and the head's parameters are free again
     }
-    // a copy still in flight when the CTA gives up is given a bounded chance to land
+    // copies still in flight when the CTA gives up are given a bounded chance to land
     if (!ok && is_control && lane == 0) {
-        for (int spin = 0; spin < (1 << 20) && !ptx::mbar_try_wait(ptx::smem_addr(&B.kv_full), (n_kv - 1u) & 1u); ++spin) {}
-        for (int spin = 0; spin < (1 << 20) && n_q > 0 && !ptx::mbar_try_wait(ptx::smem_addr(&B.q_full), (n_q - 1u) & 1u); ++spin) {}
+        auto drain = [&](uint64_t* bar, uint32_t issued) {               // the last phase of a barrier that was armed `issued` times
+            for (int spin = 0; spin < (1 << 20) && issued > 0 && !ptx::mbar_try_wait(ptx::smem_addr(bar), (issued - 1u) & 1u); ++spin) {}
+        };
+        drain(&B.q_full, i_q);
+        drain(&B.k_full[0], (i_k + 1u) >> 1);
+        drain(&B.k_full[1], i_k >> 1);
+        drain(&B.v_full, i_v);
     }
     ptx::tc_fence_before();
     __syncthreads();
@@ -308,7 +336,7 @@ inline uint32_t al_up(uint32_t v, uint32_t a) { return (v + a - 1) / a * a; }
 }  // namespace
 
 // Launcher shared with attention_core_launch: byte-stored codes, more than 256 tokens, table already in `table`.
-int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tokens, int smax, const float* table, float p_step,
+int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tokens, int smax, const float* table, float cs, float p_step,
                           float p_qp, const float* alpha_o, const float* beta_o, const vitint_codes* o_out, cudaStream_t st) {
     const int64_t D = (int64_t)heads * 64;
     LongParams P{};
@@ -323,6 +351,7 @@ int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tok
     P.part_bytes = (int)D;
     P.table = table;
     P.p_step = p_step; P.p_qp = p_qp;
+    P.c2 = (float)((double)cs * 1.4426950408889634);
     P.alpha_o = alpha_o; P.beta_o = beta_o;
     P.out_c = codes_container(o_out);
     int qn, qp;
@@ -330,9 +359,10 @@ int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tok
     P.out_qn = (float)qn; P.out_qp = (float)qp;
     P.out = (uint8_t*)o_out->data; P.out_pitch = o_out->pitch_bytes;
     uint32_t o = 0;
-    P.off_table = o; o += al_up((uint32_t)(2 * smax + 1) * 4u, 1024);
+    P.off_table = o; o += al_up((uint32_t)(2 * smax) * 4u, 1024);
     P.off_q = o; o += 128 * 64;
-    P.off_k = o; o += al_up((uint32_t)P.chunk * 64, 1024);
+    P.k_stride = al_up((uint32_t)P.chunk * 64, 1024);
+    P.off_k = o; o += 2 * P.k_stride;
     P.off_v = o; o += al_up((uint32_t)P.chunk * 64, 1024);
     P.off_p = o; o += (uint32_t)((P.chunk + 127) / 128) * 16384u;
     P.off_z = o; o += 2 * 128 * 8;

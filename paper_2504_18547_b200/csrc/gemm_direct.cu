@@ -96,28 +96,6 @@ __device__ __forceinline__ f32x2 acc_to_float2(uint32_t v0, uint32_t v1, int shi
     return f2_pack((float)(int)v0, (float)(int)v1);
 }
 
-// Sixteen byte codes -> eight bytes of 4-bit or four bytes of 2-bit codes (element order kept).
-__device__ __forceinline__ void narrow4(const uint32_t (&w)[4], uint32_t (&o)[2]) {
-    uint32_t t[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const uint32_t n = w[k] & 0x0F0F0F0Fu;
-        t[k] = n | (n >> 4);                                    // bytes 0 and 2 hold two codes each
-    }
-    o[0] = __byte_perm(t[0], t[1], 0x6420);
-    o[1] = __byte_perm(t[2], t[3], 0x6420);
-}
-__device__ __forceinline__ uint32_t narrow2(const uint32_t (&w)[4]) {
-    uint32_t t[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        uint32_t n = w[k] & 0x03030303u;
-        n |= n >> 6;                                            // bytes 0 and 2: two codes in the low four bits
-        t[k] = n | (n >> 12);                                   // byte 0: four codes
-    }
-    return __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
-}
-
 // The parameters of a thread's sixteen columns of a 64-column block.
 template <bool GELU>
 struct CodeParams {

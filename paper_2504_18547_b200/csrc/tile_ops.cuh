@@ -105,4 +105,146 @@ __device__ __forceinline__ void unpack_rows64(const uint8_t* src, uint8_t* dst, 
     }
 }
 
+// ---- softmax of a block of scores by table (attention kernels) ---------------------------------------------------
+// The table holds exp(fl32(s * c)) for every integer score, as a ring: the entry of score s lies at s mod n, n = 2 smax
+// (a power of two).  Scores of signed codes reach smax = 64 * 2^(b-1) * 2^(b-1) but never -smax, so none share an entry, and
+// one AND turns 4 s into a byte offset that lies inside the table whatever the operand bytes were.
+__device__ __forceinline__ void fill_table_ring(float* ring, const float* __restrict__ linear, int smax, int tid, int nthreads) {
+    for (int i = 1 + tid; i <= 2 * smax; i += nthreads) ring[(i - smax) & (2 * smax - 1)] = __ldg(linear + i);
+}
+
+// v: scores s (SCALED: 4 s times 2^sh) -> the entries' bits; their fp64 sum goes into four interleaved partial sums (one would
+// chain N dependent additions).  MASKED: elements from n_valid on are no scores: entry 0, nothing added.
+template <int N, bool SCALED, bool MASKED>
+__device__ __forceinline__ void exp_lookup(uint32_t (&v)[N], const char* ring, uint32_t mask, int sh, int n_valid, double (&zp)[4]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t off = (SCALED ? (uint32_t)((int)v[i] >> sh) : v[i] * 4u) & mask;
+        uint32_t eb = *reinterpret_cast<const uint32_t*>(ring + off);
+        if (MASKED && i >= n_valid) eb = 0u;
+        // an entry is a positive normal float: its double is put together from the bits, one instruction on the integer unit
+        // and one on the multiplier (the conversion unit runs at a quarter of the fp64 adder's rate)
+        const uint32_t hi = (eb >> 3) + 0x38000000u;
+        uint32_t lo;
+        asm("mul.lo.u32 %0, %1, 536870912;" : "=r"(lo) : "r"(eb));                    // eb << 29
+        zp[i & 3] += __hiloint2double(MASKED && i >= n_valid ? 0 : (int)hi, (int)lo);
+        v[i] = eb;
+    }
+}
+
+// Codes min(rint(e * (rh + rl)), Qp), e * rh + RN(e * rl): two scores per instruction up to the rounding by 1.5*2^23, then
+// two 16-bit minima per instruction (the caller keeps e * r below 2^16).
+template <int N>
+__device__ __forceinline__ void quantize_entries(const uint32_t (&v)[N], f32x2 rh2, f32x2 rl2, uint32_t qp2, uint32_t (&w)[N / 4]) {
+    const f32x2 magic2 = f2_dup(12582912.0f);
+#pragma unroll
+    for (int i4 = 0; i4 < N / 4; ++i4) {
+        uint32_t h[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const f32x2 e2 = f2_pack(__uint_as_float(v[4 * i4 + 2 * j]), __uint_as_float(v[4 * i4 + 2 * j + 1]));
+            float c0, c1;
+            f2_unpack(f2_add(f2_fma(e2, rh2, f2_mul(e2, rl2)), magic2), c0, c1);
+            const uint32_t both = __byte_perm(__float_as_uint(c0), __float_as_uint(c1), 0x5410);
+            asm("min.u16x2 %0, %1, %2;" : "=r"(h[j]) : "r"(both), "r"(qp2));
+        }
+        w[i4] = __byte_perm(h[0], h[1], 0x6420);
+    }
+}
+
+// The same codes straight from the scores, without the table: a = 2^(s c2 + l), l = log2(1 / (Z s_P)), in fp32 with the
+// hardware's exp2.  a differs from the quantizer's own argument by a relative error below the bound that the caller turned
+// into `limit` (a little less than 1/2): where |a - rint(a)| stays below it both round to the same code, where it does not
+// (about one score in 2^14) the function returns false and the caller takes the table.
+template <int N>
+__device__ __forceinline__ bool quantize_scores(const uint32_t (&v)[N], f32x2 c2, f32x2 l2, float qp, float limit, uint32_t (&w)[N / 4]) {
+    const f32x2 magic2 = f2_dup(12582912.0f), nmagic2 = f2_dup(-12582912.0f), neg1 = f2_dup(-1.0f);
+    float dev = 0.0f;
+#pragma unroll
+    for (int i4 = 0; i4 < N / 4; ++i4) {
+        uint32_t c[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const f32x2 s = f2_add(f2_pack(__uint_as_float(0x4B400000u + v[4 * i4 + 2 * j]), __uint_as_float(0x4B400000u + v[4 * i4 + 2 * j + 1])), nmagic2);
+            float t0, t1, a0, a1, c0, c1, d0, d1;
+            f2_unpack(f2_fma(s, c2, l2), t0, t1);
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a0) : "f"(t0));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a1) : "f"(t1));
+            const f32x2 a = f2_pack(fminf(a0, qp), fminf(a1, qp)), m = f2_add(a, magic2);
+            f2_unpack(f2_fma(f2_add(m, nmagic2), neg1, a), d0, d1);
+            dev = fmaxf(dev, fmaxf(fabsf(d0), fabsf(d1)));
+            f2_unpack(m, c0, c1);
+            c[2 * j] = __float_as_uint(c0);
+            c[2 * j + 1] = __float_as_uint(c1);
+        }
+        w[i4] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+    }
+    return dev < limit;
+}
+
+// Requantizes 32 columns of an accumulator row (|acc| < 2^22, scaled by 2^sh) to byte codes in two's complement:
+// clamp(rint(fma(acc, a, b))).  pa, pb: the columns' parameters in shared memory, 16-byte aligned.
+__device__ __forceinline__ void requantize_row32(const uint32_t (&v)[32], int sh, const float* pa, const float* pb, float qn, float qp,
+                                                 uint32_t (&w)[8]) {
+    const f32x2 magic2 = f2_dup(12582912.0f), nmagic2 = f2_dup(-12582912.0f);
+#pragma unroll
+    for (int i4 = 0; i4 < 8; ++i4) {
+        const float4 a4 = *reinterpret_cast<const float4*>(pa + 4 * i4), b4 = *reinterpret_cast<const float4*>(pb + 4 * i4);
+        uint32_t c[4];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const f32x2 f = f2_add(f2_pack(__int_as_float(0x4B400000 + ((int)v[4 * i4 + 2 * p] >> sh)),
+                                           __int_as_float(0x4B400000 + ((int)v[4 * i4 + 2 * p + 1] >> sh))), nmagic2);
+            float y0, y1, c0, c1;
+            f2_unpack(f2_fma(f, p ? f2_pack(a4.z, a4.w) : f2_pack(a4.x, a4.y), p ? f2_pack(b4.z, b4.w) : f2_pack(b4.x, b4.y)), y0, y1);
+            f2_unpack(f2_add(f2_pack(fminf(fmaxf(y0, qn), qp), fminf(fmaxf(y1, qn), qp)), magic2), c0, c1);
+            c[2 * p] = __float_as_uint(c0);
+            c[2 * p + 1] = __float_as_uint(c1);
+        }
+        w[i4] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+    }
+}
+
+// Sixteen byte codes -> eight bytes of 4-bit or four bytes of 2-bit codes (element order kept).
+__device__ __forceinline__ void narrow4(const uint32_t (&w)[4], uint32_t (&o)[2]) {
+    uint32_t t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t n = w[k] & 0x0F0F0F0Fu;
+        t[k] = n | (n >> 4);                                    // bytes 0 and 2 hold two codes each
+    }
+    o[0] = __byte_perm(t[0], t[1], 0x6420);
+    o[1] = __byte_perm(t[2], t[3], 0x6420);
+}
+__device__ __forceinline__ uint32_t narrow2(const uint32_t (&w)[4]) {
+    uint32_t t[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        uint32_t n = w[k] & 0x03030303u;
+        n |= n >> 6;                                            // bytes 0 and 2: two codes in the low four bits
+        t[k] = n | (n >> 12);                                   // byte 0: four codes
+    }
+    return __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
+}
+// Stores 32 byte codes of a row in the output's container (o: 4 * out_c bytes, 16-byte aligned for out_c >= 4, else 8).
+__device__ __forceinline__ void store_row32(uint8_t* o, const uint32_t (&w)[8], int out_c) {
+    const uint32_t lo[4] = {w[0], w[1], w[2], w[3]}, hi[4] = {w[4], w[5], w[6], w[7]};
+    if (out_c == 8) {
+        if ((reinterpret_cast<uintptr_t>(o) & 31u) == 0) {
+            // one 32-byte store: a warp's store touches 32 different rows whatever its width
+            ptx::st_global_32B(o, lo, hi);
+        } else {
+            reinterpret_cast<uint4*>(o)[0] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            reinterpret_cast<uint4*>(o)[1] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        }
+    } else if (out_c == 4) {
+        uint32_t a[2], b[2];
+        narrow4(lo, a);
+        narrow4(hi, b);
+        *reinterpret_cast<uint4*>(o) = make_uint4(a[0], a[1], b[0], b[1]);
+    } else {
+        *reinterpret_cast<uint2*>(o) = make_uint2(narrow2(lo), narrow2(hi));
+    }
+}
+
 }  // namespace vitint

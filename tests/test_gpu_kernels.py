@@ -271,3 +271,30 @@ def test_qkv_norm_tiles_and_references(M, heads, bits, packed):
         want = [compare_reference(y[:, k * D:(k + 1) * D].reshape(M * heads, 64), refs[k], flips[k], n_eps, bits).reshape(M, D)
                 for k in range(2)] + [vo.epilogue_requant(acc[:, 2 * D:], alpha, beta, bits, True)]
         assert np.array_equal(from_codes(got), np.concatenate(want, axis=1)) and padding_is_zero(got)
+
+
+# ---- fused attention core: every remainder of the column walk, a quantizer step whose unclamped codes exceed 16 bits -------
+@pytest.mark.parametrize("tokens", [1, 7, 8, 9, 31, 33, 63, 64, 72, 128, 129, 160, 192, 200, 225, 255, 256, 257, 320, 415])
+@pytest.mark.parametrize("bits,p_scale", [(4, 1.0), (2, 1.0), (4, 1e-5)])
+def test_attention_core_column_walk(tokens, bits, p_scale):
+    """Against the oracle's Q K^T, softmax band and P V: O inside the interval that the band of P reaches."""
+    from oracle import pipeline as vp
+    batch, heads = 2, 2
+    D, n = 64 * heads, batch * heads
+    qkv = rand_codes(500 + tokens, (batch * tokens, 3 * D), bits, True)
+    s_q = np.float32(0.25 if bits == 4 else 0.75)
+    s_p = np.float32(p_scale * 2.0 / (tokens * np.sqrt(2 ** bits - 1)))
+    q, k, v = (vp.split_heads(qkv, batch, tokens, heads, 64, i * D) for i in range(3))
+    S = vo.qk(q, k)
+    _, pc, plo, phi = vo.softmax_quantize(S.reshape(n * tokens, tokens), vp.softmax_scale(s_q, s_q, 64), s_p, bits)
+    if p_scale != 1.0:
+        assert (pc == 2 ** bits - 1).mean() > 0.5                          # codes far beyond the clamp
+    alpha, beta = np.full(D, np.float32(0.05 / tokens ** 0.5), np.float32), si.normal(501, (D,), 0.0, 0.5)
+    want = []
+    for a, b in ((plo, phi), (phi, plo)):
+        acc = vo.pv(a.reshape(n, tokens, tokens), np.maximum(v, 0)) + vo.pv(b.reshape(n, tokens, tokens), np.minimum(v, 0))
+        want.append(vo.epilogue_requant(vp.merge_heads(acc, batch, tokens, heads, 64), alpha, beta, bits, True))
+    got = vt.vitint_attention_core(byte_codes(qkv, bits, True), batch, heads, tokens, float(s_q), float(s_q), float(s_p), bits,
+                                   dev(alpha), dev(beta))
+    o = from_codes(got)
+    assert ((o >= want[0]) & (o <= want[1])).all() and padding_is_zero(got)
