@@ -17,7 +17,7 @@
 // leave together), two CTAs per SM so that one's loads and MMAs run beside the other's softmax; the next chunk's K is on its
 // way while this one's scores are worked on, and V is awaited only in front of P V.  Items are numbered by query tile first,
 // so that the last tile of every head, often nearly empty, fills the last round.  Byte-stored codes.
-// 785 tokens x 12 heads, batch 16: LONG_BEFORE -> LONG_AFTER us.
+// 785 tokens x 12 heads, batch 16: 202 -> 162 us.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"
