@@ -394,7 +394,9 @@ typedef enum {
     VITINT_ATTN_SHIFT_CORE = 1,      /* vitint_attention_core_shift */
     VITINT_ATTN_EXP = 2,             /* vitint_qk -> vitint_softmax_quantize -> vitint_pv */
     VITINT_ATTN_EXP_BOUNDED = 3,     /* vitint_qk -> vitint_softmax_quantize_bounded -> vitint_pv */
-    VITINT_ATTN_SHIFT = 4            /* vitint_qk -> vitint_softmax_shift_quantize -> vitint_pv */
+    VITINT_ATTN_SHIFT = 4,           /* vitint_qk -> vitint_softmax_shift_quantize -> vitint_pv */
+    VITINT_ATTN_EXP_CORE_ANY = 5     /* the result of VITINT_ATTN_EXP in one launch: codes stored one per byte (8-bit ones
+                                        included), at most 256 tokens; `scores`, `p` and `table` are not used */
 } vitint_attention_kind;
 
 typedef struct {

@@ -49,7 +49,7 @@ class _EncoderLayerDesc(Structure):
                 + [("scores", c_void_p), ("ld_scores", c_int64), ("h", c_void_p), ("table", c_void_p), ("table_bytes", c_size_t)])
 
 
-ATTN_EXP_CORE, ATTN_SHIFT_CORE, ATTN_EXP, ATTN_EXP_BOUNDED, ATTN_SHIFT = range(5)
+ATTN_EXP_CORE, ATTN_SHIFT_CORE, ATTN_EXP, ATTN_EXP_BOUNDED, ATTN_SHIFT, ATTN_EXP_CORE_ANY = range(6)
 
 
 class _AttentionDesc(Structure):

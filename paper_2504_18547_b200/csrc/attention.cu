@@ -106,6 +106,10 @@ extern "C" int vitint_attention_block(const vitint_codes* x, const vitint_attent
     if (!dbg_p && L.tab_bytes)
         fused = vitint_attention_core(&qkv, d->batch, d->heads, d->tokens, d->q_step, d->k_step, d->p_step, d->p_bits,
                                       d->alpha_o, d->beta_o, &o, ws + L.off_tab, L.tab_bytes, stream);
+    // 8-bit codes (no table): exp evaluated inside the core
+    if (!dbg_p && d->bits == 8 && d->tokens <= 256)
+        fused = attention_core_general(&qkv, d->batch, d->heads, d->tokens, d->q_step, d->k_step, d->p_step, d->p_bits, d->alpha_o,
+                                       d->beta_o, &o, stream);
     if (fused != VITINT_OK && fused != VITINT_ERR_UNSUPPORTED) return fused;
     if (fused == VITINT_ERR_UNSUPPORTED && wide_qkv) return fused;      // (the unfused kernels read bit-packed slabs)
     if (fused == VITINT_ERR_UNSUPPORTED) {

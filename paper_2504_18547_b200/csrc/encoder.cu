@@ -27,6 +27,9 @@ int attention_stage(const vitint_encoder_layer_desc& L, void* stream) {
     if (L.attention == VITINT_ATTN_SHIFT_CORE)
         return vitint_attention_core_shift(&L.qkv, L.batch, L.heads, L.tokens, L.q_step, L.k_step, L.p_step, L.bits, L.alpha_o,
                                            nullptr, &L.o, L.table, L.table_bytes, 1, stream);
+    if (L.attention == VITINT_ATTN_EXP_CORE_ANY)
+        return attention_core_general(&L.qkv, L.batch, L.heads, L.tokens, L.q_step, L.k_step, L.p_step, L.bits, L.alpha_o, nullptr, &L.o,
+                                      stream);
     const int c = container_bits(L.bits);
     vitint_slabs q{L.qkv.data, L.qkv.pitch_bytes, L.qkv.pitch_bytes * L.tokens, 64 * c / 8, L.bits, 1};
     vitint_slabs k = q, v = q;
@@ -101,7 +104,7 @@ bool valid_stack(const vitint_encoder_layer_desc* layers, int n, float* const bu
     if (!layers || n <= 0 || (n > 1 && (!buf || !buf[0] || (n > 2 && !buf[1])))) return false;
     for (int i = 0; i < n; ++i) {
         const vitint_encoder_layer_desc& L = layers[i];
-        if (L.batch <= 0 || L.tokens <= 0 || L.heads <= 0 || !L.h || L.attention < VITINT_ATTN_EXP_CORE || L.attention > VITINT_ATTN_SHIFT)
+        if (L.batch <= 0 || L.tokens <= 0 || L.heads <= 0 || !L.h || L.attention < VITINT_ATTN_EXP_CORE || L.attention > VITINT_ATTN_EXP_CORE_ANY)
             return false;
     }
     return true;

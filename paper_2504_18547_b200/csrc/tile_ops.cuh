@@ -182,8 +182,9 @@ __device__ __forceinline__ bool quantize_scores(const uint32_t (&v)[N], f32x2 c2
     return dev < limit;
 }
 
-// Requantizes 32 columns of an accumulator row (|acc| < 2^22, scaled by 2^sh) to byte codes in two's complement:
+// Requantizes 32 columns of an accumulator row (scaled by 2^sh; SMALL: |acc| < 2^22) to byte codes in two's complement:
 // clamp(rint(fma(acc, a, b))).  pa, pb: the columns' parameters in shared memory, 16-byte aligned.
+template <bool SMALL = true>
 __device__ __forceinline__ void requantize_row32(const uint32_t (&v)[32], int sh, const float* pa, const float* pb, float qn, float qp,
                                                  uint32_t (&w)[8]) {
     const f32x2 magic2 = f2_dup(12582912.0f), nmagic2 = f2_dup(-12582912.0f);
@@ -193,8 +194,9 @@ __device__ __forceinline__ void requantize_row32(const uint32_t (&v)[32], int sh
         uint32_t c[4];
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-            const f32x2 f = f2_add(f2_pack(__int_as_float(0x4B400000 + ((int)v[4 * i4 + 2 * p] >> sh)),
-                                           __int_as_float(0x4B400000 + ((int)v[4 * i4 + 2 * p + 1] >> sh))), nmagic2);
+            const int u0 = (int)v[4 * i4 + 2 * p] >> sh, u1 = (int)v[4 * i4 + 2 * p + 1] >> sh;
+            const f32x2 f = SMALL ? f2_add(f2_pack(__int_as_float(0x4B400000 + u0), __int_as_float(0x4B400000 + u1)), nmagic2)
+                                  : f2_pack((float)u0, (float)u1);
             float y0, y1, c0, c1;
             f2_unpack(f2_fma(f, p ? f2_pack(a4.z, a4.w) : f2_pack(a4.x, a4.y), p ? f2_pack(b4.z, b4.w) : f2_pack(b4.x, b4.y)), y0, y1);
             f2_unpack(f2_add(f2_pack(fminf(fmaxf(y0, qn), qp), fminf(fmaxf(y1, qn), qp)), magic2), c0, c1);

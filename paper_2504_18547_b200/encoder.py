@@ -46,6 +46,9 @@ class EncoderLayer:
                                 and ((softmax == "exp" and (tokens <= 256 or (wide_activations and tokens <= 4096)))
                                      or (softmax == "shift" and wide_activations and tokens <= 256)))
         self.stages = STAGES_FUSED if self.fused_attention else STAGES_UNFUSED
+        # 8-bit scores have no table: Q K^T, softmax and P V one by one (as forward() with events times them), or, in the
+        # recorded layer, the fused core that evaluates exp per score -- the same codes without S and P in memory
+        self._any_core = fused_attention and bits == 8 and softmax == "exp" and tokens <= 256
         d = lambda a: _dev(a, device)
         f = lambda k: float(prm[k])
         self.s_ln, self.s_q, self.s_k, self.s_v = f("s_ln"), f("s_q"), f("s_k"), f("s_v")
@@ -170,7 +173,7 @@ class EncoderLayer:
             elif self.sm_table is not None:
                 d.attention, d.c, d.score_bound, table = B.ATTN_EXP_BOUNDED, self.c, self.score_bound, self.sm_table
             else:
-                d.attention, d.c = B.ATTN_EXP, self.c
+                d.attention, d.c = B.ATTN_EXP_CORE_ANY if self._any_core else B.ATTN_EXP, self.c
         if table is not None:
             d.table, d.table_bytes = p(table), table.numel()
         return d

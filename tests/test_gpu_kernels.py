@@ -298,3 +298,32 @@ def test_attention_core_column_walk(tokens, bits, p_scale):
                                    dev(alpha), dev(beta))
     o = from_codes(got)
     assert ((o >= want[0]) & (o <= want[1])).all() and padding_is_zero(got)
+
+
+@pytest.mark.parametrize("tokens", [1, 9, 33, 100, 145, 197, 224, 256])
+def test_layer_8bit_core_equals_three_kernels(tokens):
+    """8-bit layers: the recorded pass evaluates exp inside the fused core, the launches go through S and P in memory."""
+    cfg, layer = small_layer({"bits": 8, "tokens": tokens})
+    x = dev(si.normal(600 + tokens, (cfg.rows, cfg.dim)))
+    out = torch.empty_like(x)
+    layer.forward(x, out)
+    o = layer.O.data.clone()
+    assert torch.equal(out, one_by_one(layer, x)) and torch.equal(o, layer.O.data)
+
+
+@pytest.mark.parametrize("tokens", [5, 197])
+def test_attention_block_8bit_core(tokens):
+    """vitint_attention_block with 8-bit codes: with a copy of P (three kernels) and without (the fused core)."""
+    cfg = si.BlockConfig("b8", 2, tokens, 128, 2, 8)
+    prm = si.layer_parameters(cfg)
+    xq = vt.vitint_quantize(dev(si.activations(cfg)), float(prm["s_x"]), 8, True)
+    w = {n: vt.vitint_quantize(dev(prm["w_" + n]), 0.0, 8, True, row_steps=dev(prm["s_w_" + n])) for n in ("qkv", "proj")}
+    seg = np.repeat(np.array([prm["s_q"], prm["s_k"], prm["s_v"]], np.float32), cfg.dim)
+    alpha, beta = vt.fold_requant(prm["s_x"], prm["s_w_qkv"], prm["b_qkv"], seg)
+    alpha_o, _ = vt.fold_requant(prm["s_p"], np.full(cfg.dim, prm["s_v"], np.float32), None, prm["s_o"])
+    a = vt.AttentionWeights(cfg.batch, tokens, cfg.heads, 8, w["qkv"], dev(alpha), dev(beta), float(prm["s_q"]), float(prm["s_k"]),
+                            float(prm["s_v"]), float(prm["s_p"]), float(prm["s_o"]), 8, dev(alpha_o), None, w["proj"],
+                            dev(prm["s_w_proj"]), dev(prm["b_proj"]), vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+    p = vt.Codes.empty(cfg.batch * cfg.heads * tokens, tokens, 8, False)
+    want = vt.vitint_attention_block(xq, a, dbg_p=p)
+    assert torch.equal(vt.vitint_attention_block(xq, a), want)
