@@ -272,11 +272,10 @@ int vitint_attention_core_prepared(const vitint_codes* qkv, int32_t batch, int32
  *   residual, 2^r ~ 1 + r, integer shifts; the division-free comparator quantizer of Section IV-B whose references are
  *   scaled by the row sum).  Arguments as vitint_attention_core; the codes of P and O are those of vitint_qk ->
  *   vitint_softmax_shift_quantize -> vitint_pv bit for bit (every step is an integer or a single fp32 operation).
- *   The per-score pair (floor z, mantissa of 1 + r) comes from two tables over the bounded score range, built into
- *   `workspace` (256-byte aligned, at least vitint_attention_core_shift_workspace_bytes(bits) bytes) by one small
- *   launch, unless table_ready != 0: the workspace then still holds the tables an earlier call with the same bits,
- *   q_step and k_step wrote.  The row maximum is subtracted (as shift counts), so unlike vitint_attention_core this
- *   variant has no limit on the size of the logits.
+ *   The per-score pair (floor z, mantissa of 1 + r) is computed from the score; `workspace` (256-byte aligned, at least
+ *   vitint_attention_core_shift_workspace_bytes(bits) bytes) is checked, not used, and table_ready has no effect.  The
+ *   row maximum is subtracted (as shift counts), so unlike vitint_attention_core this variant has no limit on the size
+ *   of the logits.
  *   Errors: as vitint_attention_core; UNSUPPORTED also for codes not stored one per byte (container_bits != 8). */
 size_t vitint_attention_core_shift_workspace_bytes(int32_t bits);
 int vitint_attention_core_shift(const vitint_codes* qkv, int32_t batch, int32_t heads, int32_t tokens, float q_step,
@@ -381,8 +380,8 @@ int vitint_layernorm_compare_quantize(const float* x, int64_t rows, int64_t cols
  * vitint_qk -> softmax -> vitint_pv where `attention` says so).  Layer i > 0 reads what layer i - 1 wrote: layer i writes
  * buf[i & 1], the last one `out`.
  *   vitint_encoder_forward          enqueues the launches one by one.
- *   vitint_encoder_plan_create      records the same launches once as a CUDA graph (and enqueues, on `stream`, the kernels
- *                                   that fill the tables of the Eq. 4 and bounded softmax where a layer uses them).
+ *   vitint_encoder_plan_create      records the same launches once as a CUDA graph (and enqueues, on `stream`, the kernel
+ *                                   that fills the table of the bounded softmax where a layer uses it).
  *   vitint_encoder_plan_run         runs the recorded launches with this call's x and out: one graph launch instead of
  *                                   seven or more launches per layer.  On a stream that is being captured the launches are
  *                                   enqueued one by one.  Safe to call from several threads; calls that overlap on the GPU

@@ -463,7 +463,7 @@ def vitint_attention_core_shift(qkv: Codes, batch: int, heads: int, tokens: int,
                                 out: Codes | None = None, out_bits: int | None = None,
                                 workspace: torch.Tensor | None = None, table_ready: bool = False) -> Codes:
     """The fused attention core with the Eq. 4 softmax and its division-free comparator quantizer (byte-stored codes).
-    table_ready: `workspace` still holds the table an earlier call with the same bits and steps built."""
+    The scores' integer parts and mantissas are computed, not tabulated: table_ready has no effect."""
     if out is None:
         out = Codes.empty(batch * tokens, heads * 64, qkv.bits if out_bits is None else out_bits, True, qkv.data.device)
     if workspace is None:

@@ -49,12 +49,11 @@ struct AttnParams {
     int kv_rows;                 // tokens rounded up to 32: K extent of P V, rows of the V tile
     int smax;                    // table covers scores -smax .. smax
     int part_bytes;              // bytes of one of the Q / K / V column blocks in a QKV row
-    uint32_t off_table, off_ftab, off_group, group_bytes;         // shared-memory layout
+    uint32_t off_table, off_group, group_bytes;         // shared-memory layout
     uint32_t off_pq, off_pk, off_pv, off_q, off_k, off_v, off_p, off_col, off_z, off_mx;   // within a group
     const float* table;          // global copy of the exp table, 2*smax+1 floats
-    uint32_t ftab_word;          // Eq. 4: word offset of the 16-bit table of integer parts behind the 32-bit table
     float p_step, p_qp;
-    float scale;                 // softmax scale c (GENERAL)
+    float scale;                 // softmax scale c (GENERAL), c log2 e (SHIFT)
     const float* alpha_o;        // [D]
     const float* beta_o;         // [D] or null
     int out_c;
@@ -66,20 +65,6 @@ struct AttnParams {
 struct AttnBars {
     uint64_t packed_full, v_full, ops_ready, s_full, p_ready, o_full, o_done, grp_sync, z_sync;
 };
-
-// Eq. 4's split of every integer score: z = fl32(s * c2), f = floor z (16-bit table behind the 32-bit one),
-// M = trunc((1 + (z - f)) * 2^23), the 24-bit mantissa of 2^r ~ 1 + r (2^24 in the one case where 1 + r rounds to 2).
-__global__ void shift_table_kernel(uint32_t* mtab, short* ftab, int smax, float c2) {
-    grid_dependency_wait();        // an earlier kernel may still read the table
-    grid_dependency_launch();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i > 2 * smax) return;
-    const float z = __fmul_rn((float)(i - smax), c2);
-    const float fl = floorf(z);
-    const float res = __fsub_rn(z, fl);
-    mtab[i] = (uint32_t)__fmul_rn(__fadd_rn(1.0f, res), 8388608.0f);
-    ftab[i] = (short)(int)fl;
-}
 
 // exp(fl32(s * c)) for every integer score, correctly rounded to fp32 (fp64 exp, one rounding).
 __global__ void exp_table_kernel(float* table, int smax, float c) {
@@ -96,10 +81,10 @@ __global__ void exp_table_kernel(float* table, int smax, float c) {
 enum AttnMode { AM_TABLE = 0, AM_SHIFT = 1, AM_GENERAL = 2 };
 
 // SHIFT: the softmax of Eq. 4 (2^z with z split into integer part and residual, 2^r ~ 1 + r, integer shifts, the
-// division-free comparator quantizer) instead of exp.  With integer scores of bounded range the pair (floor z,
-// mantissa of 1 + r) is one table entry per score, so the arithmetic left per score is the shift, the exact 64-bit
-// row sum and the comparison against references scaled by that sum -- every step an integer or a single fp32
-// operation in the order of the stand-alone kernel, hence the same codes bit for bit.
+// division-free comparator quantizer) instead of exp, every step with the result of the stand-alone kernel's integer or
+// single fp32 operation, hence the same codes bit for bit.  Two tables of the scores (floor z; the mantissa of 1 + r), 64-bit
+// shifts and two comparisons a score took 79 us for 197 tokens x 12 heads at batch 64; computed in pairs, summed in
+// doubles and compared only near a tie, 50 us (198 tokens x 6 heads: 42 -> 27).
 template <int C, int MODE>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kv,
@@ -147,15 +132,8 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     {
         float* tab = reinterpret_cast<float*>(smem_gen + P.off_table);
         if constexpr (MODE == AM_TABLE) fill_table_ring(tab, P.table, P.smax, threadIdx.x, AT_THREADS);
-        if constexpr (SHIFT) {
-            for (int i = threadIdx.x; i <= 2 * P.smax; i += AT_THREADS) tab[i] = __ldg(P.table + i);
-            // the 16-bit table of integer parts sits behind the 32-bit one, in the workspace and here
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(P.table) + P.ftab_word;
-            uint32_t* dst = reinterpret_cast<uint32_t*>(smem_gen + P.off_ftab);
-            for (int i = threadIdx.x; i <= P.smax; i += AT_THREADS) dst[i] = __ldg(src + i);
-        }
     }
-    if constexpr (!SHIFT) {
+    {
         // P columns behind the last block of eight that holds a token are never written: zero for good
         for (int i = threadIdx.x; i < AT_GROUPS * 128 * 16; i += AT_THREADS) {
             const int gr = i / 2048, cc = (i >> 7) & 15, r = i & 127;
@@ -319,27 +297,33 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             // a warp whose 32 query rows all lie past the last token has nothing to compute: its P rows
             // only feed accumulator rows that are never stored (whatever int8 they hold)
             const bool warp_live = qt * 128 + wq * 32 < T;
-            if constexpr (SHIFT) {
-                // Two tables over the score range: M[s] = trunc((1 + (z - floor z)) * 2^23) (32-bit) and f[s] = floor z
-                // (16-bit), z = fl32(s * c2).  floor z increases with s, so the row's largest score carries the row's
-                // largest integer part m and pass 0 needs no lookup at all.
+            if constexpr (SHIFT || GENERAL) {
+                // pass 0: the row's largest score (Eq. 4: the smallest as well).  fl32(S_j c) increases with S_j (c > 0), so the
+                // largest score has the largest logit.
                 int* const mx = reinterpret_cast<int*>(ggen + P.off_mx);
-                unsigned long long* const sx = reinterpret_cast<unsigned long long*>(ggen + P.off_z);
-                const uint32_t* const mtab = reinterpret_cast<const uint32_t*>(smem_gen + P.off_table);
-                const short* const ftab = reinterpret_cast<const short*>(smem_gen + P.off_ftab);
-                const uint32_t top = (uint32_t)(2 * P.smax);
-                // pass 0: the row's largest score
-                int smx = INT_MIN;
-                for (int ch = hf; warp_live && ch < chunks; ch += 2) {
-                    uint32_t v[32];
-                    ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
-                    ptx::tmem_ld_wait();
-                    if (ch < full_chunks) {
+                int smx = INT_MIN, smn = INT_MAX;
+                if (warp_live) {
+#pragma unroll 1
+                    for (int ch = hf; ch < full_chunks; ch += 2) {
+                        uint32_t v[32];
+                        ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
+                        ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) smx = max(smx, (int)v[i]);
-                    } else {
+                        for (int i = 0; i < 32; ++i) {
+                            smx = max(smx, (int)v[i]);
+                            if (SHIFT) smn = min(smn, (int)v[i]);
+                        }
+                    }
+#pragma unroll 1
+                    for (int k = tail0; k < tail_blocks; k += 2) {
+                        uint32_t v[8];
+                        ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                        ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) smx = max(smx, ch * 32 + i < T ? (int)v[i] : INT_MIN);
+                        for (int i = 0; i < 8; ++i) {
+                            smx = max(smx, 8 * k + i < tail ? (int)v[i] : INT_MIN);
+                            if (SHIFT) smn = min(smn, 8 * k + i < tail ? (int)v[i] : INT_MAX);
+                        }
                     }
                 }
                 mx[hf * 128 + row] = smx;
@@ -348,40 +332,94 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 0u, abort_ptr);       // two phases per item: parities 0, 1
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 smx = max(mx[row], mx[128 + row]);
-                // pass 1: E_j = M_j << (30 + f_j - m) (>> for the few scores more than 30 octaves down), exact 64-bit
-                // row sum, float(E_j) put together from its bits and parked in TMEM over the score
-                const int c0 = 30 - (int)ftab[min((uint32_t)(max(smx, -P.smax) + P.smax), top)];
-                // Straight-line per score (rows with a wide spread of scores take the right-shift form often, so a
-                // branch would mostly run both sides): the 64-bit term is (M * 2^32) >> (32 - sh) with sh kept above
-                // -32 (further down everything is shifted out anyway); float(E) is float(M) * 2^sh put together from
-                // its bits for sh >= 0, and the conversion of the small remainder by the 2^23 trick otherwise.
-                uint32_t sg_lo = 0u, sg_hi = 0u;
-                auto term = [&](uint32_t score, bool valid) -> uint32_t {
-                    const uint32_t idx = min((uint32_t)((int)score + P.smax), top);
-                    const uint32_t m24 = valid ? mtab[idx] : 0u;                       // a real entry is at least 2^23
-                    const int sh = max((int)ftab[idx] + c0, -31);
-                    const unsigned long long big = ((unsigned long long)m24 << 32) >> (32 - sh);
-                    const uint32_t lo = (uint32_t)big, hi = (uint32_t)(big >> 32);
-                    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;" : "+r"(sg_lo), "+r"(sg_hi) : "r"(lo), "r"(hi));
-                    const uint32_t up = m24 + 0x4A800000u + ((uint32_t)sh << 23);
-                    const uint32_t dn = __float_as_uint(__fadd_rn(__uint_as_float(0x4B000000u + lo), -8388608.0f));
-                    return valid ? (sh >= 0 ? up : dn) : 0u;
+                const f32x2 c2 = f2_dup(P.scale), nmagic2 = f2_dup(-12582912.0f), magic2 = f2_dup(12582912.0f);
+                uint8_t* const prow = ggen + P.off_p + row * 128;
+                const int sw = row & 7;
+                if constexpr (SHIFT) {
+                // pass 1: z_j = fl32(S_j c log2 e), f_j = floor z_j (an addition that rounds down), E_j = trunc((1 + (z_j - f_j)) 2^23)
+                // << (30 + f_j - m), m the row's largest f (>> when negative).  While nothing is shifted out, float(E_j) is the float
+                // 1 + (z_j - f_j) with 53 + f_j - m added to its exponent; that integer rides in the addend that rounds z_j down.
+                // Where the warp's rows spread over at most 21 octaves every E_j is a multiple of 2^9 and a row's sum stays below
+                // 2^62, so the 53 bits of a double carry it exactly; otherwise 64-bit integers do.
+                const float m = floorf(__fmul_rn((float)smx, P.scale));
+                const float addend = 12582912.0f + (53.0f - m);
+                const f32x2 add2 = f2_dup(addend), nadd2 = f2_dup(-addend), neg1 = f2_dup(-1.0f), one2 = f2_dup(1.0f);
+                auto split = [&](uint32_t a, uint32_t b, f32x2& t, f32x2& r1) {           // t: 1.5 * 2^23 + 53 + f - m; r1: 1 + (z - f)
+                    const f32x2 sf = f2_add(f2_pack(__uint_as_float(0x4B400000u + a), __uint_as_float(0x4B400000u + b)), nmagic2);
+                    const f32x2 z = f2_mul(sf, c2);
+                    t = f2_add_rm(z, add2);
+                    r1 = f2_add(f2_fma(f2_add(t, nadd2), neg1, z), one2);
                 };
-                for (int ch = hf; warp_live && ch < chunks; ch += 2) {
-                    uint32_t v[32];
-                    ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
-                    ptx::tmem_ld_wait();
-                    if (ch < full_chunks) {
+                unsigned long long sigma = 0ull;
+                if (warp_live) {
+                    const bool wide = floorf(__fmul_rn((float)min(smn, smx), P.scale)) < m - 21.0f;
+                    if (!__any_sync(0xffffffffu, wide)) {
+                        double zp[2] = {0.0, 0.0};
+                        auto term_pair = [&](uint32_t& a, uint32_t& b, bool va, bool vb) {
+                            f32x2 t, r1;
+                            float t0, t1, x0, x1;
+                            split(a, b, t, r1);
+                            f2_unpack(t, t0, t1);
+                            f2_unpack(r1, x0, x1);
+                            a = va ? __float_as_uint(x0) + (__float_as_uint(t0) << 23) : 0u;
+                            b = vb ? __float_as_uint(x1) + (__float_as_uint(t1) << 23) : 0u;
+                            // the doubles from the bits; a zero becomes 2^-127, which the sum rounds away
+                            zp[0] += __hiloint2double((int)((a >> 3) + 0x38000000u), (int)(a << 29));
+                            zp[1] += __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+                        };
+#pragma unroll 1
+                        for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {     // halves of the thread's chunks
+                            uint32_t v[16];
+                            ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
+                            ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] = term(v[i], true);
+                            for (int i = 0; i < 16; i += 2) term_pair(v[i], v[i + 1], true, true);
+                            ptx::tmem_st16(t_row + (uint32_t)(pc * 16), v);
+                        }
+#pragma unroll 1
+                        for (int k = tail0; k < tail_blocks; k += 2) {
+                            uint32_t v[8];
+                            ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                            ptx::tmem_ld_wait();
+#pragma unroll
+                            for (int i = 0; i < 8; i += 2) term_pair(v[i], v[i + 1], 8 * k + i < tail, 8 * k + i + 1 < tail);
+                            ptx::tmem_st8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                        }
+                        sigma = (unsigned long long)__double2ll_rn(zp[0] + zp[1]);
                     } else {
+                        // the 64-bit term is (M * 2^32) >> (32 - sh) with sh = 30 + f - m kept above -32 (further down everything is
+                        // shifted out anyway); what is left of a mantissa shifted right converts by the 2^23 trick
+#pragma unroll 1
+                        for (int blk = 0; blk < 4 * full_chunks + tail_blocks; ++blk) {           // blocks of eight columns
+                            if (blk < 4 * full_chunks ? ((blk >> 2) & 1) != hf : ((blk - 4 * full_chunks) & 1) != tail0) continue;
+                            uint32_t v[8];
+                            ptx::tmem_ld8(t_row + (uint32_t)(blk * 8), v);
+                            ptx::tmem_ld_wait();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) v[i] = term(v[i], ch * 32 + i < T);      // no score past the last token
+                            for (int i = 0; i < 8; i += 2) {
+                                f32x2 t, r1;
+                                float t0, t1, x0, x1;
+                                split(v[i], v[i + 1], t, r1);
+                                f2_unpack(t, t0, t1);
+                                f2_unpack(r1, x0, x1);
+#pragma unroll
+                                for (int j = 0; j < 2; ++j) {
+                                    const bool valid = blk * 8 + i + j < T;
+                                    const uint32_t x = __float_as_uint(j ? x1 : x0);
+                                    const int sh = max((int)__float_as_uint(j ? t1 : t0) - 0x4B400000 - 23, -31);
+                                    const unsigned long long big = ((unsigned long long)(x - 0x3F000000u) << 32) >> (32 - sh);
+                                    const uint32_t up = x + ((uint32_t)(sh + 23) << 23);
+                                    const uint32_t dn = __float_as_uint(__fadd_rn(__uint_as_float(0x4B000000u + (uint32_t)big), -8388608.0f));
+                                    sigma += valid ? big : 0ull;
+                                    v[i + j] = valid ? (sh >= 0 ? up : dn) : 0u;
+                                }
+                            }
+                            ptx::tmem_st8(t_row + (uint32_t)(blk * 8), v);
+                        }
                     }
-                    ptx::tmem_st32(t_row + (uint32_t)(ch * 32), v);
+                    ptx::tmem_st_wait();
                 }
-                unsigned long long sigma = ((unsigned long long)sg_hi << 32) | sg_lo;
-                ptx::tmem_st_wait();
+                unsigned long long* const sx = reinterpret_cast<unsigned long long*>(ggen + P.off_z);
                 sx[hf * 128 + row] = sigma;
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
@@ -390,78 +428,82 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 sigma = sx[row] + sx[128 + row];
                 const float sig_f = __ull2float_rn(sigma);
                 // pass 2: the code is the number of references fl32(fl32((k - 1/2) s_P) * Sigma) that float(E_j) exceeds.
-                // k0 = rint(min(E_j / (s_P Sigma), Qp - 3/4)) is at most one off and never Qp, so the two references
-                // around it decide: code = k0 - 1 + [E > ref(k0)] + [E > ref(k0 + 1)], references formed with the two
-                // fp32 multiplications of the definition.  The sum is taken in the float that carries k0 in its low
-                // mantissa bits (1.5 * 2^23 - 1 + k0 + the two tests): small integers, exact.
+                // k0 = rint(u), u = min(E_j / (s_P Sigma), Qp), is that number unless u lies within (Qp + 1) 2^-21 of some k - 1/2:
+                // u is off by less than 3.1 * 2^-24 of itself, a reference by less than 2.1 * 2^-24.  Columns that come that
+                // close are compared with the two references around them: k0' = rint(min(u, Qp - 3/4)) is at most one off and
+                // never Qp, code = k0' - 1 + [E > ref(k0')] + [E > ref(k0' + 1)], in the float that carries k0' in its mantissa.
                 const float inv = warp_live ? __frcp_rn(__fmul_rn(P.p_step, sig_f)) : 0.0f;
-                const float u_top = P.p_qp - 0.75f;
-                const f32x2 inv2 = f2_dup(inv), magic2 = f2_dup(12582912.0f), nmagic2 = f2_dup(-12582912.0f), neg1 = f2_dup(-1.0f);
-                const f32x2 half2 = f2_dup(0.5f), nhalf2 = f2_dup(-0.5f), ps2 = f2_dup(P.p_step), sg2 = f2_dup(sig_f);
-                uint8_t* const prow = ggen + P.off_p + row * 128;
-                const int sw = row & 7;
-                for (int ch = hf; warp_live && ch < chunks; ch += 2) {
-                    uint32_t v[32];
-                    ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
-                    ptx::tmem_ld_wait();
-                    uint32_t wd[8];
+                const float near_tie = 0.5f - (P.p_qp + 1.0f) * 4.76837158e-07f;
+                const f32x2 inv2 = f2_dup(inv);
+                auto codes = [&](const uint32_t* v, uint32_t* wd, auto count) {
+                    constexpr int N = decltype(count)::value;
+                    float far = 0.0f;
 #pragma unroll
-                    for (int i4 = 0; i4 < 8; ++i4) {
+                    for (int i4 = 0; i4 < N / 4; ++i4) {
                         uint32_t cb[4];
 #pragma unroll
                         for (int j = 0; j < 4; j += 2) {
-                            const float e0 = __uint_as_float(v[4 * i4 + j]), e1 = __uint_as_float(v[4 * i4 + j + 1]);
-                            float u0, u1;
-                            f2_unpack(f2_mul(f2_pack(e0, e1), inv2), u0, u1);
-                            const f32x2 um = f2_add(f2_pack(fminf(u0, u_top), fminf(u1, u_top)), magic2);   // 1.5*2^23 + k0
-                            const f32x2 kf = f2_add(um, nmagic2);
-                            float l0, l1, h0, h1;
-                            f2_unpack(f2_mul(f2_mul(f2_add(kf, nhalf2), ps2), sg2), l0, l1);
-                            f2_unpack(f2_mul(f2_mul(f2_add(kf, half2), ps2), sg2), h0, h1);
-                            const f32x2 t_lo = f2_pack(e0 > l0 ? 1.0f : 0.0f, e1 > l1 ? 1.0f : 0.0f);
-                            const f32x2 t_hi = f2_pack(e0 > h0 ? 1.0f : 0.0f, e1 > h1 ? 1.0f : 0.0f);
-                            float c0f, c1f;
-                            f2_unpack(f2_add(f2_add(um, neg1), f2_add(t_lo, t_hi)), c0f, c1f);
-                            cb[j] = __float_as_uint(c0f);                                          // code in the low byte
-                            cb[j + 1] = __float_as_uint(c1f);
+                            float u0, u1, c0, c1, d0, d1;
+                            f2_unpack(f2_mul(f2_pack(__uint_as_float(v[4 * i4 + j]), __uint_as_float(v[4 * i4 + j + 1])), inv2), u0, u1);
+                            const f32x2 u = f2_pack(fminf(u0, P.p_qp), fminf(u1, P.p_qp)), um = f2_add(u, magic2);
+                            f2_unpack(f2_fma(f2_add(um, nmagic2), neg1, u), d0, d1);
+                            far = fmaxf(far, fmaxf(fabsf(d0), fabsf(d1)));
+                            f2_unpack(um, c0, c1);
+                            cb[j] = __float_as_uint(c0);                                          // code in the low byte
+                            cb[j + 1] = __float_as_uint(c1);
                         }
                         wd[i4] = __byte_perm(__byte_perm(cb[0], cb[1], 0x4040), __byte_perm(cb[2], cb[3], 0x4040), 0x5410);
                     }
-                    const int cc = 2 * ch;
-                    uint8_t* const blk = prow + (cc >> 3) * 16384;
-                    *reinterpret_cast<uint4*>(blk + (((cc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                    *reinterpret_cast<uint4*>(blk + ((((cc + 1) & 7) ^ sw) << 4)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-                }
-            } else if constexpr (GENERAL) {
-                // t_j = fl32(S_j c) increases with S_j (c > 0), so the row's largest score gives the largest t.  Then exp(t_j - max)
-                // by reduction and polynomial, row sum in fp64, p = e / Z with 1/Z as two floats, one exact division by s_P.
-                int* const mx = reinterpret_cast<int*>(ggen + P.off_mx);
-                int smx = INT_MIN;
+                    if (__any_sync(0xffffffffu, far > near_tie)) {
+                        const float u_top = P.p_qp - 0.75f;
+                        const f32x2 half2 = f2_dup(0.5f), nhalf2 = f2_dup(-0.5f), ps2 = f2_dup(P.p_step), sg2 = f2_dup(sig_f);
+#pragma unroll
+                        for (int i4 = 0; i4 < N / 4; ++i4) {
+                            uint32_t cb[4];
+#pragma unroll
+                            for (int j = 0; j < 4; j += 2) {
+                                const float e0 = __uint_as_float(v[4 * i4 + j]), e1 = __uint_as_float(v[4 * i4 + j + 1]);
+                                float u0, u1;
+                                f2_unpack(f2_mul(f2_pack(e0, e1), inv2), u0, u1);
+                                const f32x2 um = f2_add(f2_pack(fminf(u0, u_top), fminf(u1, u_top)), magic2);   // 1.5*2^23 + k0'
+                                const f32x2 kf = f2_add(um, nmagic2);
+                                float l0, l1, h0, h1;
+                                f2_unpack(f2_mul(f2_mul(f2_add(kf, nhalf2), ps2), sg2), l0, l1);
+                                f2_unpack(f2_mul(f2_mul(f2_add(kf, half2), ps2), sg2), h0, h1);
+                                const f32x2 t_lo = f2_pack(e0 > l0 ? 1.0f : 0.0f, e1 > l1 ? 1.0f : 0.0f);
+                                const f32x2 t_hi = f2_pack(e0 > h0 ? 1.0f : 0.0f, e1 > h1 ? 1.0f : 0.0f);
+                                float c0, c1;
+                                f2_unpack(f2_add(f2_add(um, neg1), f2_add(t_lo, t_hi)), c0, c1);
+                                cb[j] = __float_as_uint(c0);
+                                cb[j + 1] = __float_as_uint(c1);
+                            }
+                            wd[i4] = __byte_perm(__byte_perm(cb[0], cb[1], 0x4040), __byte_perm(cb[2], cb[3], 0x4040), 0x5410);
+                        }
+                    }
+                };
                 if (warp_live) {
 #pragma unroll 1
-                    for (int ch = hf; ch < full_chunks; ch += 2) {
-                        uint32_t v[32];
-                        ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
+                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {
+                        uint32_t v[16], wd[4];
+                        ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
                         ptx::tmem_ld_wait();
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) smx = max(smx, (int)v[i]);
+                        codes(v, wd, std::integral_constant<int, 16>{});
+                        *reinterpret_cast<uint4*>(prow + (pc >> 3) * 16384 + (((pc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
                     }
 #pragma unroll 1
                     for (int k = tail0; k < tail_blocks; k += 2) {
-                        uint32_t v[8];
-                        ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                        uint32_t v[8], wd[2];
+                        const int col = full_chunks * 32 + k * 8, cc = col >> 4;
+                        ptx::tmem_ld8(t_row + (uint32_t)col, v);
                         ptx::tmem_ld_wait();
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) smx = max(smx, 8 * k + i < tail ? (int)v[i] : INT_MIN);
+                        codes(v, wd, std::integral_constant<int, 8>{});
+                        *reinterpret_cast<uint2*>(prow + (cc >> 3) * 16384 + (((cc & 7) ^ sw) << 4) + (col & 8)) = make_uint2(wd[0], wd[1]);
                     }
                 }
-                mx[hf * 128 + row] = smx;
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
-                w = mbar_wait(ptx::smem_addr(&B.z_sync), 0u, abort_ptr);       // two phases per item: parities 0, 1
-                if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-                smx = max(mx[row], mx[128 + row]);
-                const f32x2 c2 = f2_dup(P.scale), nmx2 = f2_dup(-__fmul_rn((float)smx, P.scale)), nmagic2 = f2_dup(-12582912.0f);
+                } else {
+                // exp(t_j - max) by reduction and polynomial, row sum in fp64, p = e / Z with 1/Z as two floats, one exact division
+                // by s_P
+                const f32x2 nmx2 = f2_dup(-__fmul_rn((float)smx, P.scale));
                 double zp[2] = {0.0, 0.0};
                 auto exp_pair = [&](uint32_t& a, uint32_t& b, bool va, bool vb) {
                     const f32x2 sf = f2_add(f2_pack(__uint_as_float(0x4B400000u + a), __uint_as_float(0x4B400000u + b)), nmagic2);   // |S| <= 2^20
@@ -502,9 +544,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 const double z = zx[row] + zx[128 + row];
                 const double r0 = (double)__frcp_rn((float)z), rz = r0 * (2.0 - z * r0);
                 const float rzh = (float)rz, rzl = (float)(rz - (double)(float)rz);
-                const f32x2 rzh2 = f2_dup(rzh), rzl2 = f2_dup(rzl), dr2 = f2_dup(p_div.r), ndb2 = f2_dup(-p_div.b), magic2 = f2_dup(12582912.0f);
-                uint8_t* const prow = ggen + P.off_p + row * 128;
-                const int sw = row & 7;
+                const f32x2 rzh2 = f2_dup(rzh), rzl2 = f2_dup(rzl), dr2 = f2_dup(p_div.r), ndb2 = f2_dup(-p_div.b);
                 auto code_pair = [&](uint32_t a, uint32_t b) -> uint32_t {                     // two codes in 16-bit halves
                     const f32x2 e = f2_pack(__uint_as_float(a), __uint_as_float(b));
                     const f32x2 p = f2_fma(e, rzh2, f2_mul(e, rzl2));
@@ -542,6 +582,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                                        __byte_perm(code_pair(v[4], v[5]), code_pair(v[6], v[7]), 0x6420));
                     }
                 }
+                }   // Eq. 4 / exp per score
             } else {
             // pass 1: e_j = EXP[S_j], row sum in fp64, e_j parked in TMEM over S_j; whole chunks of 32 columns, then the tail
             // by blocks of eight (197 tokens: 200 columns walked instead of 224)
@@ -622,7 +663,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     *reinterpret_cast<uint2*>(prow + (cc >> 3) * 16384 + (((cc & 7) ^ sw) << 4) + (col & 8)) = make_uint2(wd[0], wd[1]);
                 }
             }
-            }   // exp / Eq. 4
+            }
             ptx::fence_proxy_async_smem();
             ptx::tc_fence_before();
             __syncwarp();
@@ -683,17 +724,6 @@ extern "C" size_t vitint_attention_core_workspace_bytes(int32_t bits) {
 }
 
 namespace vitint {
-// Fills the tables of vitint_attention_core_shift for these steps.
-int attention_shift_table(int bits, float q_step, float k_step, void* table, size_t table_bytes, cudaStream_t st) {
-    const size_t need = vitint_attention_core_shift_workspace_bytes(bits);
-    if (need == 0) return VITINT_ERR_UNSUPPORTED;
-    if (!table || (reinterpret_cast<uintptr_t>(table) & 255u) || table_bytes < need) return VITINT_ERR_WORKSPACE;
-    const int m = 1 << (container_bits(bits) - 1), smax = 64 * m * m;
-    const float c2 = (float)((double)(float)((double)q_step * (double)k_step / 8.0) * 1.4426950408889634);
-    launch_kernel(shift_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (uint32_t*)table,
-                  reinterpret_cast<short*>((uint32_t*)table + (2 * smax + 1)), smax, c2);
-    return cuda_status(cudaGetLastError());
-}
 int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tokens, int smax, const float* table, float cs, float p_step,
                           float p_qp, const float* alpha_o, const float* beta_o, const vitint_codes* o_out, cudaStream_t st);
 }
@@ -727,8 +757,8 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
     // (the table itself is sized by the container so that any bit pattern indexes inside it)
     const int mq = 1 << (qkv->bits - 1);
     if (mode == AM_TABLE && 64.0 * mq * mq * (double)cs > 80.0) return VITINT_ERR_UNSUPPORTED;
-    // Eq. 4: z = S * c2 with c2 = c * log2 e; the row maximum is subtracted (as shifts), so the only range limit is the
-    // 16-bit table of floor z.  Byte-stored codes only.
+    // Eq. 4: z = S * c2 with c2 = c * log2 e; the row maximum is subtracted (as shifts), so the only range limit is that floor z
+    // is added in the integers between 2^23 and 2^24.  Byte-stored codes only.
     const float c2 = (float)((double)cs * 1.4426950408889634);
     if (shift && (c != 8 || (double)smax * (double)c2 > 30000.0)) return VITINT_ERR_UNSUPPORTED;
     if (!general && (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) ||
@@ -755,7 +785,7 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
     P.n_k = (tokens + 15) / 16 * 16;
     P.kv_rows = (tokens + 31) / 32 * 32;
     P.smax = smax;
-    P.scale = cs;
+    P.scale = shift ? c2 : cs;
     P.part_bytes = (int)(D * c / 8);
     P.table = (const float*)workspace;
     P.p_step = p_step;
@@ -770,13 +800,7 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
     // shared-memory layout
     const uint32_t hb = 8u * c;
     P.off_table = 0;
-    P.off_group = general ? 0u : up((uint32_t)(2 * smax + 1) * 4u, 1024);
-    if (shift) {
-        // 32-bit mantissas, then (from the next whole word on) the 16-bit integer parts
-        P.ftab_word = (uint32_t)(2 * smax + 1);
-        P.off_ftab = (uint32_t)(2 * smax + 1) * 4u;
-        P.off_group = up(P.off_ftab + (uint32_t)(2 * smax + 2) * 2u, 1024);
-    }
+    P.off_group = mode != AM_TABLE ? 0u : up((uint32_t)(2 * smax + 1) * 4u, 1024);
     uint32_t o = 0;
     P.off_q = o; o += 128 * 64;
     P.off_k = o; o += up((uint32_t)(c == 8 ? P.kv_rows : P.n_k) * 64, 1024);   // byte codes: the K box is kv_rows high
@@ -815,10 +839,8 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return VITINT_ERR_CUDA;
     }
-    if (build_table) {
-        if (shift) {
-            if (int rc = attention_shift_table(qkv->bits, q_step, k_step, workspace, workspace_bytes, st)) return rc;
-        } else launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
+    if (build_table && mode == AM_TABLE) {
+        launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
         if (cudaGetLastError() != cudaSuccess) return VITINT_ERR_CUDA;
     }
     int grid = sm_count();

@@ -153,8 +153,6 @@ extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layer
     p->buf[1] = buf ? buf[1] : nullptr;
     int rc = VITINT_OK;
     for (const vitint_encoder_layer_desc& L : p->layers) {
-        if (rc == VITINT_OK && L.attention == VITINT_ATTN_SHIFT_CORE)
-            rc = attention_shift_table(L.bits, L.q_step, L.k_step, L.table, L.table_bytes, (cudaStream_t)stream);
         if (rc == VITINT_OK && L.attention == VITINT_ATTN_EXP_BOUNDED)
             rc = softmax_bounded_table(L.c, L.score_bound, L.table, L.table_bytes, (cudaStream_t)stream);
     }

@@ -88,9 +88,8 @@ class EncoderLayer:
         self.qkv = B.Codes.empty(M, 3 * D, bits, True, device, container=cq)
         self.ld_s = (tokens + 3) // 4 * 4
         if self.fused_attention and softmax == "shift":
-            # the table of Eq. 4's (integer part, mantissa) pairs is built by the first call and reused
+            # (the workspace that the entry point's contract asks for)
             self.attn_table = torch.empty(B.vitint_attention_core_shift_workspace_bytes(bits), dtype=torch.uint8, device=device)
-            self.attn_table_ready = False
         elif self.fused_attention:
             # the exp table of the fused core depends only on the code width and the steps of Q and K: filled once
             self.attn_table = B.vitint_attention_exp_table(bits, self.s_q, self.s_k, device=device)
@@ -180,9 +179,7 @@ class EncoderLayer:
 
     def _tables_filled(self):
         """Making a plan fills the tables of the attention variants that build theirs on first use."""
-        if self.fused_attention and self.softmax == "shift":
-            self.attn_table_ready = True
-        elif not self.fused_attention and self.sm_table is not None:
+        if not self.fused_attention and self.sm_table is not None:
             self.sm_table_ready = True
 
     def _replan(self):
@@ -226,8 +223,7 @@ class EncoderLayer:
         mark()
         if self.fused_attention and self.softmax == "shift":
             B.vitint_attention_core_shift(self.qkv, b, h, t, self.s_q, self.s_k, self.s_p, self.bits, self.alpha_o, None,
-                                          out=self.O, workspace=self.attn_table, table_ready=self.attn_table_ready)
-            self.attn_table_ready = True
+                                          out=self.O, workspace=self.attn_table)
         elif self.fused_attention:
             B.vitint_attention_core_prepared(self.qkv, b, h, t, self.s_q, self.s_k, self.s_p, self.bits, self.alpha_o,
                                              None, out=self.O, table=self.attn_table)
@@ -374,7 +370,6 @@ class NormedAttention:
             # byte-stored QKV codes: the operand form of the fused core
             self.qkv = B.Codes.empty(M, 3 * D, bits, True, device, container=8)
             self.core_ws = torch.empty(B.vitint_attention_core_shift_workspace_bytes(bits), dtype=torch.uint8, device=device)
-            self.core_ws_ready = False
             self.slabs = self.v_slabs = None
         elif fused:
             self.qkv = B.Codes.empty(M, 3 * D, bits, True, device)
@@ -416,8 +411,7 @@ class NormedAttention:
                                        out_signed=True), out=self.v)
         if self.fused_core:
             B.vitint_attention_core_shift(self.qkv, b, h, t, self.s_qn, self.s_kn, self.s_p, self.bits, self.alpha_o, None,
-                                          out=self.O, workspace=self.core_ws, table_ready=self.core_ws_ready)
-            self.core_ws_ready = True
+                                          out=self.O, workspace=self.core_ws)
             return self.O
         B.vitint_qk(self.slabs[0], self.slabs[1], b, h, t, out=self.S, ld_s=self.ld_s)
         B.vitint_softmax_shift_quantize(self.S, t, self.c2, self.s_p, self.bits, out=self.P)

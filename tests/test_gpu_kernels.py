@@ -6,6 +6,7 @@ import torch
 import oracle as vo
 import paper_2504_18547_b200 as vt
 import synth_inputs as si
+from oracle import pipeline as vp
 from gpu_util import GELU_TOL_REL, dev, from_codes, padding_is_zero, rand_codes, to_codes
 
 pytestmark = pytest.mark.gpu
@@ -327,3 +328,32 @@ def test_attention_block_8bit_core(tokens):
     p = vt.Codes.empty(cfg.batch * cfg.heads * tokens, tokens, 8, False)
     want = vt.vitint_attention_block(xq, a, dbg_p=p)
     assert torch.equal(vt.vitint_attention_block(xq, a), want)
+
+
+@pytest.mark.parametrize("tokens", [1, 8, 9, 33, 40, 129, 197, 256])
+@pytest.mark.parametrize("bits,p_bits", [(4, 4), (4, 8), (2, 2)])
+def test_shift_core_equals_three_kernels(tokens, bits, p_bits):
+    """Eq. 4 inside the fused core: rows whose scores lie within a few octaves (summed in doubles), rows spread over hundreds
+    (64-bit integers, terms shifted out) and rows of equal scores, whose quantizer arguments sit on ties when T p_step 2 = 1."""
+    batch, heads, D = 2, 2, 128
+    rng = np.random.default_rng(900 + tokens + bits)
+    lo, hi = si.code_range(bits, True)
+    qkv = rng.integers(lo, hi + 1, (batch * tokens, 3 * D)).astype(np.int16)
+    qkv[::3, :D] //= 2                                    # narrow rows beside wide ones; image 1 mixes them in every warp
+    qkv[1::5, :D] = 0                                     # equal scores
+    packed = to_codes(qkv, bits, True)
+    codes = vt.vitint_widen(packed)
+    slabs = [vt.Slabs.of_qkv(packed, tokens, D, i) for i in range(3)]
+    alpha = dev(rng.uniform(0.01, 0.05, D).astype(np.float32))
+    for scale in (0.02, 0.3, 1.5):
+        for p_step in (np.float32(2.0 / tokens / (2 ** p_bits - 1) ** 0.5), np.float32(2.0 / tokens)):
+            step = np.float32(scale * 4.0 / (hi + 1))
+            c2 = np.float32(np.float64(vp.softmax_scale(step, step, 64)) * np.log2(np.e))
+            S = vt.vitint_qk(slabs[0], slabs[1], batch, heads, tokens)
+            P = vt.vitint_softmax_shift_quantize(S.view(batch * heads * tokens, -1), tokens, c2, p_step, p_bits)
+            epi = vt.Epilogue(mode=vt.EPI_REQUANT, alpha=alpha, out_bits=8, out_signed=True)
+            want = from_codes(vt.vitint_pv(P, slabs[2], batch, heads, tokens, 1.0, 1.0, epi))
+            out = vt.Codes.empty(batch * tokens, D, 8, True)
+            got = from_codes(vt.vitint_attention_core_shift(codes, batch, heads, tokens, step, step, p_step, p_bits, alpha, None,
+                                                            out=out))
+            assert np.array_equal(got, want), (scale, p_step)
