@@ -149,7 +149,15 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t tmem_grp = tmem_base_slot + (uint32_t)g * 256u;
 
     const int T = P.tokens;
-    const int item0 = blockIdx.x * AT_GROUPS + g, item_stride = gridDim.x * AT_GROUPS;
+    // Whole waves give every group an item; a remainder of at most one item a CTA goes to one group of as many CTAs as it takes
+    // (197 tokens x 12 heads, batch 128: 21 items in the busiest CTA instead of 22, 68.1 -> 65.0 us; batch 1: 24 CTAs instead of
+    // 12, 9.2 -> 7.7 us)
+    const int wave = gridDim.x * AT_GROUPS, full = P.total_items / wave;
+    const int last = full * wave + (P.total_items - full * wave <= (int)gridDim.x ? g * (int)gridDim.x + (int)blockIdx.x
+                                                                                  : (int)blockIdx.x * AT_GROUPS + g);
+    auto item_at = [&](int n) {                              // the group's n-th item; total_items when there is none
+        return n < full ? n * wave + (int)blockIdx.x * AT_GROUPS + g : n == full ? min(last, P.total_items) : P.total_items;
+    };
     constexpr bool DIRECT = (C == 8);                  // byte codes: no packed staging, no unpack
     const int head_bytes = 8 * C;                      // 64 codes
     const uint32_t q_bytes = 128u * head_bytes, kv_bytes = (uint32_t)P.kv_rows * head_bytes;   // TMA boxes
@@ -191,21 +199,21 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             const int pv_steps = P.kv_rows / 32;
             bool ok = true;
             int pending = -1, pending_v = -1;       // local index of the item whose loads are in flight
-            if (item0 < P.total_items) {
-                issue_loads(item0); pending = 0;
-                if (DIRECT) { issue_v(item0); pending_v = 0; }
+            if (item_at(0) < P.total_items) {
+                issue_loads(item_at(0)); pending = 0;
+                if (DIRECT) { issue_v(item_at(0)); pending_v = 0; }
             }
-            int n = 0;
-            for (int item = item0; ok && item < P.total_items; item += item_stride, ++n) {
+            for (int n = 0; ok && item_at(n) < P.total_items; ++n) {
                 const uint32_t ph = (uint32_t)n & 1u;
-                const bool has_next = item + item_stride < P.total_items;
+                const int next = item_at(n + 1);
+                const bool has_next = next < P.total_items;
                 if (DIRECT) {
                     if (!mbar_wait(ptx::smem_addr(&B.packed_full), ph, abort_ptr)) { ok = false; break; }
                     pending = -1;
                 } else {
                     if (!mbar_wait(ptx::smem_addr(&B.ops_ready), ph, abort_ptr)) { ok = false; break; }
                     pending = -1;
-                    if (has_next) { issue_loads(item + item_stride); pending = n + 1; }
+                    if (has_next) { issue_loads(next); pending = n + 1; }
                 }
                 if (n > 0 && !mbar_wait(ptx::smem_addr(&B.o_done), ph ^ 1u, abort_ptr)) { ok = false; break; }
                 ptx::tc_fence_after();
@@ -215,7 +223,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (DIRECT) {
                     // Q K^T has been read out of the Q and K tiles once s_full completes
                     if (!mbar_wait(ptx::smem_addr(&B.s_full), ph, abort_ptr)) { ok = false; break; }
-                    if (has_next) { issue_loads(item + item_stride); pending = n + 1; }
+                    if (has_next) { issue_loads(next); pending = n + 1; }
                 }
                 if (!mbar_wait(ptx::smem_addr(&B.p_ready), ph, abort_ptr)) { ok = false; break; }
                 if (DIRECT) {
@@ -232,7 +240,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (DIRECT && has_next) {
                     // P V has been read out of the V tile once o_full completes
                     if (!mbar_wait(ptx::smem_addr(&B.o_full), ph, abort_ptr)) { ok = false; break; }
-                    issue_v(item + item_stride); pending_v = n + 1;
+                    issue_v(next); pending_v = n + 1;
                 }
             }
             if (!ok) {
@@ -266,11 +274,10 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const double inv_p_step = 1.0 / (double)P.p_step;
         const Divisor p_div = make_divisor(P.p_step);               // (GENERAL)
         bool ok = true;
-        int n = 0;
-        for (int item = item0; ok && item < P.total_items; item += item_stride, ++n) {
+        for (int n = 0; ok && item_at(n) < P.total_items; ++n) {
             const uint32_t ph = (uint32_t)n & 1u;
             int b, h, qt;
-            item_coords(item, b, h, qt);
+            item_coords(item_at(n), b, h, qt);
             // the head's output parameters; the copy of the other parity may still be read by a warp that is
             // finishing the previous item, and every reader of this one passes z_sync first
             float* const colp = colp2 + (n & 1) * 128;
@@ -844,8 +851,8 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
         if (cudaGetLastError() != cudaSuccess) return VITINT_ERR_CUDA;
     }
     int grid = sm_count();
-    const int want = (P.total_items + AT_GROUPS - 1) / AT_GROUPS;
-    if (grid > want) grid = want;
+    if (grid >= P.total_items) grid = P.total_items;                         // one item a CTA
+    else if (grid > (P.total_items + 1) / 2) grid = (P.total_items + 1) / 2; // one item a group
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
     static bool attr_set_dev[MAX_DEVICES][5] = {};
