@@ -96,7 +96,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t* const smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     volatile int* abort_ptr = &abort_flag;
@@ -146,7 +146,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_grp = tmem_base_slot + (uint32_t)g * 256u;
+    const uint32_t tmem_grp = __shfl_sync(0xffffffffu, tmem_base_slot, 0) + (uint32_t)g * 256u;
 
     const int T = P.tokens;
     // Whole waves give every group an item; a remainder of at most one item a CTA goes to one group of as many CTAs as it takes
@@ -171,7 +171,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 
     if (is_control) {
         // --------------------------- control: TMA + MMA issue ----------------------------
-        if (lane == 0) {
+        {
             // packed codes: one barrier for the three slabs, which the compute warps unpack.
             // byte codes: Q and K land in their operand tiles under packed_full, V under v_full, so that each
             // buffer is refilled as soon as the MMA that read it has completed.
@@ -200,47 +200,64 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             bool ok = true;
             int pending = -1, pending_v = -1;       // local index of the item whose loads are in flight
             if (item_at(0) < P.total_items) {
-                issue_loads(item_at(0)); pending = 0;
-                if (DIRECT) { issue_v(item_at(0)); pending_v = 0; }
+                if (ptx::elect_one()) issue_loads(item_at(0));
+                pending = 0;
+                if (DIRECT) {
+                    if (ptx::elect_one()) issue_v(item_at(0));
+                    pending_v = 0;
+                }
             }
             for (int n = 0; ok && item_at(n) < P.total_items; ++n) {
                 const uint32_t ph = (uint32_t)n & 1u;
                 const int next = item_at(n + 1);
                 const bool has_next = next < P.total_items;
                 if (DIRECT) {
-                    if (!mbar_wait(ptx::smem_addr(&B.packed_full), ph, abort_ptr)) { ok = false; break; }
+                    if (!mbar_wait_warp(ptx::smem_addr(&B.packed_full), ph, abort_ptr)) { ok = false; break; }
                     pending = -1;
                 } else {
-                    if (!mbar_wait(ptx::smem_addr(&B.ops_ready), ph, abort_ptr)) { ok = false; break; }
+                    if (!mbar_wait_warp(ptx::smem_addr(&B.ops_ready), ph, abort_ptr)) { ok = false; break; }
                     pending = -1;
-                    if (has_next) { issue_loads(next); pending = n + 1; }
+                    if (has_next) {
+                        if (ptx::elect_one()) issue_loads(next);
+                        pending = n + 1;
+                    }
                 }
-                if (n > 0 && !mbar_wait(ptx::smem_addr(&B.o_done), ph ^ 1u, abort_ptr)) { ok = false; break; }
+                if (n > 0 && !mbar_wait_warp(ptx::smem_addr(&B.o_done), ph ^ 1u, abort_ptr)) { ok = false; break; }
                 ptx::tc_fence_after();
-                for (int k = 0; k < 2; ++k)                        // K = 64 -> two MMAs of 32
-                    ptx::mma_i8(tmem_grp, q_desc + (uint64_t)(k * 2), k_desc + (uint64_t)(k * 2), idesc_qk, k);
-                ptx::mma_commit(ptx::smem_addr(&B.s_full));
+                if (ptx::elect_one()) {
+                    for (int k = 0; k < 2; ++k)                    // K = 64 -> two MMAs of 32
+                        ptx::mma_i8(tmem_grp, q_desc + (uint64_t)(k * 2), k_desc + (uint64_t)(k * 2), idesc_qk, k);
+                    ptx::mma_commit(ptx::smem_addr(&B.s_full));
+                }
+                __syncwarp();
                 if (DIRECT) {
                     // Q K^T has been read out of the Q and K tiles once s_full completes
-                    if (!mbar_wait(ptx::smem_addr(&B.s_full), ph, abort_ptr)) { ok = false; break; }
-                    if (has_next) { issue_loads(next); pending = n + 1; }
+                    if (!mbar_wait_warp(ptx::smem_addr(&B.s_full), ph, abort_ptr)) { ok = false; break; }
+                    if (has_next) {
+                        if (ptx::elect_one()) issue_loads(next);
+                        pending = n + 1;
+                    }
                 }
-                if (!mbar_wait(ptx::smem_addr(&B.p_ready), ph, abort_ptr)) { ok = false; break; }
+                if (!mbar_wait_warp(ptx::smem_addr(&B.p_ready), ph, abort_ptr)) { ok = false; break; }
                 if (DIRECT) {
-                    if (!mbar_wait(ptx::smem_addr(&B.v_full), ph, abort_ptr)) { ok = false; break; }
+                    if (!mbar_wait_warp(ptx::smem_addr(&B.v_full), ph, abort_ptr)) { ok = false; break; }
                     pending_v = -1;
                 }
                 ptx::tc_fence_after();
-                for (int ks = 0; ks < pv_steps; ++ks) {
-                    const uint64_t p_desc = ptx::smem_desc(gbase + P.off_p + (uint32_t)(ks >> 2) * 16384u, 16, 1024,
-                                                           ptx::SWIZZLE_128B) + (uint64_t)((ks & 3) * 2);
-                    ptx::mma_i8(tmem_grp, p_desc, v_desc + (uint64_t)(ks * 128), idesc_pv, ks);
+                if (ptx::elect_one()) {
+                    for (int ks = 0; ks < pv_steps; ++ks) {
+                        const uint64_t p_desc = ptx::smem_desc(gbase + P.off_p + (uint32_t)(ks >> 2) * 16384u, 16, 1024,
+                                                               ptx::SWIZZLE_128B) + (uint64_t)((ks & 3) * 2);
+                        ptx::mma_i8(tmem_grp, p_desc, v_desc + (uint64_t)(ks * 128), idesc_pv, ks);
+                    }
+                    ptx::mma_commit(ptx::smem_addr(&B.o_full));
                 }
-                ptx::mma_commit(ptx::smem_addr(&B.o_full));
+                __syncwarp();
                 if (DIRECT && has_next) {
                     // P V has been read out of the V tile once o_full completes
-                    if (!mbar_wait(ptx::smem_addr(&B.o_full), ph, abort_ptr)) { ok = false; break; }
-                    issue_v(next); pending_v = n + 1;
+                    if (!mbar_wait_warp(ptx::smem_addr(&B.o_full), ph, abort_ptr)) { ok = false; break; }
+                    if (ptx::elect_one()) issue_v(next);
+                    pending_v = n + 1;
                 }
             }
             if (!ok) {

@@ -592,7 +592,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t* const smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     const uint32_t stage_i = P.ia_bytes + P.ib_bytes, stage_p = P.pa_bytes + P.pb_bytes;
@@ -627,15 +627,15 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_slot, 0);      // warp-uniform, as is `warp`
     const uint32_t acc_stride = P.tmem_cols >> 1;
     grid_dependency_wait();        // operands, parameters and the residual may come from the previous kernel
     grid_dependency_launch();
 
     if (warp == WARP_TMA) {
         // ------------------------------ TMA producer -------------------------------
-        if (lane == 0) {
-            VT_TRACER(tr, 0);
+        {
+            VT_TRACER(tr, lane == 0 ? 0 : -1);
             VT_STAMP(tr, TT_START);
             int it = 0;
             bool ok = true;
@@ -653,12 +653,15 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     const int m0 = m_tile * BM, n0 = n_tile * P.bn;
                     for (int kb = 0; kb < k_blocks; ++kb, ++it) {
                         VT_STAMP(tr, TT_WAIT_EMPTY);
-                        if (!mbar_wait(empty0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
+                        if (!mbar_wait_warp(empty0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
                         VT_STAMP(tr, TT_GOT_EMPTY);
                         const uint32_t full = full0 + 8u * (uint32_t)s;
-                        ptx::mbar_arrive_expect_tx(full, direct_bytes);
-                        ptx::tma_load_4d(dst, &map_a, full, kb * BK, m0, inner, outer);
-                        ptx::tma_load_4d(dst + P.ia_bytes, &map_b, full, kb * BK, n0, inner, outer);
+                        if (ptx::elect_one()) {
+                            ptx::mbar_arrive_expect_tx(full, direct_bytes);
+                            ptx::tma_load_4d(dst, &map_a, full, kb * BK, m0, inner, outer);
+                            ptx::tma_load_4d(dst + P.ia_bytes, &map_b, full, kb * BK, n0, inner, outer);
+                        }
+                        __syncwarp();
                         if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_i;
                     }
                 }
@@ -673,23 +676,27 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                     const uint32_t p_dst = smem_base + packed_off + (uint32_t)sp * stage_p;
                     const uint32_t i_dst = smem_base + (uint32_t)si * stage_i;
                     if (any_packed) {
-                        if (!mbar_wait(ptx::smem_addr(&bars.p_empty[sp]), php ^ 1u, abort_ptr)) { ok = false; break; }
-                        ptx::mbar_arrive_expect_tx(p_full, packed_bytes);
+                        if (!mbar_wait_warp(ptx::smem_addr(&bars.p_empty[sp]), php ^ 1u, abort_ptr)) { ok = false; break; }
+                        if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(p_full, packed_bytes);
                     }
                     if (any_direct) {
                         VT_STAMP(tr, TT_WAIT_EMPTY);
-                        if (!mbar_wait(ptx::smem_addr(&bars.i_empty[si]), phi ^ 1u, abort_ptr)) { ok = false; break; }
+                        if (!mbar_wait_warp(ptx::smem_addr(&bars.i_empty[si]), phi ^ 1u, abort_ptr)) { ok = false; break; }
                         VT_STAMP(tr, TT_GOT_EMPTY);
-                        ptx::mbar_arrive_expect_tx(i_full, direct_bytes);
+                        if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(i_full, direct_bytes);
                     }
-                    if (P.a_direct) ptx::tma_load_4d(i_dst, &map_a, i_full, kb * BK, m_tile * BM, inner, outer);
-                    else ptx::tma_load_4d(p_dst, &map_a, p_full, kb * 16 * P.ca, m_tile * BM, inner, outer);
-                    if (P.b_direct)
-                        ptx::tma_load_4d(i_dst + P.ia_bytes, &map_b, i_full, kb * BK, n_tile * P.bn, inner, outer);
-                    else if (P.b_mn_major)
-                        ptx::tma_load_4d(p_dst + P.pa_bytes, &map_b, p_full, 0, kb * BK, inner, outer);
-                    else
-                        ptx::tma_load_4d(p_dst + P.pa_bytes, &map_b, p_full, kb * 16 * P.cb, n_tile * P.bn, inner, outer);
+                    __syncwarp();
+                    if (ptx::elect_one()) {
+                        if (P.a_direct) ptx::tma_load_4d(i_dst, &map_a, i_full, kb * BK, m_tile * BM, inner, outer);
+                        else ptx::tma_load_4d(p_dst, &map_a, p_full, kb * 16 * P.ca, m_tile * BM, inner, outer);
+                        if (P.b_direct)
+                            ptx::tma_load_4d(i_dst + P.ia_bytes, &map_b, i_full, kb * BK, n_tile * P.bn, inner, outer);
+                        else if (P.b_mn_major)
+                            ptx::tma_load_4d(p_dst + P.pa_bytes, &map_b, p_full, 0, kb * BK, inner, outer);
+                        else
+                            ptx::tma_load_4d(p_dst + P.pa_bytes, &map_b, p_full, kb * 16 * P.cb, n_tile * P.bn, inner, outer);
+                    }
+                    __syncwarp();
                 }
             }
             if (!ok) {
@@ -708,14 +715,13 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         }
     } else if (warp == WARP_MMA) {
         // ------------------------------- MMA issuer --------------------------------
-        if (lane == 0) {
+        {
             const uint32_t idesc = ptx::idesc_i8(BM, P.bn, P.a_signed, P.b_signed, P.b_mn_major);
-            VT_TRACER(tr, 1);
+            VT_TRACER(tr, lane == 0 ? 1 : -1);
             VT_STAMP(tr, TT_START);
-            // This one thread feeds the tensor core, and a lone thread runs its dependent scalar instructions a few
-            // cycles apart: everything the loop needs is therefore kept in registers and advanced by additions (no
-            // division for the ring slot, no descriptor rebuilt per K block); the four MMAs of a whole K block are
-            // issued back to back.
+            // This one warp feeds the tensor core: everything the loop needs is kept in (uniform) registers and advanced by
+            // additions (no division for the ring slot, no descriptor rebuilt per K block); the four MMAs of a whole K block
+            // are issued back to back by an elected thread.
             const uint64_t a_desc0 = ptx::smem_desc(smem_base, 16, 1024, ptx::SWIZZLE_128B);
             const uint64_t b_desc0 = P.b_mn_major ? ptx::smem_desc(smem_base + P.ia_bytes, 16, 512, ptx::SWIZZLE_64B)
                                                   : ptx::smem_desc(smem_base + P.ia_bytes, 16, 1024, ptx::SWIZZLE_128B);
@@ -732,31 +738,34 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 const int buf = tl & 1;
                 const uint32_t acc_ph = (uint32_t)(tl >> 1) & 1u;
                 VT_STAMP(tr, TT_WAIT_EMPTY);
-                if (!mbar_wait(ptx::smem_addr(&bars.acc_empty[buf]), acc_ph ^ 1u, abort_ptr)) { ok = false; break; }
+                if (!mbar_wait_warp(ptx::smem_addr(&bars.acc_empty[buf]), acc_ph ^ 1u, abort_ptr)) { ok = false; break; }
                 VT_STAMP(tr, TT_GOT_EMPTY);
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * acc_stride;
                 for (int kb = 0; kb < k_blocks; ++kb) {
                     VT_STAMP(tr, TT_WAIT_FULL);
-                    if (!mbar_wait(full0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
+                    if (!mbar_wait_warp(full0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
                     VT_STAMP(tr, TT_GOT_FULL);
                     ptx::tc_fence_after();
                     // 32 int8 of K per MMA: 32 bytes along a swizzled row, or four 8-row
                     // groups (4 * 512 bytes) when K is the slow axis of the B tile
-                    if (kb + 1 < k_blocks || last_steps == 4) {
-                        ptx::mma_i8(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u);
-                        ptx::mma_i8(d_tmem, a_desc + 2u, b_desc + b_kstep, idesc, 1u);
-                        ptx::mma_i8(d_tmem, a_desc + 4u, b_desc + 2u * b_kstep, idesc, 1u);
-                        ptx::mma_i8(d_tmem, a_desc + 6u, b_desc + 3u * b_kstep, idesc, 1u);
-                    } else {
-                        for (int k = 0; k < last_steps; ++k)
-                            ptx::mma_i8(d_tmem, a_desc + (uint64_t)(k * 2), b_desc + (uint64_t)k * b_kstep, idesc, (kb | k) != 0 ? 1u : 0u);
+                    if (ptx::elect_one()) {
+                        if (kb + 1 < k_blocks || last_steps == 4) {
+                            ptx::mma_i8(d_tmem, a_desc, b_desc, idesc, kb != 0 ? 1u : 0u);
+                            ptx::mma_i8(d_tmem, a_desc + 2u, b_desc + b_kstep, idesc, 1u);
+                            ptx::mma_i8(d_tmem, a_desc + 4u, b_desc + 2u * b_kstep, idesc, 1u);
+                            ptx::mma_i8(d_tmem, a_desc + 6u, b_desc + 3u * b_kstep, idesc, 1u);
+                        } else {
+                            for (int k = 0; k < last_steps; ++k)
+                                ptx::mma_i8(d_tmem, a_desc + (uint64_t)(k * 2), b_desc + (uint64_t)k * b_kstep, idesc, (kb | k) != 0 ? 1u : 0u);
+                        }
+                        ptx::mma_commit(empty0 + 8u * (uint32_t)s);
                     }
-                    ptx::mma_commit(empty0 + 8u * (uint32_t)s);
+                    __syncwarp();
                     if (++s == ns) { s = 0; ph ^= 1u; a_desc = a_desc0; b_desc = b_desc0; }
                     else { a_desc += stage_step; b_desc += stage_step; }
                 }
-                if (ok) ptx::mma_commit(ptx::smem_addr(&bars.acc_full[buf]));
+                if (ok && ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&bars.acc_full[buf]));
                 VT_STAMP(tr, TT_ISSUED);
             }
         }

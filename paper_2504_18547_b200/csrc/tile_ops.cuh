@@ -28,6 +28,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// The same for a whole converged warp; the answer is warp-uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+
 // 8 four-bit codes of one word -> 8 bytes in natural order.
 template <int SGN>
 __device__ __forceinline__ void unpack4(uint32_t w, uint32_t& o0, uint32_t& o1) {
