@@ -602,12 +602,20 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         bool ok = true;
         VT_TRACER(tr, (lane == 0 && warp == 0) ? 2 : ((lane == 0 && warp == EPI_W - 1) ? 3 : -1));
         VT_STAMP(tr, TT_START);
-        float res[2][2][8];                                                   // fp32 kinds: the next block's residual, per half
-        auto request_residual = [&](int tile, int blk, int half) {
-            int m_tile, col_t, cols;
-            direct_tile<KIND>(P, tile, m_tile, col_t, cols);
-            const int n0 = col_t + blk * BLK, row0 = m_tile * BM + q4 * 32 + 16 * half;
-            if (tile < P.total_tiles && blk * BLK < cols) direct_residual(P, lane, row0, P.M - row0, n0, res[half]);
+        // fp32 kinds: the residual of the warp's next two units of 16 rows x 32 columns, requested two units ahead across tiles
+        float res[2][2][8];
+        int ahead_tile = blockIdx.x, ahead_u = slice;
+        auto request_residual = [&](float (&r)[2][8]) {
+            for (; ahead_tile < P.total_tiles; ahead_tile += gridDim.x, ahead_u = slice) {
+                int m_tile, col_t, cols;
+                direct_tile<KIND>(P, ahead_tile, m_tile, col_t, cols);
+                if ((ahead_u >> 1) * BLK < cols) {
+                    const int row0 = m_tile * BM + q4 * 32 + 16 * (ahead_u & 1);
+                    direct_residual(P, lane, row0, P.M - row0, col_t + (ahead_u >> 1) * BLK, r);
+                    ahead_u += SLICES;
+                    break;
+                }
+            }
         };
         if constexpr (KIND == EK_QKV_NORM) {
             // read by every epilogue warp after the first tile's group barrier
@@ -627,8 +635,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             }
         }
         if (KIND == EK_DEQUANT && RES) {
-            request_residual(blockIdx.x, slice, 0);
-            request_residual(blockIdx.x, slice, 1);
+            request_residual(res[0]);
+            request_residual(res[1]);
         }
         for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x, ++tl) {
             int m_tile, col_t, cols;
@@ -654,23 +662,26 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             const uint32_t t_quarter = tmem_base + (uint32_t)buf * acc_stride + ((uint32_t)(q4 * 32) << 16);
             const int n_blk = cols / BLK;
             if constexpr (KIND == EK_DEQUANT) {
+                // Units of half a block: 192 columns are three for every slice, where whole blocks were two for half of the slices
+                // (25,344 x 384 -> 384: 19.0 -> 17.4 us, 12,608 x 768 -> 768: 20.0 -> 18.6)
+                auto unit = [&](int u, const float (&r)[2][8]) {
+                    uint32_t v[16];
+                    const int blk = u >> 1, half = u & 1;
+                    ptx::tmem_ld_frag32(t_quarter + ((uint32_t)half << 20) + (uint32_t)(blk * BLK), v);
+                    ptx::tmem_ld_wait();
+                    direct_f32<SMALL, RES, PACKED>(P, v, epi_params, buf, blk * BLK, lane, row_q + 16 * half, rows_q - 16 * half, col_t + blk * BLK, r);
+                };
 #pragma unroll 1
-                for (int blk = slice; blk < n_blk; blk += SLICES) {
-                    const int n0 = col_t + blk * BLK;
-                    const bool more = blk + SLICES < n_blk;
+                for (int u = slice; u < 2 * n_blk; u += 2 * SLICES) {
+                    unit(u, res[0]);
+                    if (u + SLICES < 2 * n_blk) {
+                        if (RES) request_residual(res[0]);
+                        unit(u + SLICES, res[1]);
+                    } else if (RES) {                                         // an odd number: the next tile starts with the other half
 #pragma unroll
-                    for (int half = 0; half < 2; ++half) {
-                        uint32_t v[16];
-                        ptx::tmem_ld_frag32(t_quarter + ((uint32_t)half << 20) + (uint32_t)(blk * BLK), v);
-                        ptx::tmem_ld_wait();
-                        direct_f32<SMALL, RES, PACKED>(P, v, epi_params, buf, blk * BLK, lane, row_q + 16 * half, rows_q - 16 * half, n0, res[half]);
-                        // the warp's next block (of this tile or the next) is on its way from here on
-                        if (RES) request_residual(more ? tile : next_tile, more ? blk + SLICES : slice, half);
+                        for (int i = 0; i < 16; ++i) res[0][i >> 3][i & 7] = res[1][i >> 3][i & 7];
                     }
-                }
-                if (RES && slice >= n_blk) {                                  // no block of this tile was this warp's
-                    request_residual(next_tile, slice, 0);
-                    request_residual(next_tile, slice, 1);
+                    if (RES) request_residual(res[1]);
                 }
             } else {
                 bool norm = false;
@@ -745,23 +756,25 @@ bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_maj
 }
 
 // Tile width: the multiple of the column block with the least estimated time
-//     fill (K blocks x 0.27 us) + (waves - 1) x max(K blocks x 0.32 us, epilogue) + epilogue
-// where the epilogue takes 0.2 us and 9.8 (requantize), 14.8 (GELU) or 12.9 ns (fp32) a column, as measured at M = 197 ..
-// 25,344 and widths 32 .. 256: a K block costs the same at every width (four MMAs of one issuing thread), so a grid that
-// does not fill the chip takes narrow tiles (197 x 768 x 768 fp32: 7.3 us at 256 columns, 4.4 at 32) and a full one the
-// widest that does not add a wave.
+//     fill (K blocks x 0.17 us) + (waves - 1) x max(K blocks x max(0.17, 0.00125 columns) us, epilogue) + epilogue
+// where the epilogue takes 0.55 us and 8 ns a column (requantize), 0.85 and 12.4 (GELU) or 0.8 and 15.5 (fp32), as measured at
+// M = 197 .. 25,344 and widths 32 .. 256: below 136 columns a K block costs the same at every width, so a grid that does not
+// fill the chip takes narrow tiles (197 x 768 x 768 fp32: 7.1 us at 256 columns, 3.6 at 32) and a full one the widest that does
+// not add a wave (25,344 x 384 -> 1152: 20.9 us at 192 columns in nine waves, 19.3 at 256 in seven; 6304 x 768 -> 768 fp32:
+// 10.0 at 192, 9.4 at 160, both two waves).
 int direct_tile_columns(const GemmParams& P) {
     const int block = gd_block(P.kind), sms = sm_count();
     const int segments = P.kind == EK_QKV_NORM ? 3 : 1, width = P.N / segments;
-    const float per_col = P.kind == EK_QKV_NORM ? 0.017f : P.kind == EK_REQUANT ? 0.0098f : P.kind == EK_DEQUANT ? 0.0129f : 0.0148f;
-    const float k_fill = 0.27f * (float)P.k_blocks, k_main = 0.32f * (float)P.k_blocks;
+    const float per_col = P.kind == EK_QKV_NORM ? 0.017f : P.kind == EK_REQUANT ? 0.008f : P.kind == EK_DEQUANT ? 0.0155f : 0.0124f;
+    const float per_tile = P.kind == EK_QKV_NORM ? 0.2f : P.kind == EK_REQUANT ? 0.55f : P.kind == EK_DEQUANT ? 0.8f : 0.85f;
     int best = 0;
     float best_t = 0.0f;
     for (int bn = P.kind == EK_QKV_NORM ? 192 : MAX_BN; bn >= block; bn -= block) {
         if (bn > width && bn - block >= width) continue;
         const long long tiles = (long long)P.m_tiles * ((width + bn - 1) / bn) * segments;
-        const float waves = (float)((tiles + sms - 1) / sms), epi = 0.2f + per_col * (float)bn;
-        const float t = k_fill + (waves - 1.0f) * (k_main > epi ? k_main : epi) + epi;
+        const float waves = (float)((tiles + sms - 1) / sms), epi = per_tile + per_col * (float)bn;
+        const float k_main = (float)P.k_blocks * (bn > 136 ? 0.00125f * (float)bn : 0.17f);
+        const float t = 0.17f * (float)P.k_blocks + (waves - 1.0f) * (k_main > epi ? k_main : epi) + epi;
         if (!best || t < best_t) { best = bn; best_t = t; }
     }
     return best;
