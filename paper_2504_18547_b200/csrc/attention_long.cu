@@ -14,10 +14,11 @@
 // so the codes are the same.
 //
 // One pipeline per CTA, steps in sequence (every thread passes the same barriers; an expired wait makes the whole CTA
-// leave together), two CTAs per SM so that one's loads and MMAs run beside the other's softmax; the next chunk's K is on its
-// way while this one's scores are worked on, and V is awaited only in front of P V.  Items are numbered by query tile first,
+// leave together), two CTAs per SM so that one's loads and MMAs run beside the other's softmax.  A step ends with one barrier
+// of the CTA, behind which the control warp issues P V of this chunk and Q K^T of the next (of the other pass, of the next
+// item) under one completion; the K behind that is requested at the same time, and V is awaited only in front of P V.  Items are numbered by query tile first,
 // so that the last tile of every head, often nearly empty, fills the last round.  Byte-stored codes.
-// 785 tokens x 12 heads, batch 16: 202 -> 162 us.
+// 785 tokens x 12 heads, batch 16: 202 -> 160 us (with a wait and a barrier more per chunk, Q K^T issued behind them, 162).
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"
@@ -48,7 +49,7 @@ struct LongParams {
 };
 
 struct LongBars {
-    uint64_t q_full, k_full[2], v_full, s_full, o_full;
+    uint64_t q_full, k_full[2], v_full, s_full;
 };
 
 __global__ void __launch_bounds__(AL_THREADS, 2)
@@ -59,7 +60,7 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(al_smem_raw) + 1023u) & ~1023u;
     uint8_t* const smem_gen = al_smem_raw + (smem_base - ptx::smem_addr(al_smem_raw));
     volatile int* abort_ptr = &abort_flag;
@@ -72,7 +73,6 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         ptx::mbar_init(ptx::smem_addr(&B.k_full[1]), 1);
         ptx::mbar_init(ptx::smem_addr(&B.v_full), 1);
         ptx::mbar_init(ptx::smem_addr(&B.s_full), 1);
-        ptx::mbar_init(ptx::smem_addr(&B.o_full), 1);
         ptx::fence_mbar_init();
         ptx::fence_proxy_async_smem();
     }
@@ -89,7 +89,7 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    const uint32_t tmem = tmem_base_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_base_slot, 0);
 
     const int T = P.tokens, CH = P.chunk;
     const uint32_t q_bytes = 128u * 64u, kv_bytes = (uint32_t)CH * 64u;
@@ -117,9 +117,9 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     uint8_t* const prow = smem_gen + P.off_p + row * 128;
     const int sw = row & 7;
 
-    uint32_t n_q = 0, n_k = 0, n_v = 0, n_s = 0, n_o = 0;        // completed phases of each barrier (parity = count & 1; K alternates)
-    uint32_t i_q = 0, i_k = 0, i_v = 0;                          // copies issued (control lane)
-    bool ok = true;
+    uint32_t n_q = 0, n_k = 0, n_v = 0, n_s = 0;                 // completed phases of each barrier (parity = count & 1; K alternates)
+    uint32_t i_q = 0, i_k = 0, i_v = 0;                          // copies issued (control warp)
+    bool ok = true, w = true;                                    // w: every wait of this thread has been granted
     const int per_tile = P.batch * P.heads;
     auto coords = [&](int item, int& b, int& h, int& qt) {
         qt = item / per_tile;
@@ -127,30 +127,65 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         b = bh / P.heads;
         h = bh - b * P.heads;
     };
-    auto load_q = [&](int b, int h, int qt) {
-        ptx::mbar_arrive_expect_tx(ptx::smem_addr(&B.q_full), q_bytes);
-        ptx::tma_load_3d(smem_base + P.off_q, &map_q, ptx::smem_addr(&B.q_full), h * 64, qt * 128, b);
+    // A step is one chunk of one pass over an item.
+    struct Step { int item, pass, c; };
+    auto step_after = [&](Step t) {
+        if (++t.c == P.n_chunks) {
+            t.c = 0;
+            if (t.pass == 0) t.pass = 1;
+            else { t.pass = 0; t.item += (int)gridDim.x; }
+        }
+        return t;
+    };
+    auto load_q = [&](int item) {
+        int b, h, qt;
+        coords(item, b, h, qt);
+        if (ptx::elect_one()) {
+            ptx::mbar_arrive_expect_tx(ptx::smem_addr(&B.q_full), q_bytes);
+            ptx::tma_load_3d(smem_base + P.off_q, &map_q, ptx::smem_addr(&B.q_full), h * 64, qt * 128, b);
+        }
         ++i_q;
     };
-    auto load_k = [&](int b, int h, int c) {
+    auto load_k = [&](Step t) {
+        int b, h, qt;
+        coords(t.item, b, h, qt);
         const uint32_t bar = ptx::smem_addr(&B.k_full[i_k & 1u]);
-        ptx::mbar_arrive_expect_tx(bar, kv_bytes);
-        ptx::tma_load_3d(smem_base + P.off_k + (i_k & 1u) * P.k_stride, &map_kv, bar, P.part_bytes + h * 64, c * CH, b);
+        if (ptx::elect_one()) {
+            ptx::mbar_arrive_expect_tx(bar, kv_bytes);
+            ptx::tma_load_3d(smem_base + P.off_k + (i_k & 1u) * P.k_stride, &map_kv, bar, P.part_bytes + h * 64, t.c * CH, b);
+        }
         ++i_k;
     };
-    if (is_control && lane == 0 && (int)blockIdx.x < P.total_items) {
-        int b, h, qt;
-        coords(blockIdx.x, b, h, qt);
-        load_q(b, h, qt);
-        load_k(b, h, 0);
+    // Q K^T of step t into S, and the K of the step behind it (the other K buffer was read by the product before this one, which
+    // has been awaited)
+    auto issue_qk = [&](Step t) {
+        if (t.pass == 0 && t.c == 0) { w = w && mbar_wait_warp(ptx::smem_addr(&B.q_full), n_q & 1u, abort_ptr); ++n_q; }
+        w = w && mbar_wait_warp(ptx::smem_addr(&B.k_full[n_k & 1u]), (n_k >> 1) & 1u, abort_ptr);
+        if (!w) return;
+        ptx::tc_fence_after();
+        const uint64_t kd = k_desc[n_k & 1u];
+        if (ptx::elect_one()) {
+            for (int k = 0; k < 2; ++k)
+                ptx::mma_i8(tmem, q_desc + (uint64_t)(k * 2), kd + (uint64_t)(k * 2), idesc_qk, k);
+        }
+        __syncwarp();
+        ++n_k;
+        const Step next = step_after(t);
+        if (next.item < P.total_items) load_k(next);
+    };
+    if (is_control && (int)blockIdx.x < P.total_items) {
+        const Step first{(int)blockIdx.x, 0, 0};
+        load_q(first.item);
+        load_k(first);
+        issue_qk(first);
+        if (w && ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&B.s_full));
+        __syncwarp();
     }
+    w = w && mbar_wait(ptx::smem_addr(&B.s_full), 0u, abort_ptr);
+    n_s = 1;
     for (int item = blockIdx.x; ok && item < P.total_items; item += gridDim.x) {
         int b, h, qt;
         coords(item, b, h, qt);
-        if (!is_control) {
-            if (tid_c < 64) colp[tid_c] = __ldg(P.alpha_o + h * 64 + tid_c);
-            else if (tid_c < 128) colp[tid_c] = P.beta_o ? __ldg(P.beta_o + h * 64 + (tid_c - 64)) : 0.0f;
-        }
         double zp[4] = {0.0, 0.0, 0.0, 0.0};
         f32x2 rzh2 = f2_dup(0.0f), rzl2 = f2_dup(0.0f), l2 = f2_dup(0.0f);
         float limit = 0.0f, e_top = 0.0f;
@@ -158,46 +193,21 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         for (int pass = 0; ok && pass < 2; ++pass) {
             for (int c = 0; ok && c < P.n_chunks; ++c) {
                 const int key0 = c * CH;
-                // ---- S_c = Q K_c^T; the next chunk's K and this one's V are requested behind it -------------------------
-                bool w = true;
-                if (is_control && lane == 0) {
-                    if (pass == 0 && c == 0) w = mbar_wait(ptx::smem_addr(&B.q_full), n_q & 1u, abort_ptr);
-                    w = w && mbar_wait(ptx::smem_addr(&B.k_full[n_k & 1u]), (n_k >> 1) & 1u, abort_ptr);
-                    if (w) {
-                        ptx::tc_fence_after();
-                        const uint64_t kd = k_desc[n_k & 1u];
-                        for (int k = 0; k < 2; ++k)
-                            ptx::mma_i8(tmem, q_desc + (uint64_t)(k * 2), kd + (uint64_t)(k * 2), idesc_qk, k);
-                        ptx::mma_commit(ptx::smem_addr(&B.s_full));
-                        // (the other K buffer was read by the product before this one, which every thread has awaited)
-                        if (c + 1 < P.n_chunks) load_k(b, h, c + 1);
-                        else if (pass == 0) load_k(b, h, 0);
-                        else if (item + (int)gridDim.x < P.total_items) {
-                            int b2, h2, q2;
-                            coords(item + gridDim.x, b2, h2, q2);
-                            load_k(b2, h2, 0);
-                        }
-                        if (pass) {
-                            // (the V before it has been read: the last P V has been awaited)
+                w = __all_sync(0xffffffffu, w);
+                if (is_control && w) {
+                    if (pass) {
+                        // (the V before it has been read: P V completed with the scores at hand)
+                        if (ptx::elect_one()) {
                             ptx::mbar_arrive_expect_tx(ptx::smem_addr(&B.v_full), kv_bytes);
                             ptx::tma_load_3d(smem_base + P.off_v, &map_kv, ptx::smem_addr(&B.v_full), 2 * P.part_bytes + h * 64, key0, b);
-                            ++i_v;
                         }
+                        ++i_v;
+                        // Q has been read for the last time
+                        if (c + 1 == P.n_chunks && item + (int)gridDim.x < P.total_items) load_q(item + (int)gridDim.x);
                     }
                 }
-                if (pass == 0 && c == 0) ++n_q;
-                ++n_k;
-                w = w && mbar_wait(ptx::smem_addr(&B.s_full), n_s & 1u, abort_ptr);
-                ++n_s;
-                if (!__syncthreads_and(w ? 1 : 0)) { ok = false; break; }
                 ptx::tc_fence_after();
-                if (is_control && lane == 0 && pass == 1 && c + 1 == P.n_chunks && item + (int)gridDim.x < P.total_items) {
-                    // Q has been read for the last time
-                    int b2, h2, q2;
-                    coords(item + gridDim.x, b2, h2, q2);
-                    load_q(b2, h2, q2);
-                }
-                if (!is_control && warp_live) {
+                if (!is_control && w && warp_live) {
                     if (pass == 0) {
                         // ---- pass A: row sum of the table entries ------------------------------------------
 #pragma unroll 1
@@ -245,36 +255,39 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                         ptx::fence_proxy_async_smem();
                     }
                 }
+                const bool last = c + 1 == P.n_chunks;
+                if (pass == 0 && last && !is_control) {
+                    zx[hf * 128 + row] = (zp[0] + zp[1]) + (zp[2] + zp[3]);
+                    // the head's output parameters: at least two chunks, so a barrier lies behind the last item's use of them
+                    if (tid_c < 64) colp[tid_c] = __ldg(P.alpha_o + h * 64 + tid_c);
+                    else if (tid_c < 128) colp[tid_c] = P.beta_o ? __ldg(P.beta_o + h * 64 + (tid_c - 64)) : 0.0f;
+                }
                 ptx::tc_fence_before();
-                __syncthreads();                                        // S has been read; the P tile is complete
-                if (pass == 1) {
-                    // ---- O += P_c V_c ----------------------------------------------------------------------
-                    w = true;
-                    if (is_control && lane == 0) {
-                        w = mbar_wait(ptx::smem_addr(&B.v_full), n_v & 1u, abort_ptr);
+                if (!__syncthreads_and(w ? 1 : 0)) { ok = false; break; }        // S has been read; the P tile is complete
+                if (is_control) {
+                    if (pass == 1) {
+                        // ---- O += P_c V_c ----------------------------------------------------------------------
+                        w = mbar_wait_warp(ptx::smem_addr(&B.v_full), n_v & 1u, abort_ptr);
+                        ++n_v;
                         if (w) {
                             ptx::tc_fence_after();
-                            for (int ks = 0; ks < pv_steps; ++ks) {
-                                const uint64_t p_desc = ptx::smem_desc(smem_base + P.off_p + (uint32_t)(ks >> 2) * 16384u, 16, 1024,
-                                                                       ptx::SWIZZLE_128B) + (uint64_t)((ks & 3) * 2);
-                                ptx::mma_i8(tmem + AL_O_COL, p_desc, v_desc + (uint64_t)(ks * 128), idesc_pv, (c > 0 || ks > 0) ? 1 : 0);
+                            if (ptx::elect_one()) {
+                                for (int ks = 0; ks < pv_steps; ++ks) {
+                                    const uint64_t p_desc = ptx::smem_desc(smem_base + P.off_p + (uint32_t)(ks >> 2) * 16384u, 16, 1024,
+                                                                           ptx::SWIZZLE_128B) + (uint64_t)((ks & 3) * 2);
+                                    ptx::mma_i8(tmem + AL_O_COL, p_desc, v_desc + (uint64_t)(ks * 128), idesc_pv, (c > 0 || ks > 0) ? 1 : 0);
+                                }
                             }
-                            ptx::mma_commit(ptx::smem_addr(&B.o_full));
+                            __syncwarp();
                         }
                     }
-                    ++n_v;
-                    // V and the P tile are reused by the next chunk: everyone waits for the MMAs that read them
-                    w = w && mbar_wait(ptx::smem_addr(&B.o_full), n_o & 1u, abort_ptr);
-                    ++n_o;
-                    if (!__syncthreads_and(w ? 1 : 0)) { ok = false; break; }
+                    const Step next = step_after(Step{item, pass, c});
+                    if (next.item < P.total_items && w) issue_qk(next);
+                    if (w && ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&B.s_full));
+                    __syncwarp();
                 }
-            }
-            if (!ok) break;
-            if (pass == 0) {
-                // the row's two threads add their partial sums; r = 1 / (Z s_P) as a two-float number
-                if (!is_control) zx[hf * 128 + row] = (zp[0] + zp[1]) + (zp[2] + zp[3]);
-                __syncthreads();
-                if (!is_control) {
+                if (pass == 0 && last && !is_control) {
+                    // the row's two threads add their partial sums; r = 1 / (Z s_P) as a two-float number
                     const double z = zx[row] + zx[128 + row];
                     const double rz = warp_live ? inv_p_step / z : 0.0;
                     const float rzh = (float)rz;
@@ -288,13 +301,15 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     l2 = f2_dup(l);
                     limit = 0.5f - (P.p_qp + 1.0f) * 1.25f * ((4.0f * fabsf(l) + 40.0f) * 4.1316e-8f + 2.4e-7f);
                 }
-                __syncthreads();                                        // zx may be rewritten by the next item
+                // the next step's scores (the last step of all: P V alone)
+                w = w && mbar_wait(ptx::smem_addr(&B.s_full), n_s & 1u, abort_ptr);
+                ++n_s;
             }
         }
         if (!ok) break;
         // ---- requantize O and store -------------------------------------------------------------------------
         ptx::tc_fence_after();
-        if (!is_control) {
+        if (!is_control && __all_sync(0xffffffffu, w)) {
             const int token = qt * 128 + row;
             uint32_t v[32], ow[8];
             ptx::tmem_ld32(t_row + AL_O_COL + (uint32_t)(hf * 32), v);
@@ -309,11 +324,11 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 }
             }
         }
-        ptx::tc_fence_before();
-        __syncthreads();                                                // O and the head's parameters are free again
+        ptx::tc_fence_before();                                         // (O is written again a whole pass of barriers later)
     }
+    ok = ok && w;
     // copies still in flight when the CTA gives up are given a bounded chance to land
-    if (!ok && is_control && lane == 0) {
+    if (!ok && is_control) {
         auto drain = [&](uint64_t* bar, uint32_t issued) {               // the last phase of a barrier that was armed `issued` times
             for (int spin = 0; spin < (1 << 20) && issued > 0 && !ptx::mbar_try_wait(ptx::smem_addr(bar), (issued - 1u) & 1u); ++spin) {}
         };
