@@ -87,12 +87,15 @@ extern "C" int vitint_attention_block(const vitint_codes* x, const vitint_attent
     uint8_t* ws = (uint8_t*)workspace;
     const int cbits = container_bits(d->bits);
 
-    // 1. QKV linear, requantized per output channel (three per-tensor steps).  Beyond 256 tokens, when no copy of QKV
-    // or P is asked for and the logits' range allows the table-driven core, the codes are stored one per byte: the form
-    // the chunked two-pass core takes (S and P then never reach HBM).
+    // 1. QKV linear, requantized per output channel (three per-tensor steps).  Where no copy of QKV or P is asked for and the
+    // logits' range allows the table-driven core, the codes are stored one per byte: the only form that core takes beyond 256
+    // tokens (S and P then never reach HBM), and the faster one below, where its tiles need no unpacking (197 tokens x 6 heads,
+    // batch 64: 20.1 against 24.7 us) -- as long as they fit where the unfused sequence would keep QKV, S and P (all but the
+    // shortest sequences).
     const int mq = 1 << (d->bits - 1);
-    const bool wide_qkv = d->tokens > 256 && d->tokens <= 4096 && !dbg_qkv && !dbg_p && L.tab_bytes && d->bits != 8 &&
-                          64.0 * mq * mq * (double)(float)((double)d->q_step * (double)d->k_step / 8.0) <= 80.0;
+    const bool wide_qkv = !dbg_qkv && !dbg_p && L.tab_bytes && d->bits != 8 &&
+                          64.0 * mq * mq * (double)(float)((double)d->q_step * (double)d->k_step / 8.0) <= 80.0 &&
+                          (d->tokens > 256 ? d->tokens <= 4096 : d->batch <= 65535 && (size_t)(L.M * L.pitch_qkv_wide) <= L.off_o - L.off_qkv);
     vitint_codes qkv{ws + L.off_qkv, L.M, 3 * L.D, wide_qkv ? L.pitch_qkv_wide : L.pitch_qkv, d->bits, 1, wide_qkv ? 8 : 0, 0};
     vitint_epilogue e1{};
     e1.mode = VITINT_EPI_REQUANT; e1.alpha = d->alpha_qkv; e1.beta = d->beta_qkv;
@@ -104,8 +107,8 @@ extern "C" int vitint_attention_block(const vitint_codes* x, const vitint_attent
     // 2-4 fused when the shape allows and no copy of P is wanted
     int fused = VITINT_ERR_UNSUPPORTED;
     if (!dbg_p && L.tab_bytes)
-        fused = vitint_attention_core(&qkv, d->batch, d->heads, d->tokens, d->q_step, d->k_step, d->p_step, d->p_bits,
-                                      d->alpha_o, d->beta_o, &o, ws + L.off_tab, L.tab_bytes, stream);
+        fused = attention_core_behind_linear(&qkv, d->batch, d->heads, d->tokens, d->q_step, d->k_step, d->p_step, d->p_bits,
+                                             d->alpha_o, d->beta_o, &o, ws + L.off_tab, L.tab_bytes, stream);
     // 8-bit codes (no table): exp evaluated inside the core
     if (!dbg_p && d->bits == 8 && d->tokens <= 256)
         fused = attention_core_general(&qkv, d->batch, d->heads, d->tokens, d->q_step, d->k_step, d->p_step, d->p_bits, d->alpha_o,

@@ -357,3 +357,35 @@ def test_shift_core_equals_three_kernels(tokens, bits, p_bits):
             got = from_codes(vt.vitint_attention_core_shift(codes, batch, heads, tokens, step, step, p_step, p_bits, alpha, None,
                                                             out=out))
             assert np.array_equal(got, want), (scale, p_step)
+
+
+@pytest.mark.parametrize("tokens,bits", [(1, 4), (15, 2), (16, 4), (24, 4), (32, 2), (40, 3), (197, 4), (256, 3)])
+def test_attention_block_qkv_form(tokens, bits):
+    """QKV stored one code per byte where its room is that of the unfused sequence, packed otherwise or when a copy is asked for:
+    the same output and the same O, twice in a row with the workspace reused (the exp table is filled beside the QKV linear)."""
+    cfg = si.BlockConfig("form", 3, tokens, 192, 3, bits)
+    prm = si.layer_parameters(cfg)
+    xq = vt.vitint_quantize(dev(si.activations(cfg)), float(prm["s_x"]), bits, True)
+    w = {n: vt.vitint_quantize(dev(prm["w_" + n]), 0.0, bits, True, row_steps=dev(prm["s_w_" + n])) for n in ("qkv", "proj")}
+    seg = np.repeat(np.array([prm["s_q"], prm["s_k"], prm["s_v"]], np.float32), cfg.dim)
+    alpha, beta = vt.fold_requant(prm["s_x"], prm["s_w_qkv"], prm["b_qkv"], seg)
+    alpha_o, _ = vt.fold_requant(prm["s_p"], np.full(cfg.dim, prm["s_v"], np.float32), None, prm["s_o"])
+
+    def block(step):
+        return vt.AttentionWeights(cfg.batch, tokens, cfg.heads, bits, w["qkv"], dev(alpha), dev(beta), step, step, float(prm["s_v"]),
+                                   float(prm["s_p"]), float(prm["s_o"]), bits, dev(alpha_o), None, w["proj"], dev(prm["s_w_proj"]),
+                                   dev(prm["b_proj"]), vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+
+    a, b = block(float(prm["s_q"])), block(0.5 * float(prm["s_q"]))
+    work = torch.empty(vt.vitint_attention_block_workspace_bytes(a), dtype=torch.uint8, device="cuda")
+    want = []
+    for d in (a, b):
+        copy = vt.Codes.empty(cfg.rows, 3 * cfg.dim, bits, True)
+        want.append(vt.vitint_attention_block(xq, d, workspace=work, dbg_qkv=copy))
+    got = [vt.vitint_attention_block(xq, d, workspace=work) for _ in range(4) for d in (a, b)]
+    assert all(torch.equal(g, want[i % 2]) for i, g in enumerate(got))
+    o = [vt.Codes.empty(cfg.rows, cfg.dim, bits, True) for _ in range(2)]
+    p = vt.Codes.empty(cfg.batch * cfg.heads * tokens, tokens, bits, False)
+    vt.vitint_attention_block(xq, a, workspace=work, dbg_o=o[0])
+    vt.vitint_attention_block(xq, a, workspace=work, dbg_o=o[1], dbg_p=p)
+    assert torch.equal(o[0].data, o[1].data)
