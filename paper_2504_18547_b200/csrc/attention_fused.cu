@@ -66,18 +66,10 @@ struct AttnBars {
     uint64_t packed_full, v_full, ops_ready, s_full, p_ready, o_full, o_done, grp_sync, z_sync;
 };
 
-// exp(fl32(s * c)) for every integer score, correctly rounded to fp32 (fp64 exp, one rounding).  beside: the kernel in front does
-// not use the table and started after everything before it had finished (as every kernel here does), so the table is filled
-// beside that kernel and only the completion waits for it.
-__global__ void exp_table_kernel(float* table, int smax, float c, int beside) {
-    if (!beside) grid_dependency_wait();        // an earlier kernel may still read the table
+__global__ void exp_table_kernel(float* table, int smax, float c) {
+    grid_dependency_wait();        // an earlier kernel may still read the table
     grid_dependency_launch();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i <= 2 * smax) {
-        const float t = __fmul_rn((float)(i - smax), c);
-        table[i] = (float)exp((double)t);
-    }
-    if (beside) grid_dependency_wait();
+    fill_exp_table(table, smax, c, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
 // What the compute warps make of the scores: exp from the table; Eq. 4; or exp evaluated per score, for any logits (8-bit codes,
@@ -761,7 +753,7 @@ int attention_long_launch(const vitint_codes* qkv, int batch, int heads, int tok
 static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t heads, int32_t tokens,
                                  float q_step, float k_step, float p_step, int32_t p_bits, const float* alpha_o,
                                  const float* beta_o, const vitint_codes* o_out, void* workspace,
-                                 size_t workspace_bytes, bool build_table, void* stream, int mode = AM_TABLE, int beside = 0) {
+                                 size_t workspace_bytes, bool build_table, void* stream, int mode = AM_TABLE) {
     const bool shift = mode == AM_SHIFT, general = mode == AM_GENERAL;
     if (int rc = check_codes(qkv)) return rc;
     if (int rc = check_codes(o_out)) return rc;
@@ -796,7 +788,7 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
     cudaStream_t st = (cudaStream_t)stream;
     if (long_seq) {
         if (build_table) {
-            launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs, beside);
+            launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
             if (cudaGetLastError() != cudaSuccess) return VITINT_ERR_CUDA;
         }
         int pqn, pqp;
@@ -868,7 +860,7 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
             return VITINT_ERR_CUDA;
     }
     if (build_table && mode == AM_TABLE) {
-        launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs, beside);
+        launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
         if (cudaGetLastError() != cudaSuccess) return VITINT_ERR_CUDA;
     }
     int grid = sm_count();
@@ -914,14 +906,6 @@ int attention_core_general(const vitint_codes* qkv, int batch, int heads, int to
     return attention_core_launch(qkv, batch, heads, tokens, q_step, k_step, p_step, p_bits, alpha_o, beta_o, o_out, nullptr, 0, false,
                                  stream, AM_GENERAL);
 }
-
-// vitint_attention_core right behind a vitint_linear that wrote qkv.
-int attention_core_behind_linear(const vitint_codes* qkv, int batch, int heads, int tokens, float q_step, float k_step, float p_step,
-                                 int p_bits, const float* alpha_o, const float* beta_o, const vitint_codes* o_out, void* workspace,
-                                 size_t workspace_bytes, void* stream) {
-    return attention_core_launch(qkv, batch, heads, tokens, q_step, k_step, p_step, p_bits, alpha_o, beta_o, o_out, workspace,
-                                 workspace_bytes, true, stream, AM_TABLE, 1);
-}
 }  // namespace vitint
 
 extern "C" int vitint_attention_core_shift(const vitint_codes* qkv, int32_t batch, int32_t heads, int32_t tokens,
@@ -942,7 +926,7 @@ extern "C" int vitint_attention_exp_table(int32_t bits, float q_step, float k_st
     const int smax = 64 * m * m;
     const float cs = (float)((double)q_step * (double)k_step / 8.0);
     launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, (cudaStream_t)stream, (float*)table,
-                  smax, cs, 0);
+                  smax, cs);
     return cuda_status(cudaGetLastError());
 }
 

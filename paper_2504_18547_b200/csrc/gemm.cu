@@ -72,6 +72,9 @@ struct GemmParams {
     float* norm_stats;                 // [2][M * heads][2] (mu, V) or null
     const float* v_alpha;              // [D] requantization of the V segment
     const float* v_beta;               // [D] or null
+    float* exp_table;             // requantizing linear in front of an attention core: also fills the core's exp table (or null)
+    int exp_smax;
+    float exp_c;
 };
 
 struct Bars {
@@ -1138,8 +1141,9 @@ extern "C" int vitint_trace_words(void) { return TRACE_CTAS * TRACE_ROLES * TRAC
 extern "C" int vitint_trace_max_ctas(int n) { g_trace_max_ctas = n; return VITINT_OK; }
 #endif
 
-extern "C" int vitint_linear(const vitint_codes* x, float x_step, const vitint_codes* w, const float* w_step,
-                             const float* bias, const vitint_epilogue* epi, void* out, int64_t ld_out, void* stream) {
+static int linear_launch(const vitint_codes* x, float x_step, const vitint_codes* w, const float* w_step, const float* bias,
+                         const vitint_epilogue* epi, void* out, int64_t ld_out, float* exp_table, int exp_smax, float exp_c,
+                         void* stream) {
     if (int rc = check_codes(x)) return rc;
     if (int rc = check_codes(w)) return rc;
     if (x->cols != w->cols) return VITINT_ERR_INVALID_ARG;
@@ -1149,6 +1153,7 @@ extern "C" int vitint_linear(const vitint_codes* x, float x_step, const vitint_c
     if ((epi->mode == VITINT_EPI_DEQUANT_F32 || (epi->mode == VITINT_EPI_REQUANT && epi->act == 1)) && !w_step)
         return VITINT_ERR_INVALID_ARG;
     P.row_off_outer = 0; P.row_off_inner = 0; P.col_off_inner = 0;
+    P.exp_table = exp_table; P.exp_smax = exp_smax; P.exp_c = exp_c;
     Operand A{x->data, x->bits, x->is_signed, codes_container(x), (uint64_t)codes_row_bytes(x, x->cols), (uint64_t)x->rows,
               (uint64_t)x->pitch_bytes, (uint64_t)x->pitch_bytes * (uint64_t)x->rows,
               (uint64_t)x->pitch_bytes * (uint64_t)x->rows};
@@ -1157,6 +1162,22 @@ extern "C" int vitint_linear(const vitint_codes* x, float x_step, const vitint_c
               (uint64_t)w->pitch_bytes * (uint64_t)w->rows};
     return launch_gemm(A, B, (int)x->rows, (int)w->rows, (int)x->cols, 1, 1, 0, P, (cudaStream_t)stream);
 }
+
+extern "C" int vitint_linear(const vitint_codes* x, float x_step, const vitint_codes* w, const float* w_step,
+                             const float* bias, const vitint_epilogue* epi, void* out, int64_t ld_out, void* stream) {
+    return linear_launch(x, x_step, w, w_step, bias, epi, out, ld_out, nullptr, 0, 0.0f, stream);
+}
+
+namespace vitint {
+// vitint_linear with a requantizing epilogue and a multiple of 64 output channels (so that gemm_direct_kernel takes it), whose
+// epilogue warps fill an exp table of 2 smax + 1 entries while they wait for the first accumulators: one launch less in front
+// of an attention core.
+int linear_and_exp_table(const vitint_codes* x, const vitint_codes* w, const vitint_epilogue* epi, void* out, int64_t ld_out,
+                         float* table, int smax, float c, void* stream) {
+    if (epi->mode != VITINT_EPI_REQUANT || epi->act != 0 || w->rows % 64 != 0) return VITINT_ERR_INVALID_ARG;
+    return linear_launch(x, 1.0f, w, nullptr, nullptr, epi, out, ld_out, table, smax, c, stream);
+}
+}  // namespace vitint
 
 extern "C" int vitint_linear_qkv_norm(const vitint_codes* x, float x_step, const vitint_codes* w_qkv, const float* w_step,
                                       const float* bias, const float* refs, const uint8_t* flip, float n_eps,

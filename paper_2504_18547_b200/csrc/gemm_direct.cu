@@ -598,6 +598,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             fetch_params(blockIdx.x, tid_e, a, b, q);
             put_params(blockIdx.x, 0, a, b, q);
         }
+        if (KIND == EK_REQUANT && P.exp_table != nullptr)
+            fill_exp_table(P.exp_table, P.exp_smax, P.exp_c, blockIdx.x * (EPI_W * 32) + tid_e, gridDim.x * (EPI_W * 32));
         int tl = 0;
         bool ok = true;
         VT_TRACER(tr, (lane == 0 && warp == 0) ? 2 : ((lane == 0 && warp == EPI_W - 1) ? 3 : -1));

@@ -102,7 +102,7 @@ int launch_softmax_table(const int32_t* s, int64_t rows, int cols, int64_t ld_s,
 int softmax_bounded_table(float c, int score_bound, void* table, size_t table_bytes, cudaStream_t st) {
     if (!table || (reinterpret_cast<uintptr_t>(table) & 255u) || table_bytes < vitint_softmax_table_workspace_bytes(score_bound))
         return VITINT_ERR_WORKSPACE;
-    launch_kernel(exp_table_kernel, dim3((2 * score_bound + 1 + 255) / 256), dim3(256), 0, st, (float*)table, score_bound, c, 0);
+    launch_kernel(exp_table_kernel, dim3((2 * score_bound + 1 + 255) / 256), dim3(256), 0, st, (float*)table, score_bound, c);
     return cuda_status(cudaGetLastError());
 }
 

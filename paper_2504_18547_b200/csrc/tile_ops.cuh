@@ -33,6 +33,12 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
 }
 
+// exp(fl32(s * c)) for every integer score s = -smax .. smax, correctly rounded to fp32 (fp64 exp, one rounding); thread `first` of
+// `threads` that share the table.
+__device__ __forceinline__ void fill_exp_table(float* table, int smax, float c, int first, int threads) {
+    for (int i = first; i <= 2 * smax; i += threads) table[i] = (float)exp((double)__fmul_rn((float)(i - smax), c));
+}
+
 // 8 four-bit codes of one word -> 8 bytes in natural order.
 template <int SGN>
 __device__ __forceinline__ void unpack4(uint32_t w, uint32_t& o0, uint32_t& o1) {
