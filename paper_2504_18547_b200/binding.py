@@ -2,7 +2,8 @@
 from __future__ import annotations
 
 import ctypes
-from ctypes import POINTER, Structure, byref, c_char_p, c_float, c_int32, c_int64, c_size_t, c_void_p
+import struct
+from ctypes import POINTER, Structure, byref, c_char_p, c_float, c_int32, c_int64, c_size_t, c_void_p, sizeof
 from dataclasses import dataclass
 from pathlib import Path
 
@@ -59,6 +60,9 @@ class _AttentionDesc(Structure):
                 ("o_step", c_float), ("p_bits", c_int32), ("alpha_o", c_void_p), ("beta_o", c_void_p),
                 ("w_proj", _Codes), ("w_proj_step", c_void_p), ("b_proj", c_void_p), ("proj_epi", _Epilogue)]
 
+
+_PACK_ATTENTION = struct.Struct("@4i P3q4i 2P 5fi 2P P3q4i 2P 2iPq3P4i").pack      # the fields of _AttentionDesc in order
+assert struct.calcsize("@4i P3q4i 2P 5fi 2P P3q4i 2P 2iPq3P4i") == sizeof(_AttentionDesc)
 
 _lib = None
 
@@ -559,10 +563,19 @@ class AttentionWeights:
     proj_epi: Epilogue
 
     def desc(self) -> _AttentionDesc:
-        return _AttentionDesc(self.batch, self.tokens, self.heads, self.bits, self.w_qkv.desc(),
-                              _ptr(self.alpha_qkv), _ptr(self.beta_qkv), self.q_step, self.k_step, self.v_step,
-                              self.p_step, self.o_step, self.p_bits, _ptr(self.alpha_o), _ptr(self.beta_o),
-                              self.w_proj.desc(), _ptr(self.w_proj_step), _ptr(self.b_proj), self.proj_epi.desc())
+        # one packing call instead of a constructor per nested structure (6.3 -> 3.5 us of the host per block)
+        q, o, e = self.w_qkv, self.w_proj, self.proj_epi
+        d = _AttentionDesc.from_buffer_copy(_PACK_ATTENTION(
+            self.batch, self.tokens, self.heads, self.bits,
+            q.data.data_ptr(), q.rows, q.cols, q.pitch, q.bits, q.signed, q.container, 0,
+            _ptr(self.alpha_qkv) or 0, _ptr(self.beta_qkv) or 0, 0.0, 0.0, 0.0, 0.0, 0.0,
+            self.p_bits, _ptr(self.alpha_o) or 0, _ptr(self.beta_o) or 0,
+            o.data.data_ptr(), o.rows, o.cols, o.pitch, o.bits, o.signed, o.container, 0,
+            _ptr(self.w_proj_step) or 0, _ptr(self.b_proj) or 0,
+            e.mode, e.act, _ptr(e.residual) or 0, 0 if e.residual is None else _ld(e.residual), _ptr(e.alpha) or 0,
+            _ptr(e.beta) or 0, _ptr(e.inv_out_step) or 0, e.out_bits, e.out_signed, e.out_container, 0))
+        d.q_step, d.k_step, d.v_step, d.p_step, d.o_step = self.q_step, self.k_step, self.v_step, self.p_step, self.o_step
+        return d
 
 
 def vitint_attention_block_workspace_bytes(a: AttentionWeights) -> int:
