@@ -389,3 +389,22 @@ def test_attention_block_qkv_form(tokens, bits):
     vt.vitint_attention_block(xq, a, workspace=work, dbg_o=o[0])
     vt.vitint_attention_block(xq, a, workspace=work, dbg_o=o[1], dbg_p=p)
     assert torch.equal(o[0].data, o[1].data)
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 5), (1183, 768), (1185, 768), (2369, 200), (9473, 33), (4737, 127), (12608, 20)])
+@pytest.mark.parametrize("bits", [2, 3, 4, 8])
+def test_quantize_rows_per_thread(rows, cols, bits):
+    """Around the row counts from which a thread walks several rows (a remainder of the rows it takes at a time included), values
+    on ties, at and beyond the end levels, non-finite."""
+    x = si.normal(700 + rows, (rows, cols), 0.0, 3.0)
+    step = np.float32(0.25)
+    x[::3] = (np.round(x[::3] * 8) / 8).astype(np.float32)                  # ties of the quotient
+    flat = x.reshape(-1)
+    special = np.array([np.nan, np.inf, -np.inf, 3e38, -3e38, -0.0], np.float32)[:flat.size]
+    flat[:special.size] = special
+    for signed in (True, False):
+        for container in (0, 8):
+            out = vt.Codes.empty(rows, cols, bits, signed, container=container)
+            out.data.fill_(0x5A)
+            vt.vitint_quantize(dev(x), float(step), bits, signed, out=out)
+            assert np.array_equal(from_codes(out), vo.quantize(x, step, bits, signed)) and padding_is_zero(out)
