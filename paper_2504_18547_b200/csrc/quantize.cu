@@ -281,10 +281,10 @@ extern "C" int vitint_quantize(const float* x, int64_t rows, int64_t cols, int64
     int64_t gy = (rows + by - 1) / by;
     if (gy > 16384) gy = 16384;
     // Byte codes: about the threads the chip holds, each walking rows (a thread's four values are less work than its divisor).
-    // Packed codes keep one row a thread: in front of a linear, from a cold L2, the walk gained nothing (12,608 x 768 with the
-    // linear behind it 60.4 us as it is, 61.0 walking).
-    const int64_t resident = (8 * sm_count() + gx - 1) / gx;
-    const bool walks = c == 8 && !row_steps && gy > resident;
+    // 4-bit packed codes walk from more than eight rows a thread on (25,344 x 768 17.8 -> 14.2 us); below, in front of a linear and
+    // from a cold L2, one row a thread is the better form (12,608 x 768 with the linear behind it 60.4 us, walking 61.0).
+    const int64_t all_rows = (rows + by - 1) / by, resident = (8 * sm_count() + gx - 1) / gx;
+    const bool walks = !row_steps && (c == 8 ? all_rows > resident : c == 4 && all_rows > 8 * resident);
     if (walks) gy = resident;
     dim3 grid(gx, (unsigned)gy);
     cudaStream_t st = (cudaStream_t)stream;
@@ -294,7 +294,7 @@ extern "C" int vitint_quantize(const float* x, int64_t rows, int64_t cols, int64
                       (float)qn, (float)qp, vec_ok);
     };
     if (c == 2) row_steps ? launch(quantize_pack_kernel<2, true, 1>) : launch(quantize_pack_kernel<2, false, 1>);
-    else if (c == 4) row_steps ? launch(quantize_pack_kernel<4, true, 1>) : launch(quantize_pack_kernel<4, false, 1>);
+    else if (c == 4) row_steps ? launch(quantize_pack_kernel<4, true, 1>) : walks ? launch(quantize_pack_kernel<4, false, 2>) : launch(quantize_pack_kernel<4, false, 1>);
     else row_steps ? launch(quantize_pack_kernel<8, true, 1>) : walks ? launch(quantize_pack_kernel<8, false, 4>) : launch(quantize_pack_kernel<8, false, 1>);
     return cuda_status(cudaGetLastError());
 }

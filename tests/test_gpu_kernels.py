@@ -391,7 +391,7 @@ def test_attention_block_qkv_form(tokens, bits):
     assert torch.equal(o[0].data, o[1].data)
 
 
-@pytest.mark.parametrize("rows,cols", [(1, 5), (1183, 768), (1185, 768), (2369, 200), (9473, 33), (4737, 127), (12608, 20)])
+@pytest.mark.parametrize("rows,cols", [(1, 5), (1183, 768), (1185, 768), (2369, 200), (9473, 33), (4737, 127), (12608, 20), (75781, 12)])
 @pytest.mark.parametrize("bits", [2, 3, 4, 8])
 def test_quantize_rows_per_thread(rows, cols, bits):
     """Around the row counts from which a thread walks several rows (a remainder of the rows it takes at a time included), values
