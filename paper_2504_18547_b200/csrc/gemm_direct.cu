@@ -536,8 +536,13 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         int kb = grp, tile = blockIdx.x;
         while (kb >= P.k_blocks) { kb -= P.k_blocks; tile += gridDim.x; }
         while (ok && tile < P.total_tiles) {
-            bool w = mbar_wait(ptx::smem_addr(&bars.p_full[sp]), php, abort_ptr);
-            w = w && mbar_wait(ptx::smem_addr(&bars.empty[s]), ph, abort_ptr);
+            // The operand slot first: a parity tells a phase only from the one before it, and the phase of p_full[sp] before this
+            // block's is block it - ns_p, the other group's where ns_p is odd.  Once block it - ns has been contracted (blocks are
+            // contracted in order) every block up to it has landed, it - ns_p among them unless ns_p = 2 < ns, where that one is
+            // this group's own.  Asked first, the packed slot could answer for block it - 3 of a ring of three before that block
+            // had landed, and the old bytes would be expanded.
+            bool w = mbar_wait(ptx::smem_addr(&bars.empty[s]), ph, abort_ptr);
+            w = w && mbar_wait(ptx::smem_addr(&bars.p_full[sp]), php, abort_ptr);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             ptx::tc_fence_after();
             const uint8_t* pa = smem_gen + packed_off + (size_t)sp * stage_packed;

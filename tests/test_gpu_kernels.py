@@ -196,6 +196,39 @@ def test_linear_packed_large_sums():
     assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
 
 
+# ---- sizes whose packed ring has three slots (the launcher's arithmetic: 224 columns of fp32 output or 192 of the norm kind with
+# ---- both operands packed, 256 columns with one of them byte-stored or 2-bit), many K blocks, several tiles a CTA
+@pytest.mark.parametrize("M,K,N,bx,bw,kind", [(4000, 1100, 896, 4, 4, "fp32"), (12608, 896, 896, 4, 4, "fp32"), (4000, 1100, 896, 2, 4, "fp32"),
+                                              (4000, 1100, 1024, 8, 4, "codes"), (4000, 1100, 1024, 4, 2, "codes"),
+                                              (2000, 1100, 1344, 4, 4, "norm")])
+def test_linear_packed_three_slot_ring(M, K, N, bx, bw, kind):
+    qx, qw = rand_codes(141, (M, K), bx, True), rand_codes(142, (N, K), bw, True)
+    acc = vo.matmul_i32(qx, qw)
+    spread = max(float(np.abs(acc).mean()), 1.0)
+    alpha = ((np.abs(si.normal(143, (N,), 0.0, 0.2)) + 0.5) * 2 / spread).astype(np.float32)
+    beta = si.normal(144, (N,), 0.0, 0.3)
+    x, w = to_codes(qx, bx, True), to_codes(qw, bw, True)
+    for _ in range(5):                                      # the order in which copies land differs from run to run
+        if kind == "codes":
+            q = vt.vitint_linear(x, 1.0, w, None, None, vt.Epilogue(mode=vt.EPI_REQUANT, alpha=dev(alpha), beta=dev(beta), out_bits=4,
+                                                                    out_signed=True))
+            assert np.array_equal(from_codes(q), vo.epilogue_requant(acc, alpha, beta, 4, True))
+        elif kind == "fp32":
+            y = vt.vitint_linear(x, 0.75, w, dev(alpha), dev(beta), vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+            want = vo.epilogue_dequant(acc, np.float32(0.75), alpha, beta)
+            assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
+        else:
+            D = N // 3
+            rf = [compare_case(2, 64, 4, 480 + k) for k in range(2)]
+            refs, flips, n_eps = [r for _, r, _, _ in rf], [f for _, _, f, _ in rf], rf[0][3]
+            got, _ = vt.vitint_linear_qkv_norm(x, 0.5, w, dev(alpha), dev(beta), dev(np.stack(refs)), dev(np.stack(flips)), n_eps,
+                                               dev(alpha[2 * D:]), dev(beta[2 * D:]), 4)
+            y = vo.epilogue_dequant(acc, np.float32(0.5), alpha, beta)
+            want = [compare_reference(y[:, k * D:(k + 1) * D].reshape(M * D // 64, 64), refs[k], flips[k], n_eps, 4).reshape(M, D)
+                    for k in range(2)] + [vo.epilogue_requant(acc[:, 2 * D:], alpha[2 * D:], beta[2 * D:], 4, True)]
+            assert np.array_equal(from_codes(got), np.concatenate(want, axis=1))
+
+
 # ---- comparator LayerNorm: column slabs, staged chunks and rounds of rows; references no uniform quantizer would give ------
 def compare_case(rows, cols, bits, seed, refs=None):
     x = si.normal(seed, (rows, cols), 0.3, 1.7)
