@@ -314,7 +314,8 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             uint32_t v[32], ow[8];
             ptx::tmem_ld32(t_row + AL_O_COL + (uint32_t)(hf * 32), v);
             ptx::tmem_ld_wait();
-            requantize_row32(v, 0, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
+            // (once an item, so the conversion instruction: 8-bit P over more than 2056 tokens can take |O| past 2^22)
+            requantize_row32<false>(v, 0, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
             if (token < T) {
                 store_row32(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c), ow, P.out_c);
                 if (h == P.heads - 1 && hf == 1) {

@@ -334,6 +334,22 @@ def test_attention_core_column_walk(tokens, bits, p_scale):
     assert ((o >= want[0]) & (o <= want[1])).all() and padding_is_zero(got)
 
 
+@pytest.mark.parametrize("tokens,bits", [(2056, 4), (2057, 4), (2400, 4), (4096, 4), (4096, 2)])
+def test_long_attention_sums_beyond_22_bits(tokens, bits):
+    """8-bit P saturated over thousands of tokens, where |O| passes 2^22: all scores equal, so every code of P is 255 and
+    O = 255 T v."""
+    D = 64
+    lo, hi = si.code_range(bits, True)
+    qkv = np.zeros((tokens, 3 * D), np.int16)
+    qkv[:, 2 * D:] = v = (np.arange(D) % (hi - lo + 1) + lo).astype(np.int16)
+    acc = np.broadcast_to((255 * tokens * v.astype(np.int64)).astype(np.int32), (tokens, D)).copy()
+    alpha, beta = np.full(D, np.float32(100.0 / (255.0 * 8 * tokens)), np.float32), np.linspace(-20, 20, D).astype(np.float32)
+    out = vt.Codes.empty(tokens, D, 8, True)
+    vt.vitint_attention_core(byte_codes(qkv, bits, True), 1, 1, tokens, 0.25, 0.25, 1.0 / (300.0 * tokens), 8, dev(alpha), dev(beta),
+                             out=out)
+    assert np.array_equal(from_codes(out), vo.epilogue_requant(acc, alpha, beta, 8, True))
+
+
 @pytest.mark.parametrize("tokens", [1, 9, 33, 100, 145, 197, 224, 256])
 def test_layer_8bit_core_equals_three_kernels(tokens):
     """8-bit layers: the recorded pass evaluates exp inside the fused core, the launches go through S and P in memory."""
