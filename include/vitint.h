@@ -379,7 +379,8 @@ int vitint_layernorm_compare_quantize(const float* x, int64_t rows, int64_t cols
  * each stage exactly the entry point of this header that the fields name (the attention core is one fused launch, or
  * vitint_qk -> softmax -> vitint_pv where `attention` says so).  Layer i > 0 reads what layer i - 1 wrote: layer i writes
  * buf[i & 1], the last one `out`.
- *   vitint_encoder_forward          enqueues the launches one by one.
+ *   vitint_encoder_forward          enqueues the launches one by one (with VITINT_ATTN_EXP_BOUNDED also the one that fills the
+ *                                   layer's table).
  *   vitint_encoder_plan_create      records the same launches once as a CUDA graph (and enqueues, on `stream`, the kernel
  *                                   that fills the table of the bounded softmax where a layer uses it).
  *   vitint_encoder_plan_run         runs the recorded launches with this call's x and out: one graph launch instead of

@@ -19,7 +19,8 @@ struct RecorderScope {
     ~RecorderScope() { t_recorder = nullptr; }
 };
 
-int attention_stage(const vitint_encoder_layer_desc& L, void* stream) {
+// tables_ready: the table of the bounded softmax has been filled (by vitint_encoder_plan_create); otherwise the softmax fills it.
+int attention_stage(const vitint_encoder_layer_desc& L, bool tables_ready, void* stream) {
     const int64_t D = (int64_t)L.heads * 64;
     if (L.attention == VITINT_ATTN_EXP_CORE)
         return vitint_attention_core_prepared(&L.qkv, L.batch, L.heads, L.tokens, L.q_step, L.k_step, L.p_step, L.bits, L.alpha_o,
@@ -42,7 +43,7 @@ int attention_stage(const vitint_encoder_layer_desc& L, void* stream) {
         rc = vitint_softmax_shift_quantize(L.scores, rows, L.tokens, L.ld_scores, L.c, L.p_step, &L.p, stream);
     else if (L.attention == VITINT_ATTN_EXP_BOUNDED)
         rc = vitint_softmax_quantize_bounded(L.scores, rows, L.tokens, L.ld_scores, L.c, L.p_step, L.score_bound, &L.p, nullptr, 0,
-                                             L.table, L.table_bytes, 1, stream);
+                                             L.table, L.table_bytes, tables_ready ? 1 : 0, stream);
     else
         rc = vitint_softmax_quantize(L.scores, rows, L.tokens, L.ld_scores, L.c, L.p_step, &L.p, nullptr, 0, stream);
     if (rc) return rc;
@@ -51,7 +52,7 @@ int attention_stage(const vitint_encoder_layer_desc& L, void* stream) {
     return vitint_pv(&L.p, &v, L.batch, L.heads, L.tokens, L.p_step, L.v_step, &e, L.o.data, L.o.pitch_bytes, stream);
 }
 
-int run_stage(const vitint_encoder_layer_desc& L, int stage, const float* x, float* out, void* stream) {
+int run_stage(const vitint_encoder_layer_desc& L, int stage, const float* x, float* out, bool tables_ready, void* stream) {
     const int64_t D = (int64_t)L.heads * 64, M = (int64_t)L.batch * L.tokens;
     vitint_epilogue e{};
     switch (stage) {
@@ -71,7 +72,7 @@ int run_stage(const vitint_encoder_layer_desc& L, int stage, const float* x, flo
             e.out_bits = L.qkv.bits; e.out_signed = 1; e.out_container_bits = L.qkv.container_bits;
             return vitint_linear(&L.x1, L.ln_step, &L.w_qkv, nullptr, nullptr, &e, L.qkv.data, L.qkv.pitch_bytes, stream);
         case ST_ATTENTION:
-            return attention_stage(L, stream);
+            return attention_stage(L, tables_ready, stream);
         case ST_PROJ:
             e.mode = VITINT_EPI_DEQUANT_F32; e.residual = x; e.ld_res = D;
             return vitint_linear(&L.o, L.o_step, &L.w_proj, L.proj_step, L.proj_bias, &e, L.h, D, stream);
@@ -86,13 +87,13 @@ int run_stage(const vitint_encoder_layer_desc& L, int stage, const float* x, flo
 }
 
 // stage_end, when given, receives the number of launches recorded up to the end of every stage.
-int run_stack(const vitint_encoder_layer_desc* layers, int n, float* const buf[2], const float* x, float* out, void* stream,
-              std::vector<size_t>* stage_end = nullptr) {
+int run_stack(const vitint_encoder_layer_desc* layers, int n, float* const buf[2], const float* x, float* out, bool tables_ready,
+              void* stream, std::vector<size_t>* stage_end = nullptr) {
     const float* cur = x;
     for (int i = 0; i < n; ++i) {
         float* const dst = i + 1 == n ? out : buf[i & 1];
         for (int s = 0; s < NUM_STAGES; ++s) {
-            if (int rc = run_stage(layers[i], s, cur, dst, stream)) return rc;
+            if (int rc = run_stage(layers[i], s, cur, dst, tables_ready, stream)) return rc;
             if (stage_end) stage_end->push_back(t_recorder->next);
         }
         cur = dst;
@@ -132,7 +133,7 @@ struct vitint_encoder_plan {
         LaunchRecorder r;
         r.exec = exec; r.nodes = &nodes; r.next = first;
         RecorderScope scope(&r);
-        if (int rc = run_stage(layers[(size_t)layer], stage, x, out, nullptr)) return rc;
+        if (int rc = run_stage(layers[(size_t)layer], stage, x, out, true, nullptr)) return rc;
         return r.error == cudaSuccess && r.next == stage_end[at] ? VITINT_OK : VITINT_ERR_CUDA;
     }
 };
@@ -140,7 +141,7 @@ struct vitint_encoder_plan {
 extern "C" int vitint_encoder_forward(const vitint_encoder_layer_desc* layers, int32_t n_layers, float* const buf[2], const float* x,
                                       float* out, void* stream) {
     if (!valid_stack(layers, n_layers, buf) || !x || !out) return VITINT_ERR_INVALID_ARG;
-    return run_stack(layers, n_layers, buf, x, out, stream);
+    return run_stack(layers, n_layers, buf, x, out, false, stream);
 }
 
 extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layers, int32_t n_layers, float* const buf[2], void* stream,
@@ -163,7 +164,7 @@ extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layer
         r.graph = p->graph; r.nodes = &p->nodes;
         RecorderScope scope(&r);
         float* const io = p->layers[0].h;
-        rc = run_stack(p->layers.data(), n_layers, p->buf, io, io, nullptr, &p->stage_end);
+        rc = run_stack(p->layers.data(), n_layers, p->buf, io, io, true, nullptr, &p->stage_end);
         if (rc == VITINT_OK && r.error != cudaSuccess) rc = VITINT_ERR_CUDA;
     }
     if (rc == VITINT_OK && cudaGraphInstantiate(&p->exec, p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
@@ -180,7 +181,7 @@ extern "C" int vitint_encoder_plan_run(vitint_encoder_plan* plan, const float* x
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing((cudaStream_t)stream, &capturing) != cudaSuccess) return VITINT_ERR_CUDA;
     const int n = (int)plan->layers.size();
-    if (capturing != cudaStreamCaptureStatusNone) return run_stack(plan->layers.data(), n, plan->buf, x, out, stream);
+    if (capturing != cudaStreamCaptureStatusNone) return run_stack(plan->layers.data(), n, plan->buf, x, out, true, stream);
     std::lock_guard<std::mutex> guard(plan->lock);
     if (int rc = plan->update(0, ST_LN1, x, nullptr)) return rc;
     if (int rc = plan->update(0, ST_PROJ, x, nullptr)) return rc;

@@ -109,6 +109,29 @@ def test_layer_plan_equals_its_launches(kw):
     assert torch.equal(odd, one_by_one(layer, x)) and not torch.equal(odd, out)
 
 
+@pytest.mark.parametrize("kw", [{}, {"softmax": "shift"}, {"fused_attention": False, "bits": 8}, {"fused_attention": False},
+                                {"softmax": "shift", "fused_attention": False}, {"bits": 8}],
+                         ids=["exp_core", "shift_core", "exp", "exp_bounded", "shift", "exp_core_any"])
+def test_encoder_forward_equals_the_plan(kw):
+    """vitint_encoder_forward for every kind of attention, on one and three layers, the table of the bounded softmax not filled."""
+    import ctypes
+    from paper_2504_18547_b200 import binding as B
+    from paper_2504_18547_b200.encoder import EncoderStack
+    kw = dict(kw)
+    cfg = si.BlockConfig("forward", 2, 50, 128, 2, kw.pop("bits", 4), mlp_dim=320)
+    x = dev(si.normal(330, (cfg.rows, cfg.dim)))
+    for n in (1, 3):
+        stack = EncoderStack([si.layer_parameters(cfg, l) for l in range(n)], cfg.batch, cfg.tokens, cfg.heads, cfg.mlp_dim, cfg.bits, **kw)
+        want, out = stack.forward(x, torch.empty_like(x)), torch.full_like(x, float("nan"))
+        assert stack._plan is not None
+        for l in stack.layers:
+            if getattr(l, "sm_table", None) is not None:
+                l.sm_table.zero_()
+        descs, bufs = (B._EncoderLayerDesc * n)(*[l._desc() for l in stack.layers]), (ctypes.c_void_p * 2)(*[b.data_ptr() for b in stack.buf])
+        assert B.lib().vitint_encoder_forward(descs, n, bufs, x.data_ptr(), out.data_ptr(), B._stream()) == 0
+        assert torch.equal(out, want)
+
+
 def test_layer_plan_inside_a_captured_graph():
     cfg, layer = small_layer({})
     x, out = dev(si.normal(310, (cfg.rows, cfg.dim))), torch.empty((cfg.rows, cfg.dim), device="cuda")
