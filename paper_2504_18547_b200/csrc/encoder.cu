@@ -101,14 +101,25 @@ int run_stack(const vitint_encoder_layer_desc* layers, int n, float* const buf[2
     return VITINT_OK;
 }
 
-bool valid_stack(const vitint_encoder_layer_desc* layers, int n, float* const buf[2]) {
-    if (!layers || n <= 0 || (n > 1 && (!buf || !buf[0] || (n > 2 && !buf[1])))) return false;
+// What no stage checks by itself: that a layer's matrices have the rows the stages around them write or read, and the table that
+// vitint_encoder_plan_create fills in front of any stage.
+int check_stack(const vitint_encoder_layer_desc* layers, int n, float* const buf[2]) {
+    if (!layers || n <= 0 || (n > 1 && (!buf || !buf[0] || (n > 2 && !buf[1])))) return VITINT_ERR_INVALID_ARG;
     for (int i = 0; i < n; ++i) {
         const vitint_encoder_layer_desc& L = layers[i];
         if (L.batch <= 0 || L.tokens <= 0 || L.heads <= 0 || !L.h || L.attention < VITINT_ATTN_EXP_CORE || L.attention > VITINT_ATTN_EXP_CORE_ANY)
-            return false;
+            return VITINT_ERR_INVALID_ARG;
+        const int64_t D = (int64_t)L.heads * 64, M = (int64_t)L.batch * L.tokens;
+        if (L.qkv.rows != M || L.o.rows != M || L.g.rows != M || L.w_qkv.rows != 3 * D || L.w_proj.rows != D || L.w_fc1.rows != L.g.cols ||
+            L.w_fc2.rows != D)
+            return VITINT_ERR_INVALID_ARG;
+        if (L.attention == VITINT_ATTN_EXP_BOUNDED) {
+            const size_t need = vitint_softmax_table_workspace_bytes(L.score_bound);
+            if (need == 0) return L.score_bound <= 0 ? VITINT_ERR_INVALID_ARG : VITINT_ERR_UNSUPPORTED;
+            if (!L.table || (reinterpret_cast<uintptr_t>(L.table) & 255u) || L.table_bytes < need) return VITINT_ERR_WORKSPACE;
+        }
     }
-    return true;
+    return VITINT_OK;
 }
 
 }  // namespace
@@ -140,23 +151,21 @@ struct vitint_encoder_plan {
 
 extern "C" int vitint_encoder_forward(const vitint_encoder_layer_desc* layers, int32_t n_layers, float* const buf[2], const float* x,
                                       float* out, void* stream) {
-    if (!valid_stack(layers, n_layers, buf) || !x || !out) return VITINT_ERR_INVALID_ARG;
+    if (int rc = check_stack(layers, n_layers, buf)) return rc;
+    if (!x || !out) return VITINT_ERR_INVALID_ARG;
     return run_stack(layers, n_layers, buf, x, out, false, stream);
 }
 
 extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layers, int32_t n_layers, float* const buf[2], void* stream,
                                           vitint_encoder_plan** plan) {
-    if (!plan || !valid_stack(layers, n_layers, buf)) return VITINT_ERR_INVALID_ARG;
+    if (!plan) return VITINT_ERR_INVALID_ARG;
+    if (int rc = check_stack(layers, n_layers, buf)) return rc;
     *plan = nullptr;
     vitint_encoder_plan* p = new vitint_encoder_plan;
     p->layers.assign(layers, layers + n_layers);
     p->buf[0] = buf ? buf[0] : nullptr;
     p->buf[1] = buf ? buf[1] : nullptr;
     int rc = VITINT_OK;
-    for (const vitint_encoder_layer_desc& L : p->layers) {
-        if (rc == VITINT_OK && L.attention == VITINT_ATTN_EXP_BOUNDED)
-            rc = softmax_bounded_table(L.c, L.score_bound, L.table, L.table_bytes, (cudaStream_t)stream);
-    }
     if (rc == VITINT_OK && cudaGraphCreate(&p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
     if (rc == VITINT_OK) {
         // recorded with the intermediate buffer in place of x and out; every run sets its own
@@ -166,6 +175,11 @@ extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layer
         float* const io = p->layers[0].h;
         rc = run_stack(p->layers.data(), n_layers, p->buf, io, io, true, nullptr, &p->stage_end);
         if (rc == VITINT_OK && r.error != cudaSuccess) rc = VITINT_ERR_CUDA;
+    }
+    // (behind the stages' own checks, which recording has run)
+    for (const vitint_encoder_layer_desc& L : p->layers) {
+        if (rc == VITINT_OK && L.attention == VITINT_ATTN_EXP_BOUNDED)
+            rc = softmax_bounded_table(L.c, L.score_bound, L.table, L.table_bytes, (cudaStream_t)stream);
     }
     if (rc == VITINT_OK && cudaGraphInstantiate(&p->exec, p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
     if (rc != VITINT_OK) {

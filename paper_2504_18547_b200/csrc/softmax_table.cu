@@ -98,7 +98,7 @@ int launch_softmax_table(const int32_t* s, int64_t rows, int cols, int64_t ld_s,
 
 }  // namespace
 
-// Fills the table of vitint_softmax_quantize_bounded.
+// Fills the table of vitint_softmax_quantize_bounded; score_bound in 1 .. 8192, checked by the callers.
 int softmax_bounded_table(float c, int score_bound, void* table, size_t table_bytes, cudaStream_t st) {
     if (!table || (reinterpret_cast<uintptr_t>(table) & 255u) || table_bytes < vitint_softmax_table_workspace_bytes(score_bound))
         return VITINT_ERR_WORKSPACE;

@@ -150,3 +150,40 @@ def test_layernorm_reference_folding_matches_the_oracle_side(L):
         assert np.array_equal(np.signbit(refs) & (refs != 0), (neg != 0) & (ref != 0))
         assert np.array_equal(flip_b, flip) and flip_b.sum() == 2
         assert np.all(np.diff(refs.astype(np.float64), axis=1) >= 0)      # ascending along the thresholds
+
+
+def _layer_desc(L, fake, **kw):
+    """A consistent layer descriptor, none of whose pointers is dereferenced on the host."""
+    d = L._EncoderLayerDesc()
+    d.batch, d.tokens, d.heads, d.bits, d.attention = 2, 16, 1, 4, L.ATTN_EXP
+    codes = lambda rows, cols, s=1: L._Codes(fake, rows, cols, max(32, cols // 2), 4, s, 0, 0)
+    d.w_qkv, d.w_proj, d.w_fc1, d.w_fc2 = codes(192, 64), codes(64, 64), codes(128, 64), codes(64, 128)
+    d.x1, d.qkv, d.o, d.x2, d.g, d.p = codes(32, 64), codes(32, 192), codes(32, 64), codes(32, 64), codes(32, 128, 0), codes(32, 16, 0)
+    d.h = d.scores = d.table = fake
+    d.ld_scores, d.table_bytes, d.c, d.score_bound = 16, 4096, 0.001, 256
+    for k, v in kw.items():
+        setattr(d, k, v)
+    return d
+
+
+def test_encoder_descriptors_are_checked_before_anything_is_launched(L):
+    lib, fake = L.lib(), 0x7000_0000_0000
+    plan = ctypes.c_void_p()
+
+    def create(**kw):
+        d = _layer_desc(L, fake, **kw)
+        return lib.vitint_encoder_plan_create(ctypes.byref(d), 1, None, None, ctypes.byref(plan)), \
+            lib.vitint_encoder_forward(ctypes.byref(d), 1, None, fake, fake, None)
+
+    bounded = {"attention": L.ATTN_EXP_BOUNDED}
+    assert create(**bounded, score_bound=9000) == (-2, -2)          # more entries than any table has
+    assert create(**bounded, score_bound=0) == (-1, -1)
+    assert create(**bounded, score_bound=8192) == (-5, -5)          # 65,792 bytes
+    assert create(**bounded, table=fake + 16) == (-5, -5)
+    assert create(**bounded, table=None) == (-5, -5)
+    rows = lambda n, cols: L._Codes(fake, n, cols, 64, 4, 1, 0, 0)
+    for name, codes in (("qkv", rows(64, 192)), ("o", rows(64, 64)), ("g", rows(64, 128)), ("w_proj", rows(128, 64)), ("w_fc2", rows(128, 128)),
+                        ("w_qkv", rows(64, 64)), ("w_fc1", rows(256, 64))):
+        assert create(**{name: codes}) == (-1, -1), name
+    assert create(attention=6) == (-1, -1) and create(h=None) == (-1, -1)
+    assert plan.value is None
