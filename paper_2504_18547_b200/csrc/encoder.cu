@@ -4,6 +4,8 @@
 // kernels run for 3 to 9 us each, so launches one by one are what a small batch waits for.  A graph launch costs the host
 // little per kernel; x and out of a call enter through the parameters of the first layer's LayerNorm and projection and the
 // last layer's fc2, which are rewritten before each launch.
+#include <exception>
+#include <memory>
 #include <mutex>
 
 #include "common.cuh"
@@ -13,6 +15,16 @@ namespace vitint {
 namespace {
 
 enum Stage { ST_LN1, ST_QKV, ST_ATTENTION, ST_PROJ, ST_LN2, ST_FC1, ST_FC2, NUM_STAGES };
+
+// What the C++ library throws (no host memory, a lock that fails) ends here as a status: a plan's functions are called from C.
+template <typename F>
+int no_exceptions(F&& f) {
+    try {
+        return f();
+    } catch (const std::exception&) {
+        return VITINT_ERR_CUDA;
+    }
+}
 
 struct RecorderScope {
     explicit RecorderScope(LaunchRecorder* r) { t_recorder = r; }
@@ -161,33 +173,31 @@ extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layer
     if (!plan) return VITINT_ERR_INVALID_ARG;
     if (int rc = check_stack(layers, n_layers, buf)) return rc;
     *plan = nullptr;
-    vitint_encoder_plan* p = new vitint_encoder_plan;
-    p->layers.assign(layers, layers + n_layers);
-    p->buf[0] = buf ? buf[0] : nullptr;
-    p->buf[1] = buf ? buf[1] : nullptr;
-    int rc = VITINT_OK;
-    if (rc == VITINT_OK && cudaGraphCreate(&p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
-    if (rc == VITINT_OK) {
-        // recorded with the intermediate buffer in place of x and out; every run sets its own
-        LaunchRecorder r;
-        r.graph = p->graph; r.nodes = &p->nodes;
-        RecorderScope scope(&r);
-        float* const io = p->layers[0].h;
-        rc = run_stack(p->layers.data(), n_layers, p->buf, io, io, true, nullptr, &p->stage_end);
-        if (rc == VITINT_OK && r.error != cudaSuccess) rc = VITINT_ERR_CUDA;
-    }
-    // (behind the stages' own checks, which recording has run)
-    for (const vitint_encoder_layer_desc& L : p->layers) {
-        if (rc == VITINT_OK && L.attention == VITINT_ATTN_EXP_BOUNDED)
-            rc = softmax_bounded_table(L.c, L.score_bound, L.table, L.table_bytes, (cudaStream_t)stream);
-    }
-    if (rc == VITINT_OK && cudaGraphInstantiate(&p->exec, p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
-    if (rc != VITINT_OK) {
-        delete p;
+    return no_exceptions([&]() -> int {
+        std::unique_ptr<vitint_encoder_plan> p(new vitint_encoder_plan);
+        p->layers.assign(layers, layers + n_layers);
+        p->buf[0] = buf ? buf[0] : nullptr;
+        p->buf[1] = buf ? buf[1] : nullptr;
+        int rc = VITINT_OK;
+        if (rc == VITINT_OK && cudaGraphCreate(&p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
+        if (rc == VITINT_OK) {
+            // recorded with the intermediate buffer in place of x and out; every run sets its own
+            LaunchRecorder r;
+            r.graph = p->graph; r.nodes = &p->nodes;
+            RecorderScope scope(&r);
+            float* const io = p->layers[0].h;
+            rc = run_stack(p->layers.data(), n_layers, p->buf, io, io, true, nullptr, &p->stage_end);
+            if (rc == VITINT_OK && r.error != cudaSuccess) rc = VITINT_ERR_CUDA;
+        }
+        // (behind the stages' own checks, which recording has run)
+        for (const vitint_encoder_layer_desc& L : p->layers) {
+            if (rc == VITINT_OK && L.attention == VITINT_ATTN_EXP_BOUNDED)
+                rc = softmax_bounded_table(L.c, L.score_bound, L.table, L.table_bytes, (cudaStream_t)stream);
+        }
+        if (rc == VITINT_OK && cudaGraphInstantiate(&p->exec, p->graph, 0) != cudaSuccess) rc = VITINT_ERR_CUDA;
+        if (rc == VITINT_OK) *plan = p.release();
         return rc;
-    }
-    *plan = p;
-    return VITINT_OK;
+    });
 }
 
 extern "C" int vitint_encoder_plan_run(vitint_encoder_plan* plan, const float* x, float* out, void* stream) {
@@ -196,11 +206,13 @@ extern "C" int vitint_encoder_plan_run(vitint_encoder_plan* plan, const float* x
     if (cudaStreamIsCapturing((cudaStream_t)stream, &capturing) != cudaSuccess) return VITINT_ERR_CUDA;
     const int n = (int)plan->layers.size();
     if (capturing != cudaStreamCaptureStatusNone) return run_stack(plan->layers.data(), n, plan->buf, x, out, true, stream);
-    std::lock_guard<std::mutex> guard(plan->lock);
-    if (int rc = plan->update(0, ST_LN1, x, nullptr)) return rc;
-    if (int rc = plan->update(0, ST_PROJ, x, nullptr)) return rc;
-    if (int rc = plan->update(n - 1, ST_FC2, nullptr, out)) return rc;
-    return cuda_status(cudaGraphLaunch(plan->exec, (cudaStream_t)stream));
+    return no_exceptions([&]() -> int {
+        std::lock_guard<std::mutex> guard(plan->lock);
+        if (int rc = plan->update(0, ST_LN1, x, nullptr)) return rc;
+        if (int rc = plan->update(0, ST_PROJ, x, nullptr)) return rc;
+        if (int rc = plan->update(n - 1, ST_FC2, nullptr, out)) return rc;
+        return cuda_status(cudaGraphLaunch(plan->exec, (cudaStream_t)stream));
+    });
 }
 
 extern "C" void vitint_encoder_plan_destroy(vitint_encoder_plan* plan) { delete plan; }

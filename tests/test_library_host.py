@@ -2,6 +2,8 @@
 declares, and rejects bad arguments before anything is launched (no compute call is made)."""
 import ctypes
 import re
+import subprocess
+import sys
 from pathlib import Path
 
 import pytest
@@ -187,3 +189,24 @@ def test_encoder_descriptors_are_checked_before_anything_is_launched(L):
         assert create(**{name: codes}) == (-1, -1), name
     assert create(attention=6) == (-1, -1) and create(h=None) == (-1, -1)
     assert plan.value is None
+
+
+def test_no_exception_leaves_a_c_entry(L):
+    """A plan for which the host has no memory: a status, not std::bad_alloc through the C boundary (which ends the process)."""
+    script = """
+import ctypes, resource, sys
+sys.path[:0] = [{root!r}, {tests!r}]
+import paper_2504_18547_b200.binding as L
+from test_library_host import _layer_desc
+n, plan = 120000, ctypes.c_void_p()
+arr = (L._EncoderLayerDesc * n)()
+one = bytes(_layer_desc(L, 0x7000_0000_0000))
+ctypes.memmove(arr, one * n, len(one) * n)
+buf = (ctypes.c_void_p * 2)(0x7000_0000_0000, 0x7000_0000_0000)
+create = L.lib().vitint_encoder_plan_create
+pages = int(open("/proc/self/statm").read().split()[0])
+resource.setrlimit(resource.RLIMIT_AS, (pages * resource.getpagesize() + (1 << 26),) * 2)
+print("status", create(arr, n, buf, None, ctypes.byref(plan)), plan.value)
+""".format(root=str(ROOT), tests=str(ROOT / "tests"))
+    r = subprocess.run([sys.executable, "-c", script], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "status -6 None" in r.stdout, (r.returncode, r.stdout, r.stderr[-500:])
