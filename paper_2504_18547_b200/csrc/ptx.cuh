@@ -193,9 +193,10 @@ __device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, uint32_t (&v)[16]
         : "r"(taddr)
         : "memory");
 }
-// 32-byte global accesses of eight floats (address 32-byte aligned).
+// 32-byte global accesses of eight floats (address 32-byte aligned).  Not through the read-only path (.nc): a residual may be
+// the output buffer itself, and a kernel may be resident while the one in front of it still writes.
 __device__ __forceinline__ void ld_global_32B(const float* p, float (&v)[8]) {
-    asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                  : "l"(p));
 }

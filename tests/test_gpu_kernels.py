@@ -66,6 +66,18 @@ def test_linear_fp32_dispatch_boundary(M, N):
     assert np.array_equal(y.cpu().numpy().view(np.uint32), want.view(np.uint32))
 
 
+@pytest.mark.parametrize("M,K,N", [(129, 64, 96), (3000, 128, 768), (25216, 64, 768)])
+def test_linear_residual_in_place(M, K, N):
+    """out is the residual: several calls in a row on one buffer, as an accumulating caller makes them."""
+    qx, qw = rand_codes(151, (M, K), 4, True), rand_codes(152, (N, K), 4, True)
+    acc, s_w, y = vo.matmul_i32(qx, qw), np.full(N, np.float32(0.01), np.float32), si.normal(153, (M, N))
+    x, w, buf = byte_codes(qx, 4, True), byte_codes(qw, 4, True), dev(y)
+    for _ in range(6):
+        vt.vitint_linear(x, 0.75, w, dev(s_w), None, vt.Epilogue(mode=vt.EPI_DEQUANT_F32, residual=buf), out=buf)
+        y = vo.epilogue_dequant(acc, np.float32(0.75), s_w, None, y)
+    assert np.array_equal(buf.cpu().numpy().view(np.uint32), y.view(np.uint32))
+
+
 # ---- recorded layers: the plan against the same launches one by one ------------------------------------------------
 def small_layer(kw, layer=0, cfg=None):
     from paper_2504_18547_b200.encoder import EncoderLayer
