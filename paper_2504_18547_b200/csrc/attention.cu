@@ -93,8 +93,9 @@ extern "C" int vitint_attention_block(const vitint_codes* x, const vitint_attent
     // batch 64: 20.1 against 24.7 us) -- as long as they fit where the unfused sequence would keep QKV, S and P (all but the
     // shortest sequences).
     const int mq = 1 << (d->bits - 1);
-    const bool wide_qkv = !dbg_qkv && !dbg_p && L.tab_bytes && d->bits != 8 &&
-                          64.0 * mq * mq * (double)(float)((double)d->q_step * (double)d->k_step / 8.0) <= 80.0 &&
+    const float c = (float)((double)d->q_step * (double)d->k_step / 8.0);
+    const bool in_range = 64.0 * mq * mq * (double)c <= 80.0;        // else the core refuses and the unfused sequence runs
+    const bool wide_qkv = !dbg_qkv && !dbg_p && L.tab_bytes && d->bits != 8 && in_range &&
                           (d->tokens > 256 ? d->tokens <= 4096 : d->batch <= 65535 && (size_t)(L.M * L.pitch_qkv_wide) <= L.off_o - L.off_qkv);
     vitint_codes qkv{ws + L.off_qkv, L.M, 3 * L.D, wide_qkv ? L.pitch_qkv_wide : L.pitch_qkv, d->bits, 1, wide_qkv ? 8 : 0, 0};
     vitint_epilogue e1{};
@@ -102,11 +103,10 @@ extern "C" int vitint_attention_block(const vitint_codes* x, const vitint_attent
     e1.out_bits = d->bits; e1.out_signed = 1; e1.out_container_bits = wide_qkv ? 8 : 0;
     // The exp table of the core is filled by the same launch, one less for the host, whose launches set the pace of small blocks
     // (197 tokens: one image x 3 heads 24.8 -> 23.5 us, 64 images x 6 heads 57.2 -> 55.7).
-    const bool table_core = !dbg_p && L.tab_bytes;
+    const bool table_core = !dbg_p && L.tab_bytes, fill = table_core && in_range && (d->tokens <= 256 || wide_qkv);
     const int half = 1 << (cbits - 1), bound = 64 * half * half;     // scores of b-bit codes, at the container's width
-    const float c = (float)((double)d->q_step * (double)d->k_step / 8.0);
-    if (int rc = table_core ? linear_and_exp_table(x, &d->w_qkv, &e1, qkv.data, qkv.pitch_bytes, (float*)(ws + L.off_tab), bound, c, stream)
-                            : vitint_linear(x, 1.0f, &d->w_qkv, nullptr, nullptr, &e1, qkv.data, qkv.pitch_bytes, stream))
+    if (int rc = fill ? linear_and_exp_table(x, &d->w_qkv, &e1, qkv.data, qkv.pitch_bytes, (float*)(ws + L.off_tab), bound, c, stream)
+                      : vitint_linear(x, 1.0f, &d->w_qkv, nullptr, nullptr, &e1, qkv.data, qkv.pitch_bytes, stream))
         return rc;
     if (int rc = copy_codes(dbg_qkv, qkv.data, L.pitch_qkv, L.M, row_bytes(3 * L.D, d->bits), st)) return rc;
 

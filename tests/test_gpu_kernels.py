@@ -475,6 +475,28 @@ def test_attention_block_qkv_form(tokens, bits):
     assert torch.equal(o[0].data, o[1].data)
 
 
+@pytest.mark.parametrize("tokens,q_step", [(40, 1.0), (300, 1.0), (40, 0.1), (300, 0.1)])
+def test_attention_block_range_of_the_logits(tokens, q_step):
+    """Logits that the exp table cannot hold (the unfused sequence) and logits that it can, with a copy of QKV beside."""
+    cfg = si.BlockConfig("range", 2, tokens, 128, 2, 4)
+    prm = si.layer_parameters(cfg)
+    xq = vt.vitint_quantize(dev(si.activations(cfg)), float(prm["s_x"]), 4, True)
+    w = {n: vt.vitint_quantize(dev(prm["w_" + n]), 0.0, 4, True, row_steps=dev(prm["s_w_" + n])) for n in ("qkv", "proj")}
+    seg = np.repeat(np.array([prm["s_q"], prm["s_k"], prm["s_v"]], np.float32), cfg.dim)
+    alpha, beta = vt.fold_requant(prm["s_x"], prm["s_w_qkv"], prm["b_qkv"], seg)
+    alpha_o, _ = vt.fold_requant(prm["s_p"], np.full(cfg.dim, prm["s_v"], np.float32), None, prm["s_o"])
+    a = vt.AttentionWeights(cfg.batch, tokens, cfg.heads, 4, w["qkv"], dev(alpha), dev(beta), q_step, q_step, float(prm["s_v"]),
+                            float(prm["s_p"]), float(prm["s_o"]), 4, dev(alpha_o), None, w["proj"], dev(prm["s_w_proj"]),
+                            dev(prm["b_proj"]), vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+    work = torch.empty(vt.vitint_attention_block_workspace_bytes(a), dtype=torch.uint8, device="cuda")
+    p = vt.Codes.empty(cfg.batch * cfg.heads * tokens, tokens, 4, False)
+    want = vt.vitint_attention_block(xq, a, dbg_p=p, workspace=work)
+    work.fill_(0xA5)
+    assert torch.equal(vt.vitint_attention_block(xq, a, workspace=work), want)
+    qkv = vt.Codes.empty(cfg.rows, 3 * cfg.dim, 4, True)
+    assert torch.equal(vt.vitint_attention_block(xq, a, workspace=work, dbg_qkv=qkv), want)
+
+
 @pytest.mark.parametrize("rows,cols", [(1, 5), (1183, 768), (1185, 768), (2369, 200), (9473, 33), (4737, 127), (12608, 20), (75781, 12)])
 @pytest.mark.parametrize("bits", [2, 3, 4, 8])
 def test_quantize_rows_per_thread(rows, cols, bits):
