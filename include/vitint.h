@@ -382,7 +382,8 @@ int vitint_layernorm_compare_quantize(const float* x, int64_t rows, int64_t cols
  *   vitint_encoder_forward          enqueues the launches one by one (with VITINT_ATTN_EXP_BOUNDED also the one that fills the
  *                                   layer's table).
  *   vitint_encoder_plan_create      records the same launches once as a CUDA graph (and enqueues, on `stream`, the kernel
- *                                   that fills the table of the bounded softmax where a layer uses it).
+ *                                   that fills the table of the bounded softmax where a layer uses it; on a stream that is
+ *                                   being captured that kernel becomes part of the capture, like any other launch).
  *   vitint_encoder_plan_run         runs the recorded launches with this call's x and out: one graph launch instead of
  *                                   seven or more launches per layer.  On a stream that is being captured the launches are
  *                                   enqueued one by one.  Safe to call from several threads; calls that overlap on the GPU

@@ -26,6 +26,14 @@ int no_exceptions(F&& f) {
     }
 }
 
+// A plan is made and destroyed in calls that a stream capture elsewhere in the process (or on this thread) would otherwise count
+// against itself: they touch no stream, so the thread leaves the capture's restrictions for their time.
+struct OutsideCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OutsideCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
 struct RecorderScope {
     explicit RecorderScope(LaunchRecorder* r) { t_recorder = r; }
     ~RecorderScope() { t_recorder = nullptr; }
@@ -174,6 +182,7 @@ extern "C" int vitint_encoder_plan_create(const vitint_encoder_layer_desc* layer
     if (int rc = check_stack(layers, n_layers, buf)) return rc;
     *plan = nullptr;
     return no_exceptions([&]() -> int {
+        OutsideCapture outside;
         std::unique_ptr<vitint_encoder_plan> p(new vitint_encoder_plan);
         p->layers.assign(layers, layers + n_layers);
         p->buf[0] = buf ? buf[0] : nullptr;
@@ -215,4 +224,7 @@ extern "C" int vitint_encoder_plan_run(vitint_encoder_plan* plan, const float* x
     });
 }
 
-extern "C" void vitint_encoder_plan_destroy(vitint_encoder_plan* plan) { delete plan; }
+extern "C" void vitint_encoder_plan_destroy(vitint_encoder_plan* plan) {
+    OutsideCapture outside;
+    delete plan;
+}

@@ -158,6 +158,40 @@ def test_layer_plan_inside_a_captured_graph():
     assert torch.equal(out, want)
 
 
+def test_plans_made_run_and_dropped_during_a_capture():
+    """Neither the capturing thread's plans nor another thread's forward() may end a capture."""
+    import threading
+    from paper_2504_18547_b200 import binding as B
+    cfg, layer = small_layer({})
+    (_, other), (_, dropped) = small_layer({}), small_layer({})
+    x = dev(si.normal(312, (cfg.rows, cfg.dim)))
+    out, elsewhere, late = (torch.zeros_like(x) for _ in range(3))
+    want = layer.forward(x, torch.empty_like(x)).clone()
+    stream, errors = torch.cuda.Stream(), []
+    torch.cuda.synchronize()
+
+    def beside():
+        try:
+            with torch.cuda.stream(stream):
+                other.forward(x, elsewhere)
+        except Exception as e:                               # noqa: BLE001 -- reported by the main thread
+            errors.append(e)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        layer.forward(x, out)
+        del dropped
+        plan = B.EncoderPlan([layer._desc()])
+        t = threading.Thread(target=beside)
+        t.start()
+        t.join()
+    assert not errors
+    graph.replay()
+    plan.run(x, late)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and torch.equal(elsewhere, want) and torch.equal(late, want)
+
+
 def test_stack_plan_from_two_threads():
     import threading
     from paper_2504_18547_b200.encoder import EncoderStack
