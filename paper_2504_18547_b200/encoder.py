@@ -23,6 +23,8 @@ def _dev(a, device):
 
 
 class EncoderLayer:
+    _any_core = False
+
     def __init__(self, batch: int, tokens: int, heads: int, mlp_dim: int, bits: int, prm: dict, device="cuda",
                  eps: float = 1e-6, widen_weights: bool = True, fused_attention: bool = True,
                  wide_activations: bool = True, softmax: str = "exp", layernorm: str = "fp32", plan: bool = True):
@@ -47,7 +49,8 @@ class EncoderLayer:
                                      or (softmax == "shift" and wide_activations and tokens <= 256)))
         self.stages = STAGES_FUSED if self.fused_attention else STAGES_UNFUSED
         # 8-bit scores have no table: Q K^T, softmax and P V one by one (as forward() with events times them), or, in the
-        # recorded layer, the fused core that evaluates exp per score -- the same codes without S and P in memory
+        # recorded layer, the fused core that evaluates exp per score -- the same codes without S and P in memory, which
+        # the layer has only once they are asked for (__getattr__)
         self._any_core = fused_attention and bits == 8 and softmax == "exp" and tokens <= 256
         d = lambda a: _dev(a, device)
         f = lambda k: float(prm[k])
@@ -94,8 +97,9 @@ class EncoderLayer:
             # the exp table of the fused core depends only on the code width and the steps of Q and K: filled once
             self.attn_table = B.vitint_attention_exp_table(bits, self.s_q, self.s_k, device=device)
         else:
-            self.S = torch.empty((batch * heads * tokens, self.ld_s), dtype=torch.int32, device=device)
-            self.P = B.Codes.empty(batch * heads * tokens, tokens, bits, False, device)
+            if not self._any_core:
+                self.S, self.P = self._new_scores()
+            self._spare_scores = None
             # scores of b-bit codes are bounded by 64 * 2^(b-1) * 2^(b-1): where the table-driven softmax takes that
             # range its exp table is built by the first call and reused afterwards
             half = 1 << ((4 if bits == 3 else bits) - 1)
@@ -120,6 +124,30 @@ class EncoderLayer:
         if plan:
             self._replan()
 
+    def _new_scores(self):
+        n = self.batch * self.heads * self.tokens
+        return (torch.empty((n, self.ld_s), dtype=torch.int32, device=self.device),
+                B.Codes.empty(n, self.tokens, self.bits, False, self.device))
+
+    def _scores(self):
+        """S and P for the three attention kernels: the layer's own, or spare ones where forward() does without."""
+        if not self._any_core:
+            return self.S, self.P
+        if self._spare_scores is None:
+            self._spare_scores = self._new_scores()
+        return self._spare_scores
+
+    def __getattr__(self, name):
+        """S and P of an 8-bit layer.  The first time one is asked for, both get the scores and codes of the last call (its QKV
+        codes are still there), and from then on forward() keeps them in memory: whoever holds them sees every later call's."""
+        if name not in ("S", "P") or not self._any_core:
+            raise AttributeError(f"{type(self).__name__!r} object has no attribute {name!r}")
+        S, P = self._scores()
+        B.vitint_qk(self.slabs[0], self.slabs[1], self.batch, self.heads, self.tokens, out=S, ld_s=self.ld_s)
+        B.vitint_softmax_quantize(S, self.tokens, self.c, self.s_p, self.bits, out=P)
+        self._any_core, self.S, self.P, self._spare_scores = False, S, P, None
+        return self.__dict__[name]
+
     def _signature(self) -> list:
         """Everything a plan takes from this layer, as plain values: the addresses of its weights, parameters and buffers,
         and its scalars.  A plan is used only while it equals the one the plan was made for."""
@@ -137,7 +165,7 @@ class EncoderLayer:
             v += [self.ln1_g.data_ptr(), self.ln1_b.data_ptr(), self.ln2_g.data_ptr(), self.ln2_b.data_ptr()]
         if self.fused_attention:
             v.append(self.attn_table.data_ptr())
-        else:
+        elif not self._any_core:
             v += [self.S.data_ptr(), self.P.data.data_ptr(), self.c, self.c2]
             if self.sm_table is not None:
                 v.append(self.sm_table.data_ptr())
@@ -165,6 +193,8 @@ class EncoderLayer:
         if self.fused_attention:
             d.attention = B.ATTN_SHIFT_CORE if self.softmax == "shift" else B.ATTN_EXP_CORE
             table = self.attn_table
+        elif self._any_core:
+            d.attention = B.ATTN_EXP_CORE_ANY
         else:
             d.scores, d.ld_scores, d.p = p(self.S), self.ld_s, self.P.desc()
             if self.softmax == "shift":
@@ -172,7 +202,7 @@ class EncoderLayer:
             elif self.sm_table is not None:
                 d.attention, d.c, d.score_bound, table = B.ATTN_EXP_BOUNDED, self.c, self.score_bound, self.sm_table
             else:
-                d.attention, d.c = B.ATTN_EXP_CORE_ANY if self._any_core else B.ATTN_EXP, self.c
+                d.attention, d.c = B.ATTN_EXP, self.c
         if table is not None:
             d.table, d.table_bytes = p(table), table.numel()
         return d
@@ -199,7 +229,8 @@ class EncoderLayer:
 
     def forward(self, x: torch.Tensor, out: torch.Tensor, events: list | None = None) -> torch.Tensor:
         """x, out: fp32 [batch*tokens, dim] on the device.  `events`, when given, receives
-        len(self.stages)+1 recorded CUDA events bracketing the stages."""
+        len(self.stages)+1 recorded CUDA events bracketing the stages (of an 8-bit layer too: Q K^T, softmax and P V, where
+        a call without events runs one kernel with the same codes)."""
         if events is None and self._plan is not None and self._plain_io(x, out):
             if self._plan_for != self._signature():
                 self._replan()
@@ -228,18 +259,19 @@ class EncoderLayer:
             B.vitint_attention_core_prepared(self.qkv, b, h, t, self.s_q, self.s_k, self.s_p, self.bits, self.alpha_o,
                                              None, out=self.O, table=self.attn_table)
         else:
-            B.vitint_qk(self.slabs[0], self.slabs[1], b, h, t, out=self.S, ld_s=self.ld_s)
+            S, P = self._scores()
+            B.vitint_qk(self.slabs[0], self.slabs[1], b, h, t, out=S, ld_s=self.ld_s)
             mark()
             if self.softmax == "shift":
-                B.vitint_softmax_shift_quantize(self.S, t, self.c2, self.s_p, self.bits, out=self.P)
+                B.vitint_softmax_shift_quantize(S, t, self.c2, self.s_p, self.bits, out=P)
             elif self.sm_table is not None:
-                B.vitint_softmax_quantize_bounded(self.S, t, self.c, self.s_p, self.bits, self.score_bound, out=self.P,
+                B.vitint_softmax_quantize_bounded(S, t, self.c, self.s_p, self.bits, self.score_bound, out=P,
                                                   workspace=self.sm_table, table_ready=self.sm_table_ready)
                 self.sm_table_ready = True
             else:
-                B.vitint_softmax_quantize(self.S, t, self.c, self.s_p, self.bits, out=self.P)
+                B.vitint_softmax_quantize(S, t, self.c, self.s_p, self.bits, out=P)
             mark()
-            B.vitint_pv(self.P, self.slabs[2], b, h, t, self.s_p, self.s_v, self.epi_o, out=self.O)
+            B.vitint_pv(P, self.slabs[2], b, h, t, self.s_p, self.s_v, self.epi_o, out=self.O)
         mark()
         B.vitint_linear(self.O, self.s_o, self.w["proj"], self.s_w["proj"], self.bias["proj"],
                         B.Epilogue(mode=B.EPI_DEQUANT_F32, residual=x), out=self.h)

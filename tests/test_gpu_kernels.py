@@ -430,6 +430,24 @@ def test_layer_8bit_core_equals_three_kernels(tokens):
     assert torch.equal(out, one_by_one(layer, x)) and torch.equal(o, layer.O.data)
 
 
+@pytest.mark.parametrize("tokens", [9, 197])
+def test_8bit_layer_keeps_scores_that_are_asked_for(tokens):
+    """S and P hold the last call's scores and codes whenever they are looked at; held references follow later calls."""
+    cfg, layer = small_layer({"bits": 8, "tokens": tokens})
+    _, three = small_layer({"bits": 8, "tokens": tokens, "fused_attention": False})
+    assert not hasattr(layer, "no_such_attribute")
+    for i in range(4):
+        x = dev(si.normal(620 + i, (cfg.rows, cfg.dim)))
+        out, want = torch.empty_like(x), torch.empty_like(x)
+        layer.forward(x, out) if i != 3 else layer.forward(x, out, events=[])
+        three.forward(x, want)
+        assert torch.equal(out, want) and layer._plan is not None
+        if i == 1:
+            S, P = layer.S, layer.P
+        if i:
+            assert torch.equal(S[:, :tokens], three.S[:, :tokens]) and torch.equal(P.data, three.P.data)
+
+
 @pytest.mark.parametrize("tokens", [5, 197])
 def test_attention_block_8bit_core(tokens):
     """vitint_attention_block with 8-bit codes: with a copy of P (three kernels) and without (the fused core)."""
