@@ -18,6 +18,10 @@ STAGES_FUSED = ("ln1_quant", "qkv_linear", "attention_core", "proj_linear", "ln2
 GEMM_STAGES = ("qkv_linear", "qk", "pv", "proj_linear", "fc1_linear", "fc2_linear")
 
 
+_NO_TENSOR = torch.empty(0)                # stands for an absent tensor where addresses are compared
+_data_ptr = torch.Tensor.data_ptr
+
+
 def _dev(a, device):
     return torch.from_numpy(np.ascontiguousarray(a)).to(device)
 
@@ -149,34 +153,50 @@ class EncoderLayer:
         return self.__dict__[name]
 
     def _signature(self) -> list:
-        """Everything a plan takes from this layer, as plain values: the addresses of its weights, parameters and buffers,
-        and its scalars.  A plan is used only while it equals the one the plan was made for."""
-        w, s, b = self.w, self.s_w, self.bias
+        """Everything the launches take from this layer, as plain values: the addresses of its weights, parameters and buffers,
+        the forms of weights and epilogues, and its scalars.  A plan is used only while it equals the one the plan was made for."""
+        w, s, b, eq, eg, none = self.w, self.s_w, self.bias, self.epi_qkv, self.epi_fc1, _NO_TENSOR
+        wq, wp, w1, w2 = w["qkv"], w["proj"], w["fc1"], w["fc2"]
+        bq, bp, b1, b2 = eq.beta, b["proj"], b["fc1"], b["fc2"]
+        t = [self.x1.data, self.qkv.data, self.O.data, self.x2.data, self.g.data, self.h, wq.data, wp.data, w1.data, w2.data,
+             s["proj"], s["fc1"], s["fc2"], eq.alpha, eg.inv_out_step, none if bq is None else bq, none if bp is None else bp, none if b1 is None else b1,
+             none if b2 is None else b2]
         v = [self.s_ln, self.s_q, self.s_k, self.s_v, self.s_p, self.s_o, self.s_g, self.eps, self.batch, self.tokens,
-             self.x1.data.data_ptr(), self.qkv.data.data_ptr(), self.O.data.data_ptr(), self.x2.data.data_ptr(),
-             self.g.data.data_ptr(), self.h.data_ptr(), self.alpha_qkv.data_ptr(), self.beta_qkv.data_ptr(),
-             self.alpha_o.data_ptr(), self.inv_s_g.data_ptr(), w["qkv"].data.data_ptr(), w["proj"].data.data_ptr(),
-             w["fc1"].data.data_ptr(), w["fc2"].data.data_ptr(), s["proj"].data_ptr(), s["fc1"].data_ptr(),
-             s["fc2"].data_ptr(), b["proj"].data_ptr(), b["fc1"].data_ptr(), b["fc2"].data_ptr()]
+             wq.container, wp.container, w1.container, w2.container, eq.mode, eq.act, eq.out_bits, eq.out_signed, eq.out_container,
+             eg.mode, eg.act, eg.out_bits, eg.out_signed, eg.out_container]
         if self.layernorm == "compare":
             (r1, f1), (r2, f2) = self.ln_refs
-            v += [r1.data_ptr(), f1.data_ptr(), r2.data_ptr(), f2.data_ptr(), self.ln_stats.data_ptr(), self.n_eps]
+            t += [r1, r2, self.ln_stats, none if f1 is None else f1, none if f2 is None else f2]
+            v.append(self.n_eps)
         else:
-            v += [self.ln1_g.data_ptr(), self.ln1_b.data_ptr(), self.ln2_g.data_ptr(), self.ln2_b.data_ptr()]
+            t += [self.ln1_g, self.ln1_b, self.ln2_g, self.ln2_b]
         if self.fused_attention:
-            v.append(self.attn_table.data_ptr())
-        elif not self._any_core:
-            v += [self.S.data_ptr(), self.P.data.data_ptr(), self.c, self.c2]
-            if self.sm_table is not None:
-                v.append(self.sm_table.data_ptr())
+            t += [self.alpha_o, self.attn_table]
+        else:
+            eo = self.epi_o
+            t += [eo.alpha, none if eo.beta is None else eo.beta]
+            v += [eo.mode, eo.act, eo.out_bits, eo.out_signed, eo.out_container, self.c, self.c2, self._any_core]
+            if not self._any_core:
+                t += [self.S, self.P.data]
+                v += [self.P.container, self.ld_s, self.score_bound]
+                if self.sm_table is not None:
+                    t.append(self.sm_table)
+        v.extend(map(_data_ptr, t))
         return v
+
+    def _recordable(self) -> bool:
+        """Whether the epilogues are of the form that a recorded layer gives them (forward() takes any)."""
+        def form(e, codes, act, signed):
+            return (e.mode, e.act, e.out_bits, bool(e.out_signed), e.out_container) == (B.EPI_REQUANT, act, codes.bits, signed, codes.container)
+        return (form(self.epi_qkv, self.qkv, 0, True) and form(self.epi_fc1, self.g, 1, False)
+                and (self.fused_attention or (form(self.epi_o, self.O, 0, True) and self.epi_o.beta is None)))
 
     def _desc(self):
         d = B._EncoderLayerDesc()
         d.batch, d.tokens, d.heads, d.bits = self.batch, self.tokens, self.heads, self.bits
         d.eps, d.ln_step, d.g_step = self.eps, self.s_ln, self.s_g
         d.q_step, d.k_step, d.v_step, d.p_step, d.o_step = self.s_q, self.s_k, self.s_v, self.s_p, self.s_o
-        p = lambda t: t.data_ptr()
+        p = B._ptr
         if self.layernorm == "compare":
             d.compare_layernorm, d.n_eps, d.ln_stats = 1, self.n_eps, p(self.ln_stats)
             (r1, f1), (r2, f2) = self.ln_refs
@@ -184,7 +204,8 @@ class EncoderLayer:
         else:
             d.ln1_gamma, d.ln1_beta, d.ln2_gamma, d.ln2_beta = p(self.ln1_g), p(self.ln1_b), p(self.ln2_g), p(self.ln2_b)
         d.w_qkv, d.w_proj, d.w_fc1, d.w_fc2 = (self.w[n].desc() for n in ("qkv", "proj", "fc1", "fc2"))
-        d.alpha_qkv, d.beta_qkv, d.alpha_o, d.inv_g_step = p(self.alpha_qkv), p(self.beta_qkv), p(self.alpha_o), p(self.inv_s_g)
+        d.alpha_qkv, d.beta_qkv, d.inv_g_step = p(self.epi_qkv.alpha), p(self.epi_qkv.beta), p(self.epi_fc1.inv_out_step)
+        d.alpha_o = p(self.alpha_o if self.fused_attention else self.epi_o.alpha)
         d.proj_step, d.fc1_step, d.fc2_step = (p(self.s_w[n]) for n in ("proj", "fc1", "fc2"))
         d.proj_bias, d.fc1_bias, d.fc2_bias = (p(self.bias[n]) for n in ("proj", "fc1", "fc2"))
         d.x1, d.qkv, d.o, d.x2, d.g = self.x1.desc(), self.qkv.desc(), self.O.desc(), self.x2.desc(), self.g.desc()
@@ -216,6 +237,8 @@ class EncoderLayer:
         """Records the layer's launches.  Where a stage does not take the layer's shape or steps there is no plan, and
         forward() reports the error of that stage."""
         self._plan_for, self._plan = self._signature(), None
+        if not self._recordable():
+            return
         try:
             self._plan = B.EncoderPlan([self._desc()])
         except B.VitintError:
@@ -326,6 +349,8 @@ class EncoderStack:
 
     def _replan(self):
         self._plan_for, self._plan = self._signature(), None
+        if not all(l._recordable() for l in self.layers):
+            return
         try:
             self._plan = B.EncoderPlan([l._desc() for l in self.layers], self.buf)
         except B.VitintError:

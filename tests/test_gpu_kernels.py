@@ -121,6 +121,43 @@ def test_layer_plan_equals_its_launches(kw):
     assert torch.equal(odd, one_by_one(layer, x)) and not torch.equal(odd, out)
 
 
+@pytest.mark.parametrize("kw", [{}, {"fused_attention": False}, {"bits": 8}], ids=["core", "three_kernels", "bits8"])
+def test_plan_follows_every_parameter_that_the_launches_read(kw):
+    cfg, layer = small_layer(dict(kw))
+    x = dev(si.normal(352, (cfg.rows, cfg.dim)))
+    seen = []
+
+    def same(changed=True):
+        out = layer.forward(x, torch.empty_like(x))
+        assert torch.equal(out, one_by_one(layer, x))
+        assert not seen or torch.equal(out, seen[-1]) != changed
+        seen.append(out)
+
+    same()
+    layer.epi_qkv.alpha = layer.epi_qkv.alpha * 0.5
+    same()
+    layer.epi_qkv.beta = None
+    same()
+    layer.epi_fc1.inv_out_step = layer.epi_fc1.inv_out_step * 0.5
+    same()
+    for name in ("proj", "fc1", "fc2"):
+        layer.bias[name] = None
+        same()
+    layer.alpha_qkv, layer.beta_qkv, layer.inv_s_g = (t * 3.0 for t in (layer.alpha_qkv, layer.beta_qkv, layer.inv_s_g))
+    same(changed=False)                                     # the launches read the epilogues
+    if layer.fused_attention:
+        layer.alpha_o = layer.alpha_o * 0.5
+        same()
+    else:
+        layer.epi_o.alpha = layer.epi_o.alpha * 0.5
+        same()
+        assert layer._plan is not None
+        layer.epi_o.beta = torch.full((cfg.dim,), 1.0, device="cuda")      # no recorded layer has it: launched one by one
+        same()
+        layer.epi_o.beta = None
+        same()
+
+
 @pytest.mark.parametrize("kw", [{}, {"softmax": "shift"}, {"fused_attention": False, "bits": 8}, {"fused_attention": False},
                                 {"softmax": "shift", "fused_attention": False}, {"bits": 8}],
                          ids=["exp_core", "shift_core", "exp", "exp_bounded", "shift", "exp_core_any"])
