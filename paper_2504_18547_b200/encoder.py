@@ -26,7 +26,23 @@ def _dev(a, device):
     return torch.from_numpy(np.ascontiguousarray(a)).to(device)
 
 
-class EncoderLayer:
+class _Recorded:
+    """What recorded layers and stacks share: the plan, and the signature of the state it was made for."""
+    _record = False
+    _plan = _plan_for = None
+
+    def _planned(self):
+        """The plan of the layer or stack as it is now.  None where a stage does not take its shape or steps: forward() then
+        launches one by one and reports the error of that stage; it is recorded again once it has changed."""
+        if not self._record:
+            return None
+        now = self._signature()
+        if now != self._plan_for:
+            self._plan_for, self._plan = now, self._new_plan()
+        return self._plan
+
+
+class EncoderLayer(_Recorded):
     _any_core = False
 
     def __init__(self, batch: int, tokens: int, heads: int, mlp_dim: int, bits: int, prm: dict, device="cuda",
@@ -124,9 +140,8 @@ class EncoderLayer:
         self.epi_o = B.Epilogue(mode=B.EPI_REQUANT, alpha=self.alpha_o, out_bits=bits, out_signed=True, out_container=ca)
         self.epi_fc1 = B.Epilogue(mode=B.EPI_REQUANT, act=1, inv_out_step=self.inv_s_g, out_bits=bits, out_signed=False,
                                   out_container=ca)
-        self._plan = self._plan_for = None
-        if plan:
-            self._replan()
+        self._record = plan
+        self._planned()
 
     def _new_scores(self):
         n = self.batch * self.heads * self.tokens
@@ -233,17 +248,15 @@ class EncoderLayer:
         if not self.fused_attention and self.sm_table is not None:
             self.sm_table_ready = True
 
-    def _replan(self):
-        """Records the layer's launches.  Where a stage does not take the layer's shape or steps there is no plan, and
-        forward() reports the error of that stage."""
-        self._plan_for, self._plan = self._signature(), None
+    def _new_plan(self):
         if not self._recordable():
-            return
+            return None
         try:
-            self._plan = B.EncoderPlan([self._desc()])
+            plan = B.EncoderPlan([self._desc()])
         except B.VitintError:
-            return
+            return None
         self._tables_filled()
+        return plan
 
     def _plain_io(self, x: torch.Tensor, out: torch.Tensor) -> bool:
         """Whether x and out are dense matrices of the layer's shape (what a plan takes)."""
@@ -254,12 +267,10 @@ class EncoderLayer:
         """x, out: fp32 [batch*tokens, dim] on the device.  `events`, when given, receives
         len(self.stages)+1 recorded CUDA events bracketing the stages (of an 8-bit layer too: Q K^T, softmax and P V, where
         a call without events runs one kernel with the same codes)."""
-        if events is None and self._plan is not None and self._plain_io(x, out):
-            if self._plan_for != self._signature():
-                self._replan()
-            if self._plan is not None:
-                self._plan.run(x, out)
-                return out
+        plan = self._planned() if events is None and self._plain_io(x, out) else None
+        if plan is not None:
+            plan.run(x, out)
+            return out
         def mark():
             if events is not None:
                 e = torch.cuda.Event(enable_timing=True)
@@ -330,7 +341,7 @@ class EncoderLayer:
                 "softmax_quant": n * T * 4 + n * ((T * c + 7) // 8)}
 
 
-class EncoderStack:
+class EncoderStack(_Recorded):
     """`layers` integerized encoder layers applied in sequence (each with its own weights and steps);
     the fp32 residual stream ping-pongs between two device buffers."""
 
@@ -340,31 +351,28 @@ class EncoderStack:
         self.layers = [EncoderLayer(batch, tokens, heads, mlp_dim, bits, prm, device, **kw) for prm in layer_params]
         rows, dim = batch * tokens, heads * 64
         self.buf = [torch.empty((rows, dim), dtype=torch.float32, device=device) for _ in range(2)]
-        self._plan = self._plan_for = None
-        if self.layers:
-            self._replan()
+        self._record = bool(self.layers)
+        self._planned()
 
     def _signature(self) -> list:
         return [l._signature() for l in self.layers] + [b.data_ptr() for b in self.buf]
 
-    def _replan(self):
-        self._plan_for, self._plan = self._signature(), None
+    def _new_plan(self):
         if not all(l._recordable() for l in self.layers):
-            return
+            return None
         try:
-            self._plan = B.EncoderPlan([l._desc() for l in self.layers], self.buf)
+            plan = B.EncoderPlan([l._desc() for l in self.layers], self.buf)
         except B.VitintError:
-            return
+            return None
         for l in self.layers:
             l._tables_filled()
+        return plan
 
     def forward(self, x: torch.Tensor, out: torch.Tensor) -> torch.Tensor:
-        if self._plan is not None and self.layers[0]._plain_io(x, out):
-            if self._plan_for != self._signature():
-                self._replan()
-            if self._plan is not None:
-                self._plan.run(x, out)
-                return out
+        plan = self._planned() if self._record and self.layers[0]._plain_io(x, out) else None
+        if plan is not None:
+            plan.run(x, out)
+            return out
         cur = x
         n = len(self.layers)
         for i, layer in enumerate(self.layers):

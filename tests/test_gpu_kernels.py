@@ -158,6 +158,21 @@ def test_plan_follows_every_parameter_that_the_launches_read(kw):
         same()
 
 
+def test_plan_comes_back_with_the_parameter_that_was_refused():
+    from paper_2504_18547_b200.encoder import EncoderStack
+    cfg, layer = small_layer({})
+    stack = EncoderStack([si.layer_parameters(cfg, l) for l in range(2)], cfg.batch, cfg.tokens, cfg.heads, cfg.mlp_dim, cfg.bits)
+    x = dev(si.normal(351, (cfg.rows, cfg.dim)))
+    for m, part in ((layer, layer), (stack, stack.layers[1])):
+        want = m.forward(x, torch.empty_like(x))
+        good, part.s_p = part.s_p, -1.0
+        with pytest.raises(vt.VitintError):
+            m.forward(x, torch.empty_like(x))
+        assert m._plan is None
+        part.s_p = good
+        assert torch.equal(m.forward(x, torch.empty_like(x)), want) and m._plan is not None
+
+
 @pytest.mark.parametrize("kw", [{}, {"softmax": "shift"}, {"fused_attention": False, "bits": 8}, {"fused_attention": False},
                                 {"softmax": "shift", "fused_attention": False}, {"bits": 8}],
                          ids=["exp_core", "shift_core", "exp", "exp_bounded", "shift", "exp_core_any"])
