@@ -38,6 +38,8 @@ class _Recorded:
             return None
         now = self._signature()
         if now != self._plan_for:
+            if torch.cuda.is_current_stream_capturing():
+                return None                # (what making a plan fills would be filled when the captured graph runs)
             self._plan_for, self._plan = now, self._new_plan()
         return self._plan
 
@@ -129,7 +131,7 @@ class EncoderLayer(_Recorded):
                     and self.score_bound * abs(self.c) <= 80.0 and tokens <= 895):
                 self.sm_table = torch.empty(B.vitint_softmax_table_workspace_bytes(self.score_bound), dtype=torch.uint8,
                                             device=device)
-                self.sm_table_ready = False
+                self.sm_table_ready, self._sm_table_c = False, None
         self.O = B.Codes.empty(M, D, bits, True, device, container=ca)
         self.h = torch.empty((M, D), dtype=torch.float32, device=device)
         self.x2 = B.Codes.empty(M, D, bits, True, device, container=ca)
@@ -246,7 +248,7 @@ class EncoderLayer(_Recorded):
     def _tables_filled(self):
         """Making a plan fills the tables of the attention variants that build theirs on first use."""
         if not self.fused_attention and self.sm_table is not None:
-            self.sm_table_ready = True
+            self.sm_table_ready, self._sm_table_c = True, self.c
 
     def _new_plan(self):
         if not self._recordable():
@@ -299,9 +301,11 @@ class EncoderLayer(_Recorded):
             if self.softmax == "shift":
                 B.vitint_softmax_shift_quantize(S, t, self.c2, self.s_p, self.bits, out=P)
             elif self.sm_table is not None:
+                ready = self.sm_table_ready and self._sm_table_c == self.c
                 B.vitint_softmax_quantize_bounded(S, t, self.c, self.s_p, self.bits, self.score_bound, out=P,
-                                                  workspace=self.sm_table, table_ready=self.sm_table_ready)
-                self.sm_table_ready = True
+                                                  workspace=self.sm_table, table_ready=ready)
+                if not ready and not torch.cuda.is_current_stream_capturing():     # (a captured launch fills it when its graph runs)
+                    self._tables_filled()
             else:
                 B.vitint_softmax_quantize(S, t, self.c, self.s_p, self.bits, out=P)
             mark()

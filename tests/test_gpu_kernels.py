@@ -210,6 +210,35 @@ def test_layer_plan_inside_a_captured_graph():
     assert torch.equal(out, want)
 
 
+@pytest.mark.parametrize("replay_first", [True, False])
+@pytest.mark.parametrize("plan", [True, False])
+@pytest.mark.parametrize("kw", [{}, {"fused_attention": False}], ids=["core", "bounded"])
+def test_layer_changed_during_a_capture(kw, plan, replay_first):
+    """A parameter replaced inside a capture: the captured launches, and eager ones before the graph has run once or after it."""
+    (cfg, layer), (_, fresh) = small_layer(dict(kw, plan=plan)), small_layer(dict(kw, plan=False))
+    x = dev(si.normal(370, (cfg.rows, cfg.dim)))
+    if plan:
+        layer.forward(x, torch.empty_like(x))
+    fresh.bias["fc2"] = bias = layer.bias["fc2"] + 1.0
+    fresh.c = c = float(np.float32(layer.c * 0.5)) if kw else layer.c
+    want = fresh.forward(x, torch.empty_like(x))
+    out, eager, graph = torch.zeros_like(x), torch.zeros_like(x), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        layer.bias["fc2"], layer.c = bias, c
+        layer.forward(x, out)
+    if replay_first:
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, want)
+    layer.forward(x, eager)
+    assert torch.equal(eager, want) and (layer._plan is not None) == plan
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+
+
 def test_plans_made_run_and_dropped_during_a_capture():
     """Neither the capturing thread's plans nor another thread's forward() may end a capture."""
     import threading
