@@ -27,7 +27,9 @@ def _dev(a, device):
 
 
 class _Recorded:
-    """What recorded layers and stacks share: the plan, and the signature of the state it was made for."""
+    """What recorded layers and stacks share: the plan, and the signature of the state it was made for.  Copies and pickles go
+    without the plan, which names the original's memory, and make their own at the next forward().  (Class-level values serve
+    objects pickled before there were plans.)"""
     _record = False
     _plan = _plan_for = None
 
@@ -43,9 +45,13 @@ class _Recorded:
             self._plan_for, self._plan = now, self._new_plan()
         return self._plan
 
+    def __getstate__(self):
+        return {k: v for k, v in self.__dict__.items() if k not in ("_plan", "_plan_for")}
+
 
 class EncoderLayer(_Recorded):
     _any_core = False
+    _sm_table_c = None
 
     def __init__(self, batch: int, tokens: int, heads: int, mlp_dim: int, bits: int, prm: dict, device="cuda",
                  eps: float = 1e-6, widen_weights: bool = True, fused_attention: bool = True,

@@ -158,6 +158,25 @@ def test_plan_follows_every_parameter_that_the_launches_read(kw):
         same()
 
 
+@pytest.mark.parametrize("kw", [{}, {"bits": 8}, {"fused_attention": False}, {"softmax": "shift", "layernorm": "compare"}],
+                         ids=["core", "bits8", "bounded", "paper"])
+def test_layers_and_stacks_can_be_copied_and_pickled(kw):
+    import copy
+    import pickle
+    from paper_2504_18547_b200.encoder import EncoderStack
+    cfg, layer = small_layer(dict(kw))
+    kw = {k: v for k, v in kw.items() if k != "bits"}
+    stack = EncoderStack([si.layer_parameters(cfg, l) for l in range(3)], cfg.batch, cfg.tokens, cfg.heads, cfg.mlp_dim, cfg.bits, **kw)
+    x = dev(si.normal(350, (cfg.rows, cfg.dim)))
+    for m in (layer, stack):
+        want = m.forward(x, torch.empty_like(x))
+        for other in (copy.deepcopy(m), copy.copy(m), pickle.loads(pickle.dumps(m))):
+            assert torch.equal(other.forward(x, torch.empty_like(x)), want)
+            assert other._plan is not None and other._plan is not m._plan
+        del other
+        assert torch.equal(m.forward(x, torch.empty_like(x)), want)
+
+
 def test_plan_comes_back_with_the_parameter_that_was_refused():
     from paper_2504_18547_b200.encoder import EncoderStack
     cfg, layer = small_layer({})
