@@ -357,11 +357,11 @@ class EncoderStack(_Recorded):
 
     def __init__(self, layer_params: list, batch: int, tokens: int, heads: int, mlp_dim: int, bits: int,
                  device="cuda", **kw):
-        kw = dict(kw, plan=False)
+        plan, kw = kw.get("plan", True), dict(kw, plan=False)       # (recorded as a whole)
         self.layers = [EncoderLayer(batch, tokens, heads, mlp_dim, bits, prm, device, **kw) for prm in layer_params]
         rows, dim = batch * tokens, heads * 64
         self.buf = [torch.empty((rows, dim), dtype=torch.float32, device=device) for _ in range(2)]
-        self._record = bool(self.layers)
+        self._record = plan and bool(self.layers)
         self._planned()
 
     def _signature(self) -> list:

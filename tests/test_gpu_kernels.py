@@ -177,6 +177,15 @@ def test_layers_and_stacks_can_be_copied_and_pickled(kw):
         assert torch.equal(m.forward(x, torch.empty_like(x)), want)
 
 
+def test_stack_without_a_plan():
+    from paper_2504_18547_b200.encoder import EncoderStack
+    cfg = si.BlockConfig("plan", 1, 40, 64, 1, 4, mlp_dim=128)
+    stacks = [EncoderStack([si.layer_parameters(cfg, l) for l in range(2)], 1, 40, 1, 128, 4, plan=plan) for plan in (True, False)]
+    x = dev(si.normal(353, (40, 64)))
+    a, b = (s.forward(x, torch.empty_like(x)) for s in stacks)
+    assert torch.equal(a, b) and stacks[0]._plan is not None and stacks[1]._plan is None
+
+
 def test_plan_comes_back_with_the_parameter_that_was_refused():
     from paper_2504_18547_b200.encoder import EncoderStack
     cfg, layer = small_layer({})
