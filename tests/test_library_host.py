@@ -210,3 +210,21 @@ print("status", create(arr, n, buf, None, ctypes.byref(plan)), plan.value)
 """.format(root=str(ROOT), tests=str(ROOT / "tests"))
     r = subprocess.run([sys.executable, "-c", script], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and "status -6 None" in r.stdout, (r.returncode, r.stdout, r.stderr[-500:])
+
+
+def test_attention_descriptor_holds_the_fields_of_its_parts(L):
+    """The packed descriptor against the structures one by one, signedness given as numpy and Python truth values."""
+    import numpy as np
+    import torch
+    t = [torch.zeros(64 + i) for i in range(8)]
+    for yes in (True, np.bool_(True), 1):
+        codes = [L.Codes(torch.zeros((r, 32), dtype=torch.uint8), r, 64, 4, yes, c) for r, c in ((192, 0), (64, 8))]
+        epi = L.Epilogue(mode=L.EPI_REQUANT, act=1, residual=torch.zeros((3, 5)), alpha=t[5], beta=t[6], inv_out_step=t[7], out_bits=3,
+                         out_signed=yes, out_container=8)
+        a = L.AttentionWeights(2, 17, 1, 4, codes[0], t[0], t[1], 0.1, 0.2, 0.3, 0.4, 0.5, 3, t[2], None, codes[1], t[3], t[4], epi)
+        d = a.desc()
+        assert bytes(d.w_qkv) == bytes(codes[0].desc()) and bytes(d.w_proj) == bytes(codes[1].desc()) and bytes(d.proj_epi) == bytes(epi.desc())
+        assert (d.batch, d.tokens, d.heads, d.bits, d.p_bits) == (2, 17, 1, 4, 3)
+        assert [d.alpha_qkv, d.beta_qkv, d.alpha_o, d.beta_o, d.w_proj_step, d.b_proj] == [
+            t[0].data_ptr(), t[1].data_ptr(), t[2].data_ptr(), None, t[3].data_ptr(), t[4].data_ptr()]
+        assert [np.float32(v) for v in (0.1, 0.2, 0.3, 0.4, 0.5)] == [d.q_step, d.k_step, d.v_step, d.p_step, d.o_step]
