@@ -274,9 +274,11 @@ int vitint_attention_core_prepared(const vitint_codes* qkv, int32_t batch, int32
  *   vitint_softmax_shift_quantize -> vitint_pv bit for bit (every step is an integer or a single fp32 operation).
  *   The per-score pair (floor z, mantissa of 1 + r) is computed from the score; `workspace` (256-byte aligned, at least
  *   vitint_attention_core_shift_workspace_bytes(bits) bytes) is checked, not used, and table_ready has no effect.  The
- *   row maximum is subtracted (as shift counts), so unlike vitint_attention_core this variant has no limit on the size
- *   of the logits.
- *   Errors: as vitint_attention_core; UNSUPPORTED also for codes not stored one per byte (container_bits != 8). */
+ *   row maximum is subtracted (as shift counts), so the logits may be far larger than vitint_attention_core takes:
+ *   64 m^2 q_step k_step log2(e) / 8 <= 30000 with m = 2, 8, 8 for 2, 3, 4 bits (floor z is formed in the integers between
+ *   2^23 and 2^24).
+ *   Errors: as vitint_attention_core, but UNSUPPORTED beyond that limit instead of at logits of 80, and for codes not stored
+ *   one per byte (container_bits != 8). */
 size_t vitint_attention_core_shift_workspace_bytes(int32_t bits);
 int vitint_attention_core_shift(const vitint_codes* qkv, int32_t batch, int32_t heads, int32_t tokens, float q_step,
                                 float k_step, float p_step, int32_t p_bits, const float* alpha_o, const float* beta_o,

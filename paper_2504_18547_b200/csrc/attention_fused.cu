@@ -1,9 +1,9 @@
 // a4 + a5 + a6 fused: per (image, head, 128-query tile)  S = Q K^T  ->  softmax + quantize  ->
 // O = P V  ->  requantize, with S, the probabilities and P never leaving the SM.
 //
-// A persistent CTA runs TWO independent pipelines ("groups"), each with four compute warps
-// (thread = query row = TMEM lane) and one control warp (TMA + MMA issue); while one group's
-// threads are busy with the softmax the other group's loads and MMAs proceed.
+// A persistent CTA runs TWO independent pipelines ("groups"), each with eight compute warps
+// (query row = TMEM lane, shared by two threads) and one control warp (TMA + MMA issue); while one
+// group's threads are busy with the softmax the other group's loads and MMAs proceed.
 //
 // Per item and group:
 //   control   TMA: packed Q [128 x 64], K [T x 64], V [T x 64] code slabs -> shared memory
@@ -280,7 +280,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const uint32_t ring_mask = 8u * (uint32_t)P.smax - 4u;
         float* const colp2 = reinterpret_cast<float*>(ggen + P.off_col);  // alpha[64], beta[64] of the head, one copy per item parity
         const int sh_idx = DIRECT ? 0 : 2 * (8 - C) - 2;            // scaled score -> byte offset 4*S
-        const int chunks = P.kv_rows / 32, full_chunks = T >> 5, tail = T & 31, tail_blocks = (tail + 7) >> 3;
+        const int full_chunks = T >> 5, tail = T & 31, tail_blocks = (tail + 7) >> 3;
         const int tail0 = (hf ^ full_chunks) & 1;                   // the thread with fewer whole chunks takes the first block of the tail
         const uint32_t qp2 = (uint32_t)P.p_qp * 0x00010001u;
         const bool steep = P.p_step < 1.0f / 65000.0f;              // codes before the clamp might not fit 16 bits
@@ -734,7 +734,7 @@ using namespace vitint;
 extern "C" size_t vitint_attention_core_shift_workspace_bytes(int32_t bits) {
     if (bits != 2 && bits != 3 && bits != 4) return 0;
     const int m = 1 << (container_bits(bits) - 1);
-    return (size_t)(2 * 64 * m * m + 2) * 6 + 256;                   // 32-bit mantissas + 16-bit integer parts
+    return (size_t)(2 * 64 * m * m + 2) * 6 + 256;                   // six bytes a score: what the contract has asked for since the kernel kept tables
 }
 
 extern "C" size_t vitint_attention_core_workspace_bytes(int32_t bits) {

@@ -404,7 +404,7 @@ class NormedAttention:
     fused=True (default): one QKV GEMM whose epilogue normalises and quantizes the Q and K heads and requantizes V,
     then the fused attention core with the Eq. 4 softmax inside (2 launches; `fused_core=False` keeps Q K^T, softmax
     and P V as three kernels with S and P in memory: 4 launches); fused=False: separate Q, K, V linears with fp32 Q
-    and K rows and a LayerNorm kernel pass each (10 launches, the fp32 rows and their statistics left in `f32` /
+    and K rows and a LayerNorm kernel each (8 launches, the fp32 rows and their statistics left in `f32` /
     `stats` for inspection)."""
 
     def __init__(self, batch: int, tokens: int, heads: int, bits: int, prm: dict, qkn: dict, device="cuda",

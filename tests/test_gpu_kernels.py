@@ -335,6 +335,45 @@ def test_stack_plan_from_two_threads():
             assert torch.equal(a, b)
 
 
+def test_one_plan_from_two_threads():
+    """Two threads run ONE plan with their own x and out on one stream: rewriting the nodes and launching are one step."""
+    import threading
+    cfg, layer = small_layer({})
+    xs = [dev(si.normal(360 + i, (cfg.rows, cfg.dim))) for i in range(8)]
+    want = [one_by_one(layer, x) for x in xs]
+    stream, errors, got, start = torch.cuda.Stream(), [], [[], []], threading.Barrier(2)
+    outs = [[torch.empty_like(xs[0]) for _ in range(200)] for _ in range(2)]
+    torch.cuda.synchronize()
+
+    def work(k):
+        try:
+            with torch.cuda.stream(stream):
+                start.wait()
+                for i, out in enumerate(outs[k]):
+                    got[k].append((layer.forward(xs[(i + 3 * k) % 8], out), (i + 3 * k) % 8))
+        except Exception as e:                               # noqa: BLE001 -- reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    torch.cuda.synchronize()
+    assert not errors and layer._plan is not None
+    assert all(torch.equal(out, want[i]) for k in range(2) for out, i in got[k])
+
+
+@pytest.mark.parametrize("bits", [2, 4])
+def test_shift_core_limit_of_the_logits(bits):
+    """64 m^2 c log2(e) <= 30000: taken right below, refused right above."""
+    heads, tokens, D, m = 1, 9, 64, 2 if bits == 2 else 8
+    codes, alpha = byte_codes(rand_codes(541, (tokens, 3 * D), bits, True), bits, True), torch.ones(D, device="cuda")
+    step = (30000.0 / (64 * m * m * np.log2(np.e)) * 8) ** 0.5
+    vt.vitint_attention_core_shift(codes, 1, heads, tokens, 0.999 * step, step, 0.05, bits, alpha, None)
+    with pytest.raises(vt.VitintError) as e:
+        vt.vitint_attention_core_shift(codes, 1, heads, tokens, 1.001 * step, step, 0.05, bits, alpha, None)
+    assert e.value.code == -2
+
+
 # ---- bit-packed operands: both packed alike (the reordered unpacking), packed unlike, one of them byte-stored; K at the
 # ---- edges of a 32-code MMA step, a 64-code chunk and a 128-code block
 @pytest.mark.parametrize("M,K,N", [(1, 16, 64), (33, 33, 64), (129, 96, 128), (130, 200, 192), (197, 1000, 320), (2000, 160, 1152)])
