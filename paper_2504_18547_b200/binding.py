@@ -563,17 +563,18 @@ class AttentionWeights:
     proj_epi: Epilogue
 
     def desc(self) -> _AttentionDesc:
-        # one packing call instead of a constructor per nested structure (6.3 -> 3.5 us of the host per block)
+        # one packing call instead of a constructor per nested structure (6.3 -> 3.5 us of the host per block); "+ 0" makes an
+        # integer of any truth type
         q, o, e = self.w_qkv, self.w_proj, self.proj_epi
         d = _AttentionDesc.from_buffer_copy(_PACK_ATTENTION(
             self.batch, self.tokens, self.heads, self.bits,
-            q.data.data_ptr(), q.rows, q.cols, q.pitch, q.bits, int(q.signed), q.container, 0,
+            q.data.data_ptr(), q.rows, q.cols, q.pitch, q.bits, q.signed + 0, q.container, 0,
             _ptr(self.alpha_qkv) or 0, _ptr(self.beta_qkv) or 0, 0.0, 0.0, 0.0, 0.0, 0.0,
             self.p_bits, _ptr(self.alpha_o) or 0, _ptr(self.beta_o) or 0,
-            o.data.data_ptr(), o.rows, o.cols, o.pitch, o.bits, int(o.signed), o.container, 0,
+            o.data.data_ptr(), o.rows, o.cols, o.pitch, o.bits, o.signed + 0, o.container, 0,
             _ptr(self.w_proj_step) or 0, _ptr(self.b_proj) or 0,
             e.mode, e.act, _ptr(e.residual) or 0, 0 if e.residual is None else _ld(e.residual), _ptr(e.alpha) or 0,
-            _ptr(e.beta) or 0, _ptr(e.inv_out_step) or 0, e.out_bits, int(e.out_signed), e.out_container, 0))
+            _ptr(e.beta) or 0, _ptr(e.inv_out_step) or 0, e.out_bits, e.out_signed + 0, e.out_container, 0))
         d.q_step, d.k_step, d.v_step, d.p_step, d.o_step = self.q_step, self.k_step, self.v_step, self.p_step, self.o_step
         return d
 
