@@ -16,9 +16,9 @@
 //   control   tcgen05.mma  O[128, 64] = P V  (V is the N-contiguous B operand) into TMEM
 //   compute   requantize O, pack, store the head's 64 columns of the [M, D] code matrix
 //
-// What bounds it: the lookups.  Random entries of a 32 KB table take 2.8 passes of the shared-memory pipe per 32 scores, and
-// with the code stores, the operand copies and the tensor core's own reads that pipe is busy 57 % of the time; instructions
-// issue in half the slots.  197 tokens x 12 heads, batch 128: 75.5 -> 65.9 us by walking the last columns in blocks of eight
+// What bounds it: the lookups.  Random entries of a 32 KB table take 2.8 passes of the shared-memory pipe per 32 scores: the
+// load/store data pipe is 42 % busy with them and the code stores, the tensor core's own reads not counted, and instructions
+// issue in 56 % of the slots.  197 tokens x 12 heads, batch 128: 75.5 -> 65.9 us by walking the last columns in blocks of eight
 // (200 instead of 224) and 20 % fewer instructions a score; 256 tokens, where nothing is padded, 45.9 -> 45.3.  Overlapping the
 // steps of neighbouring items (scores formed while O is pending, O requantized between two chunks) cost more in instructions
 // than it hid: 74.8.
@@ -899,7 +899,7 @@ extern "C" int vitint_attention_core(const vitint_codes* qkv, int32_t batch, int
 
 namespace vitint {
 // The fused core for logits of any range (no table, no workspace), byte-stored codes up to 8 bits and 256 tokens; the codes of
-// P are those of vitint_softmax_quantize.  197 tokens x 12 heads of 8-bit codes, batch 32: 39 us, against 87 us as
+// P are those of vitint_softmax_quantize.  197 tokens x 12 heads of 8-bit codes, batch 32: 34 us, against 87 us as
 // Q K^T, softmax and P V with S and P in memory.
 int attention_core_general(const vitint_codes* qkv, int batch, int heads, int tokens, float q_step, float k_step, float p_step,
                            int p_bits, const float* alpha_o, const float* beta_o, const vitint_codes* o_out, void* stream) {

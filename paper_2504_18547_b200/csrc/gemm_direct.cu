@@ -15,8 +15,8 @@
 // Measured against gemm_i8_kernel on the same operands (us, 4-bit codes, M = 25,216): 768 -> 2304 requantized 48.3 -> 40.1,
 // 768 -> 3072 GELU 79.8 -> 72.1, 3072 -> 768 fp32 60.1 -> 55.5; at M = 197, where the tile width matters, 6.6 -> 4.5, 7.7 ->
 // 4.9 and 15.0 -> 9.3, and 768 -> 768 fp32 9.9 -> 4.3.  What bounds it: the mainloop alone (no epilogue) takes 27.5, 35.9 and
-// 36.2 us at M = 25,216, the epilogue alone 28, 63 (GELU: the fp32 pipe, 58 % busy) and 38 us (its 155 MB); the two share the
-// SM's issue slots and data pipe.
+// 36.2 us at M = 25,216, the epilogue alone 28, 63 (GELU: in the whole kernel the fp32 pipe is 53 % busy, the issue slots 57 %) and
+// 38 us (its 155 MB); the two share the SM's issue slots and data pipe.
 //
 // The TMA and MMA warps run their loops as whole warps and elect a thread around each issue (see elect_one): 197 x 3072 -> 768 fp32
 // 9.3 -> 6.6 us, 197 x 768 -> 768 4.4 -> 3.7, 197 x 768 -> 2304 4.6 -> 3.8, against one lane that runs the loop alone (a K block
@@ -755,8 +755,10 @@ bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_maj
     if (P.kind == EK_REQUANT || (P.kind == EK_REQUANT_GELU && P.unit_out)) return P.N % 64 == 0;
     if (P.kind != EK_DEQUANT || P.N % 32 != 0) return false;
     // A short contraction whose residual and output exceed L2 is bound by HBM, and gemm_i8_kernel's asynchronous copies of the
-    // residual through shared memory keep more of it in flight (K = 768, N = 768: 27.8 against 30.1 us at M = 18,912, 35.7
-    // against 39.2 at 25,216; below, 24.1 against 19.2 at 12,608).
+    // residual through shared memory keep more of it in flight.  This kernel against that one, rotating buffers, residual and
+    // output together: 50 MB 15.9 / 19.4, 15.6 / 16.6 and 15.4 / 20.5 us (K = N = 768, 384, 1024), 95 MB 27.1 / 27.1, 26.5 / 29.5 and
+    // 26.7 / 29.0, 140 MB 37.2 / 34.5, 36.9 / 36.4 and 37.8 / 37.3, 400 MB 100 / 85, 100 / 95 and 100 / 93 (K = N = 192, two K
+    // blocks: 15.6 / 15.6, 29.4 / 27.5, 37.6 / 32.5, 98 / 81).
     if (P.a_direct && P.b_direct && P.residual && P.K <= 1024 && (long long)P.M * P.N * 8 > 100ll * 1000 * 1000) return false;
     auto rows32 = [](const void* p, long long ld) { return (reinterpret_cast<uintptr_t>(p) & 31u) == 0 && ld % 8 == 0; };
     return rows32(P.out, P.ld_out) && (!P.residual || rows32(P.residual, P.ld_res));

@@ -281,8 +281,10 @@ extern "C" int vitint_quantize(const float* x, int64_t rows, int64_t cols, int64
     int64_t gy = (rows + by - 1) / by;
     if (gy > 16384) gy = 16384;
     // Byte codes: about the threads the chip holds, each walking rows (a thread's four values are less work than its divisor).
-    // 4-bit packed codes walk from more than eight rows a thread on (25,344 x 768 17.8 -> 14.2 us); below, in front of a linear and
-    // from a cold L2, one row a thread is the better form (12,608 x 768 with the linear behind it 60.4 us, walking 61.0).
+    // 4-bit packed codes walk from more than eight rows a thread on, 58 MB of input (25,344 x 768 17.8 -> 14.2 us).  Rotating buffers,
+    // one row a thread / walking: 20 MB 6.6 / 6.7, 6.0 / 6.4 and 6.1 / 6.6 us (192, 768, 1536 columns), 40 MB 11.3 / 10.4, 10.0 / 9.8
+    // and 10.3 / 10.0 (with the linear behind it 12,608 x 768 takes 60.4 and 61.0), 80 MB 21.0 / 18.4, 18.1 / 17.3 and 18.7 / 17.4.
+    // 2-bit codes stay with one row a thread: 40 MB 9.1 / 10.1 and 8.5 / 9.9 us (768, 1536 columns), 160 MB 30.1 / 30.8 and 27.2 / 30.7.
     const int64_t all_rows = (rows + by - 1) / by, resident = (8 * sm_count() + gx - 1) / gx;
     const bool walks = !row_steps && (c == 8 ? all_rows > resident : c == 4 && all_rows > 8 * resident);
     if (walks) gy = resident;
