@@ -643,6 +643,35 @@ def test_shift_core_equals_three_kernels(tokens, bits, p_bits):
             assert np.array_equal(got, want), (scale, p_step)
 
 
+@pytest.mark.parametrize("tokens", [1, 9, 40, 197])
+@pytest.mark.parametrize("p_step", [1e-6, 2.0 ** -16, 1.0 / 64999.0, "tie"])
+def test_cores_with_codes_on_or_far_beyond_the_last_level(tokens, p_step):
+    """Codes proven by an interval around the reciprocal, against the three kernels: steps whose unclamped codes need more than 16
+    bits (nothing is proven, every code by comparisons or division) and a step that puts equal probabilities on a tie."""
+    step_p = np.float32(2.0 / tokens if p_step == "tie" else p_step)
+    batch, heads, D, bits = 1, 2, 128, 4
+    qkv = rand_codes(950 + tokens, (batch * tokens, 3 * D), bits, True)
+    qkv[::2, :D] = 0                                      # equal scores
+    packed = to_codes(qkv, bits, True)
+    slabs = [vt.Slabs.of_qkv(packed, tokens, D, i) for i in range(3)]
+    alpha, step = dev(np.full(D, np.float32(0.02))), np.float32(0.3)
+    c2 = np.float32(np.float64(vp.softmax_scale(step, step, 64)) * np.log2(np.e))
+    S = vt.vitint_qk(slabs[0], slabs[1], batch, heads, tokens)
+    P = vt.vitint_softmax_shift_quantize(S.view(batch * heads * tokens, -1), tokens, c2, step_p, bits)
+    want = from_codes(vt.vitint_pv(P, slabs[2], batch, heads, tokens, 1.0, 1.0,
+                                   vt.Epilogue(mode=vt.EPI_REQUANT, alpha=alpha, out_bits=8, out_signed=True)))
+    got = vt.vitint_attention_core_shift(vt.vitint_widen(packed), batch, heads, tokens, step, step, step_p, bits, alpha, None,
+                                         out=vt.Codes.empty(batch * tokens, D, 8, True))
+    assert np.array_equal(from_codes(got), want)
+    from paper_2504_18547_b200.encoder import EncoderLayer
+    cfg = si.BlockConfig("steep", 2, tokens, 128, 2, 8, mlp_dim=320)
+    layer = EncoderLayer(cfg.batch, tokens, 2, 320, 8, dict(si.layer_parameters(cfg), s_p=step_p))
+    x = dev(si.normal(951, (cfg.rows, cfg.dim)))
+    out = torch.empty_like(x)
+    layer.forward(x, out)
+    assert torch.equal(out, one_by_one(layer, x))
+
+
 @pytest.mark.parametrize("tokens,bits", [(1, 4), (15, 2), (16, 4), (24, 4), (32, 2), (40, 3), (197, 4), (256, 3)])
 def test_attention_block_qkv_form(tokens, bits):
     """QKV stored one code per byte where its room is that of the unfused sequence, packed otherwise or when a copy is asked for:
