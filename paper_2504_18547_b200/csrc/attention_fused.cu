@@ -3,7 +3,8 @@
 //
 // A persistent CTA runs TWO independent pipelines ("groups"), each with eight compute warps
 // (query row = TMEM lane, shared by two threads) and one control warp (TMA + MMA issue); while one
-// group's threads are busy with the softmax the other group's loads and MMAs proceed.
+// group's threads are busy with the softmax the other group's loads and MMAs proceed.  Where no CTA gets a second
+// item there is one group of sixteen warps, four threads a row.
 //
 // Per item and group:
 //   control   TMA: packed Q [128 x 64], K [T x 64], V [T x 64] code slabs -> shared memory
@@ -37,9 +38,9 @@
 namespace vitint {
 namespace {
 
-constexpr int AT_GROUPS = 2;
-constexpr int AT_COMPUTE_WARPS = 8;   // two warps per TMEM lane quarter: a query row is shared by two threads
-constexpr int AT_THREADS = (AT_GROUPS * AT_COMPUTE_WARPS + AT_GROUPS) * 32;   // 576
+constexpr int AT_COMPUTE_WARPS = 16;
+// Two groups of eight compute warps, or one of sixteen: a query row is shared by 2 or 4 threads, 4 GROUPS warps a TMEM lane quarter.
+__host__ __device__ constexpr int at_threads(int groups) { return (AT_COMPUTE_WARPS + groups) * 32; }
 
 struct AttnParams {
     int batch, heads, tokens, q_tiles, total_items;
@@ -81,14 +82,17 @@ enum AttnMode { AM_TABLE = 0, AM_SHIFT = 1, AM_GENERAL = 2 };
 // single fp32 operation, hence the same codes bit for bit.  Two tables of the scores (floor z; the mantissa of 1 + r), 64-bit
 // shifts and two comparisons a score took 79 us for 197 tokens x 12 heads at batch 64; computed in pairs, summed in
 // doubles and compared only near a tie, 50 us (198 tokens x 6 heads: 42 -> 27).
-template <int C, int MODE>
-__global__ void __launch_bounds__(AT_THREADS, 1)
+//
+// GROUPS: two pipelines in a CTA, or one with all the warps where no CTA gets a second item.
+template <int C, int MODE, int GROUPS>
+__global__ void __launch_bounds__(at_threads(GROUPS), 1)
 attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_kv,
                        const __grid_constant__ AttnParams P) {
     static_assert(MODE == AM_TABLE || C == 8, "only the table variant takes packed codes");
     constexpr bool SHIFT = MODE == AM_SHIFT, GENERAL = MODE == AM_GENERAL;
+    constexpr int WARPS = AT_COMPUTE_WARPS / GROUPS, H = WARPS / 4;           // compute warps of a group, threads of a row
     extern __shared__ uint8_t smem_raw[];
-    __shared__ AttnBars bars[AT_GROUPS];
+    __shared__ AttnBars bars[GROUPS];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -96,42 +100,35 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t* const smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     volatile int* abort_ptr = &abort_flag;
-    const bool is_control = warp >= AT_GROUPS * AT_COMPUTE_WARPS;
-    const int g = is_control ? warp - AT_GROUPS * AT_COMPUTE_WARPS : warp / AT_COMPUTE_WARPS;
+    const bool is_control = warp >= AT_COMPUTE_WARPS;
+    const int g = is_control ? warp - AT_COMPUTE_WARPS : warp / WARPS;
     AttnBars& B = bars[g];
     const uint32_t gbase = smem_base + P.off_group + (uint32_t)g * P.group_bytes;
     uint8_t* const ggen = smem_gen + P.off_group + (size_t)g * P.group_bytes;
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int k = 0; k < AT_GROUPS; ++k) {
+        for (int k = 0; k < GROUPS; ++k) {
             ptx::mbar_init(ptx::smem_addr(&bars[k].packed_full), 1);
             ptx::mbar_init(ptx::smem_addr(&bars[k].v_full), 1);
-            ptx::mbar_init(ptx::smem_addr(&bars[k].ops_ready), AT_COMPUTE_WARPS);
+            ptx::mbar_init(ptx::smem_addr(&bars[k].ops_ready), WARPS);
             ptx::mbar_init(ptx::smem_addr(&bars[k].s_full), 1);
-            ptx::mbar_init(ptx::smem_addr(&bars[k].p_ready), AT_COMPUTE_WARPS);
+            ptx::mbar_init(ptx::smem_addr(&bars[k].p_ready), WARPS);
             ptx::mbar_init(ptx::smem_addr(&bars[k].o_full), 1);
-            ptx::mbar_init(ptx::smem_addr(&bars[k].o_done), AT_COMPUTE_WARPS);
-            ptx::mbar_init(ptx::smem_addr(&bars[k].grp_sync), AT_COMPUTE_WARPS * 32);
-            ptx::mbar_init(ptx::smem_addr(&bars[k].z_sync), AT_COMPUTE_WARPS);
+            ptx::mbar_init(ptx::smem_addr(&bars[k].o_done), WARPS);
+            ptx::mbar_init(ptx::smem_addr(&bars[k].grp_sync), WARPS * 32);
+            ptx::mbar_init(ptx::smem_addr(&bars[k].z_sync), WARPS);
         }
         ptx::fence_mbar_init();
         ptx::fence_proxy_async_smem();
     }
-    if (warp == AT_GROUPS * AT_COMPUTE_WARPS) {          // first control warp owns the TMEM allocation
-        ptx::tmem_alloc(ptx::smem_addr(&tmem_base_slot), 512);
+    if (warp == AT_COMPUTE_WARPS) {                      // first control warp owns the TMEM allocation
+        ptx::tmem_alloc(ptx::smem_addr(&tmem_base_slot), GROUPS * 256);
         ptx::tmem_relinquish();
-    }
-    grid_dependency_wait();        // the table and the codes come from earlier kernels of the stream
-    grid_dependency_launch();
-    // the exp table: global -> shared, once per CTA
-    {
-        float* tab = reinterpret_cast<float*>(smem_gen + P.off_table);
-        if constexpr (MODE == AM_TABLE) fill_table_ring(tab, P.table, P.smax, threadIdx.x, AT_THREADS);
     }
     {
         // P columns behind the last block of eight that holds a token are never written: zero for good
-        for (int i = threadIdx.x; i < AT_GROUPS * 128 * 16; i += AT_THREADS) {
+        for (int i = threadIdx.x; i < GROUPS * 128 * 16; i += at_threads(GROUPS)) {
             const int gr = i / 2048, cc = (i >> 7) & 15, r = i & 127;
             if (cc * 16 < P.kv_rows)
                 *reinterpret_cast<uint4*>(smem_gen + P.off_group + (size_t)gr * P.group_bytes + P.off_p + (cc >> 3) * 16384 + r * 128 + (((cc & 7) ^ (r & 7)) << 4)) = make_uint4(0u, 0u, 0u, 0u);
@@ -142,17 +139,26 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
+    grid_dependency_wait();        // the table and the codes come from earlier kernels of the stream
+    grid_dependency_launch();
+    // the exp table: global -> shared, once per CTA, while the control warps' first copies and Q K^T are on their way
+    if constexpr (MODE == AM_TABLE) {
+        if (!is_control) {
+            fill_table_ring(reinterpret_cast<float*>(smem_gen + P.off_table), P.table, P.smax, threadIdx.x, AT_COMPUTE_WARPS * 32);
+            asm volatile("bar.sync 1, %0;" ::"n"(AT_COMPUTE_WARPS * 32) : "memory");
+        }
+    }
     const uint32_t tmem_grp = __shfl_sync(0xffffffffu, tmem_base_slot, 0) + (uint32_t)g * 256u;
 
     const int T = P.tokens;
     // Whole waves give every group an item; a remainder of at most one item a CTA goes to one group of as many CTAs as it takes
     // (197 tokens x 12 heads, batch 128: 21 items in the busiest CTA instead of 22, 68.1 -> 65.0 us; batch 1: 24 CTAs instead of
     // 12, 9.2 -> 7.7 us)
-    const int wave = gridDim.x * AT_GROUPS, full = P.total_items / wave;
+    const int wave = gridDim.x * GROUPS, full = P.total_items / wave;
     const int last = full * wave + (P.total_items - full * wave <= (int)gridDim.x ? g * (int)gridDim.x + (int)blockIdx.x
-                                                                                  : (int)blockIdx.x * AT_GROUPS + g);
+                                                                                  : (int)blockIdx.x * GROUPS + g);
     auto item_at = [&](int n) {                              // the group's n-th item; total_items when there is none
-        return n < full ? n * wave + (int)blockIdx.x * AT_GROUPS + g : n == full ? min(last, P.total_items) : P.total_items;
+        return n < full ? n * wave + (int)blockIdx.x * GROUPS + g : n == full ? min(last, P.total_items) : P.total_items;
     };
     constexpr bool DIRECT = (C == 8);                  // byte codes: no packed staging, no unpack
     const int head_bytes = 8 * C;                      // 64 codes
@@ -271,17 +277,17 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     } else {
         // ------------------------------ compute warps ------------------------------------
         const int wq = warp & 3;                                    // TMEM lane quarter
-        const int hf = (warp % AT_COMPUTE_WARPS) >> 2;              // which of the row's two threads: even / odd 32-column chunks
-        const int tid_g = (warp % AT_COMPUTE_WARPS) * 32 + lane;    // 0..255 within the group
+        const int hf = (warp % WARPS) >> 2;                         // which of the row's H threads: every H-th chunk of 32 columns
+        const int tid_g = (warp % WARPS) * 32 + lane;               // within the group
         const int row = wq * 32 + lane;                             // query row of the tile
-        double* const zx = reinterpret_cast<double*>(ggen + P.off_z);   // partial row sums, [2][128]
+        double* const zx = reinterpret_cast<double*>(ggen + P.off_z);   // partial row sums, [H][128]
         const uint32_t t_row = tmem_grp + ((uint32_t)(wq * 32) << 16);
         const char* const ring = reinterpret_cast<const char*>(smem_gen + P.off_table);
         const uint32_t ring_mask = 8u * (uint32_t)P.smax - 4u;
         float* const colp2 = reinterpret_cast<float*>(ggen + P.off_col);  // alpha[64], beta[64] of the head, one copy per item parity
         const int sh_idx = DIRECT ? 0 : 2 * (8 - C) - 2;            // scaled score -> byte offset 4*S
         const int full_chunks = T >> 5, tail = T & 31, tail_blocks = (tail + 7) >> 3;
-        const int tail0 = (hf ^ full_chunks) & 1;                   // the thread with fewer whole chunks takes the first block of the tail
+        const int tail0 = (hf - full_chunks) & (H - 1);             // the threads with fewer whole chunks take the first blocks of the tail
         const uint32_t qp2 = (uint32_t)P.p_qp * 0x00010001u;
         const bool steep = P.p_step < 1.0f / 65000.0f;              // codes before the clamp might not fit 16 bits
         const double inv_p_step = 1.0 / (double)P.p_step;
@@ -301,9 +307,9 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 // ---- operands: packed -> int8 ---------------------------------------------
                 w = mbar_wait(ptx::smem_addr(&B.packed_full), ph, abort_ptr);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-                unpack_rows64<C, 1>(ggen + P.off_pq, ggen + P.off_q, 128, tid_g, AT_COMPUTE_WARPS * 32);
-                unpack_rows64<C, 1>(ggen + P.off_pk, ggen + P.off_k, P.n_k, tid_g, AT_COMPUTE_WARPS * 32);
-                unpack_rows64<C, 1>(ggen + P.off_pv, ggen + P.off_v, P.kv_rows, tid_g, AT_COMPUTE_WARPS * 32);
+                unpack_rows64<C, 1>(ggen + P.off_pq, ggen + P.off_q, 128, tid_g, WARPS * 32);
+                unpack_rows64<C, 1>(ggen + P.off_pk, ggen + P.off_k, P.n_k, tid_g, WARPS * 32);
+                unpack_rows64<C, 1>(ggen + P.off_pv, ggen + P.off_v, P.kv_rows, tid_g, WARPS * 32);
                 ptx::fence_proxy_async_smem();
                 ptx::mbar_arrive(ptx::smem_addr(&B.grp_sync));
                 w = mbar_wait(ptx::smem_addr(&B.grp_sync), ph, abort_ptr);
@@ -324,7 +330,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 int smx = INT_MIN, smn = INT_MAX;
                 if (warp_live) {
 #pragma unroll 1
-                    for (int ch = hf; ch < full_chunks; ch += 2) {
+                    for (int ch = hf; ch < full_chunks; ch += H) {
                         uint32_t v[32];
                         ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
                         ptx::tmem_ld_wait();
@@ -335,7 +341,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                         }
                     }
 #pragma unroll 1
-                    for (int k = tail0; k < tail_blocks; k += 2) {
+                    for (int k = tail0; k < tail_blocks; k += H) {
                         uint32_t v[8];
                         ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
                         ptx::tmem_ld_wait();
@@ -352,6 +358,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 0u, abort_ptr);       // two phases per item: parities 0, 1
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 smx = max(mx[row], mx[128 + row]);
+                if constexpr (H == 4) smx = max(smx, max(mx[256 + row], mx[384 + row]));
                 const f32x2 c2 = f2_dup(P.scale), nmagic2 = f2_dup(-12582912.0f), magic2 = f2_dup(12582912.0f);
                 uint8_t* const prow = ggen + P.off_p + row * 128;
                 const int sw = row & 7;
@@ -388,7 +395,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                             zp[1] += __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
                         };
 #pragma unroll 1
-                        for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {     // halves of the thread's chunks
+                        for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 2 * H - 1 : 1) {     // halves of the thread's chunks
                             uint32_t v[16];
                             ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
                             ptx::tmem_ld_wait();
@@ -397,7 +404,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                             ptx::tmem_st16(t_row + (uint32_t)(pc * 16), v);
                         }
 #pragma unroll 1
-                        for (int k = tail0; k < tail_blocks; k += 2) {
+                        for (int k = tail0; k < tail_blocks; k += H) {
                             uint32_t v[8];
                             ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
                             ptx::tmem_ld_wait();
@@ -411,7 +418,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                         // shifted out anyway); what is left of a mantissa shifted right converts by the 2^23 trick
 #pragma unroll 1
                         for (int blk = 0; blk < 4 * full_chunks + tail_blocks; ++blk) {           // blocks of eight columns
-                            if (blk < 4 * full_chunks ? ((blk >> 2) & 1) != hf : ((blk - 4 * full_chunks) & 1) != tail0) continue;
+                            if (blk < 4 * full_chunks ? ((blk >> 2) & (H - 1)) != hf : ((blk - 4 * full_chunks) & (H - 1)) != tail0) continue;
                             uint32_t v[8];
                             ptx::tmem_ld8(t_row + (uint32_t)(blk * 8), v);
                             ptx::tmem_ld_wait();
@@ -446,6 +453,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 1u, abort_ptr);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
                 sigma = sx[row] + sx[128 + row];
+                if constexpr (H == 4) sigma += sx[256 + row] + sx[384 + row];
                 const float sig_f = __ull2float_rn(sigma);
                 // pass 2: the code is the number of references fl32(fl32((k - 1/2) s_P) * Sigma) that float(E_j) exceeds.
                 // k0 = rint(u), u = min(E_j / (s_P Sigma), Qp), is that number unless u lies within (Qp + 1) 2^-21 of some k - 1/2:
@@ -490,7 +498,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 };
                 if (warp_live) {
 #pragma unroll 1
-                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {
+                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 2 * H - 1 : 1) {
                         uint32_t v[16], wd[4];
                         ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
                         ptx::tmem_ld_wait();
@@ -498,7 +506,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                         *reinterpret_cast<uint4*>(prow + (pc >> 3) * 16384 + (((pc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
                     }
 #pragma unroll 1
-                    for (int k = tail0; k < tail_blocks; k += 2) {
+                    for (int k = tail0; k < tail_blocks; k += H) {
                         uint32_t v[8], wd[2];
                         const int col = full_chunks * 32 + k * 8, cc = col >> 4;
                         ptx::tmem_ld8(t_row + (uint32_t)col, v);
@@ -524,7 +532,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 };
                 if (warp_live) {
 #pragma unroll 1
-                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {     // halves of the thread's chunks
+                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 2 * H - 1 : 1) {     // halves of the thread's chunks
                         uint32_t v[16];
                         ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
                         ptx::tmem_ld_wait();
@@ -533,7 +541,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                         ptx::tmem_st16(t_row + (uint32_t)(pc * 16), v);
                     }
 #pragma unroll 1
-                    for (int k = tail0; k < tail_blocks; k += 2) {
+                    for (int k = tail0; k < tail_blocks; k += H) {
                         uint32_t v[8];
                         ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
                         ptx::tmem_ld_wait();
@@ -548,7 +556,8 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 1u, abort_ptr);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-                const double z = zx[row] + zx[128 + row];
+                double z = zx[row] + zx[128 + row];
+                if constexpr (H == 4) z += zx[256 + row] + zx[384 + row];
                 const double r0 = (double)__frcp_rn((float)z), rz = r0 * (2.0 - z * r0);
                 const float rzh = (float)rz, rzl = (float)(rz - (double)(float)rz);
                 const f32x2 rzh2 = f2_dup(rzh), rzl2 = f2_dup(rzl), dr2 = f2_dup(p_div.r), ndb2 = f2_dup(-p_div.b);
@@ -585,7 +594,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 };
                 if (warp_live) {
 #pragma unroll 1
-                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {
+                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 2 * H - 1 : 1) {
                         uint32_t v[16], wd[4];
                         ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
                         ptx::tmem_ld_wait();
@@ -593,7 +602,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                         *reinterpret_cast<uint4*>(prow + (pc >> 3) * 16384 + (((pc & 7) ^ sw) << 4)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
                     }
 #pragma unroll 1
-                    for (int k = tail0; k < tail_blocks; k += 2) {
+                    for (int k = tail0; k < tail_blocks; k += H) {
                         uint32_t v[8], wd[2];
                         const int col = full_chunks * 32 + k * 8, cc = col >> 4;
                         ptx::tmem_ld8(t_row + (uint32_t)col, v);
@@ -612,19 +621,19 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 uint32_t v0[16], v1[16];
                 if (hf < full_chunks) ptx::tmem_ld16(t_row + (uint32_t)(hf * 32), v0);
 #pragma unroll 1
-                for (int ch = hf; ch < full_chunks; ch += 2) {
+                for (int ch = hf; ch < full_chunks; ch += H) {
                     const uint32_t t_ch = t_row + (uint32_t)(ch * 32);
                     ptx::tmem_ld_wait();
                     ptx::tmem_ld16(t_ch + 16, v1);
                     exp_lookup<16, !DIRECT, false>(v0, ring, ring_mask, sh_idx, 16, zp);
                     ptx::tmem_st16(t_ch, v0);
                     ptx::tmem_ld_wait();
-                    if (ch + 2 < full_chunks) ptx::tmem_ld16(t_ch + 64, v0);
+                    if (ch + H < full_chunks) ptx::tmem_ld16(t_ch + 32 * H, v0);
                     exp_lookup<16, !DIRECT, false>(v1, ring, ring_mask, sh_idx, 16, zp);
                     ptx::tmem_st16(t_ch + 16, v1);
                 }
 #pragma unroll 1
-                for (int k = tail0; k < tail_blocks; k += 2) {
+                for (int k = tail0; k < tail_blocks; k += H) {
                     uint32_t v[8];
                     ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
                     ptx::tmem_ld_wait();
@@ -641,6 +650,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             w = mbar_wait(ptx::smem_addr(&B.z_sync), ph, abort_ptr);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             z = zx[row] + zx[128 + row];
+            if constexpr (H == 4) z += zx[256 + row] + zx[384 + row];
             // r = 1 / (Z * s_P) as a two-float number: e * r then carries the quantizer argument p / s_P to
             // about half an ulp, i.e. it is the exact-division result for a probability that differs from
             // RN(e / Z) by less than one ulp
@@ -654,7 +664,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (warp_live) {
                 const float e_top = steep ? 60000.0f / rzh : 0.0f;         // far above Qp, below 2^16
 #pragma unroll 1
-                for (int ch = hf; ch < full_chunks; ch += 2) {
+                for (int ch = hf; ch < full_chunks; ch += H) {
                     uint32_t v[32], wd[8];
                     ptx::tmem_ld32(t_row + (uint32_t)(ch * 32), v);
                     ptx::tmem_ld_wait();
@@ -670,7 +680,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     *reinterpret_cast<uint4*>(blk + ((((cc + 1) & 7) ^ sw) << 4)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
                 }
 #pragma unroll 1
-                for (int k = tail0; k < tail_blocks; k += 2) {
+                for (int k = tail0; k < tail_blocks; k += H) {
                     uint32_t v[8], wd[2];
                     const int col = full_chunks * 32 + k * 8, cc = col >> 4;
                     ptx::tmem_ld8(t_row + (uint32_t)col, v);
@@ -693,18 +703,20 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             ptx::tc_fence_after();
             const int token = qt * 128 + row;
-            // each of the row's two threads requantizes and stores 32 of the head's 64 columns (V codes that were unpacked sit
+            // each of the row's threads requantizes and stores its share of the head's 64 columns (V codes that were unpacked sit
             // in the high bits of their bytes)
             if (warp_live) {
-                uint32_t v[32], ow[8];
-                ptx::tmem_ld32(t_row + (uint32_t)(hf * 32), v);
+                constexpr int N = 64 / H;
+                uint32_t v[N], ow[N / 4];
+                if constexpr (H == 2) ptx::tmem_ld32(t_row + (uint32_t)(hf * N), v);
+                else ptx::tmem_ld16(t_row + (uint32_t)(hf * N), v);
                 ptx::tmem_ld_wait();
-                requantize_row32<!GENERAL>(v, 8 - C, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
+                requantize_row<!GENERAL, N>(v, 8 - C, colp + hf * N, colp + 64 + hf * N, P.out_qn, P.out_qp, ow);
                 if (token < T)
-                    store_row32(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c), ow, P.out_c);
+                    store_row(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (N * P.out_c / 8), ow, P.out_c);
             }
             // row padding behind the last head's columns (a caller may choose a pitch beyond the row's codes)
-            if (token < T && h == P.heads - 1 && hf == 1) {
+            if (token < T && h == P.heads - 1 && hf == H - 1) {
                 uint8_t* const orow = P.out + ((long long)b * T + token) * P.out_pitch;
                 for (long long off = (long long)P.heads * (8 * P.out_c); off + 4 <= P.out_pitch; off += 4)
                     *reinterpret_cast<uint32_t*>(orow + off) = 0u;
@@ -717,10 +729,10 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
 
     ptx::tc_fence_before();
     __syncthreads();
-    if (warp == AT_GROUPS * AT_COMPUTE_WARPS) {
+    if (warp == AT_COMPUTE_WARPS) {
         ptx::tc_fence_after();
         __syncwarp();
-        ptx::tmem_dealloc(tmem_base_slot, 512);
+        ptx::tmem_dealloc(tmem_base_slot, GROUPS * 256);
     }
 }
 
@@ -832,11 +844,15 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
         P.off_pv = o; o += up((uint32_t)P.kv_rows * hb, 128);
     }
     P.off_col = o; o += 1024;
-    P.off_z = o; o += 2 * 128 * 8;
+    // One group of sixteen warps where every item has a CTA of its own: with two groups of eight the other half of the warps has
+    // nothing to do.  197 tokens x 12 heads, one image, inside a stack of layers: 7.9 -> 6.2 us together with the copies
+    // of Q, K and V being under way while the exp table is filled (192 items on 96 CTAs of two groups, 9.3 -> 7.4 by the latter).
+    const int sms = sm_count(), groups = P.total_items <= sms ? 1 : 2, row_threads = 4 / groups;
+    P.off_z = o; o += row_threads * 128 * 8;
     P.off_mx = o;
-    if (mode != AM_TABLE) o += 2 * 128 * 4;                // partial row maxima
+    if (mode != AM_TABLE) o += row_threads * 128 * 4;      // partial row maxima
     P.group_bytes = up(o, 1024);
-    const size_t smem = (size_t)P.off_group + (size_t)AT_GROUPS * P.group_bytes + 1024;
+    const size_t smem = (size_t)P.off_group + (size_t)groups * P.group_bytes + 1024;
     if (smem > 225 * 1024) return VITINT_ERR_UNSUPPORTED;
 
     CUtensorMap map_q, map_kv;
@@ -863,30 +879,29 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
         launch_kernel(exp_table_kernel, dim3((2 * smax + 1 + 255) / 256), dim3(256), 0, st, (float*)workspace, smax, cs);
         if (cudaGetLastError() != cudaSuccess) return VITINT_ERR_CUDA;
     }
-    int grid = sm_count();
+    int grid = sms;
     if (grid >= P.total_items) grid = P.total_items;                         // one item a CTA
     else if (grid > (P.total_items + 1) / 2) grid = (P.total_items + 1) / 2; // one item a group
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
-    static bool attr_set_dev[MAX_DEVICES][5] = {};
-    bool* const attr_set = attr_set_dev[dev];
-#define VITINT_ATTN_LAUNCH(CC, SH, SLOT)                                                                           \
-    {                                                                                                              \
-        if (!attr_set[SLOT]) {                                                                                     \
-            if (cudaFuncSetAttribute(attention_fused_kernel<CC, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
-                                     225 * 1024) != cudaSuccess)                                                   \
-                return VITINT_ERR_CUDA;                                                                            \
-            attr_set[SLOT] = true;                                                                                 \
-        }                                                                                                          \
-        launch_kernel(attention_fused_kernel<CC, SH>, dim3(grid), dim3(AT_THREADS), smem, st, map_q, map_kv, P);   \
-    }
-    if (general) VITINT_ATTN_LAUNCH(8, AM_GENERAL, 4)
-    else if (shift) VITINT_ATTN_LAUNCH(8, AM_SHIFT, 3)
-    else if (c == 8) VITINT_ATTN_LAUNCH(8, AM_TABLE, 2)
-    else if (c == 4) VITINT_ATTN_LAUNCH(4, AM_TABLE, 1)
-    else VITINT_ATTN_LAUNCH(2, AM_TABLE, 0)
-#undef VITINT_ATTN_LAUNCH
-    return cuda_status(cudaGetLastError());
+    static bool attr_set[MAX_DEVICES][10] = {};
+    auto launch = [&](auto kernel, int slot) -> int {
+        if (!attr_set[dev][slot]) {
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024) != cudaSuccess) return VITINT_ERR_CUDA;
+            attr_set[dev][slot] = true;
+        }
+        launch_kernel(kernel, dim3(grid), dim3(at_threads(groups)), smem, st, map_q, map_kv, P);
+        return cuda_status(cudaGetLastError());
+    };
+    auto by_mode = [&](auto g) -> int {
+        constexpr int G = decltype(g)::value, s0 = 5 * (G - 1);
+        if (general) return launch(attention_fused_kernel<8, AM_GENERAL, G>, s0 + 4);
+        if (shift) return launch(attention_fused_kernel<8, AM_SHIFT, G>, s0 + 3);
+        if (c == 8) return launch(attention_fused_kernel<8, AM_TABLE, G>, s0 + 2);
+        if (c == 4) return launch(attention_fused_kernel<4, AM_TABLE, G>, s0 + 1);
+        return launch(attention_fused_kernel<2, AM_TABLE, G>, s0);
+    };
+    return groups == 1 ? by_mode(std::integral_constant<int, 1>{}) : by_mode(std::integral_constant<int, 2>{});
 }
 
 extern "C" int vitint_attention_core(const vitint_codes* qkv, int32_t batch, int32_t heads, int32_t tokens,

@@ -318,9 +318,9 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             ptx::tmem_ld32(t_row + AL_O_COL + (uint32_t)(hf * 32), v);
             ptx::tmem_ld_wait();
             // (once an item, so the conversion instruction: 8-bit P over more than 2056 tokens can take |O| past 2^22)
-            requantize_row32<false>(v, 0, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
+            requantize_row<false, 32>(v, 0, colp + hf * 32, colp + 64 + hf * 32, P.out_qn, P.out_qp, ow);
             if (token < T) {
-                store_row32(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c), ow, P.out_c);
+                store_row(P.out + ((long long)b * T + token) * P.out_pitch + (long long)h * (8 * P.out_c) + hf * (4 * P.out_c), ow, P.out_c);
                 if (h == P.heads - 1 && hf == 1) {
                     uint8_t* const orow = P.out + ((long long)b * T + token) * P.out_pitch;
                     for (long long off = (long long)P.heads * (8 * P.out_c); off + 4 <= P.out_pitch; off += 4)

@@ -120,8 +120,14 @@ __device__ __forceinline__ void unpack_rows64(const uint8_t* src, uint8_t* dst, 
 // The table holds exp(fl32(s * c)) for every integer score, as a ring: the entry of score s lies at s mod n, n = 2 smax
 // (a power of two).  Scores of signed codes reach smax = 64 * 2^(b-1) * 2^(b-1) but never -smax, so none share an entry, and
 // one AND turns 4 s into a byte offset that lies inside the table whatever the operand bytes were.
+// (Four entries a load; smax is a multiple of 256.)
 __device__ __forceinline__ void fill_table_ring(float* ring, const float* __restrict__ linear, int smax, int tid, int nthreads) {
-    for (int i = 1 + tid; i <= 2 * smax; i += nthreads) ring[(i - smax) & (2 * smax - 1)] = __ldg(linear + i);
+#pragma unroll 4
+    for (int i = 4 * tid; i < 2 * smax; i += 4 * nthreads) {
+        float4 v = __ldg(reinterpret_cast<const float4*>(i < smax ? linear + smax + i : linear + (i - smax)));
+        if (i == smax) v.x = __ldg(linear + 2 * smax);
+        *reinterpret_cast<float4*>(ring + i) = v;
+    }
 }
 
 // v: scores s (SCALED: 4 s times 2^sh) -> the entries' bits; their fp64 sum goes into four interleaved partial sums (one would
@@ -209,14 +215,14 @@ __device__ __forceinline__ bool quantize_scores(const uint32_t (&v)[N], f32x2 c2
     return quantize_interval<N>(a, lo2, hi2, qp2, w) == 0.0f;
 }
 
-// Requantizes 32 columns of an accumulator row (scaled by 2^sh; SMALL: |acc| < 2^22) to byte codes in two's complement:
+// Requantizes N columns of an accumulator row (scaled by 2^sh; SMALL: |acc| < 2^22) to byte codes in two's complement:
 // clamp(rint(fma(acc, a, b))).  pa, pb: the columns' parameters in shared memory, 16-byte aligned.
-template <bool SMALL = true>
-__device__ __forceinline__ void requantize_row32(const uint32_t (&v)[32], int sh, const float* pa, const float* pb, float qn, float qp,
-                                                 uint32_t (&w)[8]) {
+template <bool SMALL, int N>
+__device__ __forceinline__ void requantize_row(const uint32_t (&v)[N], int sh, const float* pa, const float* pb, float qn, float qp,
+                                               uint32_t (&w)[N / 4]) {
     const f32x2 magic2 = f2_dup(12582912.0f), nmagic2 = f2_dup(-12582912.0f);
 #pragma unroll
-    for (int i4 = 0; i4 < 8; ++i4) {
+    for (int i4 = 0; i4 < N / 4; ++i4) {
         const float4 a4 = *reinterpret_cast<const float4*>(pa + 4 * i4), b4 = *reinterpret_cast<const float4*>(pb + 4 * i4);
         uint32_t c[4];
 #pragma unroll
@@ -255,8 +261,19 @@ __device__ __forceinline__ uint32_t narrow2(const uint32_t (&w)[4]) {
     }
     return __byte_perm(__byte_perm(t[0], t[1], 0x0040), __byte_perm(t[2], t[3], 0x0040), 0x5410);
 }
-// Stores 32 byte codes of a row in the output's container (o: 4 * out_c bytes, 16-byte aligned for out_c >= 4, else 8).
-__device__ __forceinline__ void store_row32(uint8_t* o, const uint32_t (&w)[8], int out_c) {
+// Stores 16 or 32 byte codes of a row in the output's container (o: 2 or 4 * out_c bytes, aligned to 16 bytes or their number).
+__device__ __forceinline__ void store_row(uint8_t* o, const uint32_t (&w)[4], int out_c) {
+    if (out_c == 8) {
+        *reinterpret_cast<uint4*>(o) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else if (out_c == 4) {
+        uint32_t a[2];
+        narrow4(w, a);
+        *reinterpret_cast<uint2*>(o) = make_uint2(a[0], a[1]);
+    } else {
+        *reinterpret_cast<uint32_t*>(o) = narrow2(w);
+    }
+}
+__device__ __forceinline__ void store_row(uint8_t* o, const uint32_t (&w)[8], int out_c) {
     const uint32_t lo[4] = {w[0], w[1], w[2], w[3]}, hi[4] = {w[4], w[5], w[6], w[7]};
     if (out_c == 8) {
         if ((reinterpret_cast<uintptr_t>(o) & 31u) == 0) {

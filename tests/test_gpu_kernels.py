@@ -672,6 +672,30 @@ def test_cores_with_codes_on_or_far_beyond_the_last_level(tokens, p_step):
     assert torch.equal(out, one_by_one(layer, x))
 
 
+@pytest.mark.parametrize("tokens", [1, 9, 40, 96, 129, 197, 225, 256])
+@pytest.mark.parametrize("bits,form", [(4, "byte"), (4, "packed"), (2, "packed"), (4, "shift"), (8, "layer")])
+def test_core_with_one_group_and_with_two(tokens, bits, form):
+    """Every item with a CTA of its own (one group of sixteen warps) and more items than that (two groups of eight)."""
+    heads, D = 2, 128
+    batch = torch.cuda.get_device_properties(0).multi_processor_count // (2 * ((tokens + 127) // 128)) + 3
+    if form == "layer":
+        cfg, layer = small_layer({}, cfg=si.BlockConfig("groups", batch, tokens, D, heads, bits, mlp_dim=320))
+        x = dev(si.normal(961, (cfg.rows, cfg.dim)))
+        out = torch.empty_like(x)
+        layer.forward(x, out)
+        assert torch.equal(out, one_by_one(layer, x))
+        return
+    qkv = to_codes(rand_codes(960 + tokens, (batch * tokens, 3 * D), bits, True), bits, True)
+    qkv = qkv if form == "packed" else vt.vitint_widen(qkv)
+    alpha, step, p_step = dev(np.full(D, np.float32(0.05))), 0.25, float(np.float32(2.0 / tokens / (2 ** bits - 1) ** 0.5))
+    core = vt.vitint_attention_core_shift if form == "shift" else vt.vitint_attention_core
+    whole = core(qkv, batch, heads, tokens, step, step, p_step, bits, alpha, None).data
+    for first in (0, batch - 3):
+        rows = slice(first * tokens, (first + 3) * tokens)
+        part = vt.Codes(qkv.data[rows], 3 * tokens, 3 * D, bits, True, qkv.container)
+        assert torch.equal(core(part, 3, heads, tokens, step, step, p_step, bits, alpha, None).data, whole[rows])
+
+
 @pytest.mark.parametrize("tokens,bits", [(1, 4), (15, 2), (16, 4), (24, 4), (32, 2), (40, 3), (197, 4), (256, 3)])
 def test_attention_block_qkv_form(tokens, bits):
     """QKV stored one code per byte where its room is that of the unfused sequence, packed otherwise or when a copy is asked for:
