@@ -40,7 +40,12 @@ constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
 // 64 channels, takes twelve epilogue warps (three heads of a 192-column tile for each lane quarter) and 128 registers.
 constexpr int GD_UNPACK_WARPS = 8;
 __host__ __device__ constexpr int gd_epi_warps(int kind, bool packed) { return packed ? 16 - GD_UNPACK_WARPS : kind == EK_QKV_NORM ? 12 : 16; }
-__host__ __device__ constexpr int gd_threads(int kind, bool packed) { return (gd_epi_warps(kind, packed) + (packed ? GD_UNPACK_WARPS : 0) + 2) * 32; }
+// Groups of epilogue warps.  The norm kind has two, each with an accumulator buffer of its own: a thread's walk through Eq. 5 is a
+// chain, three warps a scheduler leave half of its slots empty, and a second tile beside the first fills them.
+__host__ __device__ constexpr int gd_epi_groups(int kind, bool packed) { return kind == EK_QKV_NORM && !packed ? 2 : 1; }
+__host__ __device__ constexpr int gd_threads(int kind, bool packed) {
+    return (gd_epi_groups(kind, packed) * gd_epi_warps(kind, packed) + (packed ? GD_UNPACK_WARPS : 0) + 2) * 32;
+}
 
 // Column block within which the weight rows are permuted: column 2q + 8g + e of the tensor-core block is output column
 // (B/4) q + 2g + e, e < 2, q < 4, g < B/8.
@@ -60,7 +65,7 @@ struct NormExtra { CUtensorMap map_w; };
 template <int KIND> using DirectExtra = std::conditional_t<KIND == EK_QKV_NORM, NormExtra, NoExtra>;
 
 struct DirectBars {
-    uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync, p_full[MAX_STAGES], p_empty[MAX_STAGES];
+    uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync[2], p_full[MAX_STAGES], p_empty[MAX_STAGES];
 };
 
 // One packed operand tile, `rows` rows of 16 C bytes -> rows of 128 int8 (128-byte swizzle), by 128 threads: thread t expands
@@ -227,7 +232,7 @@ __device__ __forceinline__ void direct_f32(const GemmParams& P, const uint32_t (
 // and K never exist in memory.  Both passes are rolled loops over 16 columns: unrolled over the 64 their code streams through
 // the instruction cache once per head, and that, not arithmetic, set the pace (one 197-row tile 9.8 us, of which the levels 6).
 // 12,672 x 384 -> 1152 (DeiT-S width, batch 64, 3-bit): 49 -> 31 us, 197 x 192 -> 576: 16.3 -> 6.5, against eight warps that
-// searched the references by four dependent shared-memory loads.
+// searched the references by four dependent shared-memory loads; 31 -> 27.5 us with a second group of epilogue warps.
 constexpr int GD_NORM_REFS = 18;                               // -inf, up to 15 references, +inf, padded
 struct NormTables {
     float ref[2][64][GD_NORM_REFS];
@@ -366,7 +371,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                    const __grid_constant__ DirectExtra<KIND> X, const __grid_constant__ GemmParams P) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ DirectBars bars;
-    __shared__ __align__(16) EpiParams epi_params;
+    constexpr int GROUPS = gd_epi_groups(KIND, PACKED);
+    __shared__ __align__(16) EpiParams epi_params_of[GROUPS];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     __shared__ __align__(16) std::conditional_t<KIND == EK_QKV_NORM, NormTables, float4> norm_tab[1];
@@ -395,7 +401,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             ptx::mbar_init(ptx::smem_addr(&bars.acc_full[b]), 1);
             ptx::mbar_init(ptx::smem_addr(&bars.acc_empty[b]), EPI_W);
         }
-        ptx::mbar_init(ptx::smem_addr(&bars.epi_sync), EPI_W);
+        for (int k = 0; k < GROUPS; ++k) ptx::mbar_init(ptx::smem_addr(&bars.epi_sync[k]), EPI_W);
         ptx::fence_mbar_init();
         ptx::fence_proxy_async_smem();
     }
@@ -561,8 +567,12 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             while (kb >= P.k_blocks) { kb -= P.k_blocks; tile += gridDim.x; }
         }
     } else {
-        const int q4 = warp & 3, slice = warp >> 2;
-        const int tid_e = threadIdx.x;
+        const int grp = GROUPS == 1 ? 0 : warp / EPI_W;                        // takes every GROUPS-th tile of the CTA
+        const int q4 = warp & 3, slice = (warp - grp * EPI_W) >> 2;
+        const int tid_e = threadIdx.x - grp * EPI_W * 32;
+        const int first_tile = (int)blockIdx.x + grp * (int)gridDim.x, tile_step = GROUPS * (int)gridDim.x;
+        EpiParams& epi_params = epi_params_of[grp];
+        const uint32_t epi_sync = ptx::smem_addr(&bars.epi_sync[grp]);
         const float down = __int_as_float((127 - (SMALL ? 0 : P.shift)) << 23);
         // per-column parameters of a tile (multiplier, bias, GELU output factor), column c of the tile
         auto fetch_params = [&](int tile, int c, float& a, float& b, float& q) {
@@ -598,10 +608,10 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             epi_params.b[buf][my_slot] = b;
             if (KIND == EK_REQUANT_GELU) epi_params.q[buf][my_slot] = q;
         };
-        if (my_col && (int)blockIdx.x < P.total_tiles) {
+        if (my_col && first_tile < P.total_tiles) {
             float a, b, q;
-            fetch_params(blockIdx.x, tid_e, a, b, q);
-            put_params(blockIdx.x, 0, a, b, q);
+            fetch_params(first_tile, tid_e, a, b, q);
+            put_params(first_tile, 0, a, b, q);
         }
         if (KIND == EK_REQUANT && P.exp_table != nullptr)
             fill_exp_table(P.exp_table, P.exp_smax, P.exp_c, blockIdx.x * (EPI_W * 32) + tid_e, gridDim.x * (EPI_W * 32));
@@ -611,9 +621,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
         VT_STAMP(tr, TT_START);
         // fp32 kinds: the residual of the warp's next two units of 16 rows x 32 columns, requested two units ahead across tiles
         float res[2][2][8];
-        int ahead_tile = blockIdx.x, ahead_u = slice;
+        int ahead_tile = first_tile, ahead_u = slice;
         auto request_residual = [&](float (&r)[2][8]) {
-            for (; ahead_tile < P.total_tiles; ahead_tile += gridDim.x, ahead_u = slice) {
+            for (; ahead_tile < P.total_tiles; ahead_tile += tile_step, ahead_u = slice) {
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, ahead_tile, m_tile, col_t, cols);
                 if ((ahead_u >> 1) * BLK < cols) {
@@ -645,28 +655,29 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             request_residual(res[0]);
             request_residual(res[1]);
         }
-        for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x, ++tl) {
+        for (int tile = first_tile; ok && tile < P.total_tiles; tile += tile_step, ++tl) {
             int m_tile, col_t, cols;
             direct_tile<KIND>(P, tile, m_tile, col_t, cols);
-            const int buf = tl & 1;
-            const int next_tile = tile + (int)gridDim.x;
+            const int buf = tl & 1;                                            // half of the parameters
+            const int acc = GROUPS == 1 ? buf : grp;                           // accumulator buffer
+            const int next_tile = tile + tile_step;
             const bool fetch_next = my_col && next_tile < P.total_tiles;
             float na = 0.0f, nb = 0.0f, nq = 0.0f;
             if (fetch_next) fetch_params(next_tile, tid_e, na, nb, nq);
             const int row_q = m_tile * BM + q4 * 32;
             const int rows_q = P.M - row_q;                                   // valid rows from the quarter's first one on
-            const uint32_t acc_ph = (uint32_t)(tl >> 1) & 1u;
+            const uint32_t acc_ph = (uint32_t)(GROUPS == 1 ? tl >> 1 : tl) & 1u;
             VT_STAMP(tr, TT_WAIT_ACC);
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&bars.epi_sync));
-            bool w = mbar_wait(ptx::smem_addr(&bars.epi_sync), (uint32_t)tl & 1u, abort_ptr);
+            if (lane == 0) ptx::mbar_arrive(epi_sync);
+            bool w = mbar_wait(epi_sync, (uint32_t)tl & 1u, abort_ptr);
             VT_STAMP(tr, TT_WAIT_FULL);
-            w = w && mbar_wait(ptx::smem_addr(&bars.acc_full[buf]), acc_ph, abort_ptr);
+            w = w && mbar_wait(ptx::smem_addr(&bars.acc_full[acc]), acc_ph, abort_ptr);
             VT_STAMP(tr, TT_GOT_ACC);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
             ptx::tc_fence_after();
             if (fetch_next) put_params(next_tile, buf ^ 1, na, nb, nq);                  // every warp has passed the barrier: none reads that half
-            const uint32_t t_quarter = tmem_base + (uint32_t)buf * acc_stride + ((uint32_t)(q4 * 32) << 16);
+            const uint32_t t_quarter = tmem_base + (uint32_t)acc * acc_stride + ((uint32_t)(q4 * 32) << 16);
             const int n_blk = cols / BLK;
             if constexpr (KIND == EK_DEQUANT) {
                 // Units of half a block: 192 columns are three for every slice, where whole blocks were two for half of the slices
@@ -715,7 +726,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             }
             ptx::tc_fence_before();
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&bars.acc_empty[buf]));
+            if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&bars.acc_empty[acc]));
             VT_STAMP(tr, TT_TILE_DONE);
         }
         VT_STAMP(tr, TT_END);

@@ -498,10 +498,10 @@ def test_compare_layernorm_references_that_are_not_uniform(warp):
     assert np.array_equal(from_codes(got), compare_reference(x, refs_, flip, n_eps, 4))
 
 
-@pytest.mark.parametrize("M,heads,bits", [(1, 1, 2), (129, 3, 4), (300, 5, 3), (2000, 7, 4)])
+@pytest.mark.parametrize("M,heads,bits", [(1, 1, 2), (129, 3, 4), (300, 5, 3), (2000, 7, 4), (2600, 7, 3), (6500, 7, 4)])
 @pytest.mark.parametrize("packed", [False, True])
 def test_qkv_norm_tiles_and_references(M, heads, bits, packed):
-    """Segments that end inside a tile, packed operands, and references no uniform quantizer would give."""
+    """Segments that end inside a tile, packed operands, one to four tiles a CTA, and references no uniform quantizer would give."""
     D, K = 64 * heads, 96
     qx, qw = rand_codes(461, (M, K), bits, True), rand_codes(462, (3 * D, K), bits, True)
     acc = vo.matmul_i32(qx, qw)
