@@ -4,7 +4,7 @@
 //   statistics  one thread per row walks the row in order:
 //                 delta = x_i - mu;  mu += delta / i;  S += delta * (x_i - mu)
 //               every operation a single round-to-nearest fp32 one (no contraction), the
-//               division by i exact-rounded through a reciprocal and one correction step.
+//               division by i exactly rounded from a reciprocal of two floats.
 //   comparator  level = Qn + number of references exceeded.  With d = x - mu (negated where
 //               gamma < 0) the sign logic of the figure collapses into one comparison of
 //               signed squares,  copysign(d*d, d) > V * r,  r = sgn(c) c^2 / n the caller's
@@ -13,12 +13,12 @@
 //               spaced points, so the index is guessed from d / sqrt(V) (two operations) and two comparisons around
 //               the guess, formed exactly as defined, prove it; where they do not, all references are compared.
 //
-// What bounds it.  The recurrence is a chain of five dependent fp32 operations per element (20 cycles, 768 elements: 8 us)
+// What bounds it.  The recurrence is a chain of four dependent fp32 operations per element (16 cycles, 768 elements: 6.5 us)
 // and cannot be split without changing the order of Eq. 5 and with it the bits; one CTA per SM walks all its rows at once, one
 // lane each, while TMA keeps the next chunks of columns coming and the other warps lay out the references.  Its levels it finds
 // afterwards with all warps, the rows coming from L2.  As two kernels -- statistics, then a bisection over references held in
 // registers, 42 instructions an element -- 12,608 x 768 took 39 us and 25,216 x 768 74 us; as one 25 and 38, of which the walk
-// 13 and 17.  (Requesting the next task's rows ahead of the present one's levels: no change.)
+// 13 and 17; with the quotient in two operations instead of three (2 x 1.0 us of a layer at batch 64) 24.  (Requesting the next task's rows ahead of the present one's levels: no change.)
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"
@@ -35,22 +35,37 @@ constexpr int LNC_SLAB = 768, LNC_QUARTER = LNC_SLAB / 4;     // columns whose r
 constexpr int LNC_ROW_BATCH = 4;               // rows of one comparator task: their loads are issued together
 constexpr int LNS_MAX_COLS = 4096;
 
-// One step of Eq. 5 for element xi, i = fi: every operation a single rounded fp32 one.  The update of S
+// One step of Eq. 5 for element xi, (rh, rl) = 1/i to 48 bits: every operation a single rounded fp32 one.  The update of S
 // belonging to the PREVIOUS element (its delta in pd, its value in px; mu is still that element's mean) is
 // written between the operations of this element's dependent chain delta -> quotient -> mu, so the two
 // interleave in issue order; operands and operations are exactly those of the recurrence.
-__device__ __forceinline__ void running_step(float xi, float fi, float r, float& mu, float& S, float& pd, float& px) {
+//
+// RN(delta / i) = fma(delta, rh, RN(delta rl)): what is rounded last is within 2^-48 of the quotient, and a quotient of a 24-bit
+// number by an i <= 4096 is at least ulp / 2i = 2^-37 away from a rounding boundary (it cannot lie on one: the odd part of a
+// boundary times i has 25 bits or more) -- unless the product underflows: `tiny` keeps the smallest |delta| that is not 0, as bits
+// less 1, and a row that had one below 2^-100, or did not stay finite, is walked again by running_row_slow.
+__device__ __forceinline__ void running_step(float xi, float rh, float rl, float& mu, float& S, float& pd, float& px, uint32_t& tiny) {
     const float delta = __fadd_rn(xi, -mu);
     const float tt = __fadd_rn(px, -mu);
-    // RN(delta / i): q0 = RN(delta*r), remainder exact in one FMA, one correction
-    const float q0 = __fmul_rn(delta, r);
+    const float lo = __fmul_rn(delta, rl);
     const float pp = __fmul_rn(pd, tt);
-    const float rem = __fmaf_rn(-q0, fi, delta);
+    const float q = __fmaf_rn(delta, rh, lo);
     S = __fadd_rn(S, pp);
-    const float q = __fmaf_rn(rem, r, q0);
     mu = __fadd_rn(mu, q);
+    tiny = min(tiny, (__float_as_uint(delta) & 0x7FFFFFFFu) - 1u);
     pd = delta;
     px = xi;
+}
+// The whole row from memory, RN(delta / i) as q0 = RN(delta r), an exact remainder in one FMA and one correction.
+__device__ __noinline__ float2 running_row_slow(const float* __restrict__ x, int cols) {
+    float mu = 0.0f, S = 0.0f;
+    for (int i = 0; i < cols; ++i) {
+        const float fi = (float)(i + 1), r = __frcp_rn(fi), xi = __ldg(x + i);
+        const float delta = __fadd_rn(xi, -mu), q0 = __fmul_rn(delta, r);
+        mu = __fadd_rn(mu, __fmaf_rn(__fmaf_rn(-q0, fi, delta), r, q0));
+        S = __fadd_rn(S, __fmul_rn(delta, __fadd_rn(xi, -mu)));
+    }
+    return make_float2(mu, S);
 }
 
 struct LncShape {
@@ -102,7 +117,7 @@ ln_compare_quantize_kernel(const __grid_constant__ CUtensorMap map_x, const floa
     constexpr int LANES_PER_WORD = 8 / C;                       // lanes whose 4 codes share one 32-bit word
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint8_t* const smem = lnc_raw + ((1024u - (ptx::smem_addr(lnc_raw) & 1023u)) & 1023u);
-    float2* const tab = reinterpret_cast<float2*>(smem);        // (float(i), RN(1/i)) of every column
+    float2* const tab = reinterpret_cast<float2*>(smem);        // 1/i of every column, i from 1, as a sum of two floats
     float* const s_ref = reinterpret_cast<float*>(smem + sh.off_ref);
     float* const s_col = reinterpret_cast<float*>(smem + sh.off_col);
     uint8_t* const stage = smem + sh.off_stage;
@@ -119,8 +134,8 @@ ln_compare_quantize_kernel(const __grid_constant__ CUtensorMap map_x, const floa
         ptx::fence_proxy_async_smem();
     }
     for (int i = threadIdx.x; i < cols; i += LNC_THREADS) {
-        const float fi = (float)(i + 1);
-        tab[i] = make_float2(fi, __frcp_rn(fi));
+        const float fi = (float)(i + 1), rh = __frcp_rn(fi);
+        tab[i] = make_float2(rh, __fdiv_rn(__fmaf_rn(-rh, fi, 1.0f), fi));
     }
     __syncthreads();
     grid_dependency_wait();        // x may come from the previous kernel of the stream
@@ -140,6 +155,7 @@ ln_compare_quantize_kernel(const __grid_constant__ CUtensorMap map_x, const floa
         // ---- statistics ----
         if (warp < walkers) {
             float mu = 0.0f, S = 0.0f, pd = 0.0f, px = 0.0f;
+            uint32_t tiny = 0xFFFFFFFFu;
             const int my_row = min(warp * 32 + lane, sh.rows_cta - 1), r7 = my_row & 7;
             for (int c = 0; c < n_chunks; ++c) {
                 const bool w = mbar_wait(ptx::smem_addr(&full[buf]), ph, &abort_flag);
@@ -157,10 +173,10 @@ ln_compare_quantize_kernel(const __grid_constant__ CUtensorMap map_x, const floa
 #pragma unroll 4
                 for (int v = 0; v < nv; ++v) {
                     const Four next = read(v + 1 < nv ? v + 1 : v);
-                    running_step(cur.e.x, cur.ta.x, cur.ta.y, mu, S, pd, px);
-                    running_step(cur.e.y, cur.ta.z, cur.ta.w, mu, S, pd, px);
-                    running_step(cur.e.z, cur.tb.x, cur.tb.y, mu, S, pd, px);
-                    running_step(cur.e.w, cur.tb.z, cur.tb.w, mu, S, pd, px);
+                    running_step(cur.e.x, cur.ta.x, cur.ta.y, mu, S, pd, px, tiny);
+                    running_step(cur.e.y, cur.ta.z, cur.ta.w, mu, S, pd, px, tiny);
+                    running_step(cur.e.z, cur.tb.x, cur.tb.y, mu, S, pd, px, tiny);
+                    running_step(cur.e.w, cur.tb.z, cur.tb.w, mu, S, pd, px, tiny);
                     cur = next;
                 }
                 __syncwarp();
@@ -169,6 +185,11 @@ ln_compare_quantize_kernel(const __grid_constant__ CUtensorMap map_x, const floa
             }
             if (ok && warp * 32 + lane < n_rows) {
                 S = __fadd_rn(S, __fmul_rn(pd, __fadd_rn(px, -mu)));                   // the last element's term
+                if (tiny < 0x0D800000u - 1u || !(fabsf(mu) < INFINITY)) {              // 2^-100
+                    const float2 again = running_row_slow(x + (row0 + my_row) * ldx, cols);
+                    mu = again.x;
+                    S = again.y;
+                }
                 const float2 st = make_float2(mu, __fadd_rn(S, n_eps));
                 s_stat[my_row] = st;
                 reinterpret_cast<float2*>(stats)[row0 + my_row] = st;

@@ -615,6 +615,22 @@ def test_layernorm_compare_quantize_bit_exact(rows, cols, bits, container):
     assert padding_is_zero(got)
 
 
+@pytest.mark.parametrize("scale", [2.0 ** -98, 2.0 ** -104, 2.0 ** -112, 2.0 ** -124, 2.0 ** -140])
+def test_layernorm_compare_statistics_of_tiny_values(scale):
+    """Differences down to the subnormal numbers, where the two-operation quotient of Eq. 5 gives way to the corrected one."""
+    rows, cols, bits = 70, 768, 4
+    x = (si.normal(87, (rows, cols)).astype(np.float64) * scale).astype(np.float32)
+    x[::2, 100:] += np.float32(1.0)                  # tiny differences in front of ordinary ones
+    ref, neg, flip = vo.layernorm_references(np.ones(cols, np.float32), np.zeros(cols, np.float32), 0.5, bits, True, cols)
+    q_ref, mu_ref, v_ref = vo.layernorm_compare_quantize(x, ref, neg, flip, 1e-6, bits, True, want_stats=True)
+    refs_g, flip_g = vt.fold_layernorm_references(np.ones(cols), np.zeros(cols), 0.5, bits, True, cols)
+    got, stats = vt.vitint_layernorm_compare_quantize(dev(x), dev(refs_g), dev(flip_g), float(np.float32(cols * np.float64(np.float32(1e-6)))),
+                                                      bits, True)
+    st = stats.cpu().numpy()
+    assert np.array_equal(st[:, 0].view(np.uint32), mu_ref.view(np.uint32)) and np.array_equal(st[:, 1].view(np.uint32), v_ref.view(np.uint32))
+    assert np.array_equal(from_codes(got), q_ref)
+
+
 def test_layernorm_compare_quantize_widest_row_and_single_row():
     """The widest supported row (4096 columns: the reciprocal table fills 32 KB of shared memory) and a single row."""
     rows, cols, bits = 3, 4096, 3
