@@ -91,7 +91,9 @@ quantize_pack_kernel(const float* __restrict__ x, int64_t rows, int64_t cols, in
 // two-pass mean keeps the result inside a few ulp of the exact normalisation.
 // FULL: the row is exactly NV*128 columns and no fp32 copy is written, so no access needs a guard (the guards
 // otherwise become branches around every vector: a third of the instructions at 768 columns).
-template <int C, int NV, bool FULL>
+// FEW: the gains and offsets are requested with the row (48 registers at 768 columns); otherwise they come after the statistics,
+// from L1 where a block of the SM has been there before.
+template <int C, int NV, bool FULL, bool FEW>
 __global__ void __launch_bounds__(128)
 layernorm_quantize_kernel(const float* __restrict__ x, int64_t rows, int cols, int64_t ldx,
                           const float* __restrict__ gamma, const float* __restrict__ beta, float eps, float step,
@@ -107,6 +109,16 @@ layernorm_quantize_kernel(const float* __restrict__ x, int64_t rows, int cols, i
     // instruction (each half is the scalar IEEE result), which is what this issue-bound kernel needs.
     f32x2 f[NV][2];
     f32x2 sum2 = f2_dup(0.0f);
+    float4 ga[FEW ? NV : 1], be[FEW ? NV : 1];
+    if constexpr (FEW) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int col = (v * 32 + lane) * 4;
+            const bool in = FULL || col < cols;
+            ga[v] = in ? __ldg(reinterpret_cast<const float4*>(gamma + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            be[v] = in ? __ldg(reinterpret_cast<const float4*>(beta + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const int col = (v * 32 + lane) * 4;
@@ -168,8 +180,8 @@ layernorm_quantize_kernel(const float* __restrict__ x, int64_t rows, int cols, i
         uint32_t bits = 0;
         const int col = (v * 32 + lane) * 4;
         if (FULL || col < cols) {
-            const float4 g = __ldg(reinterpret_cast<const float4*>(gamma + col));
-            const float4 b = __ldg(reinterpret_cast<const float4*>(beta + col));
+            const float4 g = FEW ? ga[FEW ? v : 0] : __ldg(reinterpret_cast<const float4*>(gamma + col));
+            const float4 b = FEW ? be[FEW ? v : 0] : __ldg(reinterpret_cast<const float4*>(beta + col));
             const f32x2 rstd2 = f2_dup(rstd), rstep2 = f2_dup(rstep), magic2 = f2_dup(magic);
             const f32x2 y01 = f2_fma(f2_mul(f2_add(f[v][0], ncorr2), rstd2), f2_pack(g.x, g.y), f2_pack(b.x, b.y));
             const f32x2 y23 = f2_fma(f2_mul(f2_add(f[v][1], ncorr2), rstd2), f2_pack(g.z, g.w), f2_pack(b.z, b.w));
@@ -240,14 +252,16 @@ static int launch_ln(int nv, const float* x, int64_t rows, int cols, int64_t ldx
     const int warps = 4;       // four rows per block: measured best (8: +1 us per call at 25,216 x 768; 16: +3 us)
     dim3 grid((unsigned)((rows + warps - 1) / warps)), block(32 * warps);
     const bool full = cols == nv * 128 && y == nullptr;
+    // Up to one wave of blocks every SM meets the gains for the first time, and they may have to come from HBM: 197 x 768 between
+    // the kernels of a twelve-layer stack 3.7 -> 1.5 us, 1576 x 768 in a layer 2.9 -> 2.0
+    const bool few = nv <= 8 && rows <= 16 * (int64_t)sm_count();
+    auto launch = [&](auto kernel) { launch_kernel(kernel, grid, block, 0, st, x, rows, cols, ldx, gamma, beta, eps, step, out, pitch, y, ld_y, qn, qp); };
 #define VITINT_LN_CASE(NVV)                                                                                     \
     case NVV:                                                                                                   \
         if (full)                                                                                               \
-            launch_kernel(layernorm_quantize_kernel<C, NVV, true>, dim3(grid), dim3(block), 0, st, x, rows, cols, ldx, gamma, beta,    \
-                          eps, step, out, pitch, y, ld_y, qn, qp);                                              \
+            few ? launch(layernorm_quantize_kernel<C, NVV, true, (NVV <= 8)>) : launch(layernorm_quantize_kernel<C, NVV, true, false>); \
         else                                                                                                    \
-            launch_kernel(layernorm_quantize_kernel<C, NVV, false>, dim3(grid), dim3(block), 0, st, x, rows, cols, ldx, gamma, beta,   \
-                          eps, step, out, pitch, y, ld_y, qn, qp);                                              \
+            few ? launch(layernorm_quantize_kernel<C, NVV, false, (NVV <= 8)>) : launch(layernorm_quantize_kernel<C, NVV, false, false>); \
         break;
     switch (nv) {
         VITINT_LN_CASE(1) VITINT_LN_CASE(2) VITINT_LN_CASE(3) VITINT_LN_CASE(4) VITINT_LN_CASE(6)
