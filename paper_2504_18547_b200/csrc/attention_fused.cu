@@ -53,6 +53,7 @@ struct AttnParams {
     uint32_t off_table, off_group, group_bytes;         // shared-memory layout
     uint32_t off_pq, off_pk, off_pv, off_q, off_k, off_v, off_p, off_col, off_z, off_mx;   // within a group
     const float* table;          // global copy of the exp table, 2*smax+1 floats
+    int at_rest;                 // the table may be read before the grid dependency
     float p_step, p_qp;
     float scale;                 // softmax scale c (GENERAL), c log2 e (SHIFT)
     const float* alpha_o;        // [D]
@@ -139,12 +140,17 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
     ptx::tc_fence_before();
     __syncthreads();
     ptx::tc_fence_after();
-    grid_dependency_wait();        // the table and the codes come from earlier kernels of the stream
+    // The exp table: global -> shared, once per CTA, while the control warps' first copies and Q K^T are on their way, or before the
+    // wait where it cannot come from the kernel in front (the codes do).
+    auto table_to_shared = [&]() {
+        fill_table_ring(reinterpret_cast<float*>(smem_gen + P.off_table), P.table, P.smax, threadIdx.x, AT_COMPUTE_WARPS * 32);
+    };
+    if (MODE == AM_TABLE && P.at_rest && !is_control) table_to_shared();
+    grid_dependency_wait();
     grid_dependency_launch();
-    // the exp table: global -> shared, once per CTA, while the control warps' first copies and Q K^T are on their way
     if constexpr (MODE == AM_TABLE) {
         if (!is_control) {
-            fill_table_ring(reinterpret_cast<float*>(smem_gen + P.off_table), P.table, P.smax, threadIdx.x, AT_COMPUTE_WARPS * 32);
+            if (!P.at_rest) table_to_shared();
             asm volatile("bar.sync 1, %0;" ::"n"(AT_COMPUTE_WARPS * 32) : "memory");
         }
     }
@@ -820,6 +826,7 @@ static int attention_core_launch(const vitint_codes* qkv, int32_t batch, int32_t
     P.scale = shift ? c2 : cs;
     P.part_bytes = (int)(D * c / 8);
     P.table = (const float*)workspace;
+    P.at_rest = parameters_at_rest() && !build_table ? 1 : 0;
     P.p_step = p_step;
     int qn, qp;
     code_range(p_bits, 0, &qn, &qp);

@@ -76,7 +76,7 @@ inline EncodeTiledFn encode_fn() {
 // be scheduled while the previous kernel of the stream is still draining, run their set-up
 // (barriers, tensor memory, descriptor prefetch) and then block in grid_dependency_wait() until
 // the previous kernel has completed and its writes are visible.  Nothing that another kernel
-// may have produced is read, and nothing is written, before that wait.
+// may have produced is read, and nothing is written, before that wait (see parameters_at_rest).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -92,6 +92,11 @@ struct LaunchRecorder {
     cudaError_t record(const cudaKernelNodeParams& p);
 };
 inline thread_local LaunchRecorder* t_recorder = nullptr;
+
+// Whether the launch being made may read its weights and parameters before grid_dependency_wait().  True inside a recorded
+// graph: no kernel of a stack writes them, the first kernel waits for all that the stream held before the graph, and a kernel's
+// CTAs start no earlier than the wait of the kernel in front has returned in every CTA.
+inline bool parameters_at_rest() { return t_recorder != nullptr; }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

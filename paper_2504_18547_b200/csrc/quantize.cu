@@ -98,27 +98,31 @@ __global__ void __launch_bounds__(128)
 layernorm_quantize_kernel(const float* __restrict__ x, int64_t rows, int cols, int64_t ldx,
                           const float* __restrict__ gamma, const float* __restrict__ beta, float eps, float step,
                           uint8_t* __restrict__ out, int64_t pitch, float* __restrict__ y_out, int64_t ld_y,
-                          float qn, float qp) {
+                          float qn, float qp, int at_rest) {
+    const int lane = threadIdx.x & 31;
+    float4 ga[FEW ? NV : 1], be[FEW ? NV : 1];
+    auto gains = [&]() {
+        if constexpr (FEW) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                const int col = (v * 32 + lane) * 4;
+                const bool in = FULL || col < cols;
+                ga[v] = in ? __ldg(reinterpret_cast<const float4*>(gamma + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                be[v] = in ? __ldg(reinterpret_cast<const float4*>(beta + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+    };
+    if (FEW && at_rest) gains();
     grid_dependency_wait();        // inputs may come from the previous kernel of the stream
     grid_dependency_launch();
-    const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
+    if (FEW && !at_rest) gains();
     const float* xr = x + row * ldx;
     // The row is held as packed pairs: adds, multiplies and fused multiply-adds below run two elements per
     // instruction (each half is the scalar IEEE result), which is what this issue-bound kernel needs.
     f32x2 f[NV][2];
     f32x2 sum2 = f2_dup(0.0f);
-    float4 ga[FEW ? NV : 1], be[FEW ? NV : 1];
-    if constexpr (FEW) {
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const int col = (v * 32 + lane) * 4;
-            const bool in = FULL || col < cols;
-            ga[v] = in ? __ldg(reinterpret_cast<const float4*>(gamma + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
-            be[v] = in ? __ldg(reinterpret_cast<const float4*>(beta + col)) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         const int col = (v * 32 + lane) * 4;
@@ -255,7 +259,7 @@ static int launch_ln(int nv, const float* x, int64_t rows, int cols, int64_t ldx
     // Up to one wave of blocks every SM meets the gains for the first time, and they may have to come from HBM: 197 x 768 between
     // the kernels of a twelve-layer stack 3.7 -> 1.5 us, 1576 x 768 in a layer 2.9 -> 2.0
     const bool few = nv <= 8 && rows <= 16 * (int64_t)sm_count();
-    auto launch = [&](auto kernel) { launch_kernel(kernel, grid, block, 0, st, x, rows, cols, ldx, gamma, beta, eps, step, out, pitch, y, ld_y, qn, qp); };
+    auto launch = [&](auto kernel) { launch_kernel(kernel, grid, block, 0, st, x, rows, cols, ldx, gamma, beta, eps, step, out, pitch, y, ld_y, qn, qp, parameters_at_rest() ? 1 : 0); };
 #define VITINT_LN_CASE(NVV)                                                                                     \
     case NVV:                                                                                                   \
         if (full)                                                                                               \

@@ -121,6 +121,34 @@ def test_layer_plan_equals_its_launches(kw):
     assert torch.equal(odd, one_by_one(layer, x)) and not torch.equal(odd, out)
 
 
+@pytest.mark.parametrize("batch,mlp", [(1, 320), (1, 1024), (3, 2176), (60, 512)])
+def test_plan_sees_weights_written_in_place_right_before_it(batch, mlp):
+    """Recorded kernels read weights and parameters ahead of the kernel in front of them, never ahead of the stream: copies into
+    the layer's own tensors and runs in turn, nothing between them.  (MLP widths whose weights fill the ring of fc2 and exceed it.)"""
+    from paper_2504_18547_b200.encoder import EncoderLayer
+    cfg = si.BlockConfig("inplace", batch, 50, 128, 2, 4, mlp_dim=mlp)
+    prm, other = si.layer_parameters(cfg, 0), si.layer_parameters(cfg, 1)
+    scalars = {k: v for k, v in prm.items() if np.ndim(v) == 0}
+    layers = [EncoderLayer(batch, 50, 2, mlp, 4, dict(p, **scalars)) for p in (prm, other)]
+
+    def tensors(layer):
+        return ([c.data for c in layer.w.values()] + list(layer.s_w.values()) + list(layer.bias.values())
+                + [layer.alpha_qkv, layer.beta_qkv, layer.alpha_o, layer.inv_s_g, layer.ln1_g, layer.ln1_b, layer.ln2_g, layer.ln2_b])
+    states = [[t.clone() for t in tensors(layer)] for layer in layers]
+    x = dev(si.normal(350 + batch, (cfg.rows, cfg.dim)))
+    want = [one_by_one(layer, x) for layer in layers]
+    assert not torch.equal(want[0], want[1])
+    outs = [torch.empty_like(x) for _ in range(8)]
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        for t, new in zip(tensors(layers[0]), states[i & 1]):
+            t.copy_(new)
+        layers[0].forward(x, out)
+    assert layers[0]._plan is not None
+    for i, out in enumerate(outs):
+        assert torch.equal(out, want[i & 1])
+
+
 @pytest.mark.parametrize("kw", [{}, {"fused_attention": False}, {"bits": 8}], ids=["core", "three_kernels", "bits8"])
 def test_plan_follows_every_parameter_that_the_launches_read(kw):
     cfg, layer = small_layer(dict(kw))
