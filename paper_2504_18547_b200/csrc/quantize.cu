@@ -115,7 +115,9 @@ layernorm_quantize_kernel(const float* __restrict__ x, int64_t rows, int cols, i
     if (FEW && at_rest) gains();
     grid_dependency_wait();        // inputs may come from the previous kernel of the stream
     grid_dependency_launch();
-    const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    // Last rows first: of an input that does not fit L2 they are what the kernel in front has left there (layer of 25,216 x 768
+    // 329.6 -> 327.0 us, DeiT-S model at batch 128 1889 -> 1875)
+    const int64_t row = (int64_t)(gridDim.x - 1 - blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= rows) return;
     if (FEW && !at_rest) gains();
     const float* xr = x + row * ldx;
