@@ -442,7 +442,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                         ptx::mbar_arrive_expect_tx(bar, stage_bytes);
                         ptx::tma_load_5d(smem_base + (uint32_t)kb * stage_bytes + P.ia_bytes, &map_b, bar, kb * BK, 0, 0, 0, col_t / BLK);
                     }
-                    for (int kb = loaded; kb < P.k_blocks; ++kb) ptx::tma_prefetch_5d(&map_b, kb * BK, 0, 0, 0, col_t / BLK);
+                    // (by the CTAs of the first row tiles: all row tiles share them)
+                    for (int kb = loaded; m_tile < 2 && kb < P.k_blocks; ++kb) ptx::tma_prefetch_5d(&map_b, kb * BK, 0, 0, 0, col_t / BLK);
                 }
                 __syncwarp();
                 dependency();
