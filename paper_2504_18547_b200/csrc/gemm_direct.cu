@@ -59,10 +59,11 @@ __device__ __forceinline__ int gd_param_slot(int c) {
     return (c - w) + (i >> 2) * 16 + q * 4 + (i & 3);
 }
 
-// What only one kind of epilogue needs: the weights in their own order for the norm kind's Q and K tiles.
+// What only some kinds of epilogue need: the weights in their own order, for the norm kind's Q and K tiles and for a tile of codes
+// that ends inside a column block.
 struct NoExtra { int unused; };
-struct NormExtra { CUtensorMap map_w; };
-template <int KIND> using DirectExtra = std::conditional_t<KIND == EK_QKV_NORM, NormExtra, NoExtra>;
+struct OrderExtra { CUtensorMap map_w; };
+template <int KIND> using DirectExtra = std::conditional_t<KIND == EK_DEQUANT, NoExtra, OrderExtra>;
 
 struct DirectBars {
     uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync[2], p_full[MAX_STAGES], p_empty[MAX_STAGES];
@@ -120,47 +121,73 @@ struct CodeParams {
     }
 };
 
+// Four codes (bytes of a word, two's complement) of four consecutive columns of a row from their accumulators and parameters.
+template <int KIND, bool SMALL, bool PACKED>
+__device__ __forceinline__ uint32_t direct_quad(const GemmParams& P, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3, const float4& a,
+                                                const float4& b, const float4& g4) {
+    const f32x2 magic = f2_dup(12582912.0f), qp2 = f2_dup(P.out_qp);
+    const float qn = P.out_qn, qp = P.out_qp;
+    uint32_t c[4];
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+        const f32x2 y = f2_fma(acc_to_float2<SMALL, PACKED>(p ? v2 : v0, p ? v3 : v1, P.shift), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
+                               p ? f2_pack(b.z, b.w) : f2_pack(b.x, b.y));
+        float y0, y1, c0, c1;
+        f2_unpack(y, y0, y1);
+        if (KIND == EK_REQUANT_GELU) {
+            // unsigned codes: the value arrives clamped to [0, 1] in units of Qp, and a negative y is code 0 whatever
+            // its GELU: t = 0 there, the term is 1 and 2w - w = w < 0 saturates to 0
+            float e0, e1, w0, w1, d0, d1;
+            gelu_erfc_term2_pos(y0, y1, e0, e1);
+            const f32x2 wq = f2_mul(y, p ? f2_pack(g4.z, g4.w) : f2_pack(g4.x, g4.y));
+            f2_unpack(wq, w0, w1);
+            f2_unpack(f2_add(wq, wq), d0, d1);
+            const float u0 = __saturatef(fmaf(-w0, e0, d0)), u1 = __saturatef(fmaf(-w1, e1, d1));
+            f2_unpack(f2_fma(f2_pack(u0, u1), qp2, magic), c0, c1);
+        } else {
+            f2_unpack(f2_add(f2_pack(fminf(fmaxf(y0, qn), qp), fminf(fmaxf(y1, qn), qp)), magic), c0, c1);
+        }
+        c[2 * p] = __float_as_uint(c0);                         // the code in two's complement is the low byte
+        c[2 * p + 1] = __float_as_uint(c1);
+    }
+    return __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+}
+
+// A tile that ends inside a column block: its weights lie in their own order (rows behind the last one zero) and a thread takes
+// sixteen columns of its own row.  Parameters behind the last column are 0, and so are the codes, which fill the row's padding.
+template <int KIND, bool SMALL, bool PACKED>
+__device__ __forceinline__ void direct_codes_row(const GemmParams& P, uint32_t taddr, const EpiParams& ep, int buf, int tile_col,
+                                                 long long row, bool row_ok, int col) {
+    uint32_t v[16], w[4];
+    ptx::tmem_ld16(taddr, v);
+    ptx::tmem_ld_wait();
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 a = *reinterpret_cast<const float4*>(&ep.a[buf][tile_col + 4 * k]), b = *reinterpret_cast<const float4*>(&ep.b[buf][tile_col + 4 * k]);
+        float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (KIND == EK_REQUANT_GELU) g4 = *reinterpret_cast<const float4*>(&ep.q[buf][tile_col + 4 * k]);
+        w[k] = direct_quad<KIND, SMALL, PACKED>(P, v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3], a, b, g4);
+    }
+    if (!row_ok) return;
+    uint8_t* const o = (uint8_t*)P.out + row * P.ld_out;
+    store_row(o + ((col * P.out_c) >> 3), w, P.out_c);
+    if (col + 16 >= P.N)
+        for (long long off = (long long)(col + 16) * P.out_c >> 3; off + 4 <= P.ld_out; off += 4) *reinterpret_cast<uint32_t*>(o + off) = 0u;
+}
+
 // Requantizing epilogue of 16 rows x 64 columns, a thread's share two rows x 16 consecutive columns.
 template <int KIND, bool SMALL, bool PACKED>
 __device__ __forceinline__ void direct_codes(const GemmParams& P, const uint32_t (&v)[32], const CodeParams<KIND == EK_REQUANT_GELU>& cp,
                                              int lane, long long row0, int rows_valid, int n0) {
     const int r = lane >> 2, q = lane & 3;
-    const f32x2 magic = f2_dup(12582912.0f), qp2 = f2_dup(P.out_qp);
-    const float qn = P.out_qn, qp = P.out_qp;
     uint32_t w[2][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const float4 a = cp.a[k], b = cp.b[k];
-        float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (KIND == EK_REQUANT_GELU) g4 = cp.q[k];
+        const float4 g4 = KIND == EK_REQUANT_GELU ? cp.q[KIND == EK_REQUANT_GELU ? k : 0] : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {                           // rows r and r + 8
-            uint32_t c[4];
-#pragma unroll
-            for (int p = 0; p < 2; ++p) {                       // columns 4k + 2p, 4k + 2p + 1 of the thread's sixteen
-                const int i = 8 * k + 4 * p + 2 * h;
-                const f32x2 y = f2_fma(acc_to_float2<SMALL, PACKED>(v[i], v[i + 1], P.shift), p ? f2_pack(a.z, a.w) : f2_pack(a.x, a.y),
-                                       p ? f2_pack(b.z, b.w) : f2_pack(b.x, b.y));
-                float y0, y1, c0, c1;
-                f2_unpack(y, y0, y1);
-                if (KIND == EK_REQUANT_GELU) {
-                    // unsigned codes: the value arrives clamped to [0, 1] in units of Qp, and a negative y is code 0 whatever
-                    // its GELU: t = 0 there, the term is 1 and 2w - w = w < 0 saturates to 0
-                    float e0, e1, w0, w1, d0, d1;
-                    gelu_erfc_term2_pos(y0, y1, e0, e1);
-                    const f32x2 wq = f2_mul(y, p ? f2_pack(g4.z, g4.w) : f2_pack(g4.x, g4.y));
-                    f2_unpack(wq, w0, w1);
-                    f2_unpack(f2_add(wq, wq), d0, d1);
-                    const float u0 = __saturatef(fmaf(-w0, e0, d0)), u1 = __saturatef(fmaf(-w1, e1, d1));
-                    f2_unpack(f2_fma(f2_pack(u0, u1), qp2, magic), c0, c1);
-                } else {
-                    f2_unpack(f2_add(f2_pack(fminf(fmaxf(y0, qn), qp), fminf(fmaxf(y1, qn), qp)), magic), c0, c1);
-                }
-                c[2 * p] = __float_as_uint(c0);                 // the code in two's complement is the low byte
-                c[2 * p + 1] = __float_as_uint(c1);
-            }
-            w[h][k] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
-        }
+        for (int h = 0; h < 2; ++h)                             // rows r and r + 8, columns 4k .. 4k + 3 of the thread's sixteen
+            w[h][k] = direct_quad<KIND, SMALL, PACKED>(P, v[8 * k + 2 * h], v[8 * k + 2 * h + 1], v[8 * k + 4 + 2 * h], v[8 * k + 5 + 2 * h],
+                                                       cp.a[k], cp.b[k], g4);
     }
     const int col = n0 + 16 * q;
     uint8_t* const o = (uint8_t*)P.out + (row0 + r) * P.ld_out + ((col * P.out_c) >> 3);
@@ -361,7 +388,7 @@ __device__ __forceinline__ void direct_tile(const GemmParams& P, int tile, int& 
     } else {
         m_tile = tile / P.n_tiles;
         col_t = (tile - m_tile * P.n_tiles) * P.bn;
-        cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;                       // whole blocks
+        cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;                       // whole blocks, but for the tile at ragged_col
     }
 }
 
@@ -431,6 +458,15 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
 
     if (warp == WARP_TMA_D) {
         {
+            // Weights of a tile: permuted within column blocks, or in their own order
+            auto load_weights = [&](uint32_t dst, uint32_t bar, int byte, int col) {
+                bool ordered = false;
+                if constexpr (KIND == EK_QKV_NORM) ordered = col < 2 * P.norm_dim;
+                else if constexpr (KIND != EK_DEQUANT) ordered = col >= P.ragged_col;
+                if constexpr (KIND != EK_DEQUANT)
+                    if (ordered) { ptx::tma_load_4d(dst, &X.map_w, bar, byte, col, 0, 0); return; }
+                ptx::tma_load_5d(dst, &map_b, bar, byte, 0, 0, 0, col / BLK);
+            };
             int loaded = 0;                                                    // K blocks of the first tile whose weights are on their way
             if (early) {
                 int m_tile, col_t, cols;
@@ -440,10 +476,11 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     for (int kb = 0; kb < loaded; ++kb) {
                         const uint32_t bar = ptx::smem_addr(&bars.full[kb]);
                         ptx::mbar_arrive_expect_tx(bar, stage_bytes);
-                        ptx::tma_load_5d(smem_base + (uint32_t)kb * stage_bytes + P.ia_bytes, &map_b, bar, kb * BK, 0, 0, 0, col_t / BLK);
+                        load_weights(smem_base + (uint32_t)kb * stage_bytes + P.ia_bytes, bar, kb * BK, col_t);
                     }
                     // (by the CTAs of the first row tiles: all row tiles share them)
-                    for (int kb = loaded; m_tile < 2 && kb < P.k_blocks; ++kb) ptx::tma_prefetch_5d(&map_b, kb * BK, 0, 0, 0, col_t / BLK);
+                    if (m_tile < 2 && (KIND == EK_DEQUANT || col_t < P.ragged_col))
+                        for (int kb = loaded; kb < P.k_blocks; ++kb) ptx::tma_prefetch_5d(&map_b, kb * BK, 0, 0, 0, col_t / BLK);
                 }
                 __syncwarp();
                 dependency();
@@ -460,7 +497,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             for (int tile = blockIdx.x; ok && tile < P.total_tiles; tile += gridDim.x) {
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, tile, m_tile, col_t, cols);
-                const int m0 = m_tile * BM, blk0 = col_t / BLK;
+                const int m0 = m_tile * BM;
                 for (int kb = 0; kb < k_blocks; ++kb, ++it) {
                     const uint32_t full = full0 + 8u * (uint32_t)s;
                     uint32_t a_dst = dst, b_dst = dst + P.ia_bytes, a_bar = full, b_bar = full;
@@ -481,12 +518,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     __syncwarp();
                     if (ptx::elect_one()) {
                         ptx::tma_load_4d(a_dst, &map_a, a_bar, kb * a_step, m0, 0, 0);
-                        if constexpr (KIND == EK_QKV_NORM) {
-                            if (col_t < 2 * P.norm_dim) ptx::tma_load_4d(b_dst, &X.map_w, b_bar, kb * b_step, col_t, 0, 0);
-                            else ptx::tma_load_5d(b_dst, &map_b, b_bar, kb * b_step, 0, 0, 0, blk0);
-                        } else {
-                            if (it >= loaded) ptx::tma_load_5d(b_dst, &map_b, b_bar, kb * b_step, 0, 0, 0, blk0);
-                        }
+                        if (it >= loaded) load_weights(b_dst, b_bar, kb * b_step, col_t);
                     }
                     __syncwarp();
                     if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_bytes;
@@ -629,6 +661,10 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, tile, m_tile, col_t, cols);
                 if (col_t < 2 * P.norm_dim) my_slot = tid_e;                  // Q and K: columns in order
+            } else if (KIND != EK_DEQUANT && P.ragged_col != INT_MAX) {
+                int m_tile, col_t, cols;
+                direct_tile<KIND>(P, tile, m_tile, col_t, cols);
+                if (col_t >= P.ragged_col) my_slot = tid_e;
             }
             epi_params.a[buf][my_slot] = a;
             epi_params.b[buf][my_slot] = b;
@@ -729,7 +765,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     if (RES) request_residual(res[1]);
                 }
             } else {
-                bool norm = false;
+                bool norm = false;                                            // the tile's weights are in their own order
                 if constexpr (KIND == EK_QKV_NORM) {
                     norm = col_t < 2 * P.norm_dim;                            // a Q or K tile
 #pragma unroll 1
@@ -738,6 +774,12 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                                                         col_t >= P.norm_dim ? 1 : 0, row_q + lane, lane < rows_q, col_t + blk * 64);
                 }
                 constexpr int CK = KIND == EK_QKV_NORM ? EK_REQUANT : KIND;
+                if constexpr (KIND != EK_QKV_NORM) {
+                    norm = col_t >= P.ragged_col;                             // not walked by blocks either
+#pragma unroll 1
+                    for (int c = 16 * slice; norm && c < cols; c += 16 * SLICES)
+                        direct_codes_row<CK, SMALL, PACKED>(P, t_quarter + (uint32_t)c, epi_params, buf, c, row_q + lane, lane < rows_q, col_t + c);
+                }
                 // One 16-row half of a block at a time: 90 registers, so that sixteen warps fit.  (Eight warps that keep the
                 // parameters of a block for both halves and read the next accumulators ahead: fc1 79 us against 72.)
 #pragma unroll 1
@@ -785,12 +827,17 @@ int make_map_permuted(CUtensorMap* map, const void* base, uint64_t row_bytes, ui
     return r == CUDA_SUCCESS ? VITINT_OK : VITINT_ERR_CUDA;
 }
 
-// Which calls this kernel takes: whole column blocks, no batch of problems, and for fp32 outputs 32-byte aligned rows of the
-// output and the residual.  Everything else stays with gemm_i8_kernel.
+// Which calls this kernel takes: codes of at least a column block, fp32 outputs of whole column blocks whose rows, and the residual's,
+// lie on 32 bytes, no batch of problems.  Everything else stays with gemm_i8_kernel.
 bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_major) {
     if (n_inner != 1 || n_outer != 1 || b_mn_major) return false;
     if (P.kind == EK_QKV_NORM) return true;
-    if (P.kind == EK_REQUANT || (P.kind == EK_REQUANT_GELU && P.unit_out)) return P.N % 64 == 0;
+    if (P.kind == EK_REQUANT || (P.kind == EK_REQUANT_GELU && P.unit_out)) {
+        // A ragged width takes a second tensor map, 0.4 us of the host's time, which a small call waits for longer than for the GPU
+        // (with a quantizer in front, 1015 x 320 -> 1290 14.0 / 14.7 us, 197 x 768 -> 1000 14.1 / 14.8) unless it is recorded; larger
+        // ones gain: 12,608 x 768 -> 1290 33.9 -> 29.4 us, 50,000 x 256 -> 70 22.4 -> 20.9, recorded 1015 x 320 -> 1290 6.8 -> 4.4.
+        return P.N % 64 == 0 || (P.N >= 64 && (parameters_at_rest() || (long long)P.M * P.N * P.K > 800ll * 1000 * 1000));
+    }
     if (P.kind != EK_DEQUANT || P.N % 32 != 0) return false;
     // A short contraction whose residual and output exceed L2 is bound by HBM, and gemm_i8_kernel's asynchronous copies of the
     // residual through shared memory keep more of it in flight.  This kernel against that one, rotating buffers, residual and
@@ -853,6 +900,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     }
     P.ns_i = ns;
     P.ns_p = ns_p;
+    P.ragged_col = P.kind != EK_DEQUANT && P.N % block != 0 ? (P.n_tiles - 1) * P.bn : INT_MAX;
     P.at_rest = !packed && P.kind != EK_QKV_NORM && parameters_at_rest() ? 1 : 0;
     uint32_t cols = 32;
     while (cols < 2u * (uint32_t)P.bn) cols <<= 1;
@@ -883,20 +931,24 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     auto by_operands = [&](auto small) -> int {
         constexpr bool S = decltype(small)::value;
         constexpr int s0 = S ? 0 : 10;
-        if (P.kind == EK_QKV_NORM) {
-            NormExtra extra;
+        OrderExtra extra{};
+        if (P.kind == EK_QKV_NORM || P.ragged_col != INT_MAX) {
             if (int rc = make_map(&extra.map_w, w, w_row_bytes, (uint64_t)P.N, 1, 1, w_pitch, w_pitch * P.N, w_pitch * P.N,
                                   P.b_direct ? (uint32_t)BK : 16u * P.cb, (uint32_t)P.bn, P.b_direct != 0))
                 return rc;
+        }
+        if (P.kind == EK_QKV_NORM)
             return packed ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, true>, s0 + 8, extra)
                           : launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false>, s0 + 9, extra);
-        }
         if (P.kind == EK_DEQUANT) {
             if (packed) return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, true>, s0) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, true>, s0 + 1);
             return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, false>, s0 + 2) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, false>, s0 + 3);
         }
-        if (P.kind == EK_REQUANT) return packed ? launch(gemm_direct_kernel<EK_REQUANT, S, false, true>, s0 + 4) : launch(gemm_direct_kernel<EK_REQUANT, S, false, false>, s0 + 5);
-        return packed ? launch(gemm_direct_kernel<EK_REQUANT_GELU, S, false, true>, s0 + 6) : launch(gemm_direct_kernel<EK_REQUANT_GELU, S, false, false>, s0 + 7);
+        if (P.kind == EK_REQUANT)
+            return packed ? launch_with(gemm_direct_kernel<EK_REQUANT, S, false, true>, s0 + 4, extra)
+                          : launch_with(gemm_direct_kernel<EK_REQUANT, S, false, false>, s0 + 5, extra);
+        return packed ? launch_with(gemm_direct_kernel<EK_REQUANT_GELU, S, false, true>, s0 + 6, extra)
+                      : launch_with(gemm_direct_kernel<EK_REQUANT_GELU, S, false, false>, s0 + 7, extra);
     };
     return P.small_acc ? by_operands(std::true_type{}) : by_operands(std::false_type{});
 }

@@ -53,6 +53,33 @@ def test_linear_direct_epilogues(M, K, N, bits):
     assert ((q >= lo) & (q <= hi)).all() and padding_is_zero(g)
 
 
+# ---- codes of a width that is no multiple of the column block: one column into a block, around sixteen columns, one short of a
+# ---- block, a last tile of several blocks, several tiles a CTA; below a block gemm_i8_kernel
+@pytest.mark.parametrize("M,K,N", [(1, 64, 65), (129, 48, 63), (300, 144, 79), (197, 256, 80), (70, 128, 127), (197, 320, 200), (600, 768, 1290),
+                                   (5000, 128, 1290), (2600, 64, 2306)])
+@pytest.mark.parametrize("bits,packed", [(2, False), (4, False), (8, False), (4, True), (2, True)])
+def test_linear_codes_of_ragged_width(M, K, N, bits, packed):
+    qx, qw = rand_codes(121 + M, (M, K), bits, True), rand_codes(122 + N, (N, K), bits, True)
+    form = to_codes if packed else byte_codes
+    x, w = form(qx, bits, True), form(qw, bits, True)
+    acc = vo.matmul_i32(qx, qw)
+    s_w = ((np.abs(si.normal(123, (N,), 0.0, 0.2)) + 0.5) / max(float(np.abs(acc).mean()), 1.0)).astype(np.float32)
+    bias = si.normal(124, (N,), 0.0, 0.3)
+    alpha = s_w * np.float32(2 ** (bits - 1))
+    for cont, pitch in ((8, None), (0, None), (8, (N + 15) // 16 * 16 + 48)):
+        out = vt.Codes.empty(M, N, bits, True, container=cont, pitch=pitch)
+        out.data.fill_(0xA5)
+        vt.vitint_linear(x, 1.0, w, None, None, vt.Epilogue(mode=vt.EPI_REQUANT, alpha=dev(alpha), beta=dev(bias), out_bits=bits,
+                                                            out_signed=True, out_container=cont), out=out)
+        assert np.array_equal(from_codes(out), vo.epilogue_requant(acc, alpha, bias, bits, True)) and padding_is_zero(out)
+    inv = np.full(N, (2 ** bits - 1) / 1.5, np.float32)
+    g = vt.vitint_linear(x, 1.0, w, dev(s_w), dev(bias), vt.Epilogue(mode=vt.EPI_REQUANT, act=1, inv_out_step=dev(inv), out_bits=bits,
+                                                                    out_signed=False, out_container=8))
+    _, lo, hi = vo.epilogue_gelu_requant(acc, 1.0, s_w, bias, inv, bits, False, GELU_TOL_REL)
+    q = from_codes(g)
+    assert ((q >= lo) & (q <= hi)).all() and padding_is_zero(g)
+
+
 @pytest.mark.parametrize("M,N", [(16300, 768), (16250, 768)])
 def test_linear_fp32_dispatch_boundary(M, N):
     """Around the size from which a short contraction with a residual takes the staged fp32 epilogue."""
