@@ -50,6 +50,7 @@ struct GemmParams {
     int a_direct, b_direct;            // operand already int8: TMA writes the operand ring itself
     int reorder;                       // gemm_direct_kernel: both operands packed alike, unpacked in the cheaper order of k
     int small_acc;                     // |acc| < 2^22: int -> float without a conversion instruction
+    int b_resident;                    // gemm_direct_kernel, both operands packed: a CTA keeps its columns' expanded weights
     int ragged_col;                    // gemm_direct_kernel, codes: column of the tile that ends inside a column block, or INT_MAX
     int at_rest;                       // gemm_direct_kernel, byte-stored operands: weights and parameters may be read before the wait
     int unit_out;                      // GELU + unsigned requantization: the GELU multiplier carries 1/Qp and values clamp to [0, 1]

@@ -36,6 +36,7 @@ namespace vitint {
 namespace {
 
 constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
+constexpr uint32_t GD_RESIDENT_BYTES = 218u * 1024u;          // rings and resident weights of packed operands
 // Epilogue, unpack, TMA and MMA warps.  Eighteen warps leave a thread 96 registers; the norm kind, whose threads hold a head's
 // 64 channels, takes twelve epilogue warps (three heads of a 192-column tile for each lane quarter) and 128 registers.
 constexpr int GD_UNPACK_WARPS = 8;
@@ -410,8 +411,10 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t* const smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
-    const uint32_t stage_bytes = P.ia_bytes + P.ib_bytes;
+    const bool resident = PACKED && P.b_resident;
+    const uint32_t stage_bytes = P.ia_bytes + (resident ? 0u : P.ib_bytes);
     const uint32_t packed_off = (uint32_t)P.ns_i * stage_bytes, stage_packed = P.pa_bytes + P.pb_bytes;     // packed operands' ring
+    const uint32_t resident_off = packed_off + (uint32_t)P.ns_p * stage_packed;
     volatile int* abort_ptr = &abort_flag;
 
     if (threadIdx.x == 0) {
@@ -504,7 +507,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     if (PACKED) {
                         if (!mbar_wait_warp(ptx::smem_addr(&bars.p_empty[sp]), php, abort_ptr)) { ok = false; break; }
                         const uint32_t p_full = ptx::smem_addr(&bars.p_full[sp]), p_dst = smem_base + packed_off + (uint32_t)sp * stage_packed;
-                        if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(p_full, stage_packed);
+                        if (ptx::elect_one()) ptx::mbar_arrive_expect_tx(p_full, resident && tile != (int)blockIdx.x ? P.pa_bytes : stage_packed);
                         if (!P.a_direct) { a_dst = p_dst; a_bar = p_full; }
                         if (!P.b_direct) { b_dst = p_dst + P.pa_bytes; b_bar = p_full; }
                         if (++sp == P.ns_p) { sp = 0; php ^= 1u; }
@@ -518,7 +521,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     __syncwarp();
                     if (ptx::elect_one()) {
                         ptx::tma_load_4d(a_dst, &map_a, a_bar, kb * a_step, m0, 0, 0);
-                        if (it >= loaded) load_weights(b_dst, b_bar, kb * b_step, col_t);
+                        if (it >= loaded && (!resident || tile == (int)blockIdx.x)) load_weights(b_dst, b_bar, kb * b_step, col_t);
                     }
                     __syncwarp();
                     if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_bytes;
@@ -545,7 +548,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             VT_TRACER(tr, lane == 0 ? 1 : -1);
             VT_STAMP(tr, TT_START);
             const uint64_t a_desc0 = ptx::smem_desc(smem_base, 16, 1024, ptx::SWIZZLE_128B);
-            const uint64_t b_desc0 = ptx::smem_desc(smem_base + P.ia_bytes, 16, 1024, ptx::SWIZZLE_128B);
+            const uint64_t b_desc0 = ptx::smem_desc(smem_base + (resident ? resident_off : P.ia_bytes), 16, 1024, ptx::SWIZZLE_128B);
             const uint64_t stage_step = (uint64_t)(stage_bytes >> 4);        // descriptor address field counts 16-byte units
             const uint32_t full0 = ptx::smem_addr(&bars.full[0]), empty0 = ptx::smem_addr(&bars.empty[0]);
             const int k_blocks = P.k_blocks, ns = P.ns_i;
@@ -564,6 +567,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 VT_STAMP(tr, TT_GOT_EMPTY);
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)buf * acc_stride;
+                if (resident) b_desc = b_desc0;
                 for (int kb = 0; kb < k_blocks; ++kb) {
                     VT_STAMP(tr, TT_WAIT_FULL);
                     if (!mbar_wait_warp(full0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
@@ -582,8 +586,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                         ptx::mma_commit(empty0 + 8u * (uint32_t)s);
                     }
                     __syncwarp();
-                    if (++s == ns) { s = 0; ph ^= 1u; a_desc = a_desc0; b_desc = b_desc0; }
-                    else { a_desc += stage_step; b_desc += stage_step; }
+                    if (resident) b_desc += (uint64_t)(P.ib_bytes >> 4);
+                    if (++s == ns) { s = 0; ph ^= 1u; a_desc = a_desc0; if (!resident) b_desc = b_desc0; }
+                    else { a_desc += stage_step; if (!resident) b_desc += stage_step; }
                 }
                 if (ok && ptx::elect_one()) ptx::mma_commit(ptx::smem_addr(&bars.acc_full[buf]));
                 VT_STAMP(tr, TT_ISSUED);
@@ -612,7 +617,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             const uint8_t* pa = smem_gen + packed_off + (size_t)sp * stage_packed;
             uint8_t* ia = smem_gen + (size_t)s * stage_bytes;
             if (!P.a_direct) direct_unpack(P.ca, P.a_signed, P.reorder, pa, ia, BM, tid_u);
-            if (!P.b_direct) direct_unpack(P.cb, P.b_signed, P.reorder, pa + P.pa_bytes, ia + P.ia_bytes, P.bn, tid_u);
+            if (!P.b_direct && (!resident || tile == (int)blockIdx.x))
+                direct_unpack(P.cb, P.b_signed, P.reorder, pa + P.pa_bytes, resident ? smem_gen + resident_off + (size_t)kb * P.ib_bytes : ia + P.ia_bytes,
+                              P.bn, tid_u);
             ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
@@ -874,22 +881,50 @@ int direct_tile_columns(const GemmParams& P) {
     return best;
 }
 
+// Both operands bit-packed alike: what a K block costs is shared-memory traffic, three passes (packed in, packed out, expanded in)
+// over each expanded operand and the tensor core's reads of both.  A CTA whose tiles lie in one column of tiles can expand their
+// weights once and keep them: per K block 384 + columns cycles instead of 3 (128 + columns).  Returns the tile width where that
+// is the cheaper way (0: nowhere): the weights fit beside two operand slots and two packed ones, and the grid, a whole number of CTAs
+// for each column of tiles, wastes less than is won.  12,608 x 768 -> 3072 requantized (with the quantizer in front) 58.9 -> 49.3 us,
+// 25,216 x 768 -> 2304 90.9 -> 78.4, 6304 x 768 -> 2000 34.5 -> 23.3 (with the ragged width); one tile a CTA gains nothing.
+int resident_tile_columns(const GemmParams& P, int bn0) {
+    const int block = gd_block(P.kind), sms = sm_count();
+    const long long tiles0 = (long long)P.m_tiles * ((P.N + bn0 - 1) / bn0);
+    if (tiles0 <= sms) return 0;
+    // fp32 results are half bound by HBM: 12,608 x 384 -> 384 (0.76 of the cycles) gains, 25,216 x 768 -> 768 (0.83) is level
+    long long best_t = (tiles0 + sms - 1) / sms * 3 * (128 + bn0) * (P.kind == EK_DEQUANT ? 80 : 95) / 100;
+    int best = 0;
+    for (int bn = MAX_BN; bn >= block; bn -= block) {
+        const int n_tiles = (P.N + bn - 1) / bn;
+        const uint32_t need = 2u * P.ia_bytes + 2u * (P.pa_bytes + (uint32_t)(bn * 16 * P.cb)) + (uint32_t)(P.k_blocks * bn * BK);
+        if (n_tiles > sms || need > GD_RESIDENT_BYTES) continue;
+        const long long per_column = sms / n_tiles, rounds = (P.m_tiles + per_column - 1) / per_column, t = rounds * (384 + bn) + 2 * bn;
+        if (t < best_t) { best_t = t; best = bn; }
+    }
+    return best;
+}
+
 int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_bytes, uint64_t w_pitch, GemmParams P,
                        cudaStream_t st) {
     const int block = gd_block(P.kind);
     const bool packed = !P.a_direct || !P.b_direct;
+    const bool alike = !P.a_direct && !P.b_direct && P.ca == P.cb;
     P.bn = direct_tile_columns(P);
+    const int resident_bn = alike && P.kind != EK_QKV_NORM ? resident_tile_columns(P, P.bn) : 0;
+    P.b_resident = resident_bn != 0 ? 1 : 0;
+    if (resident_bn) P.bn = resident_bn;
     P.n_tiles = P.kind == EK_QKV_NORM ? 3 * ((P.norm_dim + P.bn - 1) / P.bn) : (P.N + P.bn - 1) / P.bn;
     const long long tiles = (long long)P.m_tiles * P.n_tiles;
     if (tiles > 0x7fffffffll) return VITINT_ERR_UNSUPPORTED;
     P.total_tiles = (int)tiles;
     P.ib_bytes = (uint32_t)P.bn * BK;
     P.pb_bytes = P.b_direct ? 0u : (uint32_t)P.bn * 16u * (uint32_t)P.cb;
-    const uint32_t stage = P.ia_bytes + P.ib_bytes, stage_p = P.pa_bytes + P.pb_bytes;
-    const uint32_t ring = GD_RING_BYTES - (P.kind == EK_QKV_NORM ? 8u * 1024u : 0u);     // beside 12 KB of static reference tables
+    const uint32_t kept = P.b_resident ? (uint32_t)P.k_blocks * P.ib_bytes : 0u;
+    const uint32_t stage = P.ia_bytes + (P.b_resident ? 0u : P.ib_bytes), stage_p = P.pa_bytes + P.pb_bytes;
+    const uint32_t ring = P.b_resident ? GD_RESIDENT_BYTES - kept : GD_RING_BYTES - (P.kind == EK_QKV_NORM ? 8u * 1024u : 0u);     // beside 12 KB of static reference tables
     int ns, ns_p = 0;
     if (packed) {
-        P.reorder = !P.a_direct && !P.b_direct && P.ca == P.cb ? 1 : 0;
+        P.reorder = alike ? 1 : 0;
         ns = 3;
         while (ns > 2 && (uint32_t)ns * stage + 2u * stage_p > ring) --ns;
         ns_p = (int)((ring - (uint32_t)ns * stage) / stage_p);
@@ -907,12 +942,13 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     P.tmem_cols = cols;
     CUtensorMap map_b;
     if (int rc = make_map_permuted(&map_b, w, w_row_bytes, (uint64_t)P.N, w_pitch, block, P.bn, P.b_direct ? 8 : P.cb)) return rc;
-    size_t smem = (size_t)ns * stage + (size_t)ns_p * stage_p + 1024;
+    size_t smem = (size_t)ns * stage + (size_t)ns_p * stage_p + kept + 1024;
     if (smem < 120 * 1024) smem = 120 * 1024;                  // two CTAs never share an SM (and its tensor memory)
     int grid = sm_count();
+    if (P.b_resident) grid = grid / P.n_tiles * P.n_tiles;     // tile + grid lies in the same column of tiles
     if (grid > P.total_tiles) grid = P.total_tiles;
 #ifdef VITINT_TRACE
-    if (g_trace_max_ctas > 0 && grid > g_trace_max_ctas) grid = g_trace_max_ctas;
+    if (g_trace_max_ctas > 0 && grid > g_trace_max_ctas && !P.b_resident) grid = g_trace_max_ctas;
 #endif
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
@@ -920,7 +956,8 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     const int threads = gd_threads(P.kind, packed);
     auto launch_with = [&](auto kernel, int slot, const auto& extra) -> int {
         if (!attr_set[dev][slot]) {
-            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring + 1024) != cudaSuccess)
+            if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     (int)(P.kind == EK_QKV_NORM || !packed ? GD_RING_BYTES : GD_RESIDENT_BYTES) + 1024) != cudaSuccess)
                 return VITINT_ERR_CUDA;
             attr_set[dev][slot] = true;
         }

@@ -80,6 +80,21 @@ def test_linear_codes_of_ragged_width(M, K, N, bits, packed):
     assert ((q >= lo) & (q <= hi)).all() and padding_is_zero(g)
 
 
+# ---- packed operands, many row tiles: CTAs that keep their columns' expanded weights, with K blocks of one to six, partial last
+# ---- K blocks, a ragged last tile of columns; and few row tiles, which expand as they go
+@pytest.mark.parametrize("M,K,N", [(300, 256, 576), (9000, 64, 576), (14001, 200, 192), (20000, 640, 200), (14000, 768, 384), (20000, 96, 1152)])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_linear_packed_many_rows(M, K, N, bits):
+    qx, qw = rand_codes(131 + M, (M, K), bits, True), rand_codes(132 + N, (N, K), bits, True)
+    x, w, acc = to_codes(qx, bits, True), to_codes(qw, bits, True), vo.matmul_i32(qx, qw)
+    s_w = ((np.abs(si.normal(133, (N,), 0.0, 0.2)) + 0.5) / max(float(np.abs(acc).mean()), 1.0)).astype(np.float32)
+    bias, alpha = si.normal(134, (N,), 0.0, 0.3), s_w * np.float32(2 ** (bits - 1))
+    out = vt.vitint_linear(x, 1.0, w, None, None, vt.Epilogue(mode=vt.EPI_REQUANT, alpha=dev(alpha), beta=dev(bias), out_bits=bits, out_signed=True))
+    assert np.array_equal(from_codes(out), vo.epilogue_requant(acc, alpha, bias, bits, True)) and padding_is_zero(out)
+    y = vt.vitint_linear(x, 0.75, w, dev(s_w), dev(bias), vt.Epilogue(mode=vt.EPI_DEQUANT_F32))
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), vo.epilogue_dequant(acc, np.float32(0.75), s_w, bias, None).view(np.uint32))
+
+
 @pytest.mark.parametrize("M,N", [(16300, 768), (16250, 768)])
 def test_linear_fp32_dispatch_boundary(M, N):
     """Around the size from which a short contraction with a residual takes the staged fp32 epilogue."""
