@@ -54,9 +54,9 @@ def test_linear_direct_epilogues(M, K, N, bits):
 
 
 # ---- codes of a width that is no multiple of the column block: one column into a block, around sixteen columns, one short of a
-# ---- block, a last tile of several blocks, several tiles a CTA; below a block gemm_i8_kernel
+# ---- block, a last tile of several blocks, several tiles a CTA; below a block, and where there is little to do, gemm_i8_kernel
 @pytest.mark.parametrize("M,K,N", [(1, 64, 65), (129, 48, 63), (300, 144, 79), (197, 256, 80), (70, 128, 127), (197, 320, 200), (600, 768, 1290),
-                                   (5000, 128, 1290), (2600, 64, 2306)])
+                                   (5000, 128, 1290), (2600, 64, 2306), (13000, 1000, 65), (5200, 2000, 79), (20100, 320, 127)])
 @pytest.mark.parametrize("bits,packed", [(2, False), (4, False), (8, False), (4, True), (2, True)])
 def test_linear_codes_of_ragged_width(M, K, N, bits, packed):
     qx, qw = rand_codes(121 + M, (M, K), bits, True), rand_codes(122 + N, (N, K), bits, True)
@@ -163,7 +163,7 @@ def test_layer_plan_equals_its_launches(kw):
     assert torch.equal(odd, one_by_one(layer, x)) and not torch.equal(odd, out)
 
 
-@pytest.mark.parametrize("batch,mlp", [(1, 320), (1, 1024), (3, 2176), (60, 512)])
+@pytest.mark.parametrize("batch,mlp", [(1, 320), (1, 330), (1, 1024), (3, 2176), (60, 512), (60, 1290)])
 def test_plan_sees_weights_written_in_place_right_before_it(batch, mlp):
     """Recorded kernels read weights and parameters ahead of the kernel in front of them, never ahead of the stream: copies into
     the layer's own tensors and runs in turn, nothing between them.  (MLP widths whose weights fill the ring of fc2 and exceed it.)"""
