@@ -32,11 +32,12 @@
 #include "ptx.cuh"
 #include "tile_ops.cuh"
 
+#include "gemm_resident.cuh"
+
 namespace vitint {
 namespace {
 
 constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
-constexpr uint32_t GD_RESIDENT_BYTES = 218u * 1024u;          // rings and resident weights of packed operands
 // Epilogue, unpack, TMA and MMA warps.  Eighteen warps leave a thread 96 registers; the norm kind, whose threads hold a head's
 // 64 channels, takes twelve epilogue warps (three heads of a 192-column tile for each lane quarter) and 128 registers.
 constexpr int GD_UNPACK_WARPS = 8;
@@ -881,36 +882,14 @@ int direct_tile_columns(const GemmParams& P) {
     return best;
 }
 
-// Both operands bit-packed alike: what a K block costs is shared-memory traffic, three passes (packed in, packed out, expanded in)
-// over each expanded operand and the tensor core's reads of both.  A CTA whose tiles lie in one column of tiles can expand their
-// weights once and keep them: per K block 384 + columns cycles instead of 3 (128 + columns).  Returns the tile width where that
-// is the cheaper way (0: nowhere): the weights fit beside two operand slots and two packed ones, and the grid, a whole number of CTAs
-// for each column of tiles, wastes less than is won.  12,608 x 768 -> 3072 requantized (with the quantizer in front) 58.9 -> 49.3 us,
-// 25,216 x 768 -> 2304 90.9 -> 78.4, 6304 x 768 -> 2000 34.5 -> 23.3 (with the ragged width); one tile a CTA gains nothing.
-int resident_tile_columns(const GemmParams& P, int bn0) {
-    const int block = gd_block(P.kind), sms = sm_count();
-    const long long tiles0 = (long long)P.m_tiles * ((P.N + bn0 - 1) / bn0);
-    if (tiles0 <= sms) return 0;
-    // fp32 results are half bound by HBM: 12,608 x 384 -> 384 (0.76 of the cycles) gains, 25,216 x 768 -> 768 (0.83) is level
-    long long best_t = (tiles0 + sms - 1) / sms * 3 * (128 + bn0) * (P.kind == EK_DEQUANT ? 80 : 95) / 100;
-    int best = 0;
-    for (int bn = MAX_BN; bn >= block; bn -= block) {
-        const int n_tiles = (P.N + bn - 1) / bn;
-        const uint32_t need = 2u * P.ia_bytes + 2u * (P.pa_bytes + (uint32_t)(bn * 16 * P.cb)) + (uint32_t)(P.k_blocks * bn * BK);
-        if (n_tiles > sms || need > GD_RESIDENT_BYTES) continue;
-        const long long per_column = sms / n_tiles, rounds = (P.m_tiles + per_column - 1) / per_column, t = rounds * (384 + bn) + 2 * bn;
-        if (t < best_t) { best_t = t; best = bn; }
-    }
-    return best;
-}
-
 int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_bytes, uint64_t w_pitch, GemmParams P,
                        cudaStream_t st) {
     const int block = gd_block(P.kind);
     const bool packed = !P.a_direct || !P.b_direct;
     const bool alike = !P.a_direct && !P.b_direct && P.ca == P.cb;
     P.bn = direct_tile_columns(P);
-    const int resident_bn = alike && P.kind != EK_QKV_NORM ? resident_tile_columns(P, P.bn) : 0;
+    const int resident_bn = alike && P.kind != EK_QKV_NORM
+        ? resident_tile_columns(sm_count(), P.m_tiles, P.k_blocks, P.N, P.cb, block, P.bn, P.kind == EK_DEQUANT) : 0;
     P.b_resident = resident_bn != 0 ? 1 : 0;
     if (resident_bn) P.bn = resident_bn;
     P.n_tiles = P.kind == EK_QKV_NORM ? 3 * ((P.norm_dim + P.bn - 1) / P.bn) : (P.N + P.bn - 1) / P.bn;
@@ -919,7 +898,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     P.total_tiles = (int)tiles;
     P.ib_bytes = (uint32_t)P.bn * BK;
     P.pb_bytes = P.b_direct ? 0u : (uint32_t)P.bn * 16u * (uint32_t)P.cb;
-    const uint32_t kept = P.b_resident ? (uint32_t)P.k_blocks * P.ib_bytes : 0u;
+    const uint32_t kept = P.b_resident ? (uint32_t)P.k_blocks * P.ib_bytes : 0u;       // (the plan keeps it below GD_RESIDENT_BYTES)
     const uint32_t stage = P.ia_bytes + (P.b_resident ? 0u : P.ib_bytes), stage_p = P.pa_bytes + P.pb_bytes;
     const uint32_t ring = P.b_resident ? GD_RESIDENT_BYTES - kept : GD_RING_BYTES - (P.kind == EK_QKV_NORM ? 8u * 1024u : 0u);     // beside 12 KB of static reference tables
     int ns, ns_p = 0;
