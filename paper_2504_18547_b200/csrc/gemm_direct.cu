@@ -38,8 +38,8 @@ namespace vitint {
 namespace {
 
 constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
-// Epilogue, unpack, TMA and MMA warps.  Eighteen warps leave a thread 96 registers; the norm kind, whose threads hold a head's
-// 64 channels, takes twelve epilogue warps (three heads of a 192-column tile for each lane quarter) and 128 registers.
+// Epilogue warps of a group, unpack, TMA and MMA warps.  Eighteen warps leave a thread 96 registers; the norm kind takes groups
+// of twelve epilogue warps, one for each lane quarter and head of a 192-column tile (two groups: 26 warps, 72 registers).
 constexpr int GD_UNPACK_WARPS = 8;
 __host__ __device__ constexpr int gd_epi_warps(int kind, bool packed) { return packed ? 16 - GD_UNPACK_WARPS : kind == EK_QKV_NORM ? 12 : 16; }
 // Groups of epilogue warps.  The norm kind has two, each with an accumulator buffer of its own: a thread's walk through Eq. 5 is a
@@ -706,9 +706,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             }
         };
         if constexpr (KIND == EK_QKV_NORM) {
-            // read by every epilogue warp after the first tile's group barrier
+            // laid out once for all groups, which meet before any of them reads it
             const int nt = (1 << P.norm_bits) - 1;
-            for (int i = tid_e; i < 2 * 64; i += EPI_W * 32) {
+            for (int i = threadIdx.x; i < 2 * 64; i += GROUPS * EPI_W * 32) {
                 const int set = i >> 6, c = i & 63;
                 const float* r = P.norm_refs + (size_t)i * nt;
                 float* const dst = norm_tab[0].ref[set][c];
@@ -721,6 +721,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 norm_tab[0].guess[set][c] = make_float4(inv * sgn / (float)nt, (0.5f - rho0 * inv) / (float)nt, sgn, 0.0f);
                 if (set == 0) norm_tab[0].step[c] = make_float2((float)(c + 1), __frcp_rn((float)(c + 1)));
             }
+            asm volatile("bar.sync 1, %0;" ::"n"(GROUPS * EPI_W * 32) : "memory");
         }
         if (KIND == EK_DEQUANT && RES) {
             request_residual(res[0]);

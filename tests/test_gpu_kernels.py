@@ -594,6 +594,32 @@ def test_qkv_norm_tiles_and_references(M, heads, bits, packed):
         assert np.array_equal(from_codes(got), np.concatenate(want, axis=1)) and padding_is_zero(got)
 
 
+@pytest.mark.parametrize("M,heads,bits", [(1, 1, 3), (130, 3, 3), (2600, 7, 4), (6500, 7, 3), (12000, 4, 2)])
+def test_qkv_norm_statistics_and_codes_of_both_groups(M, heads, bits):
+    """No second tile in a CTA (the second group of epilogue warps has none), then one to six tiles: every Q and K head's
+    statistics, and its codes, which read tables that all groups share."""
+    D, K = 64 * heads, 64
+    qx, qw = rand_codes(481 + M, (M, K), bits, True), rand_codes(482, (3 * D, K), bits, True)
+    s_w = (np.abs(si.normal(483, (3 * D,), 0.0, 0.01)) + 1e-3).astype(np.float32)
+    bias = si.normal(484, (3 * D,), 0.0, 0.05)
+    y = vo.epilogue_dequant(vo.matmul_i32(qx, qw), np.float32(0.5), s_w, bias)
+    rf = [compare_case(2, 64, bits, 490 + k) for k in range(2)]
+    got, stats = vt.vitint_linear_qkv_norm(byte_codes(qx, bits, True), 0.5, byte_codes(qw, bits, True), dev(s_w), dev(bias),
+                                           dev(np.stack([r for _, r, _, _ in rf])), dev(np.stack([f for _, _, f, _ in rf])), rf[0][3],
+                                           dev(np.full(D, 0.3, np.float32)), None, bits)
+    codes, stats = from_codes(got), stats.cpu().numpy()
+    for k, (_, r, f, n_eps) in enumerate(rf):
+        x = y[:, k * D:(k + 1) * D].reshape(M * heads, 64)
+        assert np.array_equal(codes[:, k * D:(k + 1) * D].reshape(M * heads, 64), compare_reference(x, r, f, n_eps, bits))
+        mu, s = np.zeros(len(x), np.float32), np.zeros(len(x), np.float32)
+        for i in range(64):
+            delta = x[:, i] - mu
+            mu = mu + delta / np.float32(i + 1)
+            s = s + delta * (x[:, i] - mu)
+        assert np.array_equal(stats[k, :, 0].view(np.uint32), mu.view(np.uint32))
+        assert np.array_equal(stats[k, :, 1].view(np.uint32), (s + np.float32(n_eps)).view(np.uint32))
+
+
 # ---- fused attention core: every remainder of the column walk, a quantizer step whose unclamped codes exceed 16 bits -------
 @pytest.mark.parametrize("tokens", [1, 7, 8, 9, 31, 33, 63, 64, 72, 128, 129, 160, 192, 200, 225, 255, 256, 257, 320, 415])
 @pytest.mark.parametrize("bits,p_scale", [(4, 1.0), (2, 1.0), (4, 1e-5)])
