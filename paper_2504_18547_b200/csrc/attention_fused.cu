@@ -287,6 +287,11 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
         const int tid_g = (warp % WARPS) * 32 + lane;               // within the group
         const int row = wq * 32 + lane;                             // query row of the tile
         double* const zx = reinterpret_cast<double*>(ggen + P.off_z);   // partial row sums, [H][128]
+        // An fp64 row sum depends in its last bit on the order of its terms, so both forms keep the same partial sums: pairs of
+        // threads `pair` = 0, 1 have the even and the odd chunks, and where a row has four threads the two of a pair share the
+        // interleaved sums of one thread of the other form between them.  A row's codes are the same in a batch of any size.
+        const int pair = hf & 1, share = hf >> 1;
+        auto row_sum = [&]() { return H == 2 ? zx[row] + zx[128 + row] : (zx[row] + zx[256 % (H * 128) + row]) + (zx[128 + row] + zx[384 % (H * 128) + row]); };
         const uint32_t t_row = tmem_grp + ((uint32_t)(wq * 32) << 16);
         const char* const ring = reinterpret_cast<const char*>(smem_gen + P.off_table);
         const uint32_t ring_mask = 8u * (uint32_t)P.smax - 4u;
@@ -525,7 +530,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 // exp(t_j - max) by reduction and polynomial, row sum in fp64, p = e / Z with 1/Z as two floats, one exact division
                 // by s_P
                 const f32x2 nmx2 = f2_dup(-__fmul_rn((float)smx, P.scale));
-                double zp[2] = {0.0, 0.0};
+                double zp[H == 2 ? 2 : 1] = {};
                 auto exp_pair = [&](uint32_t& a, uint32_t& b, bool va, bool vb) {
                     const f32x2 sf = f2_add(f2_pack(__uint_as_float(0x4B400000u + a), __uint_as_float(0x4B400000u + b)), nmagic2);   // |S| <= 2^20
                     float e0, e1;
@@ -534,11 +539,39 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     b = vb ? __float_as_uint(e1) : 0u;
                     // the doubles from the bits; a zero becomes 2^-127, which a sum of at least 1 does not see
                     zp[0] += __hiloint2double((int)((a >> 3) + 0x38000000u), (int)(a << 29));
-                    zp[1] += __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+                    zp[H == 2 ? 1 : 0] += __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
                 };
-                if (warp_live) {
+                if (H == 4 && warp_live) {
+                    // a thread of two in place of one that has the chunk in the other form: the even or the odd columns
+                    const uint32_t t_own = t_row + (uint32_t)share;
 #pragma unroll 1
-                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 2 * H - 1 : 1) {     // halves of the thread's chunks
+                    for (int pc = 2 * pair; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {           // halves of the pair's chunks
+                        uint32_t v[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) ptx::tmem_ld1(t_own + (uint32_t)(pc * 16 + 2 * i), v[i]);
+                        ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 8; i += 2) exp_pair(v[i], v[i + 1], true, true);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) ptx::tmem_st1(t_own + (uint32_t)(pc * 16 + 2 * i), v[i]);
+                    }
+#pragma unroll 1
+                    for (int k = (pair - full_chunks) & 1; k < tail_blocks; k += 2) {
+                        const uint32_t t_blk = t_own + (uint32_t)(full_chunks * 32 + k * 8);
+                        uint32_t v[4];
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) ptx::tmem_ld1(t_blk + (uint32_t)(2 * i), v[i]);
+                        ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 4; i += 2) exp_pair(v[i], v[i + 1], 8 * k + 2 * i + share < tail, 8 * k + 2 * i + 2 + share < tail);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) ptx::tmem_st1(t_blk + (uint32_t)(2 * i), v[i]);
+                    }
+                    ptx::tmem_st_wait();
+                }
+                if (H == 2 && warp_live) {
+#pragma unroll 1
+                    for (int pc = 2 * hf; pc < 2 * full_chunks; pc += (pc & 1) ? 3 : 1) {             // halves of the thread's chunks
                         uint32_t v[16];
                         ptx::tmem_ld16(t_row + (uint32_t)(pc * 16), v);
                         ptx::tmem_ld_wait();
@@ -557,13 +590,14 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                     }
                     ptx::tmem_st_wait();
                 }
-                zx[hf * 128 + row] = zp[0] + zp[1];
+                zx[hf * 128 + row] = H == 2 ? zp[0] + zp[H == 2 ? 1 : 0] : zp[0];
+                if constexpr (H == 4) ptx::tc_fence_before();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
                 w = mbar_wait(ptx::smem_addr(&B.z_sync), 1u, abort_ptr);
                 if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-                double z = zx[row] + zx[128 + row];
-                if constexpr (H == 4) z += zx[256 + row] + zx[384 + row];
+                if constexpr (H == 4) ptx::tc_fence_after();         // pass 2 reads exponentials that other warps have stored
+                const double z = row_sum();
                 const double r0 = (double)__frcp_rn((float)z), rz = r0 * (2.0 - z * r0);
                 const float rzh = (float)rz, rzl = (float)(rz - (double)(float)rz);
                 const f32x2 rzh2 = f2_dup(rzh), rzl2 = f2_dup(rzl), dr2 = f2_dup(p_div.r), ndb2 = f2_dup(-p_div.b);
@@ -621,42 +655,83 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
             } else {
             // pass 1: e_j = EXP[S_j], row sum in fp64, e_j parked in TMEM over S_j; whole chunks of 32 columns, then the tail
             // by blocks of eight (197 tokens: 200 columns walked instead of 224)
-            double zp[4] = {0.0, 0.0, 0.0, 0.0};
+            double zsum = 0.0;
             if (warp_live) {
-                // sixteen columns are looked up while the next sixteen are on their way
                 uint32_t v0[16], v1[16];
-                if (hf < full_chunks) ptx::tmem_ld16(t_row + (uint32_t)(hf * 32), v0);
+                if constexpr (H == 2) {
+                    // sixteen columns are looked up while the next sixteen are on their way
+                    double zp[4] = {0.0, 0.0, 0.0, 0.0};
+                    if (hf < full_chunks) ptx::tmem_ld16(t_row + (uint32_t)(hf * 32), v0);
 #pragma unroll 1
-                for (int ch = hf; ch < full_chunks; ch += H) {
-                    const uint32_t t_ch = t_row + (uint32_t)(ch * 32);
-                    ptx::tmem_ld_wait();
-                    ptx::tmem_ld16(t_ch + 16, v1);
-                    exp_lookup<16, !DIRECT, false>(v0, ring, ring_mask, sh_idx, 16, zp);
-                    ptx::tmem_st16(t_ch, v0);
-                    ptx::tmem_ld_wait();
-                    if (ch + H < full_chunks) ptx::tmem_ld16(t_ch + 32 * H, v0);
-                    exp_lookup<16, !DIRECT, false>(v1, ring, ring_mask, sh_idx, 16, zp);
-                    ptx::tmem_st16(t_ch + 16, v1);
-                }
+                    for (int ch = hf; ch < full_chunks; ch += H) {
+                        const uint32_t t_ch = t_row + (uint32_t)(ch * 32);
+                        ptx::tmem_ld_wait();
+                        ptx::tmem_ld16(t_ch + 16, v1);
+                        exp_lookup<16, !DIRECT, false>(v0, ring, ring_mask, sh_idx, 16, zp);
+                        ptx::tmem_st16(t_ch, v0);
+                        ptx::tmem_ld_wait();
+                        if (ch + H < full_chunks) ptx::tmem_ld16(t_ch + 32 * H, v0);
+                        exp_lookup<16, !DIRECT, false>(v1, ring, ring_mask, sh_idx, 16, zp);
+                        ptx::tmem_st16(t_ch + 16, v1);
+                    }
 #pragma unroll 1
-                for (int k = tail0; k < tail_blocks; k += H) {
-                    uint32_t v[8];
-                    ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
-                    ptx::tmem_ld_wait();
-                    exp_lookup<8, !DIRECT, true>(v, ring, ring_mask, sh_idx, tail - 8 * k, zp);
-                    ptx::tmem_st8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                    for (int k = tail0; k < tail_blocks; k += H) {
+                        uint32_t v[8];
+                        ptx::tmem_ld8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                        ptx::tmem_ld_wait();
+                        exp_lookup<8, !DIRECT, true>(v, ring, ring_mask, sh_idx, tail - 8 * k, zp);
+                        ptx::tmem_st8(t_row + (uint32_t)(full_chunks * 32 + k * 8), v);
+                    }
+                    zsum = (zp[0] + zp[1]) + (zp[2] + zp[3]);
+                } else {
+                    // a thread of two in place of one that has the chunk in the other form: two of every four columns
+                    double zp[2] = {0.0, 0.0};
+                    const uint32_t t_own = t_row + (uint32_t)(2 * share);
+                    auto load = [&](int ch, uint32_t (&v)[16]) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) ptx::tmem_ld2(t_own + (uint32_t)(ch * 32 + 4 * i), v[2 * i], v[2 * i + 1]);
+                    };
+                    auto entries = [&](int ch, uint32_t (&v)[16]) {
+                        exp_lookup<16, !DIRECT, false>(v, ring, ring_mask, sh_idx, 32, zp);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) ptx::tmem_st2(t_own + (uint32_t)(ch * 32 + 4 * i), v[2 * i], v[2 * i + 1]);
+                    };
+                    if (pair < full_chunks) load(pair, v0);
+#pragma unroll 1
+                    for (int ch = pair; ch < full_chunks; ch += 4) {
+                        ptx::tmem_ld_wait();
+                        if (ch + 2 < full_chunks) load(ch + 2, v1);
+                        entries(ch, v0);
+                        if (ch + 2 < full_chunks) {
+                            ptx::tmem_ld_wait();
+                            if (ch + 4 < full_chunks) load(ch + 4, v0);
+                            entries(ch + 2, v1);
+                        }
+                    }
+#pragma unroll 1
+                    for (int k = (pair - full_chunks) & 1; k < tail_blocks; k += 2) {
+                        const uint32_t t_blk = t_own + (uint32_t)(full_chunks * 32 + k * 8);
+                        uint32_t v[4];
+                        ptx::tmem_ld2(t_blk, v[0], v[1]);
+                        ptx::tmem_ld2(t_blk + 4, v[2], v[3]);
+                        ptx::tmem_ld_wait();
+                        exp_lookup<4, !DIRECT, true>(v, ring, ring_mask, sh_idx, tail - 8 * k - 2 * share, zp);
+                        ptx::tmem_st2(t_blk, v[0], v[1]);
+                        ptx::tmem_st2(t_blk + 4, v[2], v[3]);
+                    }
+                    zsum = zp[0] + zp[1];
                 }
                 ptx::tmem_st_wait();
             }
-            // the row's two threads add their partial sums (every warp takes part in the barrier)
-            double z = (zp[0] + zp[1]) + (zp[2] + zp[3]);
-            zx[hf * 128 + row] = z;
+            // the row's threads add their partial sums (every warp takes part in the barrier)
+            zx[hf * 128 + row] = zsum;
+            if constexpr (H == 4) ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(ptx::smem_addr(&B.z_sync));
             w = mbar_wait(ptx::smem_addr(&B.z_sync), ph, abort_ptr);
             if (!__all_sync(0xffffffffu, w)) { ok = false; break; }
-            z = zx[row] + zx[128 + row];
-            if constexpr (H == 4) z += zx[256 + row] + zx[384 + row];
+            if constexpr (H == 4) ptx::tc_fence_after();             // pass 2 reads entries that other warps have stored
+            const double z = row_sum();
             // r = 1 / (Z * s_P) as a two-float number: e * r then carries the quantizer argument p / s_P to
             // about half an ulp, i.e. it is the exact-division result for a probability that differs from
             // RN(e / Z) by less than one ulp

@@ -132,19 +132,21 @@ __device__ __forceinline__ void fill_table_ring(float* ring, const float* __rest
 
 // v: scores s (SCALED: 4 s times 2^sh) -> the entries' bits; their fp64 sum goes into four interleaved partial sums (one would
 // chain N dependent additions).  MASKED: elements from n_valid on are no scores: entry 0, nothing added.
-template <int N, bool SCALED, bool MASKED>
-__device__ __forceinline__ void exp_lookup(uint32_t (&v)[N], const char* ring, uint32_t mask, int sh, int n_valid, double (&zp)[4]) {
+// Z = 2: v holds two of every four columns, and the sums are those two of the four that they belong to.
+template <int N, bool SCALED, bool MASKED, int Z>
+__device__ __forceinline__ void exp_lookup(uint32_t (&v)[N], const char* ring, uint32_t mask, int sh, int n_valid, double (&zp)[Z]) {
 #pragma unroll
     for (int i = 0; i < N; ++i) {
         const uint32_t off = (SCALED ? (uint32_t)((int)v[i] >> sh) : v[i] * 4u) & mask;
         uint32_t eb = *reinterpret_cast<const uint32_t*>(ring + off);
-        if (MASKED && i >= n_valid) eb = 0u;
+        const int column = Z == 4 ? i : 4 * (i >> 1) + (i & 1);
+        if (MASKED && column >= n_valid) eb = 0u;
         // an entry is a positive normal float: its double is put together from the bits, one instruction on the integer unit
         // and one on the multiplier (the conversion unit runs at a quarter of the fp64 adder's rate)
         const uint32_t hi = (eb >> 3) + 0x38000000u;
         uint32_t lo;
         asm("mul.lo.u32 %0, %1, 536870912;" : "=r"(lo) : "r"(eb));                    // eb << 29
-        zp[i & 3] += __hiloint2double(MASKED && i >= n_valid ? 0 : (int)hi, (int)lo);
+        zp[i & (Z - 1)] += __hiloint2double(MASKED && column >= n_valid ? 0 : (int)hi, (int)lo);
         v[i] = eb;
     }
 }
