@@ -466,21 +466,24 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_c
                 sigma = sx[row] + sx[128 + row];
                 if constexpr (H == 4) sigma += sx[256 + row] + sx[384 + row];
                 const float sig_f = __ull2float_rn(sigma);
-                // pass 2: the code is the number of references fl32(fl32((k - 1/2) s_P) * Sigma) that float(E_j) exceeds.
-                // k0 = rint(u), u = min(E_j / (s_P Sigma), Qp), is that number unless u lies within (Qp + 1) 2^-21 of some k - 1/2:
-                // u is off by less than 3.1 * 2^-24 of itself, a reference by less than 2.1 * 2^-24.  Columns that come that
-                // close are compared with the two references around them: k0' = rint(min(u, Qp - 3/4)) is at most one off and
-                // never Qp, code = k0' - 1 + [E > ref(k0')] + [E > ref(k0' + 1)], in the float that carries k0' in its mantissa.
+                // pass 2: the code is the number of references fl32(fl32((k - 1/2) s_P) * Sigma) that float(E_j) exceeds, which is
+                // k0 = rint(u), u = min(E_j / (s_P Sigma), Qp), unless u lies next to some k - 1/2: u is off by less than 3.1 units
+                // of 2^-24 of itself, a reference by less than 2.1.  An interval of 8 units on either side of u proves a code
+                // (197 tokens x 12 heads, batch 64: 44.7 -> 43.5 us against |u - rint(u)| compared with a limit; 198 x 6: 25.5 -> 24.9).
+                // Where it does not, values above the last level are kept there for a second look (the first one for a step below
+                // 1/65000: 57 us at 1e-5, as at other steps, where comparing all of them took 71), and columns still unproven are
+                // compared with the two references around them: k0' = rint(min(u, Qp - 3/4)) is at most one off and never Qp,
+                // code = k0' - 1 + [E > ref(k0')] + [E > ref(k0' + 1)], in the float that carries k0' in its mantissa.
                 const float inv = warp_live ? __frcp_rn(__fmul_rn(P.p_step, sig_f)) : 0.0f;
-                // references and reciprocal are off by 5 units of 2^-24 between them: a code is proven by an interval 8 wide on either side
-                // (197 tokens x 12 heads, batch 64: 44.7 -> 43.5 us against |u - rint(u)| compared with a limit; 198 x 6: 25.5 -> 24.9)
                 const f32x2 inv2 = f2_dup(inv), lo2 = f2_dup(inv * (1.0f - 4.76837158e-07f)), hi2 = f2_dup(inv * (1.0f + 4.76837158e-07f));
+                const float e_top = (P.p_qp + 1.0f) * __fmul_rn(P.p_step, sig_f);
                 auto codes = [&](const uint32_t* v, auto& wd, auto count) {
                     constexpr int N = decltype(count)::value;
                     f32x2 e[N / 2];
 #pragma unroll
                     for (int i = 0; i < N / 2; ++i) e[i] = f2_pack(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-                    if (__any_sync(0xffffffffu, quantize_interval<N>(e, lo2, hi2, qp2, wd) != 0.0f || steep)) {
+                    if ((steep || __any_sync(0xffffffffu, quantize_interval<N>(e, lo2, hi2, qp2, wd) != 0.0f)) &&
+                        __any_sync(0xffffffffu, quantize_interval_below<N>(e, e_top, lo2, hi2, qp2, wd) != 0.0f)) {
                         const float u_top = P.p_qp - 0.75f;
                         const f32x2 half2 = f2_dup(0.5f), nhalf2 = f2_dup(-0.5f), ps2 = f2_dup(P.p_step), sg2 = f2_dup(sig_f);
 #pragma unroll

@@ -5,8 +5,10 @@
 //   pass B   S_c again                        ->  codes = min(rint(EXP[S_j] / (Z s_P)), Qp)  ->  P_c in shared memory
 //            O += P_c V_c (tcgen05, accumulating in tensor memory across the chunks)
 // Pass A needs the table's exact entries.  Pass B only needs the level they lead to, and finds it from 2^(s c2 + log2 r) on the
-// special-function unit; blocks in which a score comes too close to a rounding boundary to be sure of take the table again
-// (577 tokens x 12 heads, batch 16: 91.7 us with |a - rint(a)| compared with a limit, 90.2 with two ends of an interval).
+// special-function unit; blocks in which a score comes too close to a rounding boundary to be sure of take the table again.
+// (Two ends of an interval as in the Eq. 4 core instead of |a - rint(a)| compared with a limit: an interval grows with a, and a
+// clamp costs what it saves.  785 tokens x 12 heads, batch 16: 162.9 us against 162.2, rows that peak at one token 163.0 against
+// 160.8, a step of 2e-5 172 against 161; 577 tokens 92.8 against 94.2.)
 // So the lookups -- 2.8 passes of the shared-memory pipe per 32 scores, what bounded the kernel with two a score -- are halved.
 // then O is requantized and stored.  S, the probabilities and P never reach HBM: the unfused sequence writes and
 // re-reads 4 T^2 bytes per head (946 MB at 785 tokens, batch 32), which is what bounds it.  The table makes the
@@ -188,8 +190,8 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         int b, h, qt;
         coords(item, b, h, qt);
         double zp[4] = {0.0, 0.0, 0.0, 0.0};
-        f32x2 rzh2 = f2_dup(0.0f), rzl2 = f2_dup(0.0f), l2 = f2_dup(0.0f), lo2 = f2_dup(0.0f), hi2 = f2_dup(0.0f);
-        float e_top = 0.0f;
+        f32x2 rzh2 = f2_dup(0.0f), rzl2 = f2_dup(0.0f), l2 = f2_dup(0.0f);
+        float limit = 0.0f, e_top = 0.0f;
         const bool warp_live = qt * 128 + wq * 32 < T;
         for (int pass = 0; ok && pass < 2; ++pass) {
             for (int c = 0; ok && c < P.n_chunks; ++c) {
@@ -240,7 +242,7 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                                 ptx::tmem_ld16(t_row + (uint32_t)(p16 * 16), v);
                                 ptx::tmem_ld_wait();
                                 bool sure = !steep && n_valid >= 16;
-                                if (sure) sure = quantize_scores<16>(v, c2, l2, lo2, hi2, qp2, wd);
+                                if (sure) sure = quantize_scores<16>(v, c2, l2, P.p_qp, limit, wd);
                                 if (!__all_sync(0xffffffffu, sure)) {
                                     double unused[4] = {0.0, 0.0, 0.0, 0.0};
                                     exp_lookup<16, false, true>(v, ring, ring_mask, 0, n_valid, unused);
@@ -300,9 +302,7 @@ attention_long_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     // and ln 2 times that, plus exp2's 2^-22, relative in the argument.
                     const float l = log2f(rzh);
                     l2 = f2_dup(l);
-                    const float eps = 1.25f * ((4.0f * fabsf(l) + 40.0f) * 4.1316e-8f + 2.4e-7f) + 1.2e-7f;     // and the rounding of 1 +- eps
-                    lo2 = f2_dup(1.0f - eps);
-                    hi2 = f2_dup(1.0f + eps);
+                    limit = 0.5f - (P.p_qp + 1.0f) * 1.25f * ((4.0f * fabsf(l) + 40.0f) * 4.1316e-8f + 2.4e-7f);
                 }
                 // the next step's scores (the last step of all: P V alone)
                 w = w && mbar_wait(ptx::smem_addr(&B.s_full), n_s & 1u, abort_ptr);

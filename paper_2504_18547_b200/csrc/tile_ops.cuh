@@ -198,23 +198,48 @@ __device__ __forceinline__ float quantize_interval(const f32x2 (&e)[N / 2], f32x
     return d0 + d1;
 }
 
-// The codes straight from the scores, without the table: a = 2^(s c2 + l), l = log2(1 / (Z s_P)), in fp32 with the hardware's
-// exp2.  a is the quantizer's own argument up to the relative error that the caller put between lo and hi around 1; false where
-// that leaves a code in doubt (about one score in 2^16), and the caller takes the table.
+// The interval grows with the value, so far beyond the last level it often holds a boundary although the code is Qp for certain.
+// The same once more, where the first look proved nothing, with values kept at `top`, about (Qp + 1) / r.
 template <int N>
-__device__ __forceinline__ bool quantize_scores(const uint32_t (&v)[N], f32x2 c2, f32x2 l2, f32x2 lo2, f32x2 hi2, uint32_t qp2, uint32_t (&w)[N / 4]) {
-    const f32x2 nmagic2 = f2_dup(-12582912.0f);
-    f32x2 a[N / 2];
+__device__ __forceinline__ float quantize_interval_below(const f32x2 (&e)[N / 2], float top, f32x2 lo2, f32x2 hi2, uint32_t qp2, uint32_t (&w)[N / 4]) {
+    f32x2 c[N / 2];
 #pragma unroll
     for (int i = 0; i < N / 2; ++i) {
-        const f32x2 s = f2_add(f2_pack(__uint_as_float(0x4B400000u + v[2 * i]), __uint_as_float(0x4B400000u + v[2 * i + 1])), nmagic2);
-        float t0, t1, a0, a1;
-        f2_unpack(f2_fma(s, c2, l2), t0, t1);
-        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a0) : "f"(t0));
-        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a1) : "f"(t1));
-        a[i] = f2_pack(a0, a1);
+        float a, b;
+        f2_unpack(e[i], a, b);
+        c[i] = f2_pack(fminf(a, top), fminf(b, top));
     }
-    return quantize_interval<N>(a, lo2, hi2, qp2, w) == 0.0f;
+    return quantize_interval<N>(c, lo2, hi2, qp2, w);
+}
+
+// The table's codes straight from the scores, without the table: a = 2^(s c2 + l), l = log2(1 / (Z s_P)), in fp32 with the
+// hardware's exp2.  a differs from the quantizer's own argument by a relative error below the bound that the caller turned
+// into `limit` (a little less than 1/2): where |a - rint(a)| stays below it both round to the same code, where it does not
+// (about one score in 2^14) the function returns false and the caller takes the table.
+template <int N>
+__device__ __forceinline__ bool quantize_scores(const uint32_t (&v)[N], f32x2 c2, f32x2 l2, float qp, float limit, uint32_t (&w)[N / 4]) {
+    const f32x2 magic2 = f2_dup(12582912.0f), nmagic2 = f2_dup(-12582912.0f), neg1 = f2_dup(-1.0f);
+    float dev = 0.0f;
+#pragma unroll
+    for (int i4 = 0; i4 < N / 4; ++i4) {
+        uint32_t c[4];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const f32x2 s = f2_add(f2_pack(__uint_as_float(0x4B400000u + v[4 * i4 + 2 * j]), __uint_as_float(0x4B400000u + v[4 * i4 + 2 * j + 1])), nmagic2);
+            float t0, t1, a0, a1, c0, c1, d0, d1;
+            f2_unpack(f2_fma(s, c2, l2), t0, t1);
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a0) : "f"(t0));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a1) : "f"(t1));
+            const f32x2 a = f2_pack(fminf(a0, qp), fminf(a1, qp)), m = f2_add(a, magic2);
+            f2_unpack(f2_fma(f2_add(m, nmagic2), neg1, a), d0, d1);
+            dev = fmaxf(dev, fmaxf(fabsf(d0), fabsf(d1)));
+            f2_unpack(m, c0, c1);
+            c[2 * j] = __float_as_uint(c0);
+            c[2 * j + 1] = __float_as_uint(c1);
+        }
+        w[i4] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+    }
+    return dev < limit;
 }
 
 // Requantizes N columns of an accumulator row (scaled by 2^sh; SMALL: |acc| < 2^22) to byte codes in two's complement:

@@ -768,6 +768,26 @@ def test_cores_with_codes_on_or_far_beyond_the_last_level(tokens, p_step):
     assert torch.equal(out, one_by_one(layer, x))
 
 
+@pytest.mark.parametrize("tokens", [33, 197, 256])
+@pytest.mark.parametrize("p_step", [1e-3, 1e-4, 2e-5, 1e-5])
+def test_shift_core_with_rows_that_peak(tokens, p_step):
+    """Keys equal to the queries: one probability near 1, thousands of steps above the last level, beside ones on every level."""
+    batch, D, bits, step = 2, 64, 4, np.float32(0.5)
+    qkv = rand_codes(970 + tokens, (batch * tokens, 3 * D), bits, True)
+    qkv[:, D:2 * D] = qkv[:, :D]
+    packed = to_codes(qkv, bits, True)
+    slabs = [vt.Slabs.of_qkv(packed, tokens, D, i) for i in range(3)]
+    alpha = dev(np.full(D, np.float32(0.02)))
+    c2 = np.float32(np.float64(vp.softmax_scale(step, step, 64)) * np.log2(np.e))
+    S = vt.vitint_qk(slabs[0], slabs[1], batch, 1, tokens)
+    P = vt.vitint_softmax_shift_quantize(S.view(batch * tokens, -1), tokens, c2, np.float32(p_step), bits)
+    assert (from_codes(P).max(axis=1) == 15).all()
+    want = from_codes(vt.vitint_pv(P, slabs[2], batch, 1, tokens, 1.0, 1.0, vt.Epilogue(mode=vt.EPI_REQUANT, alpha=alpha, out_bits=8, out_signed=True)))
+    got = vt.vitint_attention_core_shift(vt.vitint_widen(packed), batch, 1, tokens, step, step, np.float32(p_step), bits, alpha, None,
+                                         out=vt.Codes.empty(batch * tokens, D, 8, True))
+    assert np.array_equal(from_codes(got), want)
+
+
 @pytest.mark.parametrize("tokens", [1, 9, 40, 96, 129, 197, 225, 256])
 @pytest.mark.parametrize("bits,form", [(4, "byte"), (4, "packed"), (2, "packed"), (4, "shift"), (8, "layer")])
 def test_core_with_one_group_and_with_two(tokens, bits, form):
