@@ -93,10 +93,13 @@ struct LaunchRecorder {
 };
 inline thread_local LaunchRecorder* t_recorder = nullptr;
 
+// Whether launches are being recorded: their host time is then paid once, not at every run.
+inline bool launches_recorded() { return t_recorder != nullptr; }
+
 // Whether the launch being made may read its weights and parameters before grid_dependency_wait().  True inside a recorded
 // graph: no kernel of a stack writes them, the first kernel waits for all that the stream held before the graph, and a kernel's
 // CTAs start no earlier than the wait of the kernel in front has returned in every CTA.
-inline bool parameters_at_rest() { return t_recorder != nullptr; }
+inline bool parameters_at_rest() { return launches_recorded(); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,

@@ -61,11 +61,11 @@ __device__ __forceinline__ int gd_param_slot(int c) {
     return (c - w) + (i >> 2) * 16 + q * 4 + (i & 3);
 }
 
-// What only some kinds of epilogue need: the weights in their own order, for the norm kind's Q and K tiles and for a tile of codes
-// that ends inside a column block.
+// What only some kernels need: the weights in their own order, for the norm kind's Q and K tiles and for a tile of codes that ends
+// inside a column block (RAGGED).
 struct NoExtra { int unused; };
 struct OrderExtra { CUtensorMap map_w; };
-template <int KIND> using DirectExtra = std::conditional_t<KIND == EK_DEQUANT, NoExtra, OrderExtra>;
+template <int KIND, bool RAGGED> using DirectExtra = std::conditional_t<KIND == EK_QKV_NORM || RAGGED, OrderExtra, NoExtra>;
 
 struct DirectBars {
     uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], epi_sync[2], p_full[MAX_STAGES], p_empty[MAX_STAGES];
@@ -390,14 +390,16 @@ __device__ __forceinline__ void direct_tile(const GemmParams& P, int tile, int& 
     } else {
         m_tile = tile / P.n_tiles;
         col_t = (tile - m_tile * P.n_tiles) * P.bn;
-        cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;                       // whole blocks, but for the tile at ragged_col
+        cols = P.N - col_t < P.bn ? P.N - col_t : P.bn;                       // whole blocks, but for the last tile of a ragged width
     }
 }
 
-template <int KIND, bool SMALL, bool RES, bool PACKED>
+// RAGGED: codes of a width that is no multiple of the column block.  A variant of its own: with the choice made at run time and the
+// second tensor map passed to every launch, twelve layers on one image, none of them ragged, took 332 us instead of 328.
+template <int KIND, bool SMALL, bool RES, bool PACKED, bool RAGGED = false>
 __global__ void __launch_bounds__(gd_threads(KIND, PACKED), 1)
 gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                   const __grid_constant__ DirectExtra<KIND> X, const __grid_constant__ GemmParams P) {
+                   const __grid_constant__ DirectExtra<KIND, RAGGED> X, const __grid_constant__ GemmParams P) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ DirectBars bars;
     constexpr int GROUPS = gd_epi_groups(KIND, PACKED);
@@ -413,6 +415,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
     uint8_t* const smem_gen = smem_raw + (smem_base - ptx::smem_addr(smem_raw));
     const bool resident = PACKED && P.b_resident;
+    const int ragged_col = (P.n_tiles - 1) * P.bn;             // (RAGGED) column of the tile that ends inside a column block
     const uint32_t stage_bytes = P.ia_bytes + (resident ? 0u : P.ib_bytes);
     const uint32_t packed_off = (uint32_t)P.ns_i * stage_bytes, stage_packed = P.pa_bytes + P.pb_bytes;     // packed operands' ring
     const uint32_t resident_off = packed_off + (uint32_t)P.ns_p * stage_packed;
@@ -466,8 +469,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
             auto load_weights = [&](uint32_t dst, uint32_t bar, int byte, int col) {
                 bool ordered = false;
                 if constexpr (KIND == EK_QKV_NORM) ordered = col < 2 * P.norm_dim;
-                else if constexpr (KIND != EK_DEQUANT) ordered = col >= P.ragged_col;
-                if constexpr (KIND != EK_DEQUANT)
+                else if constexpr (RAGGED) ordered = col >= ragged_col;
+                if constexpr (KIND == EK_QKV_NORM || RAGGED)
                     if (ordered) { ptx::tma_load_4d(dst, &X.map_w, bar, byte, col, 0, 0); return; }
                 ptx::tma_load_5d(dst, &map_b, bar, byte, 0, 0, 0, col / BLK);
             };
@@ -483,7 +486,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                         load_weights(smem_base + (uint32_t)kb * stage_bytes + P.ia_bytes, bar, kb * BK, col_t);
                     }
                     // (by the CTAs of the first row tiles: all row tiles share them)
-                    if (m_tile < 2 && (KIND == EK_DEQUANT || col_t < P.ragged_col))
+                    if (m_tile < 2 && (!RAGGED || col_t < ragged_col))
                         for (int kb = loaded; kb < P.k_blocks; ++kb) ptx::tma_prefetch_5d(&map_b, kb * BK, 0, 0, 0, col_t / BLK);
                 }
                 __syncwarp();
@@ -669,10 +672,10 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, tile, m_tile, col_t, cols);
                 if (col_t < 2 * P.norm_dim) my_slot = tid_e;                  // Q and K: columns in order
-            } else if (KIND != EK_DEQUANT && P.ragged_col != INT_MAX) {
+            } else if (RAGGED) {
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, tile, m_tile, col_t, cols);
-                if (col_t >= P.ragged_col) my_slot = tid_e;
+                if (col_t >= ragged_col) my_slot = tid_e;
             }
             epi_params.a[buf][my_slot] = a;
             epi_params.b[buf][my_slot] = b;
@@ -783,8 +786,8 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                                                         col_t >= P.norm_dim ? 1 : 0, row_q + lane, lane < rows_q, col_t + blk * 64);
                 }
                 constexpr int CK = KIND == EK_QKV_NORM ? EK_REQUANT : KIND;
-                if constexpr (KIND != EK_QKV_NORM) {
-                    norm = col_t >= P.ragged_col;                             // not walked by blocks either
+                if constexpr (RAGGED) {
+                    norm = col_t >= ragged_col;                               // not walked by blocks either
 #pragma unroll 1
                     for (int c = 16 * slice; norm && c < cols; c += 16 * SLICES)
                         direct_codes_row<CK, SMALL, PACKED>(P, t_quarter + (uint32_t)c, epi_params, buf, c, row_q + lane, lane < rows_q, col_t + c);
@@ -845,7 +848,7 @@ bool direct_eligible(const GemmParams& P, int n_inner, int n_outer, int b_mn_maj
         // A ragged width takes a second tensor map, 0.4 us of the host's time, which a small call waits for longer than for the GPU
         // (with a quantizer in front, 1015 x 320 -> 1290 14.0 / 14.7 us, 197 x 768 -> 1000 14.1 / 14.8) unless it is recorded; larger
         // ones gain: 12,608 x 768 -> 1290 33.9 -> 29.4 us, 50,000 x 256 -> 70 22.4 -> 20.9, recorded 1015 x 320 -> 1290 6.8 -> 4.4.
-        return P.N % 64 == 0 || (P.N >= 64 && (parameters_at_rest() || (long long)P.M * P.N * P.K > 800ll * 1000 * 1000));
+        return P.N % 64 == 0 || (P.N >= 64 && (launches_recorded() || (long long)P.M * P.N * P.K > 800ll * 1000 * 1000));
     }
     if (P.kind != EK_DEQUANT || P.N % 32 != 0) return false;
     // A short contraction whose residual and output exceed L2 is bound by HBM, and gemm_i8_kernel's asynchronous copies of the
@@ -891,7 +894,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     P.bn = direct_tile_columns(P);
     const int resident_bn = alike && P.kind != EK_QKV_NORM
         ? resident_tile_columns(sm_count(), P.m_tiles, P.k_blocks, P.N, P.cb, block, P.bn, P.kind == EK_DEQUANT) : 0;
-    P.b_resident = resident_bn != 0 ? 1 : 0;
+    P.b_resident = resident_bn != 0;
     if (resident_bn) P.bn = resident_bn;
     P.n_tiles = P.kind == EK_QKV_NORM ? 3 * ((P.norm_dim + P.bn - 1) / P.bn) : (P.N + P.bn - 1) / P.bn;
     const long long tiles = (long long)P.m_tiles * P.n_tiles;
@@ -904,7 +907,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     const uint32_t ring = P.b_resident ? GD_RESIDENT_BYTES - kept : GD_RING_BYTES - (P.kind == EK_QKV_NORM ? 8u * 1024u : 0u);     // beside 12 KB of static reference tables
     int ns, ns_p = 0;
     if (packed) {
-        P.reorder = alike ? 1 : 0;
+        P.reorder = alike;
         ns = 3;
         while (ns > 2 && (uint32_t)ns * stage + 2u * stage_p > ring) --ns;
         ns_p = (int)((ring - (uint32_t)ns * stage) / stage_p);
@@ -915,8 +918,8 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     }
     P.ns_i = ns;
     P.ns_p = ns_p;
-    P.ragged_col = P.kind != EK_DEQUANT && P.N % block != 0 ? (P.n_tiles - 1) * P.bn : INT_MAX;
-    P.at_rest = !packed && P.kind != EK_QKV_NORM && parameters_at_rest() ? 1 : 0;
+    const bool ragged = P.kind != EK_QKV_NORM && P.N % block != 0;
+    P.at_rest = !packed && P.kind != EK_QKV_NORM && parameters_at_rest();
     uint32_t cols = 32;
     while (cols < 2u * (uint32_t)P.bn) cols <<= 1;
     P.tmem_cols = cols;
@@ -932,7 +935,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
 #endif
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
-    static bool attr_set[MAX_DEVICES][20] = {};
+    static bool attr_set[MAX_DEVICES][28] = {};
     const int threads = gd_threads(P.kind, packed);
     auto launch_with = [&](auto kernel, int slot, const auto& extra) -> int {
         if (!attr_set[dev][slot]) {
@@ -947,25 +950,27 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     auto launch = [&](auto kernel, int slot) -> int { return launch_with(kernel, slot, NoExtra{}); };
     auto by_operands = [&](auto small) -> int {
         constexpr bool S = decltype(small)::value;
-        constexpr int s0 = S ? 0 : 10;
-        OrderExtra extra{};
-        if (P.kind == EK_QKV_NORM || P.ragged_col != INT_MAX) {
-            if (int rc = make_map(&extra.map_w, w, w_row_bytes, (uint64_t)P.N, 1, 1, w_pitch, w_pitch * P.N, w_pitch * P.N,
-                                  P.b_direct ? (uint32_t)BK : 16u * P.cb, (uint32_t)P.bn, P.b_direct != 0))
-                return rc;
-        }
-        if (P.kind == EK_QKV_NORM)
-            return packed ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, true>, s0 + 8, extra)
-                          : launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false>, s0 + 9, extra);
+        constexpr int s0 = S ? 0 : 14;
         if (P.kind == EK_DEQUANT) {
             if (packed) return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, true>, s0) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, true>, s0 + 1);
             return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, false>, s0 + 2) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, false>, s0 + 3);
         }
-        if (P.kind == EK_REQUANT)
-            return packed ? launch_with(gemm_direct_kernel<EK_REQUANT, S, false, true>, s0 + 4, extra)
-                          : launch_with(gemm_direct_kernel<EK_REQUANT, S, false, false>, s0 + 5, extra);
-        return packed ? launch_with(gemm_direct_kernel<EK_REQUANT_GELU, S, false, true>, s0 + 6, extra)
-                      : launch_with(gemm_direct_kernel<EK_REQUANT_GELU, S, false, false>, s0 + 7, extra);
+        if (P.kind == EK_QKV_NORM || ragged) {
+            OrderExtra extra;
+            if (int rc = make_map(&extra.map_w, w, w_row_bytes, (uint64_t)P.N, 1, 1, w_pitch, w_pitch * P.N, w_pitch * P.N,
+                                  P.b_direct ? (uint32_t)BK : 16u * P.cb, (uint32_t)P.bn, P.b_direct != 0))
+                return rc;
+            if (P.kind == EK_QKV_NORM)
+                return packed ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, true>, s0 + 8, extra)
+                              : launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false>, s0 + 9, extra);
+            if (P.kind == EK_REQUANT)
+                return packed ? launch_with(gemm_direct_kernel<EK_REQUANT, S, false, true, true>, s0 + 10, extra)
+                              : launch_with(gemm_direct_kernel<EK_REQUANT, S, false, false, true>, s0 + 11, extra);
+            return packed ? launch_with(gemm_direct_kernel<EK_REQUANT_GELU, S, false, true, true>, s0 + 12, extra)
+                          : launch_with(gemm_direct_kernel<EK_REQUANT_GELU, S, false, false, true>, s0 + 13, extra);
+        }
+        if (P.kind == EK_REQUANT) return packed ? launch(gemm_direct_kernel<EK_REQUANT, S, false, true>, s0 + 4) : launch(gemm_direct_kernel<EK_REQUANT, S, false, false>, s0 + 5);
+        return packed ? launch(gemm_direct_kernel<EK_REQUANT_GELU, S, false, true>, s0 + 6) : launch(gemm_direct_kernel<EK_REQUANT_GELU, S, false, false>, s0 + 7);
     };
     return P.small_acc ? by_operands(std::true_type{}) : by_operands(std::false_type{});
 }
