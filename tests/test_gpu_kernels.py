@@ -95,6 +95,21 @@ def test_linear_packed_many_rows(M, K, N, bits):
     assert np.array_equal(y.cpu().numpy().view(np.uint32), vo.epilogue_dequant(acc, np.float32(0.75), s_w, bias, None).view(np.uint32))
 
 
+@pytest.mark.parametrize("M,K,N,bits", [(14001, 200, 192, 4), (20000, 96, 1152, 2), (14000, 640, 384, 3)])
+def test_linear_packed_many_rows_with_a_residual(M, K, N, bits):
+    """Kept weights beside a residual that is read ahead; the residual may be the output buffer."""
+    qx, qw = rand_codes(141 + M, (M, K), bits, True), rand_codes(142 + N, (N, K), bits, True)
+    acc = vo.matmul_i32(qx, qw)
+    s_w, bias, res = (np.abs(si.normal(143, (N,), 0.0, 0.02)) + 1e-3).astype(np.float32), si.normal(144, (N,), 0.0, 0.3), si.normal(145, (M, N))
+    want = vo.epilogue_dequant(acc, np.float32(0.75), s_w, bias, res).view(np.uint32)
+    x, w = to_codes(qx, bits, True), to_codes(qw, bits, True)
+    r = dev(res)
+    epi = vt.Epilogue(mode=vt.EPI_DEQUANT_F32, residual=r)
+    assert np.array_equal(vt.vitint_linear(x, 0.75, w, dev(s_w), dev(bias), epi).cpu().numpy().view(np.uint32), want)
+    vt.vitint_linear(x, 0.75, w, dev(s_w), dev(bias), epi, out=r)
+    assert np.array_equal(r.cpu().numpy().view(np.uint32), want)
+
+
 @pytest.mark.parametrize("M,N", [(16300, 768), (16250, 768)])
 def test_linear_fp32_dispatch_boundary(M, N):
     """Around the size from which a short contraction with a residual takes the staged fp32 epilogue."""
@@ -187,6 +202,31 @@ def test_plan_sees_weights_written_in_place_right_before_it(batch, mlp):
             t.copy_(new)
         layers[0].forward(x, out)
     assert layers[0]._plan is not None
+    for i, out in enumerate(outs):
+        assert torch.equal(out, want[i & 1])
+
+
+@pytest.mark.parametrize("batch", [1, 60, 160])
+@pytest.mark.parametrize("packed", [False, True])
+def test_plan_sees_an_exp_table_written_in_place_right_before_it(batch, packed):
+    """The recorded attention core reads its table ahead of the kernel in front of it, never ahead of the stream: another score
+    scale's table and runs in turn, with items for one group of warps in a CTA and for two."""
+    from paper_2504_18547_b200.encoder import EncoderLayer
+    cfg = si.BlockConfig("table", batch, 50, 128, 2, 4, mlp_dim=320)
+    layer = EncoderLayer(batch, 50, 2, 320, 4, si.layer_parameters(cfg), wide_activations=not packed)
+    tables = [layer.attn_table.clone(), vt.vitint_attention_exp_table(4, 6 * layer.s_q, layer.s_k)]
+    x = dev(si.normal(360 + batch, (cfg.rows, cfg.dim)))
+    want = []
+    for t in tables:
+        layer.attn_table.copy_(t)
+        want.append(one_by_one(layer, x))
+    assert not torch.equal(want[0], want[1])
+    outs = [torch.empty_like(x) for _ in range(8)]
+    torch.cuda.synchronize()
+    for i, out in enumerate(outs):
+        layer.attn_table.copy_(tables[i & 1])
+        layer.forward(x, out)
+    assert layer._plan is not None
     for i, out in enumerate(outs):
         assert torch.equal(out, want[i & 1])
 
