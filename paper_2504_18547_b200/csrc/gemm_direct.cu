@@ -37,7 +37,6 @@
 namespace vitint {
 namespace {
 
-constexpr uint32_t GD_RING_BYTES = 200u * 1024u;
 // Epilogue warps of a group, unpack, TMA and MMA warps.  Eighteen warps leave a thread 96 registers; the norm kind takes groups
 // of twelve epilogue warps, one for each lane quarter and head of a 192-column tile (two groups: 26 warps, 72 registers).
 constexpr int GD_UNPACK_WARPS = 8;
@@ -893,7 +892,8 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     const bool alike = !P.a_direct && !P.b_direct && P.ca == P.cb;
     P.bn = direct_tile_columns(P);
     const int resident_bn = alike && P.kind != EK_QKV_NORM
-        ? resident_tile_columns(sm_count(), P.m_tiles, P.k_blocks, P.N, P.cb, block, P.bn, P.kind == EK_DEQUANT) : 0;
+        ? resident_tile_columns(sm_count(), P.m_tiles, P.k_blocks, P.N, P.cb, block, P.bn,
+                                P.kind == EK_DEQUANT ? PE_FP32 : P.kind == EK_REQUANT ? PE_REQUANT : PE_GELU) : 0;
     P.b_resident = resident_bn != 0;
     if (resident_bn) P.bn = resident_bn;
     P.n_tiles = P.kind == EK_QKV_NORM ? 3 * ((P.norm_dim + P.bn - 1) / P.bn) : (P.N + P.bn - 1) / P.bn;
