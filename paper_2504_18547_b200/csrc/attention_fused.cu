@@ -2,7 +2,7 @@
 // O = P V  ->  requantize, with S, the probabilities and P never leaving the SM.
 //
 // A persistent CTA runs TWO independent pipelines ("groups"), each with eight compute warps
-// (query row = TMEM lane, shared by two threads) and one control warp (TMA + MMA issue); while one
+// (query row = TMEM lane, two threads a row) and one control warp (TMA + MMA issue); while one
 // group's threads are busy with the softmax the other group's loads and MMAs proceed.  Where no CTA gets a second
 // item there is one group of sixteen warps, four threads a row.
 //

@@ -27,7 +27,9 @@
 // operands are packed alike the codes of a chunk keep the order in which masks and shifts produce them (the contraction does
 // not mind), 12 operations for 32 codes instead of 20 and their sign left in the high bits.  12,608 x 768 -> 3072 of 4-bit
 // packed codes, requantized: 81 -> 48 us (one group 63, two 58, reordered 48); 3072 -> 768 fp32 104 -> 52; 197 x 192 -> 576
-// 7.6 -> 4.3.  What is left above the byte-stored form (29 us) is the expansion: ALU and shared-memory traffic.
+// 7.6 -> 4.3.  Where a CTA keeps its columns' expanded weights (gemm_resident.cuh) only the activations are expanded tile by tile,
+// 48 -> 39 us, and the eight epilogue warps beside them bound it: issue slots 42 % busy, load/store data pipe 34 % (53 and 56 % when
+// both operands were expanded for every tile).  The byte-stored form takes 29 us.
 #include "common.cuh"
 #include "ptx.cuh"
 #include "tile_ops.cuh"

@@ -40,7 +40,7 @@ constexpr int LNS_MAX_COLS = 4096;
 // written between the operations of this element's dependent chain delta -> quotient -> mu, so the two
 // interleave in issue order; operands and operations are exactly those of the recurrence.
 //
-// RN(delta / i) = fma(delta, rh, RN(delta rl)): what is rounded last is within 2^-48 of the quotient, and a quotient of a 24-bit
+// RN(delta / i) = fma(delta, rh, RN(delta rl)): what is rounded last is within 2^-47 of the quotient, and a quotient of a 24-bit
 // number by an i <= 4096 is at least ulp / 2i = 2^-37 away from a rounding boundary (it cannot lie on one: the odd part of a
 // boundary times i has 25 bits or more) -- unless the product underflows: `tiny` keeps the smallest |delta| that is not 0, as bits
 // less 1, and a row that had one below 2^-100, or did not stay finite, is walked again by running_row_slow.
