@@ -43,11 +43,8 @@ namespace {
 // of twelve epilogue warps, one for each lane quarter and head of a 192-column tile (two groups: 26 warps, 72 registers).
 constexpr int GD_UNPACK_WARPS = 8;
 __host__ __device__ constexpr int gd_epi_warps(int kind, bool packed) { return packed ? 16 - GD_UNPACK_WARPS : kind == EK_QKV_NORM ? 12 : 16; }
-// Groups of epilogue warps.  The norm kind has two, each with an accumulator buffer of its own: a thread's walk through Eq. 5 is a
-// chain, three warps a scheduler leave half of its slots empty, and a second tile beside the first fills them.
-__host__ __device__ constexpr int gd_epi_groups(int kind, bool packed) { return kind == EK_QKV_NORM && !packed ? 2 : 1; }
-__host__ __device__ constexpr int gd_threads(int kind, bool packed) {
-    return (gd_epi_groups(kind, packed) * gd_epi_warps(kind, packed) + (packed ? GD_UNPACK_WARPS : 0) + 2) * 32;
+__host__ __device__ constexpr int gd_threads(int kind, bool packed, int groups = 1) {
+    return (groups * gd_epi_warps(kind, packed) + (packed ? GD_UNPACK_WARPS : 0) + 2) * 32;
 }
 
 // Column block within which the weight rows are permuted: column 2q + 8g + e of the tensor-core block is output column
@@ -397,20 +394,23 @@ __device__ __forceinline__ void direct_tile(const GemmParams& P, int tile, int& 
 
 // RAGGED: codes of a width that is no multiple of the column block.  A variant of its own: with the choice made at run time and the
 // second tensor map passed to every launch, twelve layers on one image, none of them ragged, took 332 us instead of 328.
-template <int KIND, bool SMALL, bool RES, bool PACKED, bool RAGGED = false>
-__global__ void __launch_bounds__(gd_threads(KIND, PACKED), 1)
+// GROUPS of epilogue warps.  The norm kind has two where CTAs have several tiles, each with an accumulator buffer of its own: a thread's
+// walk through Eq. 5 is a chain, three warps a scheduler leave half of its slots empty, and a second tile beside the first fills
+// them (12,672 x 384 -> 1152 31 -> 27.5 us).  Without a second tile 832 threads only start later than 448: 198 x 64 6.7 us with two
+// groups, 6.2 with one.
+template <int KIND, bool SMALL, bool RES, bool PACKED, bool RAGGED = false, int GROUPS = 1>
+__global__ void __launch_bounds__(gd_threads(KIND, PACKED, GROUPS), 1)
 gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                    const __grid_constant__ DirectExtra<KIND, RAGGED> X, const __grid_constant__ GemmParams P) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ DirectBars bars;
-    constexpr int GROUPS = gd_epi_groups(KIND, PACKED);
     __shared__ __align__(16) EpiParams epi_params_of[GROUPS];
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
     __shared__ __align__(16) std::conditional_t<KIND == EK_QKV_NORM, NormTables, float4> norm_tab[1];
     constexpr int BLK = gd_block(KIND);
     constexpr int EPI_W = gd_epi_warps(KIND, PACKED), SLICES = EPI_W / 4;
-    constexpr int WARP_TMA_D = gd_threads(KIND, PACKED) / 32 - 2, WARP_MMA_D = WARP_TMA_D + 1;
+    constexpr int WARP_TMA_D = gd_threads(KIND, PACKED, GROUPS) / 32 - 2, WARP_MMA_D = WARP_TMA_D + 1;
 
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_base = (ptx::smem_addr(smem_raw) + 1023u) & ~1023u;
@@ -725,7 +725,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 norm_tab[0].guess[set][c] = make_float4(inv * sgn / (float)nt, (0.5f - rho0 * inv) / (float)nt, sgn, 0.0f);
                 if (set == 0) norm_tab[0].step[c] = make_float2((float)(c + 1), __frcp_rn((float)(c + 1)));
             }
-            asm volatile("bar.sync 1, %0;" ::"n"(GROUPS * EPI_W * 32) : "memory");
+            if constexpr (GROUPS > 1) asm volatile("bar.sync 1, %0;" ::"n"(GROUPS * EPI_W * 32) : "memory");
         }
         if (KIND == EK_DEQUANT && RES) {
             request_residual(res[0]);
@@ -937,8 +937,9 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
 #endif
     const int dev = current_device();
     if (dev < 0) return VITINT_ERR_CUDA;
-    static bool attr_set[MAX_DEVICES][28] = {};
-    const int threads = gd_threads(P.kind, packed);
+    static bool attr_set[MAX_DEVICES][30] = {};
+    const int groups = P.kind == EK_QKV_NORM && !packed && P.total_tiles > grid ? 2 : 1;
+    const int threads = gd_threads(P.kind, packed, groups);
     auto launch_with = [&](auto kernel, int slot, const auto& extra) -> int {
         if (!attr_set[dev][slot]) {
             if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -952,7 +953,7 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
     auto launch = [&](auto kernel, int slot) -> int { return launch_with(kernel, slot, NoExtra{}); };
     auto by_operands = [&](auto small) -> int {
         constexpr bool S = decltype(small)::value;
-        constexpr int s0 = S ? 0 : 14;
+        constexpr int s0 = S ? 0 : 15;
         if (P.kind == EK_DEQUANT) {
             if (packed) return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, true>, s0) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, true>, s0 + 1);
             return P.residual ? launch(gemm_direct_kernel<EK_DEQUANT, S, true, false>, s0 + 2) : launch(gemm_direct_kernel<EK_DEQUANT, S, false, false>, s0 + 3);
@@ -963,8 +964,9 @@ int launch_gemm_direct(const CUtensorMap& map_a, const void* w, uint64_t w_row_b
                                   P.b_direct ? (uint32_t)BK : 16u * P.cb, (uint32_t)P.bn, P.b_direct != 0))
                 return rc;
             if (P.kind == EK_QKV_NORM)
-                return packed ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, true>, s0 + 8, extra)
-                              : launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false>, s0 + 9, extra);
+                return packed        ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, true>, s0 + 8, extra)
+                       : groups == 2 ? launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false, false, 2>, s0 + 9, extra)
+                                     : launch_with(gemm_direct_kernel<EK_QKV_NORM, S, false, false>, s0 + 14, extra);
             if (P.kind == EK_REQUANT)
                 return packed ? launch_with(gemm_direct_kernel<EK_REQUANT, S, false, true, true>, s0 + 10, extra)
                               : launch_with(gemm_direct_kernel<EK_REQUANT, S, false, false, true>, s0 + 11, extra);
