@@ -475,7 +475,9 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     if (ordered) { ptx::tma_load_4d(dst, &X.map_w, bar, byte, col, 0, 0); return; }
                 ptx::tma_load_5d(dst, &map_b, bar, byte, 0, 0, 0, col / BLK);
             };
-            int loaded = 0;                                                    // K blocks of the first tile whose weights are on their way
+            // K blocks of the first tile that are on their way before the loop, which a test for them would slow down in every call
+            // (12,608 x 384 -> 384 to fp32 7.0 -> 7.4 us)
+            int loaded = 0;
             if (early) {
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, blockIdx.x, m_tile, col_t, cols);
@@ -492,13 +494,18 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 }
                 __syncwarp();
                 dependency();
+                if (ptx::elect_one())
+                    for (int kb = 0; kb < loaded; ++kb)
+                        ptx::tma_load_4d(smem_base + (uint32_t)kb * stage_bytes, &map_a, ptx::smem_addr(&bars.full[kb]), kb * BK, m_tile * BM, 0, 0);
+                __syncwarp();
             }
             VT_TRACER(tr, lane == 0 ? 0 : -1);
             VT_STAMP(tr, TT_START);
             const uint32_t full0 = ptx::smem_addr(&bars.full[0]), empty0 = ptx::smem_addr(&bars.empty[0]);
             const int k_blocks = P.k_blocks, ns = P.ns_i;
-            int s = 0, it = 0, sp = 0;
-            uint32_t ph = 1u, dst = smem_base, php = 1u;
+            const bool wrapped = loaded == ns;
+            int s = wrapped ? 0 : loaded, it = loaded, sp = 0, kb0 = loaded;
+            uint32_t ph = wrapped ? 0u : 1u, dst = smem_base + (uint32_t)s * stage_bytes, php = 1u;
             bool ok = true;
             const uint32_t direct_bytes = PACKED ? (P.a_direct ? P.ia_bytes : 0u) + (P.b_direct ? P.ib_bytes : 0u) : stage_bytes;
             const int a_step = P.a_direct ? BK : 16 * P.ca, b_step = P.b_direct ? BK : 16 * P.cb;         // bytes of a row per K block
@@ -506,7 +513,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                 int m_tile, col_t, cols;
                 direct_tile<KIND>(P, tile, m_tile, col_t, cols);
                 const int m0 = m_tile * BM;
-                for (int kb = 0; kb < k_blocks; ++kb, ++it) {
+                for (int kb = kb0; kb < k_blocks; ++kb, ++it) {
                     const uint32_t full = full0 + 8u * (uint32_t)s;
                     uint32_t a_dst = dst, b_dst = dst + P.ia_bytes, a_bar = full, b_bar = full;
                     if (PACKED) {
@@ -517,7 +524,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                         if (!P.b_direct) { b_dst = p_dst + P.pa_bytes; b_bar = p_full; }
                         if (++sp == P.ns_p) { sp = 0; php ^= 1u; }
                     }
-                    if (it >= loaded && (!PACKED || direct_bytes)) {
+                    if (!PACKED || direct_bytes) {
                         VT_STAMP(tr, TT_WAIT_EMPTY);
                         if (!mbar_wait_warp(empty0 + 8u * (uint32_t)s, ph, abort_ptr)) { ok = false; break; }
                         VT_STAMP(tr, TT_GOT_EMPTY);
@@ -526,11 +533,12 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
                     __syncwarp();
                     if (ptx::elect_one()) {
                         ptx::tma_load_4d(a_dst, &map_a, a_bar, kb * a_step, m0, 0, 0);
-                        if (it >= loaded && (!resident || tile == (int)blockIdx.x)) load_weights(b_dst, b_bar, kb * b_step, col_t);
+                        if (!resident || tile == (int)blockIdx.x) load_weights(b_dst, b_bar, kb * b_step, col_t);
                     }
                     __syncwarp();
                     if (++s == ns) { s = 0; ph ^= 1u; dst = smem_base; } else dst += stage_bytes;
                 }
+                kb0 = 0;
             }
             if (!ok) {
                 // give the copies still in flight a bounded chance to land before the CTA exits
