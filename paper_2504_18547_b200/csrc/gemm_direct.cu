@@ -456,7 +456,7 @@ gemm_direct_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_const
     // Operands, parameters and the residual may come from the previous kernel.  Where weights and parameters cannot, the producer
     // fills the ring with weights, asks for the rest of the tile's into L2, and the epilogue fetches its first parameters before
     // it waits: at small batches they come from HBM, beside the previous kernel instead of behind it (with the gains of LayerNorm
-    // and the exp table, twelve layers on one image 352 -> 326 us, a layer at batch 8 47.1 -> 45.1, 8 bits at batch 32 117.8 -> 114.8).
+    // and the exp table, twelve layers on one image 352 -> 326 us (now 321), a layer at batch 8 47.1 -> 45.1, 8 bits at batch 32 117.8 -> 114.8).
     const bool early = !PACKED && P.at_rest;
     auto dependency = [&]() {
         grid_dependency_wait();
